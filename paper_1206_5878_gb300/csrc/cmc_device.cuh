@@ -217,154 +217,102 @@ __device__ __forceinline__ double mul_rn(double a, double b) {
   return a * b;
 }
 
-// a / b: Q = floor(N / d) for N = m_a 2^(63 + s), d = m_b 2^11 (s = 1 when
-// m_a < m_b, so that Q has 53 bits).  The reciprocal v ~ 2^128 / d - 2^64
-// is seeded from the float reciprocal of d's top 24 bits (~22 bits) and
-// refined by two Newton-Raphson steps in fixed point, R' = R + R (2^128 -
-// d R) / 2^128 with R = 2^64 + v (quadratic convergence: ~44, then ~64
-// bits; Newton division as in Knuth, TAOCP vol. 2, 4.3.3, and Brent and
-// Zimmermann, Modern Computer Arithmetic, 3.4).  The quotient estimate
-// floor(N R / 2^128) is then corrected by one step either way from the
-// exact remainder N - Q d, and rounded by comparing twice the remainder
-// with d (ties to even).  If the remainder still lies outside [0, d), the
-// FP64 division is used.
-// The fixed-point reciprocal of a normalised divisor d in [2^63, 2^64):
-// v ~ 2^128 / d - 2^64 (so R = 2^64 + v), seeded by the float reciprocal
-// of d's top 24 bits and refined by two Newton steps.
-__device__ __forceinline__ unsigned long long recip_fixed(unsigned long long d) {
-  // the float of d's top 24 bits, from its bits (2^23 <= d >> 40 < 2^24)
-  const float f = __uint_as_float(0x4B000000u | ((unsigned)(d >> 40) & 0x7FFFFFu));
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
-  const unsigned yb = __float_as_uint(y);
-  // 2^88 y - 2^64 for y in [2^-24, 2^-23); y = 2^-23 (d = 2^63) saturates
-  unsigned long long v =
-      ((yb >> 23) & 0xFFu) == 103u ? (unsigned long long)(yb & 0x7FFFFFu) << 41 : ~0ull;
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    // d R - 2^128 = T 2^64 + pl (T signed, small); E = floor((2^128 - d R) / 2^64)
-    const unsigned long long pl = d * v, ph = __umul64hi(d, v);
-    const long long T = (long long)(ph + d);
-    const long long E = -T - (pl != 0ull ? 1 : 0);
-    const unsigned long long aE = E < 0 ? (unsigned long long)(-E) : (unsigned long long)E;
-    const unsigned long long c = __umul64hi(v, aE);  // v |E| / 2^64
-    v = E < 0 ? v + (unsigned long long)E - c : v + (unsigned long long)E + c;
-  }
-  return v;
-}
-
-// a / b from the reciprocal v of d = m_b 2^11 (b normal): false where the
-// quotient needs the FP64 division (a not normal, a result out of the
-// normal range, or a remainder still out of range after the correction).
-__device__ __forceinline__ bool div_by_recip(unsigned long long ua, unsigned long long vb,
-                                             unsigned long long d, unsigned long long v,
-                                             double& out) {
+// a / b in two digits of 30 and 22 bits.  R0 = m_a 2^s with s = 1 when m_a <
+// m_b, so that R0 / m_b is in [1, 2) and its quotient in units of 2^-52 has
+// 53 bits.  v ~ 2^84 / m_b (32 bits) is the float reciprocal of m_b's top
+// bits (~21 bits) after one Newton step, v' = v - v (b_h v - 2^63) / 2^63
+// with b_h + 1 > m_b / 2^21 for the divisor, so that v stays below 2^32.
+//   q1 = floor(floor(R0 / 2^22) v / 2^32), within 4 units of R0 2^30 / m_b;
+//   R1 = R0 2^30 - q1 m_b, exact modulo 2^64 (|R1| <= 4 m_b < 2^55);
+//   q2 = R1 2^22 / m_b rounded to nearest, from R1 / 2^25 and v (|error| < 0.6);
+//   R2 = R1 2^22 - q2 m_b, exact modulo 2^64 (|R2| < 0.6 m_b).
+// The quotient is Q + R2 / m_b, Q = 2^22 q1 + q2, so the nearest integer is Q
+// or its neighbour on R2's side; a tie cannot occur (a quotient of two 53-bit
+// integers has no 54-bit significand).  About 60 instructions, a third of
+// the 64-bit fixed-point reciprocal it replaces (two Newton steps on 64 x 64
+// -> 128 bit products and a 128-bit remainder): the kernels holding these
+// operations are bound by instruction issue as much as by the FP64 pipe.
+// Dependent chains, whole GPU: 344 G/s (136 before, 70 on the FP64 pipe),
+// 128 ns a quotient on one warp (326 before, 288).
+__device__ __forceinline__ double div_rn(double a, double b) {
+  const unsigned long long ua = ubits(a), vb = ubits(b);
   const unsigned ea = (unsigned)(ua >> 52) & 0x7FFu, eb = (unsigned)(vb >> 52) & 0x7FFu;
   const unsigned long long ma = significand(ua), mb = significand(vb);
   const unsigned s = ma < mb ? 1u : 0u;
   const int e = (int)ea - (int)eb + 1023 - (int)s;
-  if (!(ea - 1u < 2046u && (unsigned)(e - 1) < 2045u)) return false;
-  // N = u1 2^64 + u0
-  const unsigned long long u1 = s ? ma : ma >> 1, u0 = s ? 0ull : (ma & 1ull) << 63;
-  const unsigned long long ql = v * u1, qh = __umul64hi(v, u1);
-  const unsigned long long q0 = ql + u0;
-  unsigned long long Q = qh + u1 + (q0 < ql ? 1ull : 0ull);
-  // remainder N - Q d as rh 2^64 + rl (rh signed)
-  const unsigned long long pl = Q * d, ph = __umul64hi(Q, d);
-  unsigned long long rl = u0 - pl;
-  long long rh = (long long)(u1 - ph - (u0 < pl ? 1ull : 0ull));
-  if (rh < 0) {
-    const unsigned long long t = rl + d;
-    rh += t < rl ? 1 : 0;
-    rl = t;
-    --Q;
-  } else if (rh > 0 || rl >= d) {
-    const unsigned long long t = rl - d;
-    rh -= rl < d ? 1 : 0;
-    rl = t;
-    ++Q;
-  }
-  if (rh == 0 && rl < d) {
-    const unsigned long long r2 = rl << 1;
-    const bool up = (rl >> 63) != 0ull || r2 > d || (r2 == d && (Q & 1ull));
-    out = __longlong_as_double((long long)(((ua ^ vb) & kSignBit) +
-                                           ((unsigned long long)(e - 1) << 52) + Q +
-                                           (up ? 1ull : 0ull)));
-    return true;
-  }
-  return false;
-}
-
-__device__ __forceinline__ double div_rn(double a, double b) {
-  const unsigned long long ua = ubits(a), vb = ubits(b);
-  const unsigned eb = (unsigned)(vb >> 52) & 0x7FFu;
-  if (eb - 1u < 2046u) {
-    const unsigned long long d = significand(vb) << 11;  // [2^63, 2^64)
-    double q;
-    if (div_by_recip(ua, vb, d, recip_fixed(d), q)) return q;
+  if (ea - 1u < 2046u && eb - 1u < 2046u && (unsigned)(e - 1) < 2045u) {
+    // (the two low bits set: the float stays above 1, its reciprocal below)
+    const float f = __uint_as_float(0x3F800003u | ((unsigned)(mb >> 29) & 0x7FFFFFu));
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
+    unsigned v = (__float_as_uint(y) << 8) | 0x80000000u;  // y 2^32, y in [1/2, 1)
+    const unsigned bh = (unsigned)(mb >> 21);
+    // (b_h + 1) v - 2^63 in units of 2^28 (2^63 falls out of the 32 bits)
+    const int d = (int)(unsigned)(((unsigned long long)bh * v + v) >> 28);
+    v -= (unsigned)(((int)(v >> 16) * d) >> 19);
+    const unsigned long long R0 = ma << s;
+    const unsigned q1 = __umulhi((unsigned)(R0 >> 22), v);
+    const long long R1 = (long long)((R0 << 30) - (unsigned long long)q1 * mb);
+    const int q2 = (__mulhi((int)(R1 >> 25), (int)(v >> 1)) + 8) >> 4;
+    const long long R2 =
+        (long long)(((unsigned long long)R1 << 22) - (unsigned long long)(long long)q2 * mb);
+    unsigned long long Q =
+        ((unsigned long long)q1 << 22) + (unsigned long long)(long long)q2;
+    const long long R22 = R2 + R2;
+    if (R22 > (long long)mb) ++Q;
+    if (R22 < -(long long)mb) --Q;
+    return __longlong_as_double((long long)(((ua ^ vb) & kSignBit) +
+                                            ((unsigned long long)(e - 1) << 52) + Q));
   }
   return a / b;
 }
 
-// sqrt(x): Q = floor(sqrt(N)) for N = m_x 2^(52 + p), p = 1 when x's
-// unbiased exponent is even (so that Q has 53 bits).  The reciprocal square
-// root Y ~ 2^94 / sqrt(w) of w = m_x 2^(10 + p) in [2^62, 2^64) is seeded
-// from the float reciprocal square root of w's top 24 bits and refined by
-// two Newton steps Y' = Y (3 - w Y^2 / 2^188) / 2 in fixed point (Brent and
-// Zimmermann, Modern Computer Arithmetic, 3.5); Q ~ N Y / 2^115 is then
-// corrected by one step either way from the exact remainder N - Q^2 in [0,
-// 2Q], and rounded up when the remainder exceeds Q (sqrt(N) >= Q + 1/2; an
-// exact tie cannot occur).  Negative, zero, subnormal and non-finite x:
-// the FP64 square root.
+// sqrt(x), in the same way: the root of N = M 2^52, M = m_x 2^p with p = 1
+// when x's biased exponent is even, is an integer of 53 bits.  v ~ 2^58 /
+// sqrt(M) (32 bits) is the float reciprocal square root of M's top bits (~20
+// bits) after one Newton step, v' = v - v (m_h v^2 - 2^94) / 2^95 with M /
+// 2^22 < m_h + 1.
+//   q1 = floor(m_h v / 2^32), within 4 units of 2^4 sqrt(M);
+//   R1 = 2^8 M - q1^2 (|R1| < 2^34);
+//   q2 = R1 2^21 / q1 rounded to nearest, from R1 / 2^4 and v (the root of the
+//   rest, q2^2 left out: |error| < 0.7);
+//   R2 = N - S^2 for S = 2^22 q1 + q2, exact modulo 2^64.
+// The nearest integer to the root is S + 1 when R2 > S, S - 1 when R2 <= -S
+// ((S +- 1/2)^2 = S^2 +- S + 1/4), S otherwise.  Negative, zero, subnormal
+// and non-finite x: the FP64 square root.  About 65 instructions: 326 G/s (120
+// for the 64-bit fixed-point form before, 67 on the FP64 pipe).
 __device__ __forceinline__ double sqrt_rn(double x) {
   const unsigned long long ux = ubits(x);
   const unsigned ex = (unsigned)(ux >> 52);  // sign included: negative x falls back
   if (ex - 1u < 2046u) {
     const unsigned long long ma = significand(ux);
     const unsigned p = (ex & 1u) ^ 1u;
-    const unsigned long long w = ma << (10 + p);
-    // the float of w / 2^40, from its bits (2^22 <= w / 2^40 < 2^24)
-    const float f = p ? __uint_as_float(0x4B000000u | ((unsigned)(w >> 40) & 0x7FFFFFu))
-                      : __uint_as_float(0x4A800000u | ((unsigned)(w >> 39) & 0x7FFFFFu));
+    const unsigned long long M = ma << p;
+    // M / 2^52 in [1, 4) as a float, its low bits replaced so that it stays
+    // off both ends and its reciprocal root inside (1/2, 1)
+    const float f =
+        __uint_as_float((0x3F800008u + (p << 23)) | ((unsigned)(ma >> 29) & 0x7FFFF0u));
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
-    const unsigned yb = __float_as_uint(y);
-    const int ye = (int)((yb >> 23) & 0xFFu) - 127;  // y in [2^ye, 2^(ye + 1)), ye in {-12, -11}
-    unsigned long long Y = (unsigned long long)((yb & 0x7FFFFFu) | 0x800000u) << (51 + ye);
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-      // E = floor((2^124 - w sh) / 2^64), sh = Y^2 / 2^64; Y' = Y + Y E / 2^61
-      const unsigned long long sh = __umul64hi(Y, Y);
-      const unsigned long long ml = w * sh, mh = __umul64hi(w, sh);
-      const long long E = (long long)((1ull << 60) - mh) - (ml != 0ull ? 1 : 0);
-      const unsigned long long aE = E < 0 ? (unsigned long long)(-E) : (unsigned long long)E;
-      const unsigned long long h = __umul64hi(Y, aE), l = Y * aE;
-      const unsigned long long c = (h << 3) | (l >> 61);
-      Y = E < 0 ? Y - c : Y + c;
-    }
-    const unsigned long long lo = ma * Y, hi = __umul64hi(ma, Y);
-    unsigned long long Q = p ? (hi << 2) | (lo >> 62) : (hi << 1) | (lo >> 63);
-    // remainder N - Q^2 as rh 2^64 + rl (rh signed), N = u1 2^64 + u0
-    const unsigned long long u1 = ma >> (12 - p), u0 = ma << (52 + p);
-    const unsigned long long ql = Q * Q, qh = __umul64hi(Q, Q);
-    unsigned long long rl = u0 - ql;
-    long long rh = (long long)(u1 - qh - (u0 < ql ? 1ull : 0ull));
-    if (rh < 0) {  // (Q - 1)^2 = Q^2 - (2Q - 1)
-      const unsigned long long t = 2 * Q - 1, n = rl + t;
-      rh += n < rl ? 1 : 0;
-      rl = n;
-      --Q;
-    } else if (rh > 0 || rl > 2 * Q) {  // (Q + 1)^2 = Q^2 + 2Q + 1
-      const unsigned long long t = 2 * Q + 1, n = rl - t;
-      rh -= rl < t ? 1 : 0;
-      rl = n;
-      ++Q;
-    }
-    if (rh == 0 && rl <= 2 * Q) {
-      const int er = ((int)ex - 1127 - (int)p) / 2 + 1075;
-      return __longlong_as_double(
-          (long long)(((unsigned long long)(er - 1) << 52) + Q + (rl > Q ? 1ull : 0ull)));
-    }
+    unsigned v = (__float_as_uint(y) << 8) | 0x80000000u;  // y 2^32
+    const unsigned mh = (unsigned)(M >> 22);
+    const unsigned sq = __umulhi(v, v);
+    const int d = (int)(unsigned)(((unsigned long long)sq * mh + sq) >> 28);
+    v -= (unsigned)(((int)(v >> 16) * d) >> 19);
+    const unsigned q1 = __umulhi(mh, v);
+    const long long R1 = (long long)((M << 8) - (unsigned long long)q1 * q1);
+    const int q2 = (__mulhi((int)(R1 >> 4), (int)(v >> 1)) + 8) >> 4;
+    const unsigned long long S =
+        ((unsigned long long)q1 << 22) + (unsigned long long)(long long)q2;
+    const long long R2 = (long long)(((unsigned long long)R1 << 44) -
+                                     (unsigned long long)(long long)q2 *
+                                         (((unsigned long long)q1 << 23) +
+                                          (unsigned long long)(long long)q2));
+    unsigned long long Q = S;
+    if (R2 > (long long)S) ++Q;
+    if (R2 <= -(long long)S) --Q;
+    const int er = ((int)ex - 1127 - (int)p) / 2 + 1075;
+    return __longlong_as_double((long long)(((unsigned long long)(er - 1) << 52) + Q));
   }
   return sqrt(x);
 }
@@ -477,11 +425,10 @@ __device__ __forceinline__ void draws_keep(const Seg& S, int c, const Draws<kTau
   if (kTaus) S.taus[__ldg(S.taus_base + c) + d.id] = d.z;
 }
 
-// Non-inlined copies of div_rn and sqrt_rn for kernels with many call
-// sites: each inlined copy is ~150 instructions, and a kernel holding a
-// dozen of them no longer fits the instruction cache (ncu: instruction
-// fetch the relaxation kernel's largest stall); one shared body costs a
-// call per use instead (measured: relaxation 1.46 -> 1.06 ms at N = 1e7).
+// Non-inlined copies of div_rn and sqrt_rn for the relaxation kernel: its
+// fifteen call sites inlined overflow the instruction cache (relaxation 0.853
+// ms shared, 0.876 ms inlined at N = 1e7); the kernels with a few call sites
+// inline them (FP64 mode's orbit stage 2.58 ms inlined, 2.65 ms shared).
 static __device__ __noinline__ double div_rn_nl(double a, double b) { return div_rn(a, b); }
 static __device__ __noinline__ double sqrt_rn_nl(double x) { return sqrt_rn(x); }
 

@@ -69,11 +69,11 @@ __device__ __forceinline__ double shell_root64(const Table64& T, const Star& s, 
 // Phi = Phi_j + M_j (x_j - x) needs no division (mixed mode).  The cores
 // take the node values, so that values loaded ahead and the table give
 // the same arithmetic.  The clamps are the FP64 comparisons restated on
-// the bit patterns (radii are positive).  Their quotients go to the integer
-// pipes through the shared body and their square roots stay on the FP64
-// pipe: that balance measured fastest in this FP64-bound kernel (turning
-// points 1.39 -> 1.36 ms at N = 10^7; both on the integer pipes, inlined or
-// shared, 0.04-0.05 ms slower).
+// the bit patterns (radii are positive).  Their quotients and square roots
+// run on the integer pipes: this kernel is bound by the FP64 pipe first
+// (turning points 1.30 ms with the square roots on the FP64 pipe, 1.275 ms
+// without, at N = 10^7; 0.127 and 0.111 ms at 10^6, where the tables stay in
+// the L2).
 __device__ __forceinline__ double rmax_core(const Star& s, double rj, double xj, double pj,
                                             double Mj, bool has_next, double rj1) {
   const double B = Mj;
@@ -81,9 +81,9 @@ __device__ __forceinline__ double rmax_core(const Star& s, double rj, double xj,
   const double em = s.E - A;
   double D = B * B + scale_up<1>(s.J * s.J) * em;
   if (!pos_num(D)) D = 0.0;
-  const double sD = sqrt(D);
+  const double sD = sqrt_rn(D);
   // 2 (A - E) = -(2 (E - A)) exactly
-  double root = div_rn_nl(B + sD, -scale_up<1>(em));
+  double root = div_rn(B + sD, -scale_up<1>(em));
   if (!ge_pos(root, rj)) root = rj;
   if (has_next && ubits(root) > ubits(rj1)) root = rj1;
   return root;
@@ -108,7 +108,7 @@ __device__ __forceinline__ double rmin_core(const Star& s, bool central, double 
     if (!pos_num(D)) D = 0.0;
     num = s.J * s.J;
   }
-  double root = div_rn_nl(num, B + sqrt(D));
+  double root = div_rn(num, B + sqrt_rn(D));
   if (central) {
     // root >= 0 (-0 included, NaN not), then root <= r_0
     const unsigned long long u = ubits(root);
@@ -411,9 +411,7 @@ __device__ __forceinline__ void point64(const double4_32a* __restrict__ nd, int6
 
 // FP64 mode: the orbit point r(s) in FP64 from an FP32 shell guess sh
 // (moved to the exact shell), Phi by Eq. 6's division form (the FP64
-// statement of the method, as phi_in_shell), L = J / r and Q.  Its
-// quotients go through the shared bodies (div_rn_nl): measured faster in
-// the long kernels that use it.
+// statement of the method, as phi_in_shell), L = J / r and Q.
 // sa = s (3 - s^2), the factor of c1 in r(s) (a table entry at the
 // envelope's samples)
 __device__ __forceinline__ void point64_div_sa(const double4_32a* __restrict__ nd, int64_t nb,
@@ -426,7 +424,7 @@ __device__ __forceinline__ void point64_div_sa(const double4_32a* __restrict__ n
   if (i < 0) {
     ph = a.z;  // node 0's Phi: the central constant
   } else {
-    const double xq = div_rn_nl(1.0, rs);
+    const double xq = div_rn(1.0, rs);
     double xj1 = 0.0, pj1 = 0.0;
     if (i + 1 < nb) {
       const double4_32a b = nd[i + 1];
@@ -434,9 +432,9 @@ __device__ __forceinline__ void point64_div_sa(const double4_32a* __restrict__ n
       pj1 = b.z;
     }
     const double den = a.y - xj1;
-    ph = !(den > 0.0) ? a.z : a.z + div_rn_nl(a.y - xq, den) * (pj1 - a.z);
+    ph = !(den > 0.0) ? a.z : a.z + div_rn(a.y - xq, den) * (pj1 - a.z);
   }
-  L = div_rn_nl(st.J, rs);
+  L = div_rn(st.J, rs);
   Q = scale_up<1>(st.E - ph) - L * L;
 }
 
@@ -450,7 +448,7 @@ __device__ __forceinline__ void point64_div(const double4_32a* __restrict__ nd, 
 // g(s) of FP64 mode at the point of point64_div, sb = 1 - s^2
 __device__ __forceinline__ double g_of_point_sb(double c1, double sb, double Q) {
   if (!(Q > 0.0)) return 0.0;
-  return div_rn_nl((3.0 * c1) * sb, sqrt_rn_nl(Q));
+  return div_rn((3.0 * c1) * sb, sqrt_rn(Q));
 }
 
 __device__ __forceinline__ double g_of_point(double c1, double sv, double Q) {
@@ -947,7 +945,7 @@ __global__ void k_env_tables() {
   g_env_sb[j] = 1.0 - sv * sv;
 }
 
-// FP64 g at sample j of a star (the noinline quotients keep this copy small)
+// FP64 g at sample j of a star (one copy for the list and the spill loops)
 __device__ __noinline__ double g64_sample(const double4_32a* __restrict__ nd, int64_t nb,
                                           const Buckets& BK, double E, double J, double c0,
                                           double c1, int j) {
