@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cstddef>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -13,6 +14,25 @@
 #include "cmc_device.cuh"
 
 namespace cmc {
+
+// Launch a kernel that calls pdl_enter: it may be set up while its
+// predecessor in the stream still runs (in a captured graph the edge becomes
+// a programmatic one).  An error is left for cudaGetLastError.
+template <class... P, class... A>
+inline void launch_k(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+                            cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // Device-resident description of the segments of one state.  Offsets are
 // fixed at initialisation; nb, dt and the statistics change every step.

@@ -18,6 +18,7 @@ namespace {
 __global__ void __launch_bounds__(256) k_bins(Seg S, int bs, double pref, const double* r,
                                               const double* vr, const double* vt,
                                               const double* m, double* nbin) {
+  pdl_enter();
   __shared__ unsigned long long s_min[8];
   __shared__ int s_seg0;
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr,
                                                double* m, const uint32_t* id,
                                                const double* nbin, const uint32_t* step_p,
                                                Collide col) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= S.pair_off[S.n_seg]) return;
   const int c = seg_find(S.pair_off, S.n_seg, p);
@@ -229,6 +231,7 @@ __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr,
 // P: [4 components][32 bits b][32 columns], a column = the image of one bit.
 __global__ void k_taus_init(int64_t slots, int n_seg, const int64_t* base, const uint4* words,
                             const uint32_t* P, uint4* table) {
+  pdl_enter();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= slots) return;
   const int c = seg_find(base, n_seg, e);
@@ -262,6 +265,7 @@ __global__ void k_taus_init(int64_t slots, int n_seg, const int64_t* base, const
 __global__ void k_tcentral(Seg S, const double* r, const double* vr, const double* vt,
                            const double* m, const double* R, const double* A, double x_bb,
                            double x_bs) {
+  pdl_enter();
   const int c = blockIdx.x;
   if (threadIdx.x != 0 || c >= S.n_seg) return;
   const int64_t nb = S.nb[c], sb = S.off[c];
@@ -334,7 +338,7 @@ __global__ void k_tcentral(Seg S, const double* r, const double* vr, const doubl
 void launch_taus_init(int64_t slots, int n_seg, const int64_t* base, const uint4* words,
                       const uint32_t* P, uint4* table, cudaStream_t st) {
   if (slots > 0)
-    k_taus_init<<<(unsigned)((slots + 255) / 256), 256, 0, st>>>(slots, n_seg, base, words, P,
+    launch_k(k_taus_init, (unsigned)((slots + 255) / 256), 256, 0, st, slots, n_seg, base, words, P,
                                                                  table);
 }
 
@@ -342,13 +346,13 @@ void launch_tcentral(const SegLayout& L, const double* r, const double* vr, cons
                      const double* m, const double* R, const double* A, double x_bb,
                      double x_bs, cudaStream_t st) {
   if (!L.n || (!R && !A)) return;
-  k_tcentral<<<(unsigned)L.n_seg, 32, 0, st>>>(L.dev(), r, vr, vt, m, R, A, x_bb, x_bs);
+  launch_k(k_tcentral, (unsigned)L.n_seg, 32, 0, st, L.dev(), r, vr, vt, m, R, A, x_bb, x_bs);
 }
 
 void launch_bins(const SegLayout& L, const double* r, const double* vr, const double* vt,
                  const double* m, double* nbin, double pref, cudaStream_t st) {
   if (!L.n_bins) return;
-  k_bins<<<(unsigned)((L.n_bins + 255) / 256), 256, 0, st>>>(L.dev(), L.bin_size, pref, r, vr,
+  launch_k(k_bins, (unsigned)((L.n_bins + 255) / 256), 256, 0, st, L.dev(), L.bin_size, pref, r, vr,
                                                              vt, m, nbin);
 }
 
@@ -360,16 +364,16 @@ static void relax_shape(const SegLayout& L, double* vr, double* vt, double* m,
   // (the collision code only in the kernels that need it: it costs
   // registers)
   if (L.taus && col.R)
-    k_relax<true, kMinB, true><<<grid, 128, 0, st>>>(L.dev(), L.bin_size, vr, vt, m, id, nbin,
+    launch_k(k_relax<true, kMinB, true>, grid, 128, 0, st, L.dev(), L.bin_size, vr, vt, m, id, nbin,
                                                      step, col);
   else if (L.taus)
-    k_relax<true, kMinB, false><<<grid, 128, 0, st>>>(L.dev(), L.bin_size, vr, vt, m, id, nbin,
+    launch_k(k_relax<true, kMinB, false>, grid, 128, 0, st, L.dev(), L.bin_size, vr, vt, m, id, nbin,
                                                       step, col);
   else if (col.R)
-    k_relax<false, kMinB, true><<<grid, 128, 0, st>>>(L.dev(), L.bin_size, vr, vt, m, id, nbin,
+    launch_k(k_relax<false, kMinB, true>, grid, 128, 0, st, L.dev(), L.bin_size, vr, vt, m, id, nbin,
                                                       step, col);
   else
-    k_relax<false, kMinB, false><<<grid, 128, 0, st>>>(L.dev(), L.bin_size, vr, vt, m, id,
+    launch_k(k_relax<false, kMinB, false>, grid, 128, 0, st, L.dev(), L.bin_size, vr, vt, m, id,
                                                        nbin, step, col);
 }
 

@@ -775,6 +775,7 @@ __global__ void __launch_bounds__(256, kMinB) k_turning_mixed(
     Seg S, const double* r, const double* x, const double* phi,
     const double* Menc, const double* vr, const double* vt, BucketArgs BA, double* tp_min,
     double* tp_max, double4_32a* orb, int64_t n) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const int c = seg_find(S.off, S.n_seg, p);
@@ -938,6 +939,7 @@ constexpr uint64_t kEnvNone = ~0ull;  // a list slot left empty
 __device__ double g_env_sa[21], g_env_sb[21];
 
 __global__ void k_env_tables() {
+  pdl_enter();
   const int j = threadIdx.x;
   if (j >= 21) return;
   const double sv = c_s64[j];
@@ -991,6 +993,7 @@ __device__ __forceinline__ bool env_star(const Seg& S, const double4_32a* orb, i
 __global__ void __launch_bounds__(kEnvThreads) k_env_screen(Seg S, BucketArgs BA,
                                                             const double4_32a* orb, EnvWork W,
                                                             int64_t n) {
+  pdl_enter();
   __shared__ float s_hi[21][kEnvThreads];  // upper bounds of the samples
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
@@ -1080,6 +1083,7 @@ __device__ __forceinline__ void env_pair(const Seg& S, const BucketArgs& BA, con
 }
 
 __global__ void __launch_bounds__(kEnvThreads) k_env_eval(Seg S, BucketArgs BA, EnvWork W) {
+  pdl_enter();
   const unsigned long long cap = (unsigned long long)W.cap;
   const unsigned long long np = W.cnt[0] < cap ? W.cnt[0] : cap;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
@@ -1152,6 +1156,7 @@ __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
                                                   const double4_32a* orb,
                                                   uint64_t* keys, uint32_t* plist,
                                                   uint32_t* pcount, int64_t n, const double* Fx) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long viol = 0;
   bool pend = false;
@@ -1304,6 +1309,7 @@ __global__ void __launch_bounds__(128) k_pending64(Seg S, int max_trials, const 
                                                    const uint32_t* plist,
                                                    const uint32_t* pcount, int64_t n,
                                                    const double* Fx) {
+  pdl_enter();
   const uint32_t np = *pcount;
   for (uint32_t i0 = blockIdx.x * blockDim.x; i0 < np; i0 += gridDim.x * blockDim.x) {
     pending_star<kTaus, kExact>(S, max_trials, id, step_p, BA, orb, keys,
@@ -1344,6 +1350,7 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
                                                int64_t n, const double* Rv, double* Rp,
                                                const double* Fx, const double* Av,
                                                double* Ap, bool packed) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const int c = seg_find(S.off, S.n_seg, p);
@@ -1570,6 +1577,7 @@ __global__ void __launch_bounds__(128, 12) k_correction_mixed(Seg S, const int64
                                                           double* vr, double* vt,
                                                           const double* r_old, const double* cc,
                                                           const double* m, int64_t n) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const int c = seg_find(S.off, S.n_seg, p);
@@ -1640,6 +1648,7 @@ int64_t grid_capacity(int64_t nc) {
 __global__ void k_grid_params(Seg S, const int64_t* esc, bool sub, const double* x,
                               const double* phi, const double* Menc, const int64_t* goff,
                               int4* gprm, float4* gaux) {
+  pdl_enter();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= S.n_seg) return;
   int64_t nb = S.nb[c];
@@ -1662,6 +1671,7 @@ __global__ void k_grid_params(Seg S, const int64_t* esc, bool sub, const double*
 // written by the stars (grid_shells_of) in one pass over stars and cells.
 __global__ void k_grid_shells(Seg S, const int64_t* esc, bool sub, const double* x,
                               BucketArgs B, int* gshell, int64_t n) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const int c = seg_find(S.off, S.n_seg, p);
@@ -1684,6 +1694,7 @@ __global__ void k_grid_build(Seg S, const int64_t* esc, bool sub, const double* 
                              const double* phi, double* Menc, BucketArgs B,
                              const int* gshell, float* gphi, float4* gaux, int64_t total,
                              bool fused, const double* r, double4_32a* node, int64_t n_tiles) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned am = __ballot_sync(0xFFFFFFFFu, p < total);
   if (p >= total) {
@@ -1751,6 +1762,7 @@ __global__ void k_grid_build(Seg S, const int64_t* esc, bool sub, const double* 
 __global__ void k_table_params(Seg S, const int64_t* esc, bool sub, const double* x,
                                const int64_t* boff, uint32_t* base, int4* prm,
                                const int64_t* goff, int4* gprm, float4* gaux) {
+  pdl_enter();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= S.n_seg) return;
   int64_t nb = S.nb[c];
@@ -1792,6 +1804,7 @@ __global__ void k_table_params(Seg S, const int64_t* esc, bool sub, const double
 // the bucket count
 __global__ void k_bucket_params(Seg S, const int64_t* esc, bool sub, const float2* t32,
                                 BucketArgs B, uint32_t* base, int4* prm) {
+  pdl_enter();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= S.n_seg) return;
   int64_t nb = S.nb[c];
@@ -1814,6 +1827,7 @@ __global__ void k_bucket_params(Seg S, const int64_t* esc, bool sub, const float
 // its predecessor's bucket and its own; the last one closes the table
 __global__ void k_bucket_build(Seg S, const int64_t* esc, bool sub, const float2* t32,
                                BucketArgs B, int* start, int64_t n) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const int c = seg_find(S.off, S.n_seg, p);
@@ -1831,6 +1845,7 @@ __global__ void k_bucket_build(Seg S, const int64_t* esc, bool sub, const float2
 // have the potential but not the masses: (Phi_{k+1} - Phi_k)/(x_k - x_{k+1}),
 // with Phi = 0 at 1/r = 0 beyond the last node
 __global__ void k_slopes(int64_t n, const double* x, const double* phi, double* M) {
+  pdl_enter();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const double xj = x[k], pj = phi[k];
@@ -1842,7 +1857,7 @@ __global__ void k_slopes(int64_t n, const double* x, const double* phi, double* 
 
 void launch_slopes(int64_t n, const double* x, const double* phi, double* Menc,
                    cudaStream_t st) {
-  if (n > 0) k_slopes<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, x, phi, Menc);
+  if (n > 0) launch_k(k_slopes, (unsigned)((n + 255) / 256), 256, 0, st, n, x, phi, Menc);
 }
 
 cudaError_t alloc_buckets(BucketWork& B, const SegLayout& L, cudaStream_t st) {
@@ -1885,11 +1900,11 @@ void free_buckets(BucketWork& B, cudaStream_t st) {
 void launch_grid(const SegLayout& L, const double* x, const double* phi, const double* Menc,
                  bool nb_sub, BucketWork& B, cudaStream_t st) {
   if (!L.n || !B.gcells) return;
-  k_grid_params<<<(unsigned)((L.n_seg + 127) / 128), 128, 0, st>>>(
+  launch_k(k_grid_params, (unsigned)((L.n_seg + 127) / 128), 128, 0, st,
       L.dev(), L.esc_step, nb_sub, x, phi, Menc, B.goff, B.gprm, B.gaux);
-  k_grid_shells<<<(unsigned)((L.n + 255) / 256), 256, 0, st>>>(L.dev(), L.esc_step, nb_sub, x,
+  launch_k(k_grid_shells, (unsigned)((L.n + 255) / 256), 256, 0, st, L.dev(), L.esc_step, nb_sub, x,
                                                               B.args(), B.gshell, L.n);
-  k_grid_build<<<(unsigned)((B.gcells + 255) / 256), 256, 0, st>>>(
+  launch_k(k_grid_build, (unsigned)((B.gcells + 255) / 256), 256, 0, st,
       L.dev(), L.esc_step, nb_sub, x, phi, const_cast<double*>(Menc), B.args(), B.gshell,
       B.gphi, B.gaux, B.gcells, false, nullptr, nullptr, 0);
 }
@@ -1899,7 +1914,7 @@ void launch_potential_tables(const SegLayout& L, const double* r, const double* 
                              float2* t32, double* Menc, bool nb_sub, bool sums_ready,
                              BucketWork& B, cudaStream_t st) {
   if (!L.n) return;
-  k_table_params<<<(unsigned)((L.n_seg + 127) / 128), 128, 0, st>>>(
+  launch_k(k_table_params, (unsigned)((L.n_seg + 127) / 128), 128, 0, st,
       L.dev(), L.esc_step, nb_sub, x, B.off, B.base, B.prm, B.goff, B.gprm, B.gaux);
   TableOut T;
   T.start = B.start;
@@ -1912,7 +1927,7 @@ void launch_potential_tables(const SegLayout& L, const double* r, const double* 
   launch_potential(L, r, x, m, tile_m, tile_mx, phi, t32, Menc, nb_sub, st, B.node, B.tdf,
                    sums_ready, true, &T);
   const int64_t threads = B.gcells + L.n_tiles;
-  k_grid_build<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(
+  launch_k(k_grid_build, (unsigned)((threads + 255) / 256), 256, 0, st,
       L.dev(), L.esc_step, nb_sub, x, phi, Menc, B.args(), B.gshell, B.gphi, B.gaux, B.gcells,
       true, r, B.node, L.n_tiles);
 }
@@ -1920,9 +1935,9 @@ void launch_potential_tables(const SegLayout& L, const double* r, const double* 
 void launch_buckets(const SegLayout& L, const float2* t32, bool nb_sub, BucketWork& B,
                     cudaStream_t st) {
   if (!L.n) return;
-  k_bucket_params<<<(unsigned)((L.n_seg + 127) / 128), 128, 0, st>>>(
+  launch_k(k_bucket_params, (unsigned)((L.n_seg + 127) / 128), 128, 0, st,
       L.dev(), L.esc_step, nb_sub, t32, B.args(), B.base, B.prm);
-  k_bucket_build<<<(unsigned)((L.n + 255) / 256), 256, 0, st>>>(L.dev(), L.esc_step, nb_sub,
+  launch_k(k_bucket_build, (unsigned)((L.n + 255) / 256), 256, 0, st, L.dev(), L.esc_step, nb_sub,
                                                                t32, B.args(), B.start, L.n);
 }
 
@@ -1935,7 +1950,7 @@ cudaError_t alloc_env(EnvWork& W, int64_t n, cudaStream_t st) {
   if (!e) e = cudaMallocAsync((void**)&W.spill, sizeof(uint64_t) * m, st);
   if (!e) e = cudaMallocAsync((void**)&W.cnt, 2 * sizeof(unsigned long long), st);
   if (!e) {
-    k_env_tables<<<1, 32, 0, st>>>();
+    launch_k(k_env_tables, 1, 32, 0, st);
     e = cudaGetLastError();
   }
   return e;
@@ -1955,10 +1970,10 @@ void launch_correction_mixed(const SegLayout& L, const double* r, const double* 
                              bool div_form) {
   if (!L.n) return;
   if (div_form)
-    k_correction_mixed<true><<<(unsigned)((L.n + 127) / 128), 128, 0, st>>>(
+    launch_k(k_correction_mixed<true>, (unsigned)((L.n + 127) / 128), 128, 0, st,
         L.dev(), L.esc_step, r, x, phi, Menc, ba, vr, vt, r_old, c, m, L.n);
   else
-    k_correction_mixed<false><<<(unsigned)((L.n + 127) / 128), 128, 0, st>>>(
+    launch_k(k_correction_mixed<false>, (unsigned)((L.n + 127) / 128), 128, 0, st,
         L.dev(), L.esc_step, r, x, phi, Menc, ba, vr, vt, r_old, c, m, L.n);
 }
 
@@ -1969,7 +1984,7 @@ void launch_turning(const SegLayout& L, const double* r, const double* x, const 
   if (!L.n) return;
   if (block <= 0) block = 64;
   const unsigned grid = (unsigned)((L.n + block - 1) / block);
-  k_turning_mixed<5><<<grid, block, 0, st>>>(L.dev(), r, x, phi, Menc, vr, vt, ba, tp_min,
+  launch_k(k_turning_mixed<5>, grid, block, 0, st, L.dev(), r, x, phi, Menc, vr, vt, ba, tp_min,
                                              tp_max, orb, L.n);
 }
 
@@ -1999,10 +2014,10 @@ void launch_orbit(const SegLayout& L, int precision, int max_trials, const doubl
   // by bisection (kPrec 0)
   const bool exact = precision == 0;
 #define CMC_TURN(B)                                                                          \
-  k_turning_mixed<5><<<grid, block, 0, st>>>(L.dev(), r, x, phi, Menc, vr, vt, ba,      \
+  launch_k(k_turning_mixed<5>, grid, block, 0, st, L.dev(), r, x, phi, Menc, vr, vt, ba,      \
                                              tp_min, tp_max, orb, L.n)
 #define CMC_ORBIT(P, B, T)                                                                  \
-  k_orbit<P, B, T><<<grid, block, 0, st>>>(L.dev(), max_trials, r, x, phi, Menc, vr, vt, \
+  launch_k(k_orbit<P, B, T>, grid, block, 0, st, L.dev(), max_trials, r, x, phi, Menc, vr, vt, \
                                            m, id, step, keys, pay, L.esc_step, d, ba, tp_min, \
                                            tp_max, orb, L.n, Rv, Rp, Fx, Av, Ap, packed)
 #define CMC_SAMPLED(B, T, X)                                                                \
@@ -2010,14 +2025,14 @@ void launch_orbit(const SegLayout& L, int precision, int max_trials, const doubl
     if (with_turning) CMC_TURN(B);                                                          \
     if (X) {                                                                                \
       cudaMemsetAsync(W.cnt, 0, 2 * sizeof(unsigned long long), st);                        \
-      k_env_screen<<<(unsigned)((L.n + kEnvThreads - 1) / kEnvThreads), kEnvThreads, 0, st>>>( \
+      launch_k(k_env_screen, (unsigned)((L.n + kEnvThreads - 1) / kEnvThreads), kEnvThreads, 0, st,  \
           L.dev(), ba, orb, W, L.n);                                                         \
-      k_env_eval<<<egrid, kEnvThreads, 0, st>>>(L.dev(), ba, W);                             \
+      launch_k(k_env_eval, egrid, kEnvThreads, 0, st, L.dev(), ba, W);                             \
     }                                                                                       \
     cudaMemsetAsync(pcount, 0, sizeof(uint32_t), st);                                      \
-    k_sample32<B, T, X><<<grid, block, 0, st>>>(L.dev(), max_trials, id, step, ba, orb, keys, \
+    launch_k(k_sample32<B, T, X>, grid, block, 0, st, L.dev(), max_trials, id, step, ba, orb, keys, \
                                                 plist, pcount, L.n, Fx);                    \
-    k_pending64<T, X><<<pgrid, 128, 0, st>>>(L.dev(), max_trials, id, step, ba, orb, keys,  \
+    launch_k(k_pending64<T, X>, pgrid, 128, 0, st, L.dev(), max_trials, id, step, ba, orb, keys,  \
                                              plist, pcount, L.n, Fx);                       \
     CMC_ORBIT(X ? 2 : 1, 5, T);                                                             \
   } while (0)

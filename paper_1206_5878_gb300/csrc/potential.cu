@@ -87,6 +87,7 @@ __device__ __forceinline__ TR tile_of(const Seg& S, const int64_t* esc, int64_t 
 __global__ void k_make_keys(int64_t n, const double* r, const double* vr, const double* vt,
                             const double* m, const uint32_t* id, uint64_t* keys,
                             Payload* pay) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   double rr = r[p];
@@ -99,12 +100,14 @@ __global__ void k_make_keys(int64_t n, const double* r, const double* vr, const 
 }
 
 __global__ void k_id_keys(int64_t n, const uint32_t* id, uint64_t* keys) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n) keys[p] = (uint64_t)id[p];
 }
 
 __global__ void k_rekey_radius(int64_t n, const uint32_t* perm, const double* r,
                                const uint32_t* id, uint64_t* keys) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   uint32_t q = perm[p];
@@ -115,6 +118,7 @@ __global__ void k_gather(int64_t n, const uint64_t* __restrict__ keys,
                          const uint32_t* __restrict__ vals, const Payload* __restrict__ pay,
                          double* r, double* x, double* vr, double* vt, double* m,
                          uint32_t* id, double* r_old, double* c) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   uint64_t k = keys[p];
@@ -139,6 +143,7 @@ __global__ void __launch_bounds__(kThreads) k_gather_sums(
     double* vr, double* vt, double* m, uint32_t* id, double* r_old, double* c, double* tile_m,
     double* tile_mx, const double* Rp, double* Rout, const double* Ap, double* Aout,
     bool packed) {
+  pdl_enter();
   __shared__ double s[kThreads];
   TR R = tile_of(S, esc, blockIdx.x, true);
   double am = 0.0, ax = 0.0;
@@ -227,6 +232,7 @@ __device__ __forceinline__ float4 float_pairs(double x, double ph) {
 __global__ void __launch_bounds__(kThreads) k_tile_sums(Seg S, const int64_t* esc, bool sub,
                                                         const double* x, const double* m,
                                                         double* tile_m, double* tile_mx) {
+  pdl_enter();
   __shared__ double s[kThreads];
   TR R = tile_of(S, esc, blockIdx.x, sub);
   // all 32 loads issued before the sums, which still run in element order
@@ -401,6 +407,7 @@ __global__ void __launch_bounds__(kPotThreads) k_potential(Seg S, const int64_t*
                                                            float2* t32, double* Mout,
                                                            double4_32a* node, float4* tdf,
                                                            bool slopes, TableOut T) {
+  pdl_enter();
   extern __shared__ double smem[];
   double* s_m = smem;               // m, then M_k
   double* s_x = smem + kPad8N;      // x
@@ -521,6 +528,7 @@ __global__ void __launch_bounds__(kPotThreads) k_potential(Seg S, const int64_t*
 __global__ void k_slope_seams(Seg S, const int64_t* esc, bool sub, const double* r,
                               const double* x, const double* phi, double* M,
                               double4_32a* node, int64_t n_tiles) {
+  pdl_enter();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n_tiles) return;
   TR R = tile_of(S, esc, t, sub);
@@ -539,6 +547,7 @@ __global__ void k_correction(Seg S, const int64_t* esc, bool sub, const double* 
                              const double* x, const double* phi, double* vr, double* vt,
                              const double* r_old, const double* cc, const double* m,
                              int64_t n) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   bool active = p < n;
   int c = 0;
@@ -578,6 +587,7 @@ __global__ void __launch_bounds__(kThreads) k_energy_tiles(Seg S, const double* 
                                                            const double* tile_m,
                                                            double* tile_k, double* tile_w,
                                                            double* Mout) {
+  pdl_enter();
   __shared__ double s1[kThreads], s2[kThreads];
   TR R = tile_of(S, nullptr, blockIdx.x, false);
   const int64_t t0 = blockIdx.x - R.lt;
@@ -623,6 +633,7 @@ __global__ void __launch_bounds__(kThreads) k_energy_tiles(Seg S, const double* 
 __global__ void __launch_bounds__(kThreads) k_core_tiles(Seg S, const double* r, const double* m,
                                                          double* tile_s1, double* tile_s2,
                                                          double* tile_sr, double* tile_n) {
+  pdl_enter();
   __shared__ double s[kThreads];
   TR R = tile_of(S, nullptr, blockIdx.x, false);
   const int64_t b = R.begin + (int64_t)threadIdx.x * kPer;
@@ -658,6 +669,7 @@ __global__ void __launch_bounds__(kThreads) k_core_final(Seg S, const double* ti
                                                          const double* tile_s2,
                                                          const double* tile_sr,
                                                          const double* tile_n, double* out3) {
+  pdl_enter();
   __shared__ double s[kThreads];
   const int c = blockIdx.x;
   const int64_t t0 = S.tile_off[c], t1 = S.tile_off[c + 1];
@@ -680,6 +692,7 @@ __global__ void __launch_bounds__(kThreads) k_core_final(Seg S, const double* ti
 __global__ void __launch_bounds__(kThreads) k_energy_final(Seg S, const double* tile_k,
                                                            const double* tile_w,
                                                            double* out3) {
+  pdl_enter();
   __shared__ double s[kThreads];
   const int c = blockIdx.x;
   int64_t t0 = S.tile_off[c], t1 = S.tile_off[c + 1];
@@ -699,6 +712,7 @@ __global__ void __launch_bounds__(kThreads) k_energy_final(Seg S, const double* 
 
 __global__ void k_lagrange(Seg S, const double* r, const double* M, const double* fracs,
                            int nf, double* out) {
+  pdl_enter();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= S.n_seg * nf) return;
   int c = i / nf, q = i % nf;
@@ -715,6 +729,7 @@ __global__ void k_lagrange(Seg S, const double* r, const double* M, const double
 
 __global__ void k_validate(int64_t n, const double* r, const double* vr, const double* vt,
                            const double* m, bool allow_inf, uint32_t* err) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   double rr = r[p], a = vr[p], b = vt[p], mm = m[p];
@@ -725,6 +740,7 @@ __global__ void k_validate(int64_t n, const double* r, const double* vr, const d
 
 __global__ void k_check_ids(int64_t n, const int64_t* off, int n_seg, const uint64_t* ids,
                             uint32_t* err) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p + 1 >= n) return;
   int c = seg_find(off, n_seg, p);
@@ -736,6 +752,7 @@ __global__ void k_check_ids(int64_t n, const int64_t* off, int n_seg, const uint
 // flag bit 0 set otherwise, and the largest id of each segment.
 __global__ void k_order_check(int64_t n, const int64_t* off, int n_seg, const double* r,
                               const uint32_t* id, uint32_t* flag, unsigned int* maxid) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool live = p < n;
   int c = 0;
@@ -760,6 +777,7 @@ __global__ void k_order_check(int64_t n, const int64_t* off, int n_seg, const do
 __global__ void k_ids_bitmap(int64_t n, const int64_t* off, int n_seg, const uint32_t* id,
                              const unsigned long long* bitoff, unsigned long long* bitmap,
                              uint32_t* err) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const int c = seg_find(off, n_seg, p);
@@ -776,6 +794,7 @@ __global__ void __launch_bounds__(256) k_step_end(Seg S, int64_t* esc, uint64_t*
                                                   uint32_t* step, const double* r_old,
                                                   const double* e, const double* m,
                                                   double* esc_me) {
+  pdl_enter();
   __shared__ double s_m[256], s_e[256];
   const int c = blockIdx.x, t = threadIdx.x;
   const int64_t ne = esc[c];
@@ -821,6 +840,7 @@ __global__ void __launch_bounds__(256) k_step_end(Seg S, int64_t* esc, uint64_t*
 __global__ void k_diag_ring(Seg S, const double* out3, const uint64_t* dt_last,
                             const double* esc_me, const uint32_t* step, const uint32_t* err,
                             double* ring, int cap) {
+  pdl_enter();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= S.n_seg) return;
   const uint32_t stp = *step;
@@ -839,6 +859,7 @@ __global__ void k_diag_ring(Seg S, const double* out3, const uint64_t* dt_last,
 }
 
 __global__ void k_nb_from_keys(Seg S, const uint64_t* keys) {
+  pdl_enter();
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= S.n_seg) return;
   int64_t sb = S.off[c], se = S.off[c + 1];
@@ -851,17 +872,20 @@ __global__ void k_nb_from_keys(Seg S, const uint64_t* keys) {
 }
 
 __global__ void k_recip(int64_t n, const double* r, double* x) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n) x[p] = 1.0 / r[p];
 }
 
 __global__ void k_make_t32(int64_t n, const double* x, const double* phi, float2* t32) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n) t32[p] = make_float2((float)x[p], (float)phi[p]);
 }
 
 __global__ void k_make_nodes(int64_t n, const double* r, const double* x, const double* phi,
                              const double* M, double4_32a* node, float4* tdf) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   node[p] = make_double4_32a(r[p], x[p], phi[p], M[p]);
@@ -870,6 +894,7 @@ __global__ void k_make_nodes(int64_t n, const double* r, const double* x, const 
 
 __global__ void k_unpack_orbit(int64_t n, const uint64_t* keys, const Payload* pay,
                                double* r_new, double* vr_new, double* vt_new) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   uint64_t k = keys[p];
@@ -884,27 +909,27 @@ inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b
 }  // namespace
 
 void launch_nb_from_keys(const SegLayout& L, const uint64_t* keys, cudaStream_t st) {
-  k_nb_from_keys<<<blocks_for(L.n_seg, 128), 128, 0, st>>>(L.dev(), keys);
+  launch_k(k_nb_from_keys, blocks_for(L.n_seg, 128), 128, 0, st, L.dev(), keys);
 }
 
 void launch_recip(int64_t n, const double* r, double* x, cudaStream_t st) {
-  if (n > 0) k_recip<<<blocks_for(n, 256), 256, 0, st>>>(n, r, x);
+  if (n > 0) launch_k(k_recip, blocks_for(n, 256), 256, 0, st, n, r, x);
 }
 
 void launch_make_t32(int64_t n, const double* x, const double* phi, float2* t32,
                      cudaStream_t st) {
-  if (n > 0) k_make_t32<<<blocks_for(n, 256), 256, 0, st>>>(n, x, phi, t32);
+  if (n > 0) launch_k(k_make_t32, blocks_for(n, 256), 256, 0, st, n, x, phi, t32);
 }
 
 void launch_make_nodes(int64_t n, const double* r, const double* x, const double* phi,
                        const double* M, double4_32a* node, float4* tdf, cudaStream_t st) {
-  if (n > 0) k_make_nodes<<<blocks_for(n, 256), 256, 0, st>>>(n, r, x, phi, M, node, tdf);
+  if (n > 0) launch_k(k_make_nodes, blocks_for(n, 256), 256, 0, st, n, r, x, phi, M, node, tdf);
 }
 
 void launch_unpack_orbit(int64_t n, const uint64_t* keys, const Payload* pay, double* r_new,
                          double* vr_new, double* vt_new, cudaStream_t st) {
   if (n > 0)
-    k_unpack_orbit<<<blocks_for(n, 256), 256, 0, st>>>(n, keys, pay, r_new, vr_new, vt_new);
+    launch_k(k_unpack_orbit, blocks_for(n, 256), 256, 0, st, n, keys, pay, r_new, vr_new, vt_new);
 }
 
 // ------------------------------------------------------------------ host
@@ -979,16 +1004,16 @@ void free_layout(SegLayout& L, cudaStream_t st) {
 void launch_make_keys(const SegLayout& L, const double* r, const double* vr,
                       const double* vt, const double* m, const uint32_t* id,
                       uint64_t* keys, Payload* pay, cudaStream_t st) {
-  if (L.n) k_make_keys<<<blocks_for(L.n, 256), 256, 0, st>>>(L.n, r, vr, vt, m, id, keys, pay);
+  if (L.n) launch_k(k_make_keys, blocks_for(L.n, 256), 256, 0, st, L.n, r, vr, vt, m, id, keys, pay);
 }
 
 void launch_id_keys(const SegLayout& L, const uint32_t* id, uint64_t* keys, cudaStream_t st) {
-  if (L.n) k_id_keys<<<blocks_for(L.n, 256), 256, 0, st>>>(L.n, id, keys);
+  if (L.n) launch_k(k_id_keys, blocks_for(L.n, 256), 256, 0, st, L.n, id, keys);
 }
 
 void launch_rekey_radius(const SegLayout& L, const uint32_t* perm, const double* r,
                          const uint32_t* id, uint64_t* keys, cudaStream_t st) {
-  if (L.n) k_rekey_radius<<<blocks_for(L.n, 256), 256, 0, st>>>(L.n, perm, r, id, keys);
+  if (L.n) launch_k(k_rekey_radius, blocks_for(L.n, 256), 256, 0, st, L.n, perm, r, id, keys);
 }
 
 void launch_gather(const SegLayout& L, const uint64_t* keys, const uint32_t* vals,
@@ -998,12 +1023,12 @@ void launch_gather(const SegLayout& L, const uint64_t* keys, const uint32_t* val
                    const double* Ap, double* Aout, bool packed) {
   if (!L.n) return;
   if (tile_m && tile_mx && r_old && c && L.n_tiles)
-    k_gather_sums<<<(unsigned)L.n_tiles, kThreads, 0, st>>>(L.dev(), L.esc_step, L.n, keys, vals,
+    launch_k(k_gather_sums, (unsigned)L.n_tiles, kThreads, 0, st, L.dev(), L.esc_step, L.n, keys, vals,
                                                             pay, r, x, vr, vt, m, id, r_old, c,
                                                             tile_m, tile_mx, Rp, Rout, Ap,
                                                             Aout, packed);
   else
-    k_gather<<<blocks_for(L.n, 256), 256, 0, st>>>(L.n, keys, vals, pay, r, x, vr, vt, m, id,
+    launch_k(k_gather, blocks_for(L.n, 256), 256, 0, st, L.n, keys, vals, pay, r, x, vr, vt, m, id,
                                                   r_old, c);
 }
 
@@ -1021,14 +1046,14 @@ void launch_potential(const SegLayout& L, const double* r, const double* x, cons
   if (!L.n_tiles) return;
   Seg S = L.dev();
   if (!sums_ready)
-    k_tile_sums<<<(unsigned)L.n_tiles, kThreads, 0, st>>>(S, L.esc_step, nb_sub, x, m, tile_m,
+    launch_k(k_tile_sums, (unsigned)L.n_tiles, kThreads, 0, st, S, L.esc_step, nb_sub, x, m, tile_m,
                                                          tile_mx);
-  k_potential<<<(unsigned)L.n_tiles, kPotThreads, kPotentialSmem, st>>>(
+  launch_k(k_potential, (unsigned)L.n_tiles, kPotThreads, kPotentialSmem, st,
       S, L.esc_step, nb_sub, r, x, m, tile_m, tile_mx, phi, t32, Mout, node, tdf, slopes,
       tables ? *tables : TableOut());
   // with the tables, the seams' slopes come with the grid's values
   if (slopes && node && !tables)
-    k_slope_seams<<<blocks_for(L.n_tiles, 128), 128, 0, st>>>(S, L.esc_step, nb_sub, r, x, phi,
+    launch_k(k_slope_seams, blocks_for(L.n_tiles, 128), 128, 0, st, S, L.esc_step, nb_sub, r, x, phi,
                                                               Mout, node, L.n_tiles);
 }
 
@@ -1038,7 +1063,7 @@ void launch_correction(const SegLayout& L, const double* r, const double* x,
                        const double* m) {
   (void)err;
   if (!L.n) return;
-  k_correction<<<blocks_for(L.n, 128), 128, 0, st>>>(L.dev(), L.esc_step, nb_sub, r, x, phi,
+  launch_k(k_correction, blocks_for(L.n, 128), 128, 0, st, L.dev(), L.esc_step, nb_sub, r, x, phi,
                                                     vr, vt, r_old, c, m, L.n);
 }
 
@@ -1047,17 +1072,17 @@ void launch_energy(const SegLayout& L, const double* r, const double* vr, const 
                    double* Mbuf, double* out3, cudaStream_t st) {
   if (!L.n_tiles) return;
   Seg S = L.dev();
-  k_tile_sums<<<(unsigned)L.n_tiles, kThreads, 0, st>>>(S, L.esc_step, false, r, m, tile_m,
+  launch_k(k_tile_sums, (unsigned)L.n_tiles, kThreads, 0, st, S, L.esc_step, false, r, m, tile_m,
                                                        tile_k);
-  k_energy_tiles<<<(unsigned)L.n_tiles, kThreads, 0, st>>>(S, r, vr, vt, m, tile_m, tile_k,
+  launch_k(k_energy_tiles, (unsigned)L.n_tiles, kThreads, 0, st, S, r, vr, vt, m, tile_m, tile_k,
                                                           tile_w, Mbuf);
-  k_energy_final<<<(unsigned)L.n_seg, kThreads, 0, st>>>(S, tile_k, tile_w, out3);
+  launch_k(k_energy_final, (unsigned)L.n_seg, kThreads, 0, st, S, tile_k, tile_w, out3);
 }
 
 void launch_diag_ring(const SegLayout& L, const double* out3, const uint32_t* step,
                       const uint32_t* err, double* ring, int cap, cudaStream_t st) {
   if (!L.n_seg || cap <= 0) return;
-  k_diag_ring<<<(unsigned)((L.n_seg + 127) / 128), 128, 0, st>>>(L.dev(), out3, L.dt_last,
+  launch_k(k_diag_ring, (unsigned)((L.n_seg + 127) / 128), 128, 0, st, L.dev(), out3, L.dt_last,
                                                                 L.esc_me, step, err, ring, cap);
 }
 
@@ -1066,45 +1091,45 @@ void launch_core(const SegLayout& L, const double* r, const double* m, double* t
   if (!L.n_tiles) return;
   Seg S = L.dev();
   const int64_t t = L.n_tiles;
-  k_core_tiles<<<(unsigned)t, kThreads, 0, st>>>(S, r, m, tiles4, tiles4 + t, tiles4 + 2 * t,
+  launch_k(k_core_tiles, (unsigned)t, kThreads, 0, st, S, r, m, tiles4, tiles4 + t, tiles4 + 2 * t,
                                                   tiles4 + 3 * t);
-  k_core_final<<<(unsigned)L.n_seg, kThreads, 0, st>>>(S, tiles4, tiles4 + t, tiles4 + 2 * t,
+  launch_k(k_core_final, (unsigned)L.n_seg, kThreads, 0, st, S, tiles4, tiles4 + t, tiles4 + 2 * t,
                                                        tiles4 + 3 * t, out3);
 }
 
 void launch_lagrange(const SegLayout& L, const double* r, const double* M,
                      const double* fracs, int nf, double* out, cudaStream_t st) {
   int n = L.n_seg * nf;
-  if (n) k_lagrange<<<blocks_for(n, 128), 128, 0, st>>>(L.dev(), r, M, fracs, nf, out);
+  if (n) launch_k(k_lagrange, blocks_for(n, 128), 128, 0, st, L.dev(), r, M, fracs, nf, out);
 }
 
 void launch_validate(const SegLayout& L, const double* r, const double* vr,
                      const double* vt, const double* m, bool allow_inf, uint32_t* err,
                      cudaStream_t st) {
-  if (L.n) k_validate<<<blocks_for(L.n, 256), 256, 0, st>>>(L.n, r, vr, vt, m, allow_inf, err);
+  if (L.n) launch_k(k_validate, blocks_for(L.n, 256), 256, 0, st, L.n, r, vr, vt, m, allow_inf, err);
 }
 
 void launch_order_check(const SegLayout& L, const double* r, const uint32_t* id, uint32_t* flag,
                         unsigned int* maxid, cudaStream_t st) {
-  if (L.n) k_order_check<<<blocks_for(L.n, 256), 256, 0, st>>>(L.n, L.off, L.n_seg, r, id, flag,
+  if (L.n) launch_k(k_order_check, blocks_for(L.n, 256), 256, 0, st, L.n, L.off, L.n_seg, r, id, flag,
                                                                maxid);
 }
 
 void launch_ids_bitmap(const SegLayout& L, const uint32_t* id, const unsigned long long* bitoff,
                        unsigned long long* bitmap, uint32_t* err, cudaStream_t st) {
-  if (L.n) k_ids_bitmap<<<blocks_for(L.n, 256), 256, 0, st>>>(L.n, L.off, L.n_seg, id, bitoff,
+  if (L.n) launch_k(k_ids_bitmap, blocks_for(L.n, 256), 256, 0, st, L.n, L.off, L.n_seg, id, bitoff,
                                                               bitmap, err);
 }
 
 void launch_check_ids(const SegLayout& L, const uint64_t* sorted_ids, uint32_t* err,
                       cudaStream_t st) {
   if (L.n > 1)
-    k_check_ids<<<blocks_for(L.n, 256), 256, 0, st>>>(L.n, L.off, L.n_seg, sorted_ids, err);
+    launch_k(k_check_ids, blocks_for(L.n, 256), 256, 0, st, L.n, L.off, L.n_seg, sorted_ids, err);
 }
 
 void launch_step_end(const SegLayout& L, uint32_t* step, const double* r_old, const double* c,
                      const double* m, cudaStream_t st) {
-  k_step_end<<<L.n_seg, 256, 0, st>>>(L.dev(), L.esc_step, L.dt_last, step, r_old, c, m,
+  launch_k(k_step_end, L.n_seg, 256, 0, st, L.dev(), L.esc_step, L.dt_last, step, r_old, c, m,
                                       L.esc_me);
 }
 

@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(kThreads) k_upsweep(const int64_t* off, const 
                                                       int n_seg, const uint64_t* keys,
                                                       int first_pass, int passes,
                                                       uint32_t* hist, uint32_t* done) {
+  pdl_enter();
   __shared__ uint32_t s_warp[kWarps];
   __shared__ bool s_last;
   extern __shared__ uint32_t h[];  // [kWarps][passes][kBins]
@@ -178,6 +179,7 @@ __global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 6 : IPT <= 16 ? (kPacked
            uint64_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out, int pass, int q,
            int passes, const uint32_t* base, unsigned long long* desc, uint32_t* tickets,
            uint32_t* err) {
+  pdl_enter();
   constexpr int kTileKeys = kThreads * IPT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PassSmem<IPT, kPacked>& S = *reinterpret_cast<PassSmem<IPT, kPacked>*>(smem_raw);
@@ -316,6 +318,7 @@ __global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 6 : IPT <= 16 ? (kPacked
 __global__ void k_tiefix(const int64_t* off, int n_seg, int64_t n, uint64_t* keys,
                          uint32_t* vals, const uint32_t* ids_by_val, int id_stride, int shift,
                          uint32_t* err, unsigned long long* stats) {
+  pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   int c = seg_find(off, n_seg, p);
@@ -413,6 +416,7 @@ __device__ __forceinline__ void tiefix_packed_at(const int64_t* off, int n_seg, 
 __global__ void k_tiefix_packed(const int64_t* off, int n_seg, int64_t n, uint64_t* keys,
                                 const Payload* pay, uint32_t* err,
                                 unsigned long long* stats) {
+  pdl_enter();
   const int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (p0 >= n) return;
   uint64_t k[6];  // keys[p0 - 1 .. p0 + 4]
@@ -440,6 +444,7 @@ __global__ void k_tiefix_packed(const int64_t* off, int n_seg, int64_t n, uint64
 }
 
 __global__ void k_philox(int64_t n, const uint32_t* ctr, uint64_t seed, uint32_t* out) {
+  pdl_enter();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint4 c = reinterpret_cast<const uint4*>(ctr)[i];
@@ -460,19 +465,19 @@ void launch_pass(const SegLayout& L, SortWork& W, bool id, const uint64_t* kin,
                  int passes, uint32_t* err, cudaStream_t st, bool packed) {
   const unsigned grid = (unsigned)W.n_stiles;
   if (packed) {
-    k_pass<false, IPT, kRank, true><<<grid, kThreads, sizeof(PassSmem<IPT, true>), st>>>(
+    launch_k(k_pass<false, IPT, kRank, true>, grid, kThreads, sizeof(PassSmem<IPT, true>), st,
         L.off, W.stile_off, L.n_seg, W.n_stiles, kin, nullptr, kout, nullptr, pass, q, passes,
         W.hist, W.desc, W.tickets, err);
     return;
   }
   const size_t sm = sizeof(PassSmem<IPT, false>);
   if (id)
-    k_pass<true, IPT, kRank, false><<<grid, kThreads, sm, st>>>(L.off, W.stile_off, L.n_seg,
+    launch_k(k_pass<true, IPT, kRank, false>, grid, kThreads, sm, st, L.off, W.stile_off, L.n_seg,
                                                          W.n_stiles, kin, vin, kout, vout, pass,
                                                          q, passes, W.hist, W.desc, W.tickets,
                                                          err);
   else
-    k_pass<false, IPT, kRank, false><<<grid, kThreads, sm, st>>>(L.off, W.stile_off, L.n_seg,
+    launch_k(k_pass<false, IPT, kRank, false>, grid, kThreads, sm, st, L.off, W.stile_off, L.n_seg,
                                                           W.n_stiles, kin, vin, kout, vout,
                                                           pass, q, passes, W.hist, W.desc,
                                                           W.tickets, err);
@@ -485,11 +490,11 @@ void launch_packed_pass(const SegLayout& L, SortWork& W, const uint64_t* kin, ui
   const unsigned grid = (unsigned)W.n_stiles;
   const size_t sm = sizeof(PassSmem<IPT, true>);
   if (W.rank == kRankMatch)
-    k_pass<false, IPT, kRankMatch, true><<<grid, kThreads, sm, st>>>(
+    launch_k(k_pass<false, IPT, kRankMatch, true>, grid, kThreads, sm, st,
         L.off, W.stile_off, L.n_seg, W.n_stiles, kin, nullptr, kout, nullptr, pass, q, passes,
         W.hist, W.desc, W.tickets, err);
   else
-    k_pass<false, IPT, kRankBallot, true><<<grid, kThreads, sm, st>>>(
+    launch_k(k_pass<false, IPT, kRankBallot, true>, grid, kThreads, sm, st,
         L.off, W.stile_off, L.n_seg, W.n_stiles, kin, nullptr, kout, nullptr, pass, q, passes,
         W.hist, W.desc, W.tickets, err);
 }
@@ -607,7 +612,7 @@ cudaError_t sort_segments(const SegLayout& L, SortWork& W, uint64_t* keys, uint3
                   W.zero_head + sizeof(unsigned long long) * (size_t)passes *
                                     (size_t)W.n_stiles * kBins,
                   st);
-  k_upsweep<<<(unsigned)L.n_tiles, kThreads, sizeof(uint32_t) * kWarps * passes * kBins, st>>>(
+  launch_k(k_upsweep, (unsigned)L.n_tiles, kThreads, sizeof(uint32_t) * kWarps * passes * kBins, st,
       L.off, L.tile_off, L.n_seg, keys, first_pass, passes, W.hist, W.done);
   uint64_t* kin = keys;
   uint32_t* vin = vals;
@@ -655,7 +660,7 @@ void launch_tiefix(const SegLayout& L, uint64_t* keys, uint32_t* vals,
                    const uint32_t* ids_by_val, int id_stride, uint32_t* err,
                    cudaStream_t st, int shift) {
   if (L.n == 0) return;
-  k_tiefix<<<(unsigned)((L.n + 255) / 256), 256, 0, st>>>(
+  launch_k(k_tiefix, (unsigned)((L.n + 255) / 256), 256, 0, st,
       L.off, L.n_seg, L.n, keys, vals, ids_by_val, id_stride, shift, err, L.stats);
 }
 
@@ -663,14 +668,14 @@ void launch_tiefix_packed(const SegLayout& L, uint64_t* keys, const Payload* pay
                           uint32_t* err, cudaStream_t st) {
   if (L.n == 0) return;
   const int64_t nt = (L.n + 3) / 4;
-  k_tiefix_packed<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(L.off, L.n_seg, L.n, keys, pay,
+  launch_k(k_tiefix_packed, (unsigned)((nt + 255) / 256), 256, 0, st, L.off, L.n_seg, L.n, keys, pay,
                                                                err, L.stats);
 }
 
 void launch_philox(int64_t n, const uint32_t* ctr, uint64_t seed, uint32_t* out,
                    cudaStream_t st) {
   if (n <= 0) return;
-  k_philox<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, ctr, seed, out);
+  launch_k(k_philox, (unsigned)((n + 255) / 256), 256, 0, st, n, ctr, seed, out);
 }
 
 CMC_DEBUG_SITE_ACCESSOR
