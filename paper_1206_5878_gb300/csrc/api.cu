@@ -25,15 +25,23 @@ struct cmc_ctx {
   SortWork W;
   BucketWork bk;  // radius-bucket index, grid and node records (precision 0 and 1)
   double pref = 0.0;
-  // state (sorted SoA)
+  // state (sorted SoA); a step writes the new radii and their reciprocals to
+  // r_alt and x_alt (the energy correction still reads the old ones) and the
+  // two change places, so there is a graph for each order
   double *r = nullptr, *x = nullptr, *vr = nullptr, *vt = nullptr, *m = nullptr,
          *phi = nullptr;
+  double *r_alt = nullptr, *x_alt = nullptr;
+  int side = 0;
   uint32_t* id = nullptr;
   float2* t32 = nullptr;
   // scratch
   uint64_t* keys = nullptr;
   uint32_t* vals = nullptr;
-  Payload* pay = nullptr;
+  RecA* ra = nullptr;
+  RecB* rb = nullptr;
+  uint32_t* order = nullptr;   // the stars' old indices at their new positions
+  BinWork bins;                // the timestep's counting sort (cfg.sort_packed)
+  std::vector<unsigned int> max_id;  // per segment, as the bins have it
   double *r_old = nullptr, *cc = nullptr, *nbin = nullptr;
   double *tile_a = nullptr, *tile_b = nullptr, *tile_c = nullptr, *Mbuf = nullptr,
          *out3 = nullptr, *fr = nullptr, *lag = nullptr;
@@ -42,10 +50,9 @@ struct cmc_ctx {
   uint32_t* pcount = nullptr;  // pending stars of the sampled orbit step
   EnvWork env;                 // FP64 mode's envelope (precision 0)
   double4_32a* orb = nullptr;  // E, J, c0, c1 of every star's orbit (precision 0 and 1)
-  bool packed = false;         // the timestep sorts packed keys (cfg.sort_packed, clusters < 2^24)
   double* ring = nullptr;      // per-step diagnostics (cfg.diag_ring records per cluster)
   int64_t steps_taken = 0;
-  cudaGraphExec_t exec = nullptr;
+  cudaGraphExec_t exec[2] = {nullptr, nullptr};
   bool poisoned = false;
   std::string last_error;
   int kernels_per_step = 0;
@@ -126,8 +133,10 @@ cmc_status check_err_flags(cmc_ctx* ctx) {
 // Whether the staged stars are already in (r, id) order in every segment
 // with ids that fit a bitmap of the key scratch (64 bits per star): then
 // bitoff receives each segment's first bit.  A state read back with
-// cmc_get_state always qualifies.
-bool staged_in_order(cmc_ctx* c, std::vector<unsigned long long>& bitoff, cudaStream_t st) {
+// cmc_get_state always qualifies.  max_id (if given) receives the largest
+// id of each segment either way.
+bool staged_in_order(cmc_ctx* c, std::vector<unsigned long long>& bitoff, cudaStream_t st,
+                     std::vector<unsigned int>* max_id = nullptr) {
   const SegLayout& L = c->L;
   unsigned int* d = nullptr;  // [0] order flag, [1 + s] largest id of segment s
   if (dalloc(d, (size_t)L.n_seg + 1, st)) return false;
@@ -139,6 +148,7 @@ bool staged_in_order(cmc_ctx* c, std::vector<unsigned long long>& bitoff, cudaSt
   }
   if (!e) e = cudaStreamSynchronize(st);
   dfree(d, st);
+  if (!e && max_id) max_id->assign(h.begin() + 1, h.end());
   if (e || h[0] != 0u) return false;
   bitoff.assign((size_t)L.n_seg, 0ull);
   unsigned long long total = 0;
@@ -167,7 +177,7 @@ bool order_in_place(cmc_ctx* c, const std::vector<unsigned long long>& bitoff,
   // the bitmap lives in the key scratch (64 bits per star)
   cudaMemsetAsync(c->keys, 0, sizeof(uint64_t) * (size_t)L.n, st);
   launch_ids_bitmap(L, c->id, dbo, reinterpret_cast<unsigned long long*>(c->keys), c->err, st);
-  launch_make_keys(L, c->r, nullptr, nullptr, nullptr, c->id, c->keys, nullptr, st);
+  launch_make_keys(L, c->r, c->id, c->keys, st);
   launch_recip(L.n, c->r, c->x, st);
   cudaStreamSynchronize(st);  // bitoff lives on the caller's stack frame
   dfree(dbo, st);
@@ -198,12 +208,18 @@ void order_state(cmc_ctx* c, cudaStream_t st) {
     launch_check_ids(L, c->keys, c->err, st);
     launch_rekey_radius(L, c->vals, c->r, c->id, c->keys, st);
     sort_segments(L, c->W, c->keys, c->vals, 0, 8, false, c->err, st);
-    launch_make_keys(L, c->r, c->vr, c->vt, c->m, c->id, c->W.keys_alt, c->pay, st);
-    launch_gather(L, c->keys, c->vals, c->pay, c->r, c->x, c->vr, c->vt, c->m, c->id, nullptr,
-                  nullptr, st);
+    launch_make_records(L, c->r, c->vr, c->vt, c->m, c->id, c->ra, c->rb, st);
+    launch_gather(L, c->vals, c->ra, c->rb, c->r, c->x, c->vr, c->vt, c->m, c->id, st);
   }
   finish_order(c, st);
 }
+
+// The largest number of stars whose bins the orbit step counts itself, saving
+// a launch (2 us at N = 1e4 to 1e5).  With more the counts no longer stay in the
+// L2 beside the step's random table reads: at N = 1e6 counting in the orbit
+// kernel cost 30 us against 6 us in a kernel of its own, at 1e7 1.06 ms
+// against 0.05.
+constexpr int64_t kCountInOrbit = 262144;
 
 // stage names (cmc_step_profiled, NVTX ranges)
 const char* const kStageName[CMC_NSTAGES] = {"timestep", "relax",     "turning",
@@ -234,76 +250,85 @@ void record_step(cmc_ctx* c, cudaStream_t st, cudaEvent_t* ev = nullptr) {
     launch_turning(L, c->r, c->x, c->phi, c->Mbuf, c->vr, c->vt, c->bk.args(), nullptr,
                    nullptr, c->orb, c->cfg.orbit_block, st);
   mark(3);
+  const bool binned = c->cfg.sort_packed != 0;
+  const bool counted = L.n <= kCountInOrbit;
   launch_orbit(L, c->cfg.precision, c->cfg.max_trials, c->r, c->x, c->phi,
                tab ? c->Mbuf : nullptr, c->vr, c->vt, c->m, c->id,
-               c->step, c->keys, c->pay, nullptr, c->cfg.orbit_block, c->orbit_variant,
+               c->step, c->keys, c->ra, c->rb, nullptr, c->cfg.orbit_block, c->orbit_variant,
                c->bk.args(), c->r_old, c->cc, c->vals, c->pcount, st, false, c->R, c->Rp,
-               c->cfg.precision == 0 ? &c->env : nullptr, c->A, c->Ap, c->orb, c->packed);
+               c->cfg.precision == 0 ? &c->env : nullptr, c->A, c->Ap, c->orb,
+               binned ? &c->bins : nullptr, c->vals, counted);
   mark(4);
-  // radix passes over bits 24-63 of the radius keys; runs equal in those
-  // bits (radii within 2^-28 of each other, escapers whose ids differ in
-  // their low 4 bits) are put in (key, id) order after
-  uint64_t* sk = nullptr;
-  uint32_t* sv = nullptr;
-  sort_segments(L, c->W, c->keys, c->vals, 3, 5, true, c->err, st, &sk, &sv, c->packed);
-  if (c->packed)
-    launch_tiefix_packed(L, sk, c->pay, c->err, st);
-  else
-    launch_tiefix(L, sk, sv, &c->pay[0].id, (int)(sizeof(Payload) / sizeof(uint32_t)), c->err,
-                  st, 24);
+  uint32_t* ord = c->W.vals_alt;
+  if (binned) {
+    launch_bin_sort(L, c->bins, c->vals, c->ra, ord, c->order, counted, c->err, st);
+  } else {
+    // radix passes over bits 24-63 of the radius keys; runs equal in those
+    // bits (radii within 2^-28 of each other, escapers whose ids differ in
+    // their low 4 bits) are put in (key, id) order after
+    uint64_t* sk = nullptr;
+    sort_segments(L, c->W, c->keys, c->vals, 3, 5, true, c->err, st, &sk, &ord);
+    launch_tiefix(L, sk, ord, &c->ra[0].id, (int)(sizeof(RecA) / sizeof(uint32_t)), c->err, st,
+                  24);
+  }
   mark(5);
-  launch_gather(L, sk, sv, c->pay, c->r, c->x, c->vr, c->vt, c->m, c->id, c->r_old, c->cc, st,
-                c->tile_a, c->tile_b, c->Rp, c->R, c->Ap, c->A, c->packed);
+  launch_gather_step(L, binned ? &c->bins : nullptr, ord, c->ra, c->rb, c->r, c->r_alt, c->x_alt,
+                     c->m, c->id, c->order, c->r_old, c->cc, c->tile_a, c->tile_b, c->Rp, c->R,
+                     c->Ap, c->A, !binned, st);
   mark(6);
   // the tables carry the shell slopes of the FP64 orbit step (not the
   // scan's enclosed masses): the sampled step's turning points and points
   // are then FP64 mode's
   if (tab)
-    launch_potential_tables(L, c->r, c->x, c->m, c->tile_a, c->tile_b, c->phi, c->t32, c->Mbuf,
-                            true, true, c->bk, st);
+    launch_potential_tables(L, c->r_alt, c->x_alt, c->m, c->tile_a, c->tile_b, c->phi, c->t32,
+                            c->Mbuf, true, true, c->bk, st);
   else
-    launch_potential(L, c->r, c->x, c->m, c->tile_a, c->tile_b, c->phi, nullptr, nullptr, true,
-                     st, nullptr, nullptr, true);
+    launch_potential(L, c->r_alt, c->x_alt, c->m, c->tile_a, c->tile_b, c->phi, nullptr, nullptr,
+                     true, st, nullptr, nullptr, true);
   mark(7);
-  if (c->cfg.energy_correction) {
-    // with the tables (precision 0 and 1) the shell of r_old comes from the
-    // bucket index; FP64 mode evaluates Phi in Eq. 6's division form
-    if (tab)
-      launch_correction_mixed(L, c->r, c->x, c->phi, c->Mbuf, c->bk.args(), c->vr, c->vt,
-                              c->r_old, c->cc, c->m, st, !mixed);
-    else
-      launch_correction(L, c->r, c->x, c->phi, c->vr, c->vt, c->r_old, c->cc, true, c->err, st,
-                        c->m);
-  }
+  // (the FP64 modes evaluate Phi_new(r_old) in Eq. 6's division form)
+  const bool correct = c->cfg.energy_correction != 0;
+  if (correct)
+    launch_phi_old(L, c->r, c->x, c->r_alt, c->x_alt, c->phi, c->bk.node, c->rb, !mixed, st);
+  launch_velocities(L, c->order, c->rb, c->phi, c->m, c->vr, c->vt, correct, st);
   mark(8);
   launch_step_end(L, c->step, c->r_old, c->cc, c->m, st);
   if (c->ring) {
     // K and W of the new state (r_old is free scratch now), then the record
-    launch_energy(L, c->r, c->vr, c->vt, c->m, c->tile_a, c->tile_b, c->tile_c, c->r_old,
+    launch_energy(L, c->r_alt, c->vr, c->vt, c->m, c->tile_a, c->tile_b, c->tile_c, c->r_old,
                   c->out3, st);
     launch_diag_ring(L, c->out3, c->step, c->err, c->ring, c->cfg.diag_ring, st);
   }
   mark(9);
 }
 
+// after a step's kernels: the new radii are the state's
+void turn_sides(cmc_ctx* c) {
+  std::swap(c->r, c->r_alt);
+  std::swap(c->x, c->x_alt);
+  c->side ^= 1;
+}
+
 int count_step_kernels(const cmc_ctx* c) {
-  // bins, relax, orbit, upsweep (with the histograms' scans), 5 passes, tie fix, gather with
-  // the tile sums, potential, [precision 0 and 1: turning points, FP32
-  // sampler, FP64 continuation, the tables' parameters, the grid's values
+  // bins, relax, orbit, gather with the tile sums, potential, velocities, step
+  // end; the sort: scan, scatter, long runs [count], or upsweep (with the
+  // histograms' scans), 5 passes, tie fix; [precision 0 and 1: turning points,
+  // FP32 sampler, FP64 continuation, the tables' parameters, the grid's values
   // with the seams' slopes; precision 0: the envelope's screen and
-  // evaluation], [correction], step end
+  // evaluation], [Phi_new(r_old)]
   const int p = c->cfg.precision;
-  return 3 + ((c->R || c->A) ? 1 : 0) + (c->ring ? 4 : 0) + 1 + 5 + 1 + 1 + 1 +
-         (p == 1 ? 5 : p == 0 ? 7 : 0) +
-         (c->cfg.energy_correction ? 1 : 0) + 1;
+  const int sort = c->cfg.sort_packed ? (c->L.n <= kCountInOrbit ? 3 : 4) : 7;
+  return 7 + sort + ((c->R || c->A) ? 1 : 0) + (c->ring ? 4 : 0) +
+         (p == 1 ? 5 : p == 0 ? 7 : 0) + (c->cfg.energy_correction ? 1 : 0);
 }
 
 void free_ctx(cmc_ctx* c) {
   if (!c) return;
   DeviceGuard g(c->device);
   cudaStream_t st = c->stream;
-  if (c->exec) cudaGraphExecDestroy(c->exec);
-  double** ds[] = {&c->r, &c->x, &c->vr, &c->vt, &c->m, &c->phi, &c->r_old, &c->cc, &c->nbin,
+  for (cudaGraphExec_t e : c->exec)
+    if (e) cudaGraphExecDestroy(e);
+  double** ds[] = {&c->r_alt, &c->x_alt, &c->r, &c->x, &c->vr, &c->vt, &c->m, &c->phi, &c->r_old, &c->cc, &c->nbin,
                    &c->tile_a, &c->tile_b, &c->tile_c, &c->Mbuf, &c->out3, &c->fr, &c->lag};
   for (double** p : ds) dfree(*p, st);
   dfree(c->id, st);
@@ -314,7 +339,10 @@ void free_ctx(cmc_ctx* c) {
   dfree(c->t32, st);
   dfree(c->keys, st);
   dfree(c->vals, st);
-  dfree(c->pay, st);
+  dfree(c->ra, st);
+  dfree(c->rb, st);
+  dfree(c->order, st);
+  free_bins(c->bins, st);
   dfree(c->err, st);
   dfree(c->step, st);
   dfree(c->pcount, st);
@@ -360,9 +388,17 @@ cmc_status load_state(cmc_ctx* c, const double* r, const double* vr, const doubl
   if (e) return cuda_fail(c, e, "copy in");
   std::vector<unsigned long long> bitoff;
   bool placed = false;
-  if (L.n > 0 && staged_in_order(c, bitoff, aux) && order_in_place(c, bitoff, aux)) {
+  std::vector<unsigned int> max_id;
+  if (L.n > 0 && staged_in_order(c, bitoff, aux, &max_id) && order_in_place(c, bitoff, aux)) {
     finish_order(c, aux);
     placed = true;
+  }
+  // (ids that could not be read: bins for any id)
+  if (max_id.empty()) max_id.assign((size_t)L.n_seg, 0xFFFFFFFFu);
+  if (c->bins.cnt && max_id != c->max_id) {
+    e = set_bin_ids(c->bins, L, max_id.data(), aux);
+    if (e) return cuda_fail(c, e, "ordering the state");
+    c->max_id = max_id;
   }
   e = cudaEventRecord(c->ev_aux, aux);
   if (!e) e = cudaStreamWaitEvent(st, c->ev_aux, 0);
@@ -512,7 +548,7 @@ cmc_status autotune(cmc_ctx* c) {
   auto run_orbit = [&](int blk, int var) {
     launch_orbit(L, c->cfg.precision, c->cfg.max_trials, c->r, c->x, c->phi,
                  tab ? c->Mbuf : nullptr, c->vr, c->vt, c->m,
-                 c->id, c->step, c->keys, c->pay, nullptr, blk, var, c->bk.args(), c->r_old,
+                 c->id, c->step, c->keys, c->ra, c->rb, nullptr, blk, var, c->bk.args(), c->r_old,
                  c->cc, c->vals, c->pcount, st, true, nullptr, nullptr,
                  c->cfg.precision == 0 ? &c->env : nullptr, nullptr, nullptr, c->orb);
   };
@@ -565,24 +601,25 @@ cmc_status autotune(cmc_ctx* c) {
                     st);
   }
   run_orbit(blk_best, var_best);
-  // sort shapes on copies of the keys the orbit step produced
-  uint64_t* saved = reinterpret_cast<uint64_t*>(c->cc);  // scratch of the same size
-  cudaMemcpyAsync(saved, c->keys, sizeof(uint64_t) * L.n, cudaMemcpyDeviceToDevice, st);
-  int best_ipt = 16, best_rank = 0;
-  float tbest = 3.4e38f;
-  for (int ipt : {8, 16, 24, 32})
-    for (int rank : {0, 1}) {
-      // 24 and 32 keys per thread: packed keys only
-      if (ipt > 16 && !c->packed) continue;
-      if (sort_set_shape(L, c->W, ipt, rank, st)) continue;
-      const float ms = time_it([&] {
-        cudaMemcpyAsync(c->keys, saved, sizeof(uint64_t) * L.n, cudaMemcpyDeviceToDevice, st);
-        sort_segments(L, c->W, c->keys, c->vals, 3, 5, true, c->err, st, nullptr, nullptr,
-                      c->packed);
-      });
-      if (ms < tbest) { tbest = ms; best_ipt = ipt; best_rank = rank; }
-    }
-  cudaError_t e = sort_set_shape(L, c->W, best_ipt, best_rank, st);
+  // shapes of the radix passes (where the timestep uses them) on copies of the
+  // keys the orbit step produced
+  cudaError_t e = cudaSuccess;
+  if (!c->cfg.sort_packed) {
+    uint64_t* saved = reinterpret_cast<uint64_t*>(c->cc);  // scratch of the same size
+    cudaMemcpyAsync(saved, c->keys, sizeof(uint64_t) * L.n, cudaMemcpyDeviceToDevice, st);
+    int best_ipt = 16, best_rank = 0;
+    float tbest = 3.4e38f;
+    for (int ipt : {8, 16})
+      for (int rank : {0, 1}) {
+        if (sort_set_shape(L, c->W, ipt, rank, st)) continue;
+        const float ms = time_it([&] {
+          cudaMemcpyAsync(c->keys, saved, sizeof(uint64_t) * L.n, cudaMemcpyDeviceToDevice, st);
+          sort_segments(L, c->W, c->keys, c->vals, 3, 5, true, c->err, st);
+        });
+        if (ms < tbest) { tbest = ms; best_ipt = ipt; best_rank = rank; }
+      }
+    e = sort_set_shape(L, c->W, best_ipt, best_rank, st);
+  }
   // undo the dry run's bookkeeping
   if (!e && taus_saved)
     e = cudaMemcpyAsync(L.taus, taus_saved, sizeof(uint4) * L.taus_slots,
@@ -703,9 +740,6 @@ cmc_status cmc_init(cmc_ctx** out, const cmc_config* cfg_in, int32_t n_clusters,
 
   cmc_ctx* c = new cmc_ctx();
   c->cfg = cfg;
-  c->packed = cfg.sort_packed != 0;
-  for (int k = 0; k < n_clusters; ++k)
-    if (sizes[k] > kPackMax) c->packed = false;
   c->stream = (cudaStream_t)stream;
   c->pref = t_rel_prefactor(cfg.theta_max);
   cudaGetDevice(&c->device);
@@ -736,7 +770,11 @@ cmc_status cmc_init(cmc_ctx** out, const cmc_config* cfg_in, int32_t n_clusters,
   }
   CMC_ALLOC(c->keys, n);
   CMC_ALLOC(c->vals, n);
-  CMC_ALLOC(c->pay, n);
+  CMC_ALLOC(c->ra, n);
+  CMC_ALLOC(c->rb, n);
+  CMC_ALLOC(c->order, n);
+  CMC_ALLOC(c->r_alt, n);
+  CMC_ALLOC(c->x_alt, n);
   CMC_ALLOC(c->r_old, n);
   CMC_ALLOC(c->cc, n);
   CMC_ALLOC(c->Mbuf, n);
@@ -760,6 +798,7 @@ cmc_status cmc_init(cmc_ctx** out, const cmc_config* cfg_in, int32_t n_clusters,
   }
 #undef CMC_ALLOC
   if (!e) e = alloc_sort(c->W, L, 8, st);
+  if (!e && cfg.sort_packed) e = alloc_bins(c->bins, L, st);
   if (!e && cfg.precision != 2) e = alloc_buckets(c->bk, L, st);
   if (e) { cmc_status s = cuda_fail(nullptr, e, "cmc_init: allocation"); free_ctx(c); return s; }
   sort_prepare();
@@ -800,21 +839,33 @@ cmc_status cmc_step(cmc_ctx* c, int32_t n_steps) {
   if (n_steps == 0) return CMC_OK;
   DeviceGuard g(c->device);
   cudaError_t e;
-  if (!c->exec) {
-    cudaGraph_t graph;
-    e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
-    if (e) return cuda_fail(c, e, "cmc_step: begin capture");
-    record_step(c, c->cap);
-    e = cudaStreamEndCapture(c->cap, &graph);
-    if (e) return cuda_fail(c, e, "cmc_step: capture");
-    e = cudaGraphInstantiate(&c->exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e) { c->exec = nullptr; return cuda_fail(c, e, "cmc_step: instantiate"); }
+  // a graph for each side of the radii (see turn_sides), captured when first
+  // needed
+  const int first = c->side;
+  for (int i = 0; i < (n_steps > 1 ? 2 : 1); ++i) {
+    const int side = first ^ i;
+    if (!c->exec[side]) {
+      if (side != c->side) turn_sides(c);
+      cudaGraph_t graph;
+      e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
+      if (!e) {
+        record_step(c, c->cap);
+        e = cudaStreamEndCapture(c->cap, &graph);
+      }
+      if (!e) {
+        e = cudaGraphInstantiate(&c->exec[side], graph, 0);
+        cudaGraphDestroy(graph);
+        if (e) c->exec[side] = nullptr;
+      }
+      if (c->side != first) turn_sides(c);
+      if (e) return cuda_fail(c, e, "cmc_step: capture");
+    }
   }
   nvtxRangePushA("cmc_step");
   for (int32_t i = 0; i < n_steps; ++i) {
-    e = cudaGraphLaunch(c->exec, c->stream);
+    e = cudaGraphLaunch(c->exec[c->side], c->stream);
     if (e) { nvtxRangePop(); return cuda_fail(c, e, "cmc_step: launch"); }
+    turn_sides(c);
   }
   c->steps_taken += n_steps;
   const cmc_status s = check_err_flags(c);
@@ -829,7 +880,10 @@ cmc_status cmc_step_profiled(cmc_ctx* c, int32_t n_steps, double* stage_ms) {
   for (int i = 0; i < CMC_NSTAGES; ++i) stage_ms[i] = 0.0;
   std::vector<cudaEvent_t> ev((size_t)(CMC_NSTAGES + 1) * (n_steps > 0 ? n_steps : 1));
   for (auto& e : ev) cudaEventCreate(&e);
-  for (int32_t i = 0; i < n_steps; ++i) record_step(c, c->stream, &ev[(size_t)i * (CMC_NSTAGES + 1)]);
+  for (int32_t i = 0; i < n_steps; ++i) {
+    record_step(c, c->stream, &ev[(size_t)i * (CMC_NSTAGES + 1)]);
+    turn_sides(c);
+  }
   cudaError_t e = cudaStreamSynchronize(c->stream);
   if (!e) {
     for (int32_t i = 0; i < n_steps; ++i)
@@ -1186,7 +1240,7 @@ cmc_status cmc_sort_radius(int64_t n, const double* r, const uint32_t* id, uint3
   if (!e) {
     sort_prepare();
     cudaMemsetAsync(err, 0, sizeof(uint32_t), st);
-    launch_make_keys(S.L, r, nullptr, nullptr, nullptr, id, keys, nullptr, st);
+    launch_make_keys(S.L, r, id, keys, st);
     // as in the timestep: passes over bits 24-63, then runs equal in those
     // bits in (r, id) order
     sort_segments(S.L, W, keys, perm, 3, 5, true, err, st);
@@ -1296,13 +1350,15 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
   double *x = nullptr, *mm = nullptr;
   float2* t32 = nullptr;
   uint64_t* keys = nullptr;
-  Payload* pay = nullptr;
+  RecA* ra = nullptr;
+  RecB* rb = nullptr;
   uint32_t* dstep = nullptr;
   cudaError_t e = dalloc(x, n, st);
   if (!e) e = dalloc(mm, n, st);
   if (!e) e = dalloc(t32, n, st);
   if (!e) e = dalloc(keys, n, st);
-  if (!e) e = dalloc(pay, n, st);
+  if (!e) e = dalloc(ra, n, st);
+  if (!e) e = dalloc(rb, n, st);
   if (!e) e = dalloc(dstep, 1, st);
   if (!e) e = cudaMemsetAsync(mm, 0, sizeof(double) * n, st);
   if (!e) e = cudaMemcpyAsync(dstep, &step, sizeof(uint32_t), cudaMemcpyHostToDevice, st);
@@ -1336,7 +1392,7 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
     if (!e && precision == 0) e = alloc_env(env, n, st);
     if (!e)
       launch_orbit(S.L, precision, max_trials, r, x, phi, sl, vr, vt, mm, id, dstep, keys,
-                   pay, &d, 0, 0, bk.args(), tmin, tmax, plist, pcnt, st, true, nullptr,
+                   ra, rb, &d, 0, 0, bk.args(), tmin, tmax, plist, pcnt, st, true, nullptr,
                    nullptr, precision == 0 ? &env : nullptr, nullptr, nullptr, orb);
     free_buckets(bk, st);
     free_env(env, st);
@@ -1346,7 +1402,7 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
     dfree(orb, st);
     dfree(plist, st);
     dfree(pcnt, st);
-    launch_unpack_orbit(n, keys, pay, r_new, vr_new, vt_new, st);
+    launch_unpack_orbit(n, ra, rb, r_new, vr_new, vt_new, st);
     e = cudaGetLastError();
   }
   if (!e) e = cudaStreamSynchronize(st);
@@ -1354,7 +1410,8 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
   dfree(mm, st);
   dfree(t32, st);
   dfree(keys, st);
-  dfree(pay, st);
+  dfree(ra, st);
+  dfree(rb, st);
   dfree(dstep, st);
   return e ? cuda_fail(nullptr, e, "cmc_orbit") : CMC_OK;
 }

@@ -116,7 +116,7 @@ void free_sort(SortWork& W, cudaStream_t st);
 cudaError_t sort_segments(const SegLayout& L, SortWork& W, uint64_t* keys, uint32_t* vals,
                           int first_pass, int passes, bool vals_identity, uint32_t* err,
                           cudaStream_t st, uint64_t** keys_res = nullptr,
-                          uint32_t** vals_res = nullptr, bool packed = false);
+                          uint32_t** vals_res = nullptr);
 
 // Order every run of finite keys equal in their bits from `shift` up by
 // (key, id of the element: ids_by_val[vals[p] * id_stride]), so that after
@@ -129,28 +129,85 @@ void launch_tiefix(const SegLayout& L, uint64_t* keys, uint32_t* vals,
 void launch_philox(int64_t n, const uint32_t* ctr, uint64_t seed, uint32_t* out,
                    cudaStream_t st);
 
-// One star between the orbit step and the sort (48 B).  c: for a bound
-// star Phi_old(r_old) - Phi_old(r_new); for a star escaping in this step
-// its energy in the field of the others, Phi_k + m_k / r_k + v^2 / 2.
-struct Payload {
-  double vr, vt, m, r_old, c;
-  uint32_t id, pad;  // pad: with packed keys, the key's own low 24 bits
+// One star between the orbit step and the sorted state, in two records of
+// one 32-byte sector each.  RecA goes with the gather after the sort: the new
+// radius, its reciprocal, the mass, the id and the star's sort bin.  RecB
+// waits for the new potential: the new velocities and c (for a bound star
+// Phi_old(r_old) - Phi_old(r_new); for a star escaping in this step its
+// energy in the field of the others, Phi_k + m_k / r_k + v^2 / 2), and w,
+// Phi_new(r_old), filled in once the new potential is there.
+struct alignas(32) RecA {
+  double r, x, m;
+  uint32_t id, bin;
 };
+struct alignas(32) RecB {
+  double vr, vt, c, w;
+};
+// (each moves as one 32-byte access: two of 16 bytes fetched a random record's
+// sector twice, gather 0.37 -> 0.70 ms with three blocks to an SM)
+__device__ __forceinline__ RecA load_rec(const RecA* p) {
+  const double4_32a v = *reinterpret_cast<const double4_32a*>(p);
+  const unsigned long long u = ubits(v.w);
+  RecA a;
+  a.r = v.x; a.x = v.y; a.m = v.z; a.id = (uint32_t)u; a.bin = (uint32_t)(u >> 32);
+  return a;
+}
+__device__ __forceinline__ RecB load_rec(const RecB* p) {
+  const double4_32a v = *reinterpret_cast<const double4_32a*>(p);
+  RecB b;
+  b.vr = v.x; b.vt = v.y; b.c = v.z; b.w = v.w;
+  return b;
+}
+__device__ __forceinline__ void store_rec(RecA* p, const RecA& a) {
+  *reinterpret_cast<double4_32a*>(p) = make_double4_32a(
+      a.r, a.x, a.m,
+      __longlong_as_double((long long)(((unsigned long long)a.bin << 32) | a.id)));
+}
+__device__ __forceinline__ void store_rec(RecB* p, const RecB& b) {
+  *reinterpret_cast<double4_32a*>(p) = make_double4_32a(b.vr, b.vt, b.c, b.w);
+}
 
-// Packed sort keys (every segment below 2^24 stars): a key's low 24 bits,
-// which the timestep's radix passes do not sort, hold the star's index in
-// its segment (the key's own low bits go to the payload), so that the
-// passes move 8-byte keys and no values.
-constexpr uint64_t kPackMask = 0xFFFFFFull;
-constexpr int64_t kPackMax = (int64_t)1 << 24;
-// the tie fix of packed keys (runs equal in bits 24-63 into (key, id) order)
-void launch_tiefix_packed(const SegLayout& L, uint64_t* keys, const Payload* pay,
-                          uint32_t* err, cudaStream_t st);
+// The counting sort of a timestep.  A star's bin is the shell of the old
+// table that its new radius lies in (the orbit step has just found it):
+// bins order like radii, and since the distribution of the radii changes
+// little in a step a bin holds about one star.  So counting the bins,
+// scanning the counts and scattering the stars' indices sorts them up to the
+// order inside a bin, which the gather settles by (r, id).  Bins of segment
+// c: cbase[c] + s + 1 for the stars in shell s = -1 .. nb - 1, then the
+// escapers by id >> esh[c].  Runs of more than kRunMax stars in one bin are
+// listed and sorted by one block each.
+struct BinWork {
+  int64_t* cbase = nullptr;             // n_seg + 1 first bins
+  int* esh = nullptr;                   // per segment: ids per escaper bin (a shift)
+  uint32_t* cnt = nullptr;              // counts, then positions; zero between steps
+  unsigned long long* desc = nullptr;   // look-back words of the scan; zero between steps
+  uint32_t* ctl = nullptr;              // [0] scan tickets, [1] listed runs; zero between steps
+  uint2* runs = nullptr;                // listed runs: first position, length
+  std::vector<int64_t> h_cbase;
+  int64_t n_bins = 0, n_tiles = 0;      // bins padded to whole scan tiles
+};
+constexpr int kRunMax = 32;
+constexpr int kBinTile = 4096;          // bins per block of the scan
+cudaError_t alloc_bins(BinWork& B, const SegLayout& L, cudaStream_t st);
+void free_bins(BinWork& B, cudaStream_t st);
+// the escapers' bins for the largest id of each segment
+cudaError_t set_bin_ids(BinWork& B, const SegLayout& L, const unsigned int* max_id,
+                        cudaStream_t st);
+// order (n indices): the stars' indices in bin order, the order inside a bin
+// left to the gather except in the listed runs, which are in (r, id) order.
+// bin (n): each star's bin; counted: the orbit step has counted the bins.
+// scratch: n indices.
+void launch_bin_sort(const SegLayout& L, BinWork& B, const uint32_t* bin, const RecA* rec,
+                     uint32_t* order, uint32_t* scratch, bool counted, uint32_t* err,
+                     cudaStream_t st);
 
-// keys of the current state (radius_key of r, id) and the payload (if pay)
-void launch_make_keys(const SegLayout& L, const double* r, const double* vr,
-                      const double* vt, const double* m, const uint32_t* id,
-                      uint64_t* keys, Payload* pay, cudaStream_t st);
+// keys of the current state (radius_key of r, id)
+void launch_make_keys(const SegLayout& L, const double* r, const uint32_t* id, uint64_t* keys,
+                      cudaStream_t st);
+// records of the current state (for the initial ordering)
+void launch_make_records(const SegLayout& L, const double* r, const double* vr,
+                         const double* vt, const double* m, const uint32_t* id, RecA* ra,
+                         RecB* rb, cudaStream_t st);
 
 // keys = id (for the (r, id) order at initialisation), and radius keys of
 // the stars in the order of a permutation
@@ -158,17 +215,36 @@ void launch_id_keys(const SegLayout& L, const uint32_t* id, uint64_t* keys, cuda
 void launch_rekey_radius(const SegLayout& L, const uint32_t* perm, const double* r,
                          const uint32_t* id, uint64_t* keys, cudaStream_t st);
 
-// sorted (keys, vals) + payload -> SoA state (r, x, vr, vt, m, id, r_old, c);
-// with tile_m and tile_mx (and r_old, c) also the potential's per-tile sums
-// over the bound stars after the orbit step (launch_potential with
-// nb_sub and sums_ready then skips them)
-void launch_gather(const SegLayout& L, const uint64_t* keys, const uint32_t* vals,
-                   const Payload* pay, double* r, double* x, double* vr, double* vt,
-                   double* m, uint32_t* id, double* r_old, double* c, cudaStream_t st,
-                   double* tile_m = nullptr, double* tile_mx = nullptr,
-                   const double* Rp = nullptr, double* Rout = nullptr,
-                   const double* Ap = nullptr, double* Aout = nullptr,
-                   bool packed = false);
+// records in the order of a permutation -> SoA state (initial ordering)
+void launch_gather(const SegLayout& L, const uint32_t* perm, const RecA* ra, const RecB* rb,
+                   double* r, double* x, double* vr, double* vt, double* m, uint32_t* id,
+                   cudaStream_t st);
+// The timestep's gather: r, x, m, id in (r, id) order with the potential's
+// per-tile sums over the bound stars (launch_potential with sums_ready then
+// skips them); order_out: the star's old index at each new position; r_out and
+// x_out must not be r_in (the old radii, still wanted for the energy
+// correction).  exact: order_in is in (r, id) order already; else bin order.
+// For the escaped stars also r_old (the old radius, +inf for those that
+// escaped before) and c.  Rp -> Rout, Ap -> Aout: attributes that go along.
+// With bins, their counts and scan words are zeroed for the next step.
+void launch_gather_step(const SegLayout& L, BinWork* B, const uint32_t* order_in,
+                        const RecA* ra, const RecB* rb, const double* r_in, double* r_out,
+                        double* x_out, double* m, uint32_t* id, uint32_t* order_out,
+                        double* r_old, double* c, double* tile_m, double* tile_mx,
+                        const double* Rp, double* Rout, const double* Ap, double* Aout,
+                        bool exact, cudaStream_t st);
+// Phi_new(r_old) of every star of the old order into its RecB (w), r_in and
+// x_in the old radii and reciprocals (sorted), r, x, phi, node the new table.
+// div_form: Eq. 6's division form (FP64 modes; node may be null), else the
+// shell slope of the node records.
+void launch_phi_old(const SegLayout& L, const double* r_in, const double* x_in, const double* r,
+                    const double* x, const double* phi, const double4_32a* node, RecB* rb,
+                    bool div_form, cudaStream_t st);
+// the new velocities into place, corrected for the changing potential
+// (correct false: as they are)
+void launch_velocities(const SegLayout& L, const uint32_t* order, const RecB* rb,
+                       const double* phi, const double* m, double* vr, double* vt, bool correct,
+                       cudaStream_t st);
 
 // potential: per-tile sums then the tile-local scans (Eqs. 1-5 in scan
 // form).  nb_sub: subtract esc_step from nb (after the orbit step).
@@ -289,7 +365,8 @@ void launch_potential_tables(const SegLayout& L, const double* r, const double* 
                              BucketWork& B, cudaStream_t st);
 
 // Menc (precision 0 and 1): the slope of Phi in 1/r across shell k.
-// precision 1 (mixed): launch_orbit runs four kernels (turning points,
+// launch_orbit writes the stars' records, and with bins their sort bins (count:
+// counted too) or else their sort keys.  precision 1 (mixed): it runs four kernels (turning points,
 // FP32 sampler, FP64 continuation of the pending stars, finishing) and
 // needs n records orb (E, J, c0 = (r_max + r_min) / 2, c1 = (r_max -
 // r_min) / 4, from the turning-point kernel, for the sampling kernels), a
@@ -325,12 +402,13 @@ void launch_orbit(const SegLayout& L, int precision, int max_trials, const doubl
                   const double* x, const double* phi, const double* Menc,
                   const double* vr,
                   const double* vt, const double* m, const uint32_t* id, const uint32_t* step,
-                  uint64_t* keys, Payload* pay, const OrbitStageOut* dbg, int block,
+                  uint64_t* keys, RecA* ra, RecB* rb, const OrbitStageOut* dbg, int block,
                   int variant, const BucketArgs& ba, double* tp_min, double* tp_max,
                   uint32_t* plist, uint32_t* pcount, cudaStream_t st,
                   bool with_turning = true, const double* Rv = nullptr, double* Rp = nullptr,
                   const EnvWork* env = nullptr, const double* Av = nullptr,
-                  double* Ap = nullptr, double4_32a* orb = nullptr, bool packed = false);
+                  double* Ap = nullptr, double4_32a* orb = nullptr,
+                  const BinWork* bins = nullptr, uint32_t* bin = nullptr, bool count = false);
 // the turning-point kernel alone (mixed mode; launch_orbit(..., false)
 // then runs the sampling kernel only)
 void launch_turning(const SegLayout& L, const double* r, const double* x, const double* phi,
@@ -346,14 +424,6 @@ constexpr int kRelaxVariants = 3;  // relaxation kernel register caps (launch_re
 
 // commits the step: nb, escaper statistics and budget (from the gathered
 // r_old and c of the escaped range), dt; resets the per-step counters
-// energy correction in mixed mode: shell of r_old from the bucket index of
-// the new table (nb - esc_step bound stars), Phi from the enclosed mass
-void launch_correction_mixed(const SegLayout& L, const double* r, const double* x,
-                             const double* phi, const double* Menc,
-                             const BucketArgs& ba, double* vr, double* vt, const double* r_old,
-                             const double* c, const double* m, cudaStream_t st,
-                             bool div_form = false);
-
 void launch_step_end(const SegLayout& L, uint32_t* step, const double* r_old, const double* c,
                      const double* m, cudaStream_t st);
 
@@ -378,7 +448,7 @@ void launch_nb_from_keys(const SegLayout& L, const uint64_t* keys, cudaStream_t 
 void launch_recip(int64_t n, const double* r, double* x, cudaStream_t st);
 void launch_make_t32(int64_t n, const double* x, const double* phi, float2* t32,
                      cudaStream_t st);
-void launch_unpack_orbit(int64_t n, const uint64_t* keys, const Payload* pay, double* r_new,
+void launch_unpack_orbit(int64_t n, const RecA* ra, const RecB* rb, double* r_new,
                          double* vr_new, double* vt_new, cudaStream_t st);
 void sort_prepare();
 // look-back polls and tie-fix moves before the sort's waits give up (<= 0:

@@ -189,10 +189,11 @@ __device__ __forceinline__ int64_t bisect_rmin64(const Table64& T, const Star& s
 
 // g(s) with Phi from the FP64 table
 __device__ __forceinline__ double g64(const Table64& T, const Star& st, double c0, double c1,
-                                      double s, double& rs, double& ph, double& Q) {
+                                      double s, double& rs, double& ph, double& Q, int64_t& i) {
   rs = c0 + c1 * (s * (3.0 - s * s));
   const double drds = (3.0 * c1) * (1.0 - s * s);
-  ph = phi_of_r(T, rs);
+  i = shell_of(T, rs);
+  ph = phi_in_shell(T, i, rs);
   const double L = div_rn(st.J, rs);
   Q = scale_up<1>(st.E - ph) - L * L;
   if (!(Q > 0.0)) return 0.0;
@@ -398,10 +399,10 @@ __device__ __forceinline__ int shell32_of(const double4_32a* __restrict__ nd, in
 __device__ __forceinline__ void point64(const double4_32a* __restrict__ nd, int64_t nb,
                                         const Star& st, double c0, double c1, double sv, int sh,
                                         double& rs, double& xs, double& ph, double& L,
-                                        double& Q) {
+                                        double& Q, int& i64) {
   rs = c0 + c1 * (sv * (3.0 - sv * sv));
   double4_32a a;
-  const int64_t i64 = fix_shell_nodes(nd, nb, sh, rs, a);
+  i64 = (int)fix_shell_nodes(nd, nb, sh, rs, a);
   xs = div_rn(1.0, rs);
   ph = i64 < 0 ? a.z : a.z + a.w * (a.y - xs);
   L = st.J * xs;
@@ -417,14 +418,14 @@ __device__ __forceinline__ void point64(const double4_32a* __restrict__ nd, int6
 __device__ __forceinline__ void point64_div_sa(const double4_32a* __restrict__ nd, int64_t nb,
                                                const Star& st, double c0, double c1, double sa,
                                                int sh, double& rs, double& ph, double& Q,
-                                               double& L) {
+                                               double& L, double& xq, int& i) {
   rs = c0 + c1 * sa;
   double4_32a a;
-  const int64_t i = fix_shell_nodes(nd, nb, sh, rs, a);
+  i = (int)fix_shell_nodes(nd, nb, sh, rs, a);
+  xq = div_rn(1.0, rs);
   if (i < 0) {
     ph = a.z;  // node 0's Phi: the central constant
   } else {
-    const double xq = div_rn(1.0, rs);
     double xj1 = 0.0, pj1 = 0.0;
     if (i + 1 < nb) {
       const double4_32a b = nd[i + 1];
@@ -441,8 +442,8 @@ __device__ __forceinline__ void point64_div_sa(const double4_32a* __restrict__ n
 __device__ __forceinline__ void point64_div(const double4_32a* __restrict__ nd, int64_t nb,
                                             const Star& st, double c0, double c1, double sv,
                                             int sh, double& rs, double& ph, double& Q,
-                                            double& L) {
-  point64_div_sa(nd, nb, st, c0, c1, sv * (3.0 - sv * sv), sh, rs, ph, Q, L);
+                                            double& L, double& xq, int& i) {
+  point64_div_sa(nd, nb, st, c0, c1, sv * (3.0 - sv * sv), sh, rs, ph, Q, L, xq, i);
 }
 
 // g(s) of FP64 mode at the point of point64_div, sb = 1 - s^2
@@ -956,9 +957,10 @@ __device__ __noinline__ double g64_sample(const double4_32a* __restrict__ nd, in
   s.E = E;
   s.J = J;
   const float c0f = f32_rn(c0), c1f = f32_rn(c1);
-  double rs, ph, Q, L;
+  double rs, ph, Q, L, xq;
+  int i;
   point64_div_sa(nd, nb, s, c0, c1, g_env_sa[j],
-                 shell32_of(nd, (int)nb, BK, c0f, c1f, c_s32[j]), rs, ph, Q, L);
+                 shell32_of(nd, (int)nb, BK, c0f, c1f, c_s32[j]), rs, ph, Q, L, xq, i);
   return g_of_point_sb(c1, g_env_sb[j], Q);
 }
 
@@ -1274,12 +1276,14 @@ __device__ __forceinline__ void pending_star(Seg S, int max_trials, const uint32
               shell32_of(BA.node + sb, (int)nbc, BK, c0f, c1f, 2.0f * u01f(w.y) - 1.0f);
           double g64v;
           if (kExact) {
-            double rs, ph, Q, L;
-            point64_div(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, ph, Q, L);
+            double rs, ph, Q, L, xq;
+            int i;
+            point64_div(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, ph, Q, L, xq, i);
             g64v = g_of_point(c1, sv, Q);
           } else {
             double rs, xs, ph, L, Q;
-            point64(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, xs, ph, L, Q);
+            int i;
+            point64(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, xs, ph, L, Q, i);
             g64v = pos_num(Q) ? div_rn((3.0 * c1) * (1.0 - sv * sv), sqrt_rn(Q)) : 0.0;
           }
           ++n64;
@@ -1318,16 +1322,29 @@ __global__ void __launch_bounds__(128) k_pending64(Seg S, int max_trials, const 
   }
 }
 
-// the star's sort key and payload record; packed: the key's low 24 bits go
-// to the record and the star's index in the segment takes their place
-__device__ __forceinline__ void put_key(uint64_t* keys, Payload* pay, Payload& P, int64_t p,
-                                        int64_t sb, uint64_t key, bool packed) {
-  if (packed) {
-    P.pad = (uint32_t)(key & kPackMask);
-    key = (key & ~kPackMask) | (uint64_t)(p - sb);
+// the star's records, and its bin (counted too with cnt) or its sort key
+struct BinOut {
+  uint32_t* bin = nullptr;
+  uint32_t* cnt = nullptr;
+  const int64_t* cbase = nullptr;
+  const int* esh = nullptr;
+};
+
+// s: shell + 1 of a bound star, -1 for an escaped one
+__device__ __forceinline__ void put_star(const Seg& S, const BinOut& O, uint64_t* keys, RecA* ra,
+                                         RecB* rb, RecA& A, const RecB& B, int64_t p, int c,
+                                         int64_t s) {
+  if (O.bin) {
+    const int64_t nc = S.off[c + 1] - S.off[c];
+    if (s < 0) s = nc + 1 + (int64_t)(A.id >> O.esh[c]);
+    A.bin = (uint32_t)(O.cbase[c] + s);
+    O.bin[p] = A.bin;
+    if (O.cnt) atomicAdd(O.cnt + A.bin, 1u);
+  } else {
+    keys[p] = radius_key(A.r, A.id);
   }
-  keys[p] = key;
-  pay[p] = P;
+  store_rec(ra + p, A);
+  store_rec(rb + p, B);
 }
 
 // kPrec: 0 FP64 by bisection (Appendix A's kernels: brackets, envelope and
@@ -1343,13 +1360,13 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
                                                const double* Menc, const double* vr,
                                                const double* vt, const double* m,
                                                const uint32_t* id, const uint32_t* step_p,
-                                               uint64_t* keys, Payload* pay, int64_t* esc,
-                                               OrbitStageOut dbg, BucketArgs BA,
+                                               uint64_t* keys, RecA* ra, RecB* rb,
+                                               int64_t* esc, OrbitStageOut dbg, BucketArgs BA,
                                                const double* tp_min, const double* tp_max,
                                                const double4_32a* orb,
                                                int64_t n, const double* Rv, double* Rp,
                                                const double* Fx, const double* Av,
-                                               double* Ap, bool packed) {
+                                               double* Ap, BinOut bo) {
   pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
@@ -1359,8 +1376,13 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
   const int64_t k = p - sb;
   const double rk = r[p], vrk = vr[p], vtk = vt[p];
   const uint32_t idk = id[p];
-  Payload P;
-  P.vr = vrk; P.vt = vtk; P.m = m[p]; P.r_old = rk; P.c = 0.0; P.id = idk; P.pad = 0;
+  const double inf = __longlong_as_double((long long)kInfBits);
+  RecA A;
+  A.r = rk; A.x = 0.0; A.m = m[p]; A.id = idk; A.bin = 0u;
+  RecB B;
+  B.vr = vrk; B.vt = vtk; B.c = 0.0; B.w = 0.0;
+  double x_new = 0.0;
+  int shell = -2;  // of r_new in the current table; -2: not found on the way
   double r_new = rk, rmin = rk, rmax = rk, F = 0.0;
   int code = 0, trials = 0;
   unsigned long long viol = 0;
@@ -1370,15 +1392,15 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
   if (Ap) Ap[p] = Av[p];  // and the binary's semi-major axis
   if (k >= nbc) {
     // escaped in an earlier step: stays at the end, ordered by id
-    put_key(keys, pay, P, p, sb, radius_key(rk, idk), packed);
+    put_star(S, bo, keys, ra, rb, A, B, p, c, -1);
     if (dbg.code) dbg.code[p] = 1;
     return;
   }
   if (Rv && lt0(Rv[p])) {
     // merged into its partner in this step (sticky spheres): it leaves
     // with no mass, draws nothing, and carries off no energy
-    put_key(keys, pay, P, p, sb, radius_key(__longlong_as_double(0x7FF0000000000000ll), idk),
-            packed);
+    A.r = inf;
+    put_star(S, bo, keys, ra, rb, A, B, p, c, -1);
     if (dbg.code) dbg.code[p] = 1;
     const unsigned full = __activemask();
     const unsigned peers = __match_any_sync(full, c);
@@ -1407,9 +1429,9 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
   if (!lt0(s.E)) {
     escaped = true;
     code = 1;
-    r_new = __longlong_as_double(0x7FF0000000000000ll);
+    r_new = inf;
     // energy carried off: the star's energy in the field of the others
-    P.c = __ldg(T.phi + k) + div_rn(P.m, rk) + scale_down<1>(vrk * vrk + vtk * vtk);
+    B.c = __ldg(T.phi + k) + div_rn(A.m, rk) + scale_down<1>(vrk * vrk + vtk * vtk);
   } else {
     int64_t jmax, jmin;
     Buckets BK;
@@ -1440,7 +1462,8 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
       double gmax = 0.0;
       for (int j = 0; j <= 20; ++j) {
         double rs, ph, Q;
-        double g = g64(T, s, c0, c1, c_s64[j], rs, ph, Q);
+        int64_t i;
+        double g = g64(T, s, c0, c1, c_s64[j], rs, ph, Q, i);
         if (g > gmax) gmax = g;
       }
       F = 1.2 * gmax;
@@ -1454,12 +1477,14 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
           const double Xp = u01(w.z, w.w);
           const double sv = sym_double(sym_int(w.x, w.y));  // 2 X - 1, exact
           double rs, ph, Q;
-          const double g = g64(T, s, c0, c1, sv, rs, ph, Q);
+          int64_t i;
+          const double g = g64(T, s, c0, c1, sv, rs, ph, Q, i);
           if (g > F) ++viol;
           if (F * Xp < g) {
             rs_a = rs;
             ph_a = ph;
             Q_a = Q;
+            shell = (int)i;
             code = 0;
             trials = t + 1;
             break;
@@ -1474,9 +1499,10 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
           U4 sg = g.block(kTagSgn, 0u);
           draws_keep(S, c, g);
           r_new = rs_a;
-          P.vr = (sg.x & 1u) ? -sq : sq;
-          P.vt = div_rn(s.J, rs_a);
-          P.c = __ldg(T.phi + k) - ph_a;
+          x_new = div_rn(1.0, rs_a);
+          B.vr = (sg.x & 1u) ? -sq : sq;
+          B.vt = div_rn(s.J, rs_a);
+          B.c = __ldg(T.phi + k) - ph_a;
           ph_new = ph_a;
         }
       }
@@ -1514,26 +1540,31 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
           const double sv = sym_double(sym_int(w.x, w.y));
           const int guess = shell32_of(BA.node + sb, nb32, BK, c0f, c1f, 2.0f * u01f(w.y) - 1.0f);
           double rs, ph, Q, vtn;
-          if (kPrec == 2) {
-            point64_div(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, ph, Q, vtn);  // v_t = J / r
-          } else {
-            double xs;
-            point64(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, xs, ph, vtn, Q);
-          }
+          if (kPrec == 2)  // v_t = J / r
+            point64_div(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, ph, Q, vtn, x_new, shell);
+          else
+            point64(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, x_new, ph, vtn, Q, shell);
           if (!pos_num(Q)) Q = 0.0;
           const double sq = sqrt_rn(Q);
           U4 sg = g.block(kTagSgn, 0u);
           draws_keep(S, c, g);
           r_new = rs;
-          P.vr = (sg.x & 1u) ? -sq : sq;
-          P.vt = vtn;
-          P.c = __ldg(T.phi + k) - ph;
+          B.vr = (sg.x & 1u) ? -sq : sq;
+          B.vt = vtn;
+          B.c = __ldg(T.phi + k) - ph;
           ph_new = ph;
         }
       }
     }
   }
-  put_key(keys, pay, P, p, sb, radius_key(r_new, idk), packed);
+  // a star that stays in place has no point from the way: its shell by bisection
+  if (!escaped && shell == -2) {
+    x_new = __ldg(T.x + k);
+    if (bo.bin) shell = (int)shell_of(T, rk);
+  }
+  A.r = r_new;
+  A.x = x_new;
+  put_star(S, bo, keys, ra, rb, A, B, p, c, escaped ? -1 : shell + 1);
 
   // statistics: one atomic per counter per segment present in the warp
   const unsigned full = __activemask();
@@ -1557,79 +1588,6 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
   if (dbg.F) dbg.F[p] = F;
   if (dbg.code) dbg.code[p] = code;
   if (dbg.trials) dbg.trials[p] = trials;
-}
-
-// Energy correction (section 2.1 step 6) in mixed mode, after the new
-// potential and its bucket index: the shell of r_old in the new table from
-// the index (FP32 1/r, moved to the exact FP64 shell by integer compares of
-// the radii), Phi_new(r_old) = Phi_i + M_i (1/r_i - 1/r_old) from the
-// enclosed mass of that shell (Eq. 6 without its division), then
-// T' = T + 1/2 [(Phi_new(r_old) - Phi_new,k) - c] clamped at 0 and both
-// velocity components scaled by sqrt(T'/T), as in the FP64 kernel.
-// kDiv (FP64 mode): Phi_new(r_old) by Eq. 6's division form and the FP64
-// kernel's comparisons, as the FP64 statement computes them, the shell found
-// the same way (the shell of a radius is unique).
-template <bool kDiv>
-__global__ void __launch_bounds__(128, 12) k_correction_mixed(Seg S, const int64_t* esc,
-                                                          const double* r, const double* x,
-                                                          const double* phi,
-                                                          const double* Menc, BucketArgs BA,
-                                                          double* vr, double* vt,
-                                                          const double* r_old, const double* cc,
-                                                          const double* m, int64_t n) {
-  pdl_enter();
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const int c = seg_find(S.off, S.n_seg, p);
-  const int64_t sb = __ldg(S.off + c);
-  const int64_t nbc = S.nb[c] - esc[c];
-  if (p - sb >= nbc) return;
-  const double ro = r_old[p];
-  const double xo = div_rn(1.0, ro);
-  Buckets BK;
-  const int4 pr = BA.prm[c];
-  BK.start = BA.start + BA.off[c];
-  BK.base = BA.base[c];
-  BK.shift = pr.x;
-  BK.nbk = pr.y;
-  BK.lo = pr.z;
-  BK.hi = pr.w;
-  const float xq[1] = {f32_rn(xo)};
-  int sh[1];
-  shells32_bk<1>(NodeKeys{BA.node + sb}, (int)nbc, BK, xq, sh);
-  double4_32a nd;
-  const int64_t i = fix_shell_nodes(BA.node + sb, nbc, sh[0], ro, nd);
-  double pn;
-  if (!kDiv) {
-    pn = i < 0 ? nd.z : nd.z + nd.w * (nd.y - xo);
-  } else if (i < 0) {
-    pn = nd.z;
-  } else {
-    double xj1 = 0.0, pj1 = 0.0;
-    if (i + 1 < nbc) {
-      const double4_32a nx = BA.node[sb + i + 1];
-      xj1 = nx.y;
-      pj1 = nx.z;
-    }
-    const double den = nd.y - xj1;
-    pn = !(den > 0.0) ? nd.z : nd.z + div_rn(nd.y - xo, den) * (pj1 - nd.z);
-  }
-  const double a = vr[p], b = vt[p];
-  const double Tk = scale_down<1>(a * a + b * b);
-  const double dnew = pn - phi[p];
-  double Tp = Tk + scale_down<1>(dnew - cc[p]);
-  bool clamp = false;
-  if (kDiv ? Tp < 0.0 : lt0(Tp)) {
-    clamp_energy_add(S.stats, c, m[p], Tp);
-    Tp = 0.0;
-    clamp = true;
-  }
-  if (kDiv ? Tk > 0.0 : pos_num(Tk)) {
-    const double f = sqrt_rn(div_rn(Tp, Tk));
-    vr[p] = a * f;
-    vt[p] = b * f;
-  }
-  if (clamp) stat_add(S.stats, c, kStClamps, 1ull);
 }
 
 // ------------------------------------------------------ potential grid
@@ -1963,20 +1921,6 @@ void free_env(EnvWork& W, cudaStream_t st) {
   W = EnvWork();
 }
 
-void launch_correction_mixed(const SegLayout& L, const double* r, const double* x,
-                             const double* phi, const double* Menc,
-                             const BucketArgs& ba, double* vr, double* vt, const double* r_old,
-                             const double* c, const double* m, cudaStream_t st,
-                             bool div_form) {
-  if (!L.n) return;
-  if (div_form)
-    launch_k(k_correction_mixed<true>, (unsigned)((L.n + 127) / 128), 128, 0, st,
-        L.dev(), L.esc_step, r, x, phi, Menc, ba, vr, vt, r_old, c, m, L.n);
-  else
-    launch_k(k_correction_mixed<false>, (unsigned)((L.n + 127) / 128), 128, 0, st,
-        L.dev(), L.esc_step, r, x, phi, Menc, ba, vr, vt, r_old, c, m, L.n);
-}
-
 void launch_turning(const SegLayout& L, const double* r, const double* x, const double* phi,
                     const double* Menc, const double* vr, const double* vt,
                     const BucketArgs& ba, double* tp_min, double* tp_max, double4_32a* orb,
@@ -1992,13 +1936,20 @@ void launch_orbit(const SegLayout& L, int precision, int max_trials, const doubl
                   const double* x, const double* phi, const double* Menc,
                   const double* vr, const double* vt, const double* m, const uint32_t* id,
                   const uint32_t* step,
-                  uint64_t* keys, Payload* pay, const OrbitStageOut* dbg, int block,
+                  uint64_t* keys, RecA* ra, RecB* rb, const OrbitStageOut* dbg, int block,
                   int variant, const BucketArgs& ba, double* tp_min, double* tp_max,
                   uint32_t* plist, uint32_t* pcount, cudaStream_t st, bool with_turning,
                   const double* Rv, double* Rp, const EnvWork* env, const double* Av,
-                  double* Ap, double4_32a* orb, bool packed) {
+                  double* Ap, double4_32a* orb, const BinWork* bins, uint32_t* bin, bool count) {
   if (!L.n) return;
   OrbitStageOut d;
+  BinOut bo;
+  if (bins) {
+    bo.bin = bin;
+    bo.cnt = count ? bins->cnt : nullptr;
+    bo.cbase = bins->cbase;
+    bo.esh = bins->esh;
+  }
   EnvWork W;
   if (env) W = *env;
   double* Fx = W.gmax;
@@ -2018,8 +1969,8 @@ void launch_orbit(const SegLayout& L, int precision, int max_trials, const doubl
                                              tp_min, tp_max, orb, L.n)
 #define CMC_ORBIT(P, B, T)                                                                  \
   launch_k(k_orbit<P, B, T>, grid, block, 0, st, L.dev(), max_trials, r, x, phi, Menc, vr, vt, \
-                                           m, id, step, keys, pay, L.esc_step, d, ba, tp_min, \
-                                           tp_max, orb, L.n, Rv, Rp, Fx, Av, Ap, packed)
+           m, id, step, keys, ra, rb, L.esc_step, d, ba, tp_min, tp_max, orb, L.n, Rv, Rp, Fx, \
+           Av, Ap, bo)
 #define CMC_SAMPLED(B, T, X)                                                                \
   do {                                                                                      \
     if (with_turning) CMC_TURN(B);                                                          \

@@ -84,19 +84,24 @@ __device__ __forceinline__ TR tile_of(const Seg& S, const int64_t* esc, int64_t 
 }
 
 // --------------------------------------------------------------- gather
-__global__ void k_make_keys(int64_t n, const double* r, const double* vr, const double* vt,
-                            const double* m, const uint32_t* id, uint64_t* keys,
-                            Payload* pay) {
+__global__ void k_make_keys(int64_t n, const double* r, const uint32_t* id, uint64_t* keys) {
+  pdl_enter();
+  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p < n) keys[p] = radius_key(r[p], id[p]);
+}
+
+__global__ void k_make_records(int64_t n, const double* r, const double* vr, const double* vt,
+                               const double* m, const uint32_t* id, RecA* ra, RecB* rb) {
   pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
-  double rr = r[p];
-  uint32_t ii = id[p];
-  keys[p] = radius_key(rr, ii);
-  if (!pay) return;
-  Payload P;
-  P.vr = vr[p]; P.vt = vt[p]; P.m = m[p]; P.r_old = rr; P.c = 0.0; P.id = ii; P.pad = 0;
-  pay[p] = P;
+  const double rr = r[p];
+  RecA A;
+  A.r = rr; A.x = lt_inf(rr) ? div_rn(1.0, rr) : 0.0; A.m = m[p]; A.id = id[p]; A.bin = 0u;
+  store_rec(ra + p, A);
+  RecB B;
+  B.vr = vr[p]; B.vt = vt[p]; B.c = 0.0; B.w = 0.0;
+  store_rec(rb + p, B);
 }
 
 __global__ void k_id_keys(int64_t n, const uint32_t* id, uint64_t* keys) {
@@ -114,65 +119,357 @@ __global__ void k_rekey_radius(int64_t n, const uint32_t* perm, const double* r,
   keys[p] = radius_key(r[q], id[q]);
 }
 
-__global__ void k_gather(int64_t n, const uint64_t* __restrict__ keys,
-                         const uint32_t* __restrict__ vals, const Payload* __restrict__ pay,
+__global__ void k_gather(int64_t n, const uint32_t* perm, const RecA* ra, const RecB* rb,
                          double* r, double* x, double* vr, double* vt, double* m,
-                         uint32_t* id, double* r_old, double* c) {
+                         uint32_t* id) {
   pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
-  uint64_t k = keys[p];
-  const uint32_t v = vals[p];
+  const uint32_t v = perm[p];
   if ((int64_t)v >= n) return;  // only after a reported sort failure
-  const Payload P = pay[v];
-  double rr, xx;
-  if (key_is_escaper(k)) { rr = __longlong_as_double(0x7FF0000000000000ll); xx = 0.0; }
-  else { rr = __longlong_as_double((long long)k); xx = div_rn(1.0, rr); }
-  r[p] = rr; x[p] = xx; vr[p] = P.vr; vt[p] = P.vt; m[p] = P.m; id[p] = P.id;
-  if (r_old) r_old[p] = P.r_old;
-  if (c) c[p] = P.c;
+  const RecA A = load_rec(ra + v);
+  const RecB B = load_rec(rb + v);
+  r[p] = A.r; x[p] = A.x; vr[p] = B.vr; vt[p] = B.vt; m[p] = A.m; id[p] = A.id;
 }
 
-// The gather of one tile with the potential's per-tile sums of m and m x
-// (k_tile_sums over the bound stars after the orbit step) taken from the
-// values it has just written: the same striped element order and tree, so
-// the same sums, without reading m and x back.
-__global__ void __launch_bounds__(kThreads) k_gather_sums(
-    Seg S, const int64_t* esc, int64_t n, const uint64_t* __restrict__ keys,
-    const uint32_t* __restrict__ vals, const Payload* __restrict__ pay, double* r, double* x,
-    double* vr, double* vt, double* m, uint32_t* id, double* r_old, double* c, double* tile_m,
-    double* tile_mx, const double* Rp, double* Rout, const double* Ap, double* Aout,
-    bool packed) {
+// The timestep's gather, one block per tile of kTile new positions.  Each star
+// counts the members of its bin's run that come before it in (r, id) order --
+// runs hold one or two stars, so a few neighbours -- and writes its record to
+// its place.  A star belongs to the tile its place falls in, so the block walks
+// the tile and kRunMax positions on each side: a run of up to kRunMax stars
+// across the tile's edge is seen whole.  Longer runs are in order already
+// (k_long_runs).
+//
+// Bound by the random 32-byte reads of the records (0.215 ms at N = 1e7 for
+// those and the writes alone).  The walk is a pipeline of sub-tiles of one star
+// per thread: while the star of sub-tile k - 1 looks at its neighbours (radii
+// and bins of sub-tiles k - 2 .. k in a shared-memory ring of four), the record
+// of k + 1 and the index of k + 2 are on their way, so that the reads go on
+// through the ranking: 0.31 ms (0.42 with the whole tile loaded first).
+//
+// The potential's per-tile sums of m and m x (k_tile_sums over the bound stars
+// after the orbit step) come from the values just written, in the same
+// striped element order and tree, so they are the same sums: half the block
+// sums m, the other half m x.
+// Blocks of 512 threads, three to an SM (40 registers: a spill would miss the
+// L1 under the random reads, which made the kernel twice as slow); while there
+// are fewer tiles than SMs blocks of 1024, whose walk is half as long.
+constexpr int kGatWin = kTile + 2 * kRunMax;
+constexpr int kGatFewTiles = 152;
+
+struct GatherOut {
+  double *r, *x, *m;
+  uint32_t *id, *order;
+  double *r_old, *c;        // escaped stars only
+  double *tile_m, *tile_mx;
+  const double *Rp, *Ap;    // attributes that go along (may be null)
+  double *R, *A;
+};
+
+template <bool kExact, int kGatThreads>
+__global__ void __launch_bounds__(kGatThreads, kGatThreads == 512 ? 3 : 1) k_gather_step(
+    Seg S, const int64_t* esc, int64_t n, const uint32_t* order, const RecA* ra, const RecB* rb,
+    const double* r_in, GatherOut O, uint32_t* cnt, int64_t n_bins, unsigned long long* desc,
+    int64_t n_desc, uint32_t* ctl) {
   pdl_enter();
-  __shared__ double s[kThreads];
+  constexpr int kGatSub = (kGatWin + kGatThreads - 1) / kGatThreads;  // the last one partial
+  constexpr int kGatRing = 4 * kGatThreads;
+  static_assert(kRunMax < kGatThreads, "a run's reach is the next sub-tile");
+  static_assert(kGatThreads >= 2 * kThreads, "two trees of kThreads");
+  __shared__ unsigned long long s_r[kGatRing];
+  __shared__ uint32_t s_bin[kGatRing];
+  __shared__ double s_red[2 * kThreads];
+  const int t = threadIdx.x;
   TR R = tile_of(S, esc, blockIdx.x, true);
-  double am = 0.0, ax = 0.0;
-#pragma unroll 4
-  for (int i = 0; i < kPer; ++i) {
-    const int64_t p = R.begin + (int64_t)i * kThreads + threadIdx.x;
-    if (p >= R.end) continue;
-    uint64_t k = keys[p];
-    // packed keys: the star's index in the segment in the low 24 bits
-    const int64_t v = packed ? R.seg_begin + (int64_t)(k & kPackMask) : (int64_t)vals[p];
-    if (v >= n) continue;  // only after a reported sort failure
-    const Payload P = pay[v];
-    if (packed) k = (k & ~kPackMask) | (uint64_t)P.pad;
-    double rr, xx;
-    if (key_is_escaper(k)) { rr = __longlong_as_double(0x7FF0000000000000ll); xx = 0.0; }
-    else { rr = __longlong_as_double((long long)k); xx = div_rn(1.0, rr); }
-    r[p] = rr; x[p] = xx; vr[p] = P.vr; vt[p] = P.vt; m[p] = P.m; id[p] = P.id;
-    r_old[p] = P.r_old;
-    c[p] = P.c;
-    if (Rout) Rout[p] = Rp[v];
-    if (Aout) Aout[p] = Ap[v];
-    if (p < R.bound_end) {
-      am = am + P.m;
-      ax = ax + P.m * xx;
+  const int len = (int)(R.end - R.begin);
+  // window element w = local position w - kRunMax, within the segment
+  const int64_t w0 = R.begin - kRunMax;
+  const int wa = w0 < R.seg_begin ? (int)(R.seg_begin - w0) : 0;
+  const int64_t we = S.off[R.seg + 1] - w0;
+  const int wb = we < kGatWin ? (int)we : kGatWin;
+  constexpr uint32_t kNone = 0xFFFFFFFFu;  // no star (and a bin that no star has)
+  auto index_of = [&](int w) {
+    uint32_t v = w >= wa && w < wb ? order[w0 + w] : kNone;
+    return (int64_t)v < n ? v : kNone;  // (out of range only after a reported sort failure)
+  };
+  RecA A;
+  A.bin = kNone;
+  double px = 0.0, pm = 0.0;  // the star being placed (its r and bin are in the ring)
+  uint32_t pid = 0u, pv = kNone;
+  uint32_t v = index_of(t), v1 = index_of(t + kGatThreads);
+  if (v != kNone) A = load_rec(ra + v);
+#pragma unroll 1
+  for (int k = 0; k <= kGatSub; ++k) {
+    const int w = k * kGatThreads + t;
+    RecA A1;
+    A1.bin = kNone;
+    if (v1 != kNone) A1 = load_rec(ra + v1);
+    const uint32_t v2 = index_of(w + 2 * kGatThreads);
+    s_r[w & (kGatRing - 1)] = ubits(A.r);
+    s_bin[w & (kGatRing - 1)] = A.bin;
+    if (!kExact) __syncthreads();
+    // the star of the sub-tile before: to the start of its run plus the
+    // members before it
+    if (pv != kNone) {
+      const int wp = w - kGatThreads;
+      const unsigned long long r = s_r[wp & (kGatRing - 1)];
+      int f = wp;
+      if (!kExact) {
+        const uint32_t b = s_bin[wp & (kGatRing - 1)];
+        auto bin_at = [&](int q) { return s_bin[q & (kGatRing - 1)]; };
+        auto r_at = [&](int q) { return s_r[q & (kGatRing - 1)]; };
+        int before = 0, left = 0, right = 0, equal = 0;
+        auto look = [&](int q) {
+          const unsigned long long rq = r_at(q);
+          const bool eq = rq == r && ra[order[w0 + q]].id < pid;
+          before += rq < r || eq;
+          equal += eq;
+        };
+        for (int q = wp - 1; q >= 0 && left < kRunMax && bin_at(q) == b; --q, ++left) look(q);
+        for (int q = wp + 1; q < kGatWin && right < kRunMax && bin_at(q) == b; ++q, ++right)
+          look(q);
+        if (left + 1 + right <= kRunMax) f = wp - left + before;
+        else equal = left > 0 && r_at(wp - 1) == r ? (left > 1 && r_at(wp - 2) == r ? 2 : 1) : 0;
+        // a group of equal finite radii counts once, at its second star
+        if (equal == 1 && r < kInfBits && f >= kRunMax && f < kRunMax + len)
+          stat_add(S.stats, R.seg, kStTies, 1ull);
+      }
+      f -= kRunMax;
+      if (f >= 0 && f < len) {
+        const int64_t p = R.begin + f;
+        O.r[p] = __longlong_as_double((long long)r);
+        O.x[p] = px;
+        O.m[p] = pm;
+        O.id[p] = pid;
+        O.order[p] = pv;
+        if (O.R) O.R[p] = O.Rp[pv];
+        if (O.A) O.A[p] = O.Ap[pv];
+        if (p >= R.bound_end) {
+          // escaped: for the step's budget, the old radius of those that left
+          // in this step, and c
+          O.r_old[p] = (int64_t)pv - R.seg_begin < S.nb[R.seg]
+                           ? r_in[pv]
+                           : __longlong_as_double((long long)kInfBits);
+          O.c[p] = rb[pv].c;
+        }
+      }
+    }
+    px = A.x;
+    pm = A.m;
+    pid = A.id;
+    pv = v;
+    A = A1;
+    v = v1;
+    v1 = v2;
+  }
+  __syncthreads();
+  // the tile's sums
+  const int h = t & (kThreads - 1);
+  const bool sums = t < 2 * kThreads, second = t >= kThreads;
+  const int64_t bl = R.bound_end - R.begin;
+  const int lb = bl < len ? (int)(bl < 0 ? 0 : bl) : len;
+  const double* tm = O.m + R.begin;
+  const double* tx = O.x + R.begin;
+  double a = 0.0;
+  if (sums) {
+#pragma unroll 8
+    for (int i = 0; i < kPer; ++i) {
+      const int e = i * kThreads + h;
+      if (e < lb) a = a + (second ? tm[e] * tx[e] : tm[e]);
+    }
+    s_red[t] = a;
+  }
+  __syncthreads();
+  // block_sum's tree, its last levels in a warp's registers
+#pragma unroll
+  for (int w = kThreads / 2; w >= 32; w >>= 1) {
+    if (sums && h < w) {
+      a = a + s_red[t + w];
+      s_red[t] = a;
+    }
+    __syncthreads();
+  }
+  if (sums && h < 32) {
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) a = a + __shfl_down_sync(0xFFFFFFFFu, a, w);
+    if (h == 0) (second ? O.tile_mx : O.tile_m)[blockIdx.x] = a;
+  }
+  // the bins' counts and the scan's words, zero again for the next step
+  if (cnt) {
+    const int64_t step = (int64_t)gridDim.x * kGatThreads;
+    const int64_t g = (int64_t)blockIdx.x * kGatThreads + t;
+    uint4* c4 = reinterpret_cast<uint4*>(cnt);
+    for (int64_t i = g; i < n_bins / 4; i += step) c4[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int64_t i = g; i < n_desc; i += step) desc[i] = 0ull;
+    if (g < 2) ctl[g] = 0u;
+  }
+}
+
+// ------------------------------------------- the energy correction's halves
+// Phi_new at the old radii.  The old radii are sorted as the new table is, so
+// a stretch of old stars meets one stretch of the new table: its ends are found
+// by two warps (32 probes a round), its radii are staged, and each star
+// searches them there (a dozen probes of shared memory, four stars a thread
+// abreast) and reads one node next to its neighbours'.  Where the stretch is
+// too long to stage, the search runs on the table.  With the velocities'
+// kernel 0.42 ms at N = 1e7, 18 us at 1e5; the one kernel before them, in the new
+// order with a random search through the bucket index per star, 0.44 ms.
+constexpr int kPoThreads = 256;
+constexpr int kPoPer = 4;
+constexpr int kPoChunk = kPoThreads * kPoPer;  // stars per block
+constexpr int kPoWin = 2048;                   // staged radii at most
+static_assert(kTile % kPoChunk == 0, "whole chunks in a tile");
+
+// largest i in [0, nb) with r[i] <= q, else -1, by one warp
+__device__ __forceinline__ int64_t warp_shell(const double* r, int64_t nb, double q) {
+  const long long qb = dbits(q);
+  const int lane = threadIdx.x & 31;
+  int64_t lo = -1, hi = nb;
+  while (hi - lo > 1) {
+    const int64_t span = hi - lo;
+    const int64_t m = lo + (span * (lane + 1)) / 33;
+    const bool below = m <= lo || (m < hi && dbits(r[m]) <= qb);
+    const unsigned k = (unsigned)__popc(__ballot_sync(0xffffffffu, below));
+    // the first k probes are at or below q (probes rise with the lane)
+    const int64_t nlo = k == 0 ? lo : lo + (span * k) / 33;
+    const int64_t nhi = k == 32 ? hi : lo + (span * (k + 1)) / 33;
+    lo = nlo > lo ? nlo : lo;
+    hi = nhi < hi ? nhi : hi;
+  }
+  return lo;
+}
+
+template <bool kDiv>
+__global__ void __launch_bounds__(kPoThreads) k_phi_old(Seg S, const int64_t* esc,
+                                                        const double* r_in, const double* x_in,
+                                                        const double* r, const double* x,
+                                                        const double* phi,
+                                                        const double4_32a* node, RecB* rb) {
+  pdl_enter();
+  __shared__ long long po_r[kPoWin];
+  __shared__ int64_t s_lo, s_hi;
+  const int t = threadIdx.x;
+  constexpr int kSub = kTile / kPoChunk;
+  TR R = tile_of(S, esc, blockIdx.x / kSub, false);
+  // the old order's bound stars in this chunk; the new table
+  const int64_t begin = R.begin + (int64_t)(blockIdx.x % kSub) * kPoChunk;
+  int64_t end = begin + kPoChunk < R.end ? begin + kPoChunk : R.end;
+  end = end < R.bound_end ? end : R.bound_end;
+  if (begin >= end) return;
+  const int64_t sb = R.seg_begin, nb = S.nb[R.seg] - esc[R.seg];
+  if (nb <= 0) return;
+  double ro[kPoPer], xo[kPoPer];
+#pragma unroll
+  for (int j = 0; j < kPoPer; ++j) {
+    const int64_t p = begin + j * kPoThreads + t;
+    ro[j] = p < end ? r_in[p] : 0.0;
+    xo[j] = p < end ? x_in[p] : 0.0;
+  }
+  if (t < 64) {
+    const int64_t k = warp_shell(r + sb, nb, r_in[t < 32 ? begin : end - 1]);
+    if (t == 0) s_lo = k;
+    if (t == 32) s_hi = k;
+  }
+  __syncthreads();
+  const int64_t lo0 = s_lo, hi0 = s_hi + 1;  // shells lo0 .. hi0 - 1
+  const int64_t first = lo0 < 0 ? 0 : lo0;
+  const int staged = (int)(hi0 - first < kPoWin ? hi0 - first : kPoWin + 1);
+  int64_t at[kPoPer];
+  if (staged <= kPoWin) {
+    for (int i = t; i < staged; i += kPoThreads) po_r[i] = dbits(r[sb + first + i]);
+    __syncthreads();
+    int lo[kPoPer], hi[kPoPer];
+#pragma unroll
+    for (int j = 0; j < kPoPer; ++j) {
+      lo[j] = lo0 < 0 ? -1 : 0;  // (r[lo0] is not above the chunk's first star)
+      hi[j] = staged;
+    }
+    // every star's bracket shrinks alike: staged or staged + 1 candidates
+    for (int width = staged + 1; width > 1; width = (width + 1) >> 1) {
+#pragma unroll
+      for (int j = 0; j < kPoPer; ++j) {
+        const int mid = (lo[j] + hi[j]) >> 1;
+        if (mid > lo[j]) {
+          if (po_r[mid] <= dbits(ro[j])) lo[j] = mid; else hi[j] = mid;
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kPoPer; ++j) at[j] = first + lo[j];
+  } else {
+#pragma unroll
+    for (int j = 0; j < kPoPer; ++j) {
+      int64_t lo = lo0, hi = hi0;
+      while (hi - lo > 1) {
+        const int64_t mid = lo + ((hi - lo) >> 1);
+        if (dbits(r[sb + mid]) <= dbits(ro[j])) lo = mid; else hi = mid;
+      }
+      at[j] = lo;
     }
   }
-  double tm = block_sum(am, s);
-  double tx = block_sum(ax, s);
-  if (threadIdx.x == 0) { tile_m[blockIdx.x] = tm; tile_mx[blockIdx.x] = tx; }
+#pragma unroll
+  for (int j = 0; j < kPoPer; ++j) {
+    const int64_t p = begin + j * kPoThreads + t;
+    if (p >= end) continue;
+    const int64_t i = at[j];
+    double pn;
+    if (!kDiv) {
+      const double4_32a nd = node[sb + (i < 0 ? 0 : i)];
+      pn = i < 0 ? nd.z : nd.z + nd.w * (nd.y - xo[j]);
+    } else {
+      const int64_t q = sb + (i < 0 ? 0 : i);
+      const double pj = phi[q];
+      pn = pj;
+      if (i >= 0) {
+        const double xj = x[q];
+        double xj1 = 0.0, pj1 = 0.0;
+        if (i + 1 < nb) {
+          xj1 = x[q + 1];
+          pj1 = phi[q + 1];
+        }
+        const double den = xj - xj1;
+        if (pos_num(den)) pn = pj + div_rn(xj - xo[j], den) * (pj1 - pj);
+      }
+    }
+    rb[p].w = pn;
+  }
+}
+
+// The new velocities into the new order: T' = T + 1/2 [(Phi_new(r_old) -
+// Phi_new(r_new)) - (Phi_old(r_old) - Phi_old(r_new))], clamped at 0; both
+// components scaled by sqrt(T'/T) (section 2.1 step 6).
+template <bool kCorrect>
+__global__ void __launch_bounds__(256) k_velocities(Seg S, const int64_t* esc, int64_t n,
+                                                    const uint32_t* order, const RecB* rb,
+                                                    const double* phi, const double* m,
+                                                    double* vr, double* vt) {
+  pdl_enter();
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n) return;
+  const uint32_t v = order[p];
+  if ((int64_t)v >= n) return;  // only after a reported sort failure
+  const RecB B = load_rec(rb + v);
+  double a = B.vr, b = B.vt;
+  if (kCorrect) {
+    const int c = seg_find(S.off, S.n_seg, p);
+    if (p - S.off[c] < S.nb[c] - esc[c]) {
+      const double Tk = scale_down<1>(a * a + b * b);
+      const double dnew = B.w - phi[p];
+      double Tp = Tk + scale_down<1>(dnew - B.c);
+      if (lt0(Tp)) {
+        clamp_energy_add(S.stats, c, m[p], Tp);
+        stat_add(S.stats, c, kStClamps, 1ull);
+        Tp = 0.0;
+      }
+      if (pos_num(Tk)) {
+        const double f = sqrt_rn(div_rn(Tp, Tk));
+        a = a * f;
+        b = b * f;
+      }
+    }
+  }
+  vr[p] = a;
+  vt[p] = b;
 }
 
 // Double -> float rounding to nearest even with integer operations: the
@@ -892,16 +1189,14 @@ __global__ void k_make_nodes(int64_t n, const double* r, const double* x, const 
   tdf[p] = float_pairs(x[p], phi[p]);
 }
 
-__global__ void k_unpack_orbit(int64_t n, const uint64_t* keys, const Payload* pay,
-                               double* r_new, double* vr_new, double* vt_new) {
+__global__ void k_unpack_orbit(int64_t n, const RecA* ra, const RecB* rb, double* r_new,
+                               double* vr_new, double* vt_new) {
   pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
-  uint64_t k = keys[p];
-  r_new[p] = key_is_escaper(k) ? __longlong_as_double(0x7FF0000000000000ll)
-                               : __longlong_as_double((long long)k);
-  if (vr_new) vr_new[p] = pay[p].vr;
-  if (vt_new) vt_new[p] = pay[p].vt;
+  r_new[p] = ra[p].r;
+  if (vr_new) vr_new[p] = rb[p].vr;
+  if (vt_new) vt_new[p] = rb[p].vt;
 }
 
 inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
@@ -926,10 +1221,10 @@ void launch_make_nodes(int64_t n, const double* r, const double* x, const double
   if (n > 0) launch_k(k_make_nodes, blocks_for(n, 256), 256, 0, st, n, r, x, phi, M, node, tdf);
 }
 
-void launch_unpack_orbit(int64_t n, const uint64_t* keys, const Payload* pay, double* r_new,
+void launch_unpack_orbit(int64_t n, const RecA* ra, const RecB* rb, double* r_new,
                          double* vr_new, double* vt_new, cudaStream_t st) {
   if (n > 0)
-    launch_k(k_unpack_orbit, blocks_for(n, 256), 256, 0, st, n, keys, pay, r_new, vr_new, vt_new);
+    launch_k(k_unpack_orbit, blocks_for(n, 256), 256, 0, st, n, ra, rb, r_new, vr_new, vt_new);
 }
 
 // ------------------------------------------------------------------ host
@@ -1001,10 +1296,16 @@ void free_layout(SegLayout& L, cudaStream_t st) {
   L = SegLayout();
 }
 
-void launch_make_keys(const SegLayout& L, const double* r, const double* vr,
-                      const double* vt, const double* m, const uint32_t* id,
-                      uint64_t* keys, Payload* pay, cudaStream_t st) {
-  if (L.n) launch_k(k_make_keys, blocks_for(L.n, 256), 256, 0, st, L.n, r, vr, vt, m, id, keys, pay);
+void launch_make_keys(const SegLayout& L, const double* r, const uint32_t* id, uint64_t* keys,
+                      cudaStream_t st) {
+  if (L.n) launch_k(k_make_keys, blocks_for(L.n, 256), 256, 0, st, L.n, r, id, keys);
+}
+
+void launch_make_records(const SegLayout& L, const double* r, const double* vr,
+                         const double* vt, const double* m, const uint32_t* id, RecA* ra,
+                         RecB* rb, cudaStream_t st) {
+  if (L.n)
+    launch_k(k_make_records, blocks_for(L.n, 256), 256, 0, st, L.n, r, vr, vt, m, id, ra, rb);
 }
 
 void launch_id_keys(const SegLayout& L, const uint32_t* id, uint64_t* keys, cudaStream_t st) {
@@ -1016,20 +1317,49 @@ void launch_rekey_radius(const SegLayout& L, const uint32_t* perm, const double*
   if (L.n) launch_k(k_rekey_radius, blocks_for(L.n, 256), 256, 0, st, L.n, perm, r, id, keys);
 }
 
-void launch_gather(const SegLayout& L, const uint64_t* keys, const uint32_t* vals,
-                   const Payload* pay, double* r, double* x, double* vr, double* vt,
-                   double* m, uint32_t* id, double* r_old, double* c, cudaStream_t st,
-                   double* tile_m, double* tile_mx, const double* Rp, double* Rout,
-                   const double* Ap, double* Aout, bool packed) {
+void launch_gather(const SegLayout& L, const uint32_t* perm, const RecA* ra, const RecB* rb,
+                   double* r, double* x, double* vr, double* vt, double* m, uint32_t* id,
+                   cudaStream_t st) {
+  if (L.n)
+    launch_k(k_gather, blocks_for(L.n, 256), 256, 0, st, L.n, perm, ra, rb, r, x, vr, vt, m, id);
+}
+
+void launch_gather_step(const SegLayout& L, BinWork* B, const uint32_t* order_in,
+                        const RecA* ra, const RecB* rb, const double* r_in, double* r_out,
+                        double* x_out, double* m, uint32_t* id, uint32_t* order_out,
+                        double* r_old, double* c, double* tile_m, double* tile_mx,
+                        const double* Rp, double* Rout, const double* Ap, double* Aout,
+                        bool exact, cudaStream_t st) {
+  if (!L.n_tiles) return;
+  GatherOut O;
+  O.r = r_out; O.x = x_out; O.m = m;
+  O.id = id; O.order = order_out;
+  O.r_old = r_old; O.c = c;
+  O.tile_m = tile_m; O.tile_mx = tile_mx;
+  O.Rp = Rp; O.Ap = Ap;
+  O.R = Rout; O.A = Aout;
+  const bool few = L.n_tiles <= kGatFewTiles;
+  launch_k(exact ? (few ? k_gather_step<true, 1024> : k_gather_step<true, 512>)
+                 : (few ? k_gather_step<false, 1024> : k_gather_step<false, 512>),
+           (unsigned)L.n_tiles, few ? 1024 : 512, 0, st, L.dev(), L.esc_step, L.n, order_in, ra, rb, r_in, O,
+           B ? B->cnt : nullptr, B ? B->n_bins : 0, B ? B->desc : nullptr, B ? B->n_tiles : 0,
+           B ? B->ctl : nullptr);
+}
+
+void launch_phi_old(const SegLayout& L, const double* r_in, const double* x_in, const double* r,
+                    const double* x, const double* phi, const double4_32a* node, RecB* rb,
+                    bool div_form, cudaStream_t st) {
+  if (!L.n_tiles) return;
+  launch_k(div_form ? k_phi_old<true> : k_phi_old<false>,
+           (unsigned)(L.n_tiles * (kTile / kPoChunk)), kPoThreads, 0, st, L.dev(), L.esc_step, r_in, x_in, r, x, phi, node, rb);
+}
+
+void launch_velocities(const SegLayout& L, const uint32_t* order, const RecB* rb,
+                       const double* phi, const double* m, double* vr, double* vt, bool correct,
+                       cudaStream_t st) {
   if (!L.n) return;
-  if (tile_m && tile_mx && r_old && c && L.n_tiles)
-    launch_k(k_gather_sums, (unsigned)L.n_tiles, kThreads, 0, st, L.dev(), L.esc_step, L.n, keys, vals,
-                                                            pay, r, x, vr, vt, m, id, r_old, c,
-                                                            tile_m, tile_mx, Rp, Rout, Ap,
-                                                            Aout, packed);
-  else
-    launch_k(k_gather, blocks_for(L.n, 256), 256, 0, st, L.n, keys, vals, pay, r, x, vr, vt, m, id,
-                                                  r_old, c);
+  launch_k(correct ? k_velocities<true> : k_velocities<false>, blocks_for(L.n, 256), 256, 0, st,
+           L.dev(), L.esc_step, L.n, order, rb, phi, m, vr, vt);
 }
 
 constexpr size_t kPotentialSmem = sizeof(double) * 3 * kPad8N;
@@ -1038,6 +1368,7 @@ void potential_prepare() {
   cudaFuncSetAttribute(k_potential, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)kPotentialSmem);
 }
+
 
 void launch_potential(const SegLayout& L, const double* r, const double* x, const double* m,
                       double* tile_m, double* tile_mx, double* phi, float2* t32,

@@ -1,4 +1,8 @@
-// Key-value sort of the stars by radius (section 2.1 step 6).
+// Sort of the stars by radius (section 2.1 step 6).
+//
+// The timestep sorts by counting, on the shells of the old table (see BinWork
+// and k_bin_scan below).  States in no particular order, the stage call and
+// timesteps configured so take the radix sort:
 //
 // A stable least-significant-digit radix sort over 8-bit digits of the
 // 64-bit key, run independently inside every segment (cluster) of the
@@ -13,9 +17,9 @@
 // writes contiguous runs.
 //
 // Two shape parameters are chosen at initialisation by timing them on the
-// real keys: keys per thread (8 or 16, so tiles of 2048 or 4096) and the
-// multisplit (one __match_any_sync per key, or eight __ballot_sync
-// intersected bit by bit).
+// real keys, where the timestep uses them: keys per thread (8 or 16, so tiles
+// of 2048 or 4096) and the multisplit (one __match_any_sync per key, or nine
+// __ballot_sync intersected bit by bit).
 #include <utility>
 #include <vector>
 
@@ -142,12 +146,10 @@ __global__ void __launch_bounds__(kThreads) k_upsweep(const int64_t* off, const 
   }
 }
 
-// kPacked: keys only (each key carries its star's index in its unsorted low
-// bits), no values
-template <int IPT, bool kPacked>
+template <int IPT>
 struct PassSmem {
   uint64_t key[kThreads * IPT];
-  uint32_t val[kPacked ? 1 : kThreads * IPT];
+  uint32_t val[kThreads * IPT];
   uint32_t whist[kWarps][kBins];
   int64_t gbase[kBins];
   uint32_t dstart[kBins];
@@ -172,8 +174,8 @@ constexpr int kRankMatch = 0;   // __match_any_sync
 constexpr int kRankBallot = 1;  // nine __ballot_sync
 
 // ------------------------------------------------------------- onesweep
-template <bool kValIdentity, int IPT, int kRank, bool kPacked>
-__global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 6 : IPT <= 16 ? (kPacked ? 4 : 3) : 2))
+template <bool kValIdentity, int IPT, int kRank>
+__global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 6 : 3))
     k_pass(const int64_t* off, const int64_t* tile_off, int n_seg, int64_t n_tiles,
            const uint64_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
            uint64_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out, int pass, int q,
@@ -182,7 +184,7 @@ __global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 6 : IPT <= 16 ? (kPacked
   pdl_enter();
   constexpr int kTileKeys = kThreads * IPT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  PassSmem<IPT, kPacked>& S = *reinterpret_cast<PassSmem<IPT, kPacked>*>(smem_raw);
+  PassSmem<IPT>& S = *reinterpret_cast<PassSmem<IPT>*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int shift = 8 * pass;
 
@@ -203,7 +205,7 @@ __global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 6 : IPT <= 16 ? (kPacked
     int64_t p = R.begin + e;
     bool valid = e < n_items;
     k[i] = valid ? keys_in[p] : 0ull;
-    v[i] = (valid && !kPacked) ? (kValIdentity ? (uint32_t)p : vals_in[p]) : 0u;
+    v[i] = valid ? (kValIdentity ? (uint32_t)p : vals_in[p]) : 0u;
     dg[i] = valid ? (int)((k[i] >> shift) & 0xFF) : kBins;
   }
 
@@ -289,7 +291,7 @@ __global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 6 : IPT <= 16 ? (kPacked
     if (dg[i] < kBins) {
       uint32_t lp = S.dstart[dg[i]] + S.whist[warp][dg[i]] + rank[i];
       S.key[lp] = k[i];
-      if (!kPacked) S.val[lp] = v[i];
+      S.val[lp] = v[i];
     }
   }
   __syncthreads();
@@ -306,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 6 : IPT <= 16 ? (kPacked
       continue;
     }
     keys_out[dest] = kk;
-    if (!kPacked) vals_out[dest] = S.val[lp];
+    vals_out[dest] = S.val[lp];
   }
 }
 
@@ -362,85 +364,225 @@ __global__ void k_tiefix(const int64_t* off, int n_seg, int64_t n, uint64_t* key
   if (equal && stats) atomicAdd(stats + (size_t)c * kStStride + kStTies, 1ull);
 }
 
-// The same for packed keys: the low 24 bits of a sorted word hold its star's
-// index in the segment, the key's own low 24 bits and the id are in the
-// star's payload record (lo24 in pad); runs equal in bits 24-63 are put in
-// (key, id) order by moving the words.
-__device__ __forceinline__ void tiefix_packed_at(const int64_t* off, int n_seg, int64_t p,
-                                                 uint64_t* keys, const Payload* pay,
-                                                 uint32_t* err, unsigned long long* stats) {
-  int c = seg_find(off, n_seg, p);
-  int64_t sb = __ldg(off + c), se = __ldg(off + c + 1);
-  const uint64_t hp = keys[p] >> 24;
-  if (p + 1 >= se || (keys[p + 1] >> 24) != hp) return;
-  if (p > sb && (keys[p - 1] >> 24) == hp) return;  // not the start of the run
-  int64_t e = p + 2;
-  while (e < se && (keys[e] >> 24) == hp) ++e;
-  for (int64_t i = p; i < e; ++i)
-    if ((int64_t)(keys[i] & 0xFFFFFFull) >= se - sb) {
-      set_err(err, kErrTimeout);
-      return;
-    }
-  const Payload* P = pay + sb;
-  auto full = [&](uint64_t w) { return (w & ~0xFFFFFFull) | (uint64_t)P[w & 0xFFFFFFull].pad; };
-  auto idof = [&](uint64_t w) { return P[w & 0xFFFFFFull].id; };
-  const long long move_cap = g_tie_move_cap;
-  long long moves = 0;
-  bool equal = false;
-  for (int64_t i = p + 1; i < e; ++i) {
-    const uint64_t wv = keys[i];
-    const uint64_t kv = full(wv);
-    const uint32_t idv = idof(wv);
-    int64_t j = i - 1;
-    while (j >= p) {
-      const uint64_t wj = keys[j];
-      const uint64_t kj = full(wj);
-      if (kj == kv) equal = true;
-      if (!(kj > kv || (kj == kv && idof(wj) > idv))) break;
-      keys[j + 1] = wj;
-      --j;
-      if (++moves > move_cap) {
-        set_err(err, kErrTies);
-        keys[j + 1] = wv;
-        return;
-      }
-    }
-    keys[j + 1] = wv;
-  }
-  if (equal && stats) atomicAdd(stats + (size_t)c * kStStride + kStTies, 1ull);
-}
-
-// four positions per thread: the keys read once (two 16-byte loads), a run
-// start looked for only where two neighbours agree in bits 24-63 (a few per
-// cent of them)
-__global__ void k_tiefix_packed(const int64_t* off, int n_seg, int64_t n, uint64_t* keys,
-                                const Payload* pay, uint32_t* err,
-                                unsigned long long* stats) {
+// ------------------------------------------------------- counting sort
+// (see BinWork).  At N = 1e7: count 0.05, scan 0.02, scatter 0.12 ms, bound
+// by random atomics and 4-byte stores in the L2, against 0.54 ms for the five
+// 8-bit radix passes it replaced in the timestep (keys with the index packed
+// into their low bits, histograms, tie fix).
+__global__ void __launch_bounds__(256) k_bin_count(int64_t n, const uint32_t* bin,
+                                                   uint32_t* cnt) {
   pdl_enter();
   const int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-  if (p0 >= n) return;
-  uint64_t k[6];  // keys[p0 - 1 .. p0 + 4]
   if (p0 + 4 <= n) {
-    const uint4 a = reinterpret_cast<const uint4*>(keys + p0)[0];
-    const uint4 b = reinterpret_cast<const uint4*>(keys + p0)[1];
-    k[1] = ((uint64_t)a.y << 32) | a.x;
-    k[2] = ((uint64_t)a.w << 32) | a.z;
-    k[3] = ((uint64_t)b.y << 32) | b.x;
-    k[4] = ((uint64_t)b.w << 32) | b.z;
+    const uint4 b = *reinterpret_cast<const uint4*>(bin + p0);
+    atomicAdd(cnt + b.x, 1u);
+    atomicAdd(cnt + b.y, 1u);
+    atomicAdd(cnt + b.z, 1u);
+    atomicAdd(cnt + b.w, 1u);
   } else {
-    for (int i = 0; i < 4; ++i) k[1 + i] = p0 + i < n ? keys[p0 + i] : 0ull;
+    for (int64_t p = p0; p < n; ++p) atomicAdd(cnt + bin[p], 1u);
   }
-  k[0] = p0 > 0 ? keys[p0 - 1] : 0ull;
-  k[5] = p0 + 4 < n ? keys[p0 + 4] : 0ull;
-  bool any = false;
-  for (int i = 0; i < 4; ++i)
-    any |= p0 + i + 1 < n && (k[1 + i] >> 24) == (k[2 + i] >> 24);
-  if (!any) return;
-  // the full test (segment bounds, run start) where a run may begin; the
-  // keys are re-read there, after any earlier run in this thread moved them
-  for (int i = 0; i < 4 && p0 + i < n; ++i)
-    if (p0 + i + 1 < n && (k[1 + i] >> 24) == (k[2 + i] >> 24))
-      tiefix_packed_at(off, n_seg, p0 + i, keys, pay, err, stats);
+}
+
+// Exclusive scan of the counts in place, one pass: tiles of kBinTile bins in
+// ticket order, the sum of the tiles before by decoupled look-back, one warp
+// reading 32 tiles' words at a time.  Each wait is bounded (g_spin_cap polls
+// of a window that is not complete).  Bins with more than kRunMax stars are
+// listed.
+__global__ void __launch_bounds__(kThreads) k_bin_scan(uint32_t* cnt, unsigned long long* desc,
+                                                       uint32_t* ctl, uint2* runs,
+                                                       uint32_t* err) {
+  pdl_enter();
+  __shared__ uint32_t s_warp[kWarps];
+  __shared__ uint32_t s_tile, s_excl;
+  constexpr int kPer = kBinTile / kThreads;  // 16 consecutive bins per thread
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) s_tile = atomicAdd(ctl, 1u);
+  __syncthreads();
+  const int64_t t = s_tile;
+  uint4* mine = reinterpret_cast<uint4*>(cnt + t * kBinTile + tid * kPer);
+  uint4 c[kPer / 4];
+  uint32_t sum = 0;
+#pragma unroll
+  for (int i = 0; i < kPer / 4; ++i) {
+    c[i] = mine[i];
+    sum += c[i].x + c[i].y + c[i].z + c[i].w;
+  }
+  const uint32_t before = block_excl_scan_u32(sum, s_warp);
+  if (warp == 0) {
+    const unsigned long long total = s_warp[kWarps - 1];
+    uint32_t excl = 0;
+    if (lane == 0) atomicExch(desc + t, (t == 0 ? kFlagInc : kFlagAgg) | total);
+    const int cap = g_spin_cap;
+    int spins = 0;
+    int64_t j = t - 1;
+    while (j >= 0) {
+      const int64_t q = j - lane;
+      const unsigned long long w = q >= 0 ? ld_volatile(desc + q) : kFlagInc;
+      const unsigned ready = __ballot_sync(0xffffffffu, (w & ~kCountMask) != 0);
+      const unsigned inc = __ballot_sync(0xffffffffu, (w & ~kCountMask) == kFlagInc);
+      const unsigned use = inc ? (2u << (__ffs(inc) - 1)) - 1u : 0xffffffffu;
+      if ((ready & use) != use) {
+        if (++spins >= cap) {
+          if (lane == 0) set_err(err, kErrTimeout);
+          break;
+        }
+        if (spins > 32) __nanosleep(64);
+        continue;
+      }
+      excl += __reduce_add_sync(0xffffffffu, (use >> lane) & 1u ? (uint32_t)(w & kCountMask) : 0u);
+      if (inc) break;
+      j -= 32;
+    }
+    if (lane == 0) {
+      if (t) atomicExch(desc + t, kFlagInc | (excl + total));
+      s_excl = excl;
+    }
+  }
+  __syncthreads();
+  uint32_t at = s_excl + before;
+#pragma unroll
+  for (int i = 0; i < kPer / 4; ++i) {
+    uint32_t v[4] = {c[i].x, c[i].y, c[i].z, c[i].w}, o[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      o[k] = at;
+      if (v[k] > (uint32_t)kRunMax) runs[atomicAdd(ctl + 1, 1u)] = make_uint2(at, v[k]);
+      at += v[k];
+    }
+    mine[i] = make_uint4(o[0], o[1], o[2], o[3]);
+  }
+}
+
+// the stars' indices to their bins' positions (the order inside a bin is
+// whatever the atomics give; the gather settles it)
+__global__ void __launch_bounds__(256) k_bin_scatter(int64_t n, const uint32_t* bin,
+                                                     uint32_t* at, uint32_t* order,
+                                                     uint32_t* err) {
+  pdl_enter();
+  const int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+  auto put = [&](uint32_t pos, int64_t p) {
+    if ((int64_t)pos < n) order[pos] = (uint32_t)p;
+    else set_err(err, kErrTimeout);  // only after a timed-out look-back
+  };
+  if (p0 + 4 <= n) {
+    const uint4 b = *reinterpret_cast<const uint4*>(bin + p0);
+    const uint32_t a0 = atomicAdd(at + b.x, 1u), a1 = atomicAdd(at + b.y, 1u),
+                   a2 = atomicAdd(at + b.z, 1u), a3 = atomicAdd(at + b.w, 1u);
+    put(a0, p0);
+    put(a1, p0 + 1);
+    put(a2, p0 + 2);
+    put(a3, p0 + 3);
+  } else {
+    for (int64_t p = p0; p < n; ++p) put(atomicAdd(at + bin[p], 1u), p);
+  }
+}
+
+// The listed runs (more than kRunMax stars in one bin: new radii crowding
+// into one shell of the old table, as when a thin shell of stars spreads out)
+// in (r, id) order: one block per run, a stable radix sort of the run's
+// indices by id, then by the bits of r, over the digits that differ.  A step
+// without such runs finds the list empty.
+constexpr int kRunItems = 8;  // indices per thread and chunk
+__global__ void __launch_bounds__(kThreads) k_long_runs(int64_t n, const uint32_t* ctl,
+                                                        const uint2* runs, const RecA* rec,
+                                                        uint32_t* order, uint32_t* scratch) {
+  pdl_enter();
+  __shared__ uint32_t whist[kWarps][kBins];
+  __shared__ uint32_t base[kBins], s_warp[kWarps];
+  __shared__ unsigned long long s_dr;
+  __shared__ uint32_t s_di;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned lt_mask = lanemask_lt();
+  const uint32_t nr = ctl[1];
+  for (uint32_t l = blockIdx.x; l < nr; l += gridDim.x) {
+    const uint2 run = runs[l];
+    const uint32_t len = run.y;
+    if ((int64_t)run.x + len > n) continue;  // only after a timed-out look-back
+    uint32_t* in = order + run.x;
+    uint32_t* out = scratch + run.x;
+    // the bits in which the run's radii and ids differ
+    if (tid == 0) {
+      s_dr = 0ull;
+      s_di = 0u;
+    }
+    __syncthreads();
+    bool ok = true;
+    unsigned long long dr = 0ull;
+    uint32_t di = 0u;
+    const uint32_t first = in[0];
+    if ((int64_t)first < n) {
+      const unsigned long long r0 = ubits(rec[first].r);
+      const uint32_t i0 = rec[first].id;
+      for (uint32_t i = tid; i < len; i += kThreads) {
+        const uint32_t v = in[i];
+        if ((int64_t)v >= n) { ok = false; break; }
+        dr |= ubits(rec[v].r) ^ r0;
+        di |= rec[v].id ^ i0;
+      }
+    } else {
+      ok = false;
+    }
+    atomicOr(&s_dr, dr);
+    atomicOr(&s_di, di);
+    ok = __syncthreads_and(ok);
+    if (!ok) continue;  // only after a timed-out look-back
+    dr = s_dr;
+    di = s_di;
+    for (int q = 0; q < 12; ++q) {
+      const bool by_id = q < 4;
+      const int shift = 8 * (by_id ? q : q - 4);
+      if (!(by_id ? (di >> shift) & 255u : (uint32_t)(dr >> shift) & 255u)) continue;
+      auto digit = [&](uint32_t v) {
+        return (int)((by_id ? (unsigned long long)rec[v].id : ubits(rec[v].r)) >> shift) & 255;
+      };
+      base[tid] = 0u;
+      __syncthreads();
+      for (uint32_t i = tid; i < len; i += kThreads) atomicAdd(&base[digit(in[i])], 1u);
+      __syncthreads();
+      const uint32_t excl = block_excl_scan_u32(base[tid], s_warp);
+      __syncthreads();
+      base[tid] = excl;
+      for (uint32_t c0 = 0; c0 < len; c0 += kThreads * kRunItems) {
+        for (int i = tid; i < kWarps * kBins; i += kThreads) (&whist[0][0])[i] = 0u;
+        __syncthreads();
+        // warp w owns a contiguous stretch of the chunk (as k_pass)
+        uint32_t v[kRunItems], rank[kRunItems];
+        int dg[kRunItems];
+#pragma unroll
+        for (int i = 0; i < kRunItems; ++i) {
+          const uint32_t e = c0 + (uint32_t)(warp * (32 * kRunItems) + i * 32 + lane);
+          v[i] = e < len ? in[e] : 0u;
+          dg[i] = e < len ? digit(v[i]) : kBins;
+          const unsigned peers = __match_any_sync(0xffffffffu, dg[i]);
+          uint32_t old = 0u;
+          if (lane == __ffs(peers) - 1 && dg[i] < kBins)
+            old = atomicAdd(&whist[warp][dg[i]], (uint32_t)__popc(peers));
+          __syncwarp();
+          rank[i] = __shfl_sync(0xffffffffu, old, __ffs(peers) - 1) + __popc(peers & lt_mask);
+        }
+        __syncthreads();
+        uint32_t at = base[tid];
+        for (int w = 0; w < kWarps; ++w) {
+          const uint32_t k = whist[w][tid];
+          whist[w][tid] = at;
+          at += k;
+        }
+        base[tid] = at;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kRunItems; ++i)
+          if (dg[i] < kBins) out[whist[warp][dg[i]] + rank[i]] = v[i];
+        __syncthreads();
+      }
+      uint32_t* sw = in;
+      in = out;
+      out = sw;
+    }
+    if (in != order + run.x)
+      for (uint32_t i = tid; i < len; i += kThreads) out[i] = in[i];
+    __syncthreads();
+  }
 }
 
 __global__ void k_philox(int64_t n, const uint32_t* ctr, uint64_t seed, uint32_t* out) {
@@ -452,51 +594,21 @@ __global__ void k_philox(int64_t n, const uint32_t* ctr, uint64_t seed, uint32_t
   reinterpret_cast<uint4*>(out)[i] = make_uint4(w.x, w.y, w.z, w.w);
 }
 
-template <bool kId, int IPT, int kRank, bool kPacked>
+template <bool kId, int IPT, int kRank>
 void set_pass_smem() {
-  cudaFuncSetAttribute(k_pass<kId, IPT, kRank, kPacked>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sizeof(PassSmem<IPT, kPacked>));
+  cudaFuncSetAttribute(k_pass<kId, IPT, kRank>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)sizeof(PassSmem<IPT>));
 }
 
 template <int IPT, int kRank>
 void launch_pass(const SegLayout& L, SortWork& W, bool id, const uint64_t* kin,
                  const uint32_t* vin, uint64_t* kout, uint32_t* vout, int pass, int q,
-                 int passes, uint32_t* err, cudaStream_t st, bool packed) {
+                 int passes, uint32_t* err, cudaStream_t st) {
   const unsigned grid = (unsigned)W.n_stiles;
-  if (packed) {
-    launch_k(k_pass<false, IPT, kRank, true>, grid, kThreads, sizeof(PassSmem<IPT, true>), st,
-        L.off, W.stile_off, L.n_seg, W.n_stiles, kin, nullptr, kout, nullptr, pass, q, passes,
-        W.hist, W.desc, W.tickets, err);
-    return;
-  }
-  const size_t sm = sizeof(PassSmem<IPT, false>);
-  if (id)
-    launch_k(k_pass<true, IPT, kRank, false>, grid, kThreads, sm, st, L.off, W.stile_off, L.n_seg,
-                                                         W.n_stiles, kin, vin, kout, vout, pass,
-                                                         q, passes, W.hist, W.desc, W.tickets,
-                                                         err);
-  else
-    launch_k(k_pass<false, IPT, kRank, false>, grid, kThreads, sm, st, L.off, W.stile_off, L.n_seg,
-                                                          W.n_stiles, kin, vin, kout, vout,
-                                                          pass, q, passes, W.hist, W.desc,
-                                                          W.tickets, err);
-}
-
-// the larger tiles (24 or 32 keys per thread) of packed keys
-template <int IPT>
-void launch_packed_pass(const SegLayout& L, SortWork& W, const uint64_t* kin, uint64_t* kout,
-                        int pass, int q, int passes, uint32_t* err, cudaStream_t st) {
-  const unsigned grid = (unsigned)W.n_stiles;
-  const size_t sm = sizeof(PassSmem<IPT, true>);
-  if (W.rank == kRankMatch)
-    launch_k(k_pass<false, IPT, kRankMatch, true>, grid, kThreads, sm, st,
-        L.off, W.stile_off, L.n_seg, W.n_stiles, kin, nullptr, kout, nullptr, pass, q, passes,
-        W.hist, W.desc, W.tickets, err);
-  else
-    launch_k(k_pass<false, IPT, kRankBallot, true>, grid, kThreads, sm, st,
-        L.off, W.stile_off, L.n_seg, W.n_stiles, kin, nullptr, kout, nullptr, pass, q, passes,
-        W.hist, W.desc, W.tickets, err);
+  const size_t sm = sizeof(PassSmem<IPT>);
+  launch_k(id ? k_pass<true, IPT, kRank> : k_pass<false, IPT, kRank>, grid, kThreads, sm, st,
+           L.off, W.stile_off, L.n_seg, W.n_stiles, kin, vin, kout, vout, pass, q, passes,
+           W.hist, W.desc, W.tickets, err);
 }
 
 }  // namespace
@@ -511,22 +623,14 @@ cudaError_t set_wait_limits(int spin_polls, long long tie_moves) {
 }
 
 void sort_prepare() {
-  set_pass_smem<true, 8, kRankMatch, false>();
-  set_pass_smem<false, 8, kRankMatch, false>();
-  set_pass_smem<true, 8, kRankBallot, false>();
-  set_pass_smem<false, 8, kRankBallot, false>();
-  set_pass_smem<true, 16, kRankMatch, false>();
-  set_pass_smem<false, 16, kRankMatch, false>();
-  set_pass_smem<true, 16, kRankBallot, false>();
-  set_pass_smem<false, 16, kRankBallot, false>();
-  set_pass_smem<false, 8, kRankMatch, true>();
-  set_pass_smem<false, 8, kRankBallot, true>();
-  set_pass_smem<false, 16, kRankMatch, true>();
-  set_pass_smem<false, 16, kRankBallot, true>();
-  set_pass_smem<false, 24, kRankMatch, true>();
-  set_pass_smem<false, 24, kRankBallot, true>();
-  set_pass_smem<false, 32, kRankMatch, true>();
-  set_pass_smem<false, 32, kRankBallot, true>();
+  set_pass_smem<true, 8, kRankMatch>();
+  set_pass_smem<false, 8, kRankMatch>();
+  set_pass_smem<true, 8, kRankBallot>();
+  set_pass_smem<false, 8, kRankBallot>();
+  set_pass_smem<true, 16, kRankMatch>();
+  set_pass_smem<false, 16, kRankMatch>();
+  set_pass_smem<true, 16, kRankBallot>();
+  set_pass_smem<false, 16, kRankBallot>();
   cudaFuncSetAttribute(k_upsweep, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)(sizeof(uint32_t) * kWarps * kMaxPasses * kBins));
 }
@@ -542,7 +646,7 @@ static std::vector<int64_t> sort_tile_offsets(const SegLayout& L, int tile) {
 
 cudaError_t sort_set_shape(const SegLayout& L, SortWork& W, int ipt, int rank,
                            cudaStream_t st) {
-  if ((ipt != 8 && ipt != 16 && ipt != 24 && ipt != 32) || (rank != 0 && rank != 1))
+  if ((ipt != 8 && ipt != 16) || (rank != 0 && rank != 1))
     return cudaErrorInvalidValue;
   std::vector<int64_t> o = sort_tile_offsets(L, kThreads * ipt);
   cudaError_t e = cudaMemcpyAsync(W.stile_off, o.data(), sizeof(int64_t) * o.size(),
@@ -592,22 +696,10 @@ void free_sort(SortWork& W, cudaStream_t st) {
 
 cudaError_t sort_segments(const SegLayout& L, SortWork& W, uint64_t* keys, uint32_t* vals,
                           int first_pass, int passes, bool vals_identity, uint32_t* err,
-                          cudaStream_t st, uint64_t** keys_res, uint32_t** vals_res,
-                          bool packed) {
+                          cudaStream_t st, uint64_t** keys_res, uint32_t** vals_res) {
   if (keys_res) *keys_res = keys;
   if (vals_res) *vals_res = vals;
   if (passes <= 0 || passes > W.max_passes || L.n_tiles == 0) return cudaSuccess;
-  // tiles of 24 or 32 keys per thread exist for packed keys only: a sort of
-  // keys and values (a new state's ordering, outside any graph capture)
-  // takes tiles of 16 and then restores the shape
-  if (!packed && W.ipt > 16) {
-    const int ipt = W.ipt, rank = W.rank;
-    cudaError_t e = sort_set_shape(L, W, 16, rank, st);
-    if (!e) e = sort_segments(L, W, keys, vals, first_pass, passes, vals_identity, err, st,
-                              keys_res, vals_res, false);
-    const cudaError_t e2 = sort_set_shape(L, W, ipt, rank, st);
-    return e ? e : e2;
-  }
   cudaMemsetAsync(W.zero_base, 0,
                   W.zero_head + sizeof(unsigned long long) * (size_t)passes *
                                     (size_t)W.n_stiles * kBins,
@@ -621,22 +713,14 @@ cudaError_t sort_segments(const SegLayout& L, SortWork& W, uint64_t* keys, uint3
   for (int q = 0; q < passes; ++q) {
     const bool id = q == 0 && vals_identity;
     const int pass = first_pass + q;
-    if (packed && W.ipt == 24)
-      launch_packed_pass<24>(L, W, kin, kout, pass, q, passes, err, st);
-    else if (packed && W.ipt == 32)
-      launch_packed_pass<32>(L, W, kin, kout, pass, q, passes, err, st);
-    else if (W.ipt == 8 && W.rank == kRankMatch)
-      launch_pass<8, kRankMatch>(L, W, id, kin, vin, kout, vout, pass, q, passes, err, st,
-                                 packed);
+    if (W.ipt == 8 && W.rank == kRankMatch)
+      launch_pass<8, kRankMatch>(L, W, id, kin, vin, kout, vout, pass, q, passes, err, st);
     else if (W.ipt == 8)
-      launch_pass<8, kRankBallot>(L, W, id, kin, vin, kout, vout, pass, q, passes, err, st,
-                                  packed);
+      launch_pass<8, kRankBallot>(L, W, id, kin, vin, kout, vout, pass, q, passes, err, st);
     else if (W.rank == kRankMatch)
-      launch_pass<16, kRankMatch>(L, W, id, kin, vin, kout, vout, pass, q, passes, err, st,
-                                  packed);
+      launch_pass<16, kRankMatch>(L, W, id, kin, vin, kout, vout, pass, q, passes, err, st);
     else
-      launch_pass<16, kRankBallot>(L, W, id, kin, vin, kout, vout, pass, q, passes, err, st,
-                                   packed);
+      launch_pass<16, kRankBallot>(L, W, id, kin, vin, kout, vout, pass, q, passes, err, st);
     std::swap(kin, kout);
     std::swap(vin, vout);
   }
@@ -648,8 +732,7 @@ cudaError_t sort_segments(const SegLayout& L, SortWork& W, uint64_t* keys, uint3
       *vals_res = vin;
     } else {
       cudaMemcpyAsync(keys, kin, sizeof(uint64_t) * (size_t)L.n, cudaMemcpyDeviceToDevice, st);
-      if (!packed)
-        cudaMemcpyAsync(vals, vin, sizeof(uint32_t) * (size_t)L.n, cudaMemcpyDeviceToDevice,
+      cudaMemcpyAsync(vals, vin, sizeof(uint32_t) * (size_t)L.n, cudaMemcpyDeviceToDevice,
                         st);
     }
   }
@@ -664,12 +747,62 @@ void launch_tiefix(const SegLayout& L, uint64_t* keys, uint32_t* vals,
       L.off, L.n_seg, L.n, keys, vals, ids_by_val, id_stride, shift, err, L.stats);
 }
 
-void launch_tiefix_packed(const SegLayout& L, uint64_t* keys, const Payload* pay,
-                          uint32_t* err, cudaStream_t st) {
+cudaError_t alloc_bins(BinWork& B, const SegLayout& L, cudaStream_t st) {
+  std::vector<int64_t>& o = B.h_cbase;
+  o.assign(L.n_seg + 1, 0);
+  for (int c = 0; c < L.n_seg; ++c) {
+    const int64_t nc = L.h_off[c + 1] - L.h_off[c];
+    o[c + 1] = o[c] + (nc + 1) + (nc / 8 + 1);  // shells -1 .. nc - 1, then escapers by id
+  }
+  B.n_tiles = (o[L.n_seg] + kBinTile - 1) / kBinTile;
+  B.n_bins = B.n_tiles * kBinTile;
+  cudaError_t e;
+  if ((e = cudaMallocAsync((void**)&B.cbase, sizeof(int64_t) * o.size(), st))) return e;
+  if ((e = cudaMallocAsync((void**)&B.esh, sizeof(int) * L.n_seg, st))) return e;
+  if ((e = cudaMallocAsync((void**)&B.cnt, sizeof(uint32_t) * B.n_bins, st))) return e;
+  if ((e = cudaMallocAsync((void**)&B.desc, sizeof(unsigned long long) * B.n_tiles, st))) return e;
+  if ((e = cudaMallocAsync((void**)&B.ctl, sizeof(uint32_t) * 2, st))) return e;
+  if ((e = cudaMallocAsync((void**)&B.runs, sizeof(uint2) * (L.n / kRunMax + 1), st))) return e;
+  e = cudaMemcpyAsync(B.cbase, o.data(), sizeof(int64_t) * o.size(), cudaMemcpyHostToDevice, st);
+  if (!e) e = cudaMemsetAsync(B.cnt, 0, sizeof(uint32_t) * B.n_bins, st);
+  if (!e) e = cudaMemsetAsync(B.desc, 0, sizeof(unsigned long long) * B.n_tiles, st);
+  if (!e) e = cudaMemsetAsync(B.ctl, 0, sizeof(uint32_t) * 2, st);
+  if (e) return e;
+  const std::vector<unsigned int> any((size_t)L.n_seg, 0xFFFFFFFFu);
+  return set_bin_ids(B, L, any.data(), st);
+}
+
+void free_bins(BinWork& B, cudaStream_t st) {
+  void* ps[] = {B.cbase, B.esh, B.cnt, B.desc, B.ctl, B.runs};
+  for (void* p : ps)
+    if (p) cudaFreeAsync(p, st);
+  B = BinWork();
+}
+
+cudaError_t set_bin_ids(BinWork& B, const SegLayout& L, const unsigned int* max_id,
+                        cudaStream_t st) {
+  std::vector<int> sh((size_t)L.n_seg, 0);
+  for (int c = 0; c < L.n_seg; ++c) {
+    const int64_t nc = L.h_off[c + 1] - L.h_off[c];
+    while (((uint64_t)max_id[c] >> sh[c]) > (uint64_t)(nc / 8)) ++sh[c];
+  }
+  cudaError_t e = cudaMemcpyAsync(B.esh, sh.data(), sizeof(int) * sh.size(),
+                                  cudaMemcpyHostToDevice, st);
+  if (!e) e = cudaStreamSynchronize(st);  // sh lives on this stack
+  return e;
+}
+
+void launch_bin_sort(const SegLayout& L, BinWork& B, const uint32_t* bin, const RecA* rec,
+                     uint32_t* order, uint32_t* scratch, bool counted, uint32_t* err,
+                     cudaStream_t st) {
   if (L.n == 0) return;
-  const int64_t nt = (L.n + 3) / 4;
-  launch_k(k_tiefix_packed, (unsigned)((nt + 255) / 256), 256, 0, st, L.off, L.n_seg, L.n, keys, pay,
-                                                               err, L.stats);
+  const unsigned grid = (unsigned)((L.n + 1023) / 1024);
+  if (!counted) launch_k(k_bin_count, grid, 256, 0, st, L.n, bin, B.cnt);
+  launch_k(k_bin_scan, (unsigned)B.n_tiles, kThreads, 0, st, B.cnt, B.desc, B.ctl, B.runs, err);
+  launch_k(k_bin_scatter, grid, 256, 0, st, L.n, bin, B.cnt, order, err);
+  const int64_t most = L.n / kRunMax + 1;  // listed runs at most
+  launch_k(k_long_runs, (unsigned)(most < 152 ? most : 152), kThreads, 0, st, L.n, B.ctl, B.runs,
+           rec, order, scratch);
 }
 
 void launch_philox(int64_t n, const uint32_t* ctr, uint64_t seed, uint32_t* out,
