@@ -194,114 +194,126 @@ __device__ __forceinline__ float f32_rn(double v) {
   return __uint_as_float(((unsigned)(u >> 32) & 0x80000000u) | (top + (up ? 1u : 0u)));
 }
 
-// Correctly rounded FP64 product, quotient and square root from 64-bit
-// integer arithmetic on the significands, for normal operands with a normal
-// result (anything else: the FP64 operation).  On this GPU an FP64 division
-// or square root takes several FP64 issues; these take none, and the FP64
-// pipe is left to the additions.  Each returns the IEEE-754 round-to-
-// nearest-even result exactly (checked bit for bit against the FP64
-// operations on 3 x 2^28 operand pairs per operation: random bit patterns,
-// random values over 81 binades, and significands with random runs of
-// trailing zeros, which give exact results and ties).
+// Correctly rounded FP64 product, quotient and square root from integer
+// arithmetic on the significands, for normal operands with a normal result
+// (anything else: the FP64 operation).  On this GPU an FP64 operation occupies
+// its SM's FP64 pipe for 16 cycles, a division or square root for about a
+// hundred; these take none of it, and the FP64 pipe is left to the additions.
+// Each returns the IEEE-754 round-to-nearest-even result exactly (checked bit
+// for bit against the FP64 operations on 3 x 2^28 operand pairs per operation:
+// random bit patterns, random values over 81 binades, and significands with
+// random runs of trailing zeros, which give exact results and ties).
 //
 // The significands are integers in [2^52, 2^53); the result's significand Q
 // is an integer in the same range, its exponent follows from the operands'.
 // A result assembled as sign + ((e - 1) << 52) + Q lets a significand that
 // rounds up to 2^53 carry into the exponent.
-__device__ __forceinline__ unsigned long long significand(unsigned long long u) {
-  return (u & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+__device__ __forceinline__ unsigned long long sig_of(unsigned hi, unsigned lo) {
+  return ((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
+}
+// whether the high word of a double is a normal number's
+__device__ __forceinline__ bool normal_hi(unsigned hi) {
+  return ((hi + 0x100000u) & 0x7FFFFFFFu) >= 0x200000u;
+}
+__device__ __forceinline__ double dbl_of(unsigned hi, unsigned long long q) {
+  return __longlong_as_double((long long)(((unsigned long long)hi << 32) + q));
 }
 
-// a b: the 106-bit product of the significands, its top 53 bits rounded to
-// nearest even by the bits below them.
+// a b: the 117-bit product of one significand and the other one shifted up
+// by 11 bits, from four 32 x 32 -> 64 bit products; its high word holds 52 or
+// 53 significant bits, rounded to nearest even by the low word.
 __device__ __forceinline__ double mul_rn(double a, double b) {
   const unsigned long long ua = ubits(a), vb = ubits(b);
-  const unsigned ea = (unsigned)(ua >> 52) & 0x7FFu, eb = (unsigned)(vb >> 52) & 0x7FFu;
-  const int e = (int)ea + (int)eb - 1023;  // the result's biased exponent, before a carry
-  if (ea - 1u < 2046u && eb - 1u < 2046u && (unsigned)(e - 2) < 2043u) {
-    const unsigned long long ma = significand(ua), mb = significand(vb);
-    const unsigned long long hi = __umul64hi(ma, mb), lo = ma * mb;
-    const unsigned c = (unsigned)(hi >> 41);  // product >= 2^105
-    const unsigned long long m = (hi << (12 - c)) | (lo >> (52 + c));
-    const unsigned long long rest = lo << (12 - c);  // the dropped bits, left-aligned
-    const unsigned long long up = (rest >> 63) & ((rest << 1) != 0ull ? 1ull : (m & 1ull));
-    return __longlong_as_double((long long)(((ua ^ vb) & kSignBit) +
-                                            ((unsigned long long)(e - 1 + (int)c) << 52) + m + up));
+  const unsigned xa = (unsigned)(ua >> 32), xb = (unsigned)(vb >> 32);
+  // the result's exponent field less one, before a carry
+  const unsigned ex = (xa & 0x7FF00000u) + (xb & 0x7FF00000u) - (1024u << 20);
+  if (normal_hi(xa) && normal_hi(xb) && ex < 0x7FC00000u) {
+    const unsigned al = (unsigned)ua << 11, ah = (unsigned)(ua >> 21) | 0x80000000u;
+    const unsigned bl = (unsigned)vb, bh = (xb & 0xFFFFFu) | 0x100000u;
+    const unsigned long long p0 = (unsigned long long)al * bl;
+    const unsigned long long p1 = (unsigned long long)ah * bl + (unsigned)(p0 >> 32);
+    const unsigned long long p2 = (unsigned long long)al * bh + (unsigned)p1;
+    unsigned long long hi =
+        (unsigned long long)ah * bh + (unsigned)(p1 >> 32) + (unsigned)(p2 >> 32);
+    unsigned long long lo = (p2 << 32) | (unsigned)p0;
+    unsigned e = ex + ((xa ^ xb) & 0x80000000u);
+    if ((unsigned)(hi >> 32) >= 0x100000u) {
+      e += 0x100000u;
+    } else {
+      hi = (hi << 1) | (lo >> 63);
+      lo <<= 1;
+    }
+    lo |= hi & 1ull;  // at half, up to the even neighbour
+    return dbl_of(e, hi + (lo > (1ull << 63) ? 1ull : 0ull));
   }
   return a * b;
 }
 
 // a / b in two digits of 30 and 22 bits.  R0 = m_a 2^s with s = 1 when m_a <
 // m_b, so that R0 / m_b is in [1, 2) and its quotient in units of 2^-52 has
-// 53 bits.  v ~ 2^84 / m_b (32 bits) is the float reciprocal of m_b's top
-// bits (~21 bits) after one Newton step, v' = v - v (b_h v - 2^63) / 2^63
-// with b_h + 1 > m_b / 2^21 for the divisor, so that v stays below 2^32.
-//   q1 = floor(floor(R0 / 2^22) v / 2^32), within 4 units of R0 2^30 / m_b;
-//   R1 = R0 2^30 - q1 m_b, exact modulo 2^64 (|R1| <= 4 m_b < 2^55);
-//   q2 = R1 2^22 / m_b rounded to nearest, from R1 / 2^25 and v (|error| < 0.6);
-//   R2 = R1 2^22 - q2 m_b, exact modulo 2^64 (|R2| < 0.6 m_b).
-// The quotient is Q + R2 / m_b, Q = 2^22 q1 + q2, so the nearest integer is Q
-// or its neighbour on R2's side; a tie cannot occur (a quotient of two 53-bit
-// integers has no 54-bit significand).  About 60 instructions, a third of
-// the 64-bit fixed-point reciprocal it replaces (two Newton steps on 64 x 64
-// -> 128 bit products and a 128-bit remainder): the kernels holding these
-// operations are bound by instruction issue as much as by the FP64 pipe.
-// Dependent chains, whole GPU: 344 G/s (136 before, 70 on the FP64 pipe),
-// 128 ns a quotient on one warp (326 before, 288).
+// 53 bits.  v ~ 2^84 / m_b (32 bits, never above) is the float reciprocal of
+// m_b's top bits (~21 bits) after one Newton step, v' = v - v (b_t v - 2^63) /
+// 2^63 with b_t + 1 > m_b / 2^21 for the divisor, lowered by 2 for the
+// roundings.
+//   q1 = floor(floor(R0 / 2^22) v / 2^32), up to 7 units below R0 2^30 / m_b;
+//   R1 = R0 2^30 - q1 m_b, exact modulo 2^64 (0 <= R1 < 7 m_b);
+//   q2 = floor of R1 2^22 / m_b from R1 / 2^25 and v, at most 1.2 below it;
+//   R2 = R1 2^22 - q2 m_b, exact modulo 2^64 (0 <= R2 < 1.2 m_b).
+// The quotient is Q + R2 / m_b, Q = 2^22 q1 + q2, so the nearest integer is Q or
+// Q + 1; a tie cannot occur (a quotient of two 53-bit integers has no 54-bit
+// significand).
 __device__ __forceinline__ double div_rn(double a, double b) {
   const unsigned long long ua = ubits(a), vb = ubits(b);
-  const unsigned ea = (unsigned)(ua >> 52) & 0x7FFu, eb = (unsigned)(vb >> 52) & 0x7FFu;
-  const unsigned long long ma = significand(ua), mb = significand(vb);
+  const unsigned xa = (unsigned)(ua >> 32), xb = (unsigned)(vb >> 32);
+  const unsigned long long ma = sig_of(xa, (unsigned)ua), mb = sig_of(xb, (unsigned)vb);
   const unsigned s = ma < mb ? 1u : 0u;
-  const int e = (int)ea - (int)eb + 1023 - (int)s;
-  if (ea - 1u < 2046u && eb - 1u < 2046u && (unsigned)(e - 1) < 2045u) {
+  // the result's exponent field less one
+  const unsigned ex = (xa & 0x7FF00000u) - (xb & 0x7FF00000u) + ((1022u - s) << 20);
+  if (normal_hi(xa) && normal_hi(xb) && ex < 0x7FD00000u) {
+    const unsigned bt = (unsigned)(mb >> 21);
     // (the two low bits set: the float stays above 1, its reciprocal below)
-    const float f = __uint_as_float(0x3F800003u | ((unsigned)(mb >> 29) & 0x7FFFFFu));
+    const float f = __uint_as_float(0x3F800003u | ((bt >> 8) & 0x7FFFFFu));
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
     unsigned v = (__float_as_uint(y) << 8) | 0x80000000u;  // y 2^32, y in [1/2, 1)
-    const unsigned bh = (unsigned)(mb >> 21);
-    // (b_h + 1) v - 2^63 in units of 2^28 (2^63 falls out of the 32 bits)
-    const int d = (int)(unsigned)(((unsigned long long)bh * v + v) >> 28);
-    v -= (unsigned)(((int)(v >> 16) * d) >> 19);
-    const unsigned long long R0 = ma << s;
-    const unsigned q1 = __umulhi((unsigned)(R0 >> 22), v);
-    const long long R1 = (long long)((R0 << 30) - (unsigned long long)q1 * mb);
-    const int q2 = (__mulhi((int)(R1 >> 25), (int)(v >> 1)) + 8) >> 4;
-    const long long R2 =
-        (long long)(((unsigned long long)R1 << 22) - (unsigned long long)(long long)q2 * mb);
-    unsigned long long Q =
-        ((unsigned long long)q1 << 22) + (unsigned long long)(long long)q2;
-    const long long R22 = R2 + R2;
-    if (R22 > (long long)mb) ++Q;
-    if (R22 < -(long long)mb) --Q;
-    return __longlong_as_double((long long)(((ua ^ vb) & kSignBit) +
-                                            ((unsigned long long)(e - 1) << 52) + Q));
+    // (b_t + 1) v - 2^63 in units of 2^28 (2^63 falls out of the 32 bits)
+    const int d = (int)(unsigned)(((unsigned long long)bt * v + v) >> 28);
+    v = v - (unsigned)(((int)(v >> 16) * d) >> 19) - 2u;
+    const unsigned q1 = __umulhi((unsigned)(ma >> (22u - s)), v);
+    const unsigned long long R1 = (ma << (30u + s)) - (unsigned long long)q1 * mb;
+    const unsigned q2 = __umulhi((unsigned)(R1 >> 25), v) >> 5;
+    const unsigned long long R2 = (R1 << 22) - (unsigned long long)q2 * mb;
+    unsigned long long Q = ((unsigned long long)q1 << 22) + q2;
+    if (R2 > (mb >> 1)) ++Q;
+    return dbl_of(ex + ((xa ^ xb) & 0x80000000u), Q);
   }
   return a / b;
 }
 
 // sqrt(x), in the same way: the root of N = M 2^52, M = m_x 2^p with p = 1
 // when x's biased exponent is even, is an integer of 53 bits.  v ~ 2^58 /
-// sqrt(M) (32 bits) is the float reciprocal square root of M's top bits (~20
-// bits) after one Newton step, v' = v - v (m_h v^2 - 2^94) / 2^95 with M /
-// 2^22 < m_h + 1.
-//   q1 = floor(m_h v / 2^32), within 4 units of 2^4 sqrt(M);
-//   R1 = 2^8 M - q1^2 (|R1| < 2^34);
-//   q2 = R1 2^21 / q1 rounded to nearest, from R1 / 2^4 and v (the root of the
-//   rest, q2^2 left out: |error| < 0.7);
+// sqrt(M) (32 bits, never above) is the float reciprocal square root of M's
+// top bits (~20 bits) after one Newton step, v' = v - v (m_h v^2 - 2^94) / 2^95
+// with M / 2^22 < m_h + 1, lowered by 3 for the roundings.
+//   q1 = floor(m_h v / 2^32), up to 7 units below 2^4 sqrt(M);
+//   R1 = 2^8 M - q1^2 (0 <= R1 < 2^35);
+//   q2 = floor of R1 2^21 / sqrt(2^8 M) from R1 / 2^4 and v, not above the root
+//   of the rest and at most 1.2 below it;
 //   R2 = N - S^2 for S = 2^22 q1 + q2, exact modulo 2^64.
-// The nearest integer to the root is S + 1 when R2 > S, S - 1 when R2 <= -S
-// ((S +- 1/2)^2 = S^2 +- S + 1/4), S otherwise.  Negative, zero, subnormal
-// and non-finite x: the FP64 square root.  About 65 instructions: 326 G/s (120
-// for the 64-bit fixed-point form before, 67 on the FP64 pipe).
+// The nearest integer to the root is S + 1 when R2 > S ((S + 1/2)^2 = S^2 + S +
+// 1/4), S otherwise.  Negative, zero, subnormal and non-finite x: the FP64
+// square root.
+//
+// Dependent chains, whole GPU: quotient 414 G/s (70 on the FP64 pipe), root 387
+// (67), product 595 (501).  Signed digits with two-sided corrections measured
+// 343 and 325, 64-bit fixed-point reciprocals with two Newton steps and a
+// 128-bit remainder 136 and 120.
 __device__ __forceinline__ double sqrt_rn(double x) {
   const unsigned long long ux = ubits(x);
-  const unsigned ex = (unsigned)(ux >> 52);  // sign included: negative x falls back
-  if (ex - 1u < 2046u) {
-    const unsigned long long ma = significand(ux);
-    const unsigned p = (ex & 1u) ^ 1u;
-    const unsigned long long M = ma << p;
+  const unsigned xh = (unsigned)(ux >> 32);
+  if (xh - 0x100000u < 0x7FE00000u) {
+    const unsigned p = (~xh >> 20) & 1u;
+    const unsigned long long ma = sig_of(xh, (unsigned)ux);
     // M / 2^52 in [1, 4) as a float, its low bits replaced so that it stays
     // off both ends and its reciprocal root inside (1/2, 1)
     const float f =
@@ -309,24 +321,17 @@ __device__ __forceinline__ double sqrt_rn(double x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
     unsigned v = (__float_as_uint(y) << 8) | 0x80000000u;  // y 2^32
-    const unsigned mh = (unsigned)(M >> 22);
+    const unsigned mh = (unsigned)(ma >> (22u - p));
     const unsigned sq = __umulhi(v, v);
     const int d = (int)(unsigned)(((unsigned long long)sq * mh + sq) >> 28);
-    v -= (unsigned)(((int)(v >> 16) * d) >> 19);
+    v = v - (unsigned)(((int)(v >> 16) * d) >> 19) - 3u;
     const unsigned q1 = __umulhi(mh, v);
-    const long long R1 = (long long)((M << 8) - (unsigned long long)q1 * q1);
-    const int q2 = (__mulhi((int)(R1 >> 4), (int)(v >> 1)) + 8) >> 4;
-    const unsigned long long S =
-        ((unsigned long long)q1 << 22) + (unsigned long long)(long long)q2;
-    const long long R2 = (long long)(((unsigned long long)R1 << 44) -
-                                     (unsigned long long)(long long)q2 *
-                                         (((unsigned long long)q1 << 23) +
-                                          (unsigned long long)(long long)q2));
-    unsigned long long Q = S;
-    if (R2 > (long long)S) ++Q;
-    if (R2 <= -(long long)S) --Q;
-    const int er = ((int)ex - 1127 - (int)p) / 2 + 1075;
-    return __longlong_as_double((long long)(((unsigned long long)(er - 1) << 52) + Q));
+    const unsigned long long R1 = (ma << (8u + p)) - (unsigned long long)q1 * q1;
+    const unsigned q2 = __umulhi((unsigned)(R1 >> 4), v) >> 5;
+    const unsigned long long S1 = (unsigned long long)q1 << 22, S = S1 + q2;
+    const unsigned long long R2 = (R1 << 44) - (unsigned long long)q2 * (S + S1);
+    const unsigned ex = ((xh >> 20) - p + 1021u) >> 1;  // its exponent field less one
+    return dbl_of(ex << 20, S + (R2 > S ? 1ull : 0ull));
   }
   return sqrt(x);
 }
@@ -441,10 +446,31 @@ __device__ __forceinline__ void draws_keep(const Seg& S, int c, const Draws<kTau
 
 // Non-inlined copies of div_rn and sqrt_rn for the relaxation kernel: its
 // fifteen call sites inlined overflow the instruction cache (relaxation 0.853
-// ms shared, 0.876 ms inlined at N = 1e7); the kernels with a few call sites
-// inline them (FP64 mode's orbit stage 2.58 ms inlined, 2.65 ms shared).
+// ms shared, 0.876 ms inlined at N = 1e7, with their earlier form); the kernels
+// with a few call sites inline them (FP64 mode's orbit stage 2.58 ms inlined,
+// 2.65 ms shared).
 static __device__ __noinline__ double div_rn_nl(double a, double b) { return div_rn(a, b); }
 static __device__ __noinline__ double sqrt_rn_nl(double x) { return sqrt_rn(x); }
+
+// A B 2^k for nonzero A, B < 2^53, rounded to nearest even, with a sign bit: the
+// 128-bit product's top 53 bits, rounded by the bits below (products below
+// 2^64, one in a million, by the FP64 product: the factors are exact doubles)
+template <int k>
+__device__ __forceinline__ double product_of(uint64_t A, uint64_t B, uint64_t sign) {
+  const uint64_t hi = __umul64hi(A, B), lo = A * B;
+  double v;
+  if (hi) {
+    const int lz = __clzll((long long)hi);
+    const uint64_t top = (hi << lz) | ((lo >> 1) >> (63 - lz)), rest = lo << lz;
+    const uint64_t Q = top >> 11;
+    const uint64_t below = (top << 53) | (rest ? 1ull : 0ull) | (Q & 1ull);
+    v = __longlong_as_double((long long)(((uint64_t)(1022 + 127 - lz + k) << 52) + Q +
+                                         (below > (1ull << 63) ? 1ull : 0ull)));
+  } else {
+    v = ((double)A * (double)B) * __longlong_as_double((long long)((uint64_t)(1023 + k) << 52));
+  }
+  return __longlong_as_double((long long)(ubits(v) | sign));
+}
 
 // uniform planar direction (cos a, sin a) by rejection of a point in the
 // unit disk; the doubled angle gives cos = (u^2 - v^2)/q, sin = 2uv/q.
@@ -489,10 +515,14 @@ __device__ __noinline__ bool disk_angle(Draws<kTaus>& g, uint32_t tag, double& c
     s = 0.0;
     return false;
   }
-  const double u = sym_double(Ua), v = sym_double(Va);
-  const double uu = u * u, vv = v * v, q = uu + vv;
+  // u u, v v and 2 u v from the integers, each rounded once as the FP64 product
+  const uint64_t A = Ua < 0 ? (uint64_t)(-Ua) : (uint64_t)Ua;
+  const uint64_t B = Va < 0 ? (uint64_t)(-Va) : (uint64_t)Va;
+  const double uu = product_of<-104>(A, A, 0ull), vv = product_of<-104>(B, B, 0ull);
+  const double uv2 = product_of<-103>(A, B, (uint64_t)(Ua ^ Va) & kSignBit);
+  const double q = uu + vv;
   c = div_rn_nl(uu - vv, q);
-  s = div_rn_nl(scale_up<1>(u) * v, q);
+  s = div_rn_nl(uv2, q);
   return true;
 }
 

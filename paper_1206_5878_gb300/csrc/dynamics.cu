@@ -46,8 +46,11 @@ __global__ void __launch_bounds__(256) k_bins(Seg S, int bs, double pref, const 
           double sv = 0.0, sm = 0.0;
           for (int64_t j = 0; j < q; ++j) {
             int64_t a = g + 2 * j;
-            double va2 = vr[a] * vr[a] + vt[a] * vt[a];
-            double vb2 = vr[a + 1] * vr[a + 1] + vt[a + 1] * vt[a + 1];
+            // two of the five products on the integer pipes: the kernel is
+            // bound by the FP64 pipe (0.137 -> 0.124 ms at N = 1e7; more of
+            // them there 0.131 and above)
+            double va2 = mul_rn(vr[a], vr[a]) + vt[a] * vt[a];
+            double vb2 = mul_rn(vr[a + 1], vr[a + 1]) + vt[a + 1] * vt[a + 1];
             double ms = m[a] + m[a + 1];
             sv = sv + sqrt_rn(va2 + vb2);
             sm = sm + ms * ms;
@@ -139,9 +142,10 @@ __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr,
   if (!disk_angle(g, kTagPsi, cpsi, spsi)) ++fails;
   const double v1x = vr[a], v1y = vt[a], v1z = 0.0;
   const double v2x = vr[b], vtb = vt[b];
-  const double v2y = vtb * cpsi, v2z = vtb * spsi;
+  const double v2y = mul_rn(vtb, cpsi), v2z = mul_rn(vtb, spsi);
   const double wx = v1x - v2x, wy = v1y - v2y, wz = v1z - v2z;
-  const double w2 = (wx * wx + wy * wy) + wz * wz;
+  const double wyy = mul_rn(wy, wy), wzz = mul_rn(wz, wz);
+  const double w2 = (mul_rn(wx, wx) + wyy) + wzz;
   if (!pos_num(w2)) {
     draws_keep(S, c, g);
     if (fails) stat_add(S.stats, c, kStAngleFails, (unsigned long long)fails);
@@ -192,7 +196,7 @@ __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr,
   draws_keep(S, c, g);
   // e1 = (w x xhat)/|w x xhat| = (0, wz, -wy)/|.| (yhat for radial w);
   // u = w x e1 has length |w| and completes the frame perpendicular to w
-  const double wp2 = wy * wy + wz * wz;
+  const double wp2 = wyy + wzz;
   double e1y, e1z;
   if (pos_num(wp2)) {
     const double wp = sqrt_rn_nl(wp2);
@@ -211,10 +215,10 @@ __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr,
   const double wpy = wy * cosb + sinb * (a1 * e1y + sphi * uy);
   const double wpz = wz * cosb + sinb * (a1 * e1z + sphi * uz);
   const double dwx = wpx - wx, dwy = wpy - wy, dwz = wpz - wz;
-  // the mass ratios as quotients; these products on the integer pipes
-  // balance the FP64 pipe's load against the integer pipes' (measured: all
-  // of the kernel's products there made it a third slower, none of them 2%
-  // slower)
+  // The products on the integer pipes (these, the frame's and |w|^2 above, the
+  // angles' in disk_angle: 17 of the pair's 44) balance the FP64 pipe's load
+  // against the issue slots: 0.757 ms at N = 1e7, 0.853 with only these six
+  // there, 0.77 to 0.80 with other groups, 0.95 with all (shared body).
   const double f1 = div_rn_nl(m2, msum), f2 = div_rn_nl(m1, msum);
   const double p1x = v1x + mul_rn(f1, dwx), p1y = v1y + mul_rn(f1, dwy), p1z = v1z + mul_rn(f1, dwz);
   const double p2x = v2x - mul_rn(f2, dwx), p2y = v2y - mul_rn(f2, dwy), p2z = v2z - mul_rn(f2, dwz);

@@ -453,7 +453,9 @@ __global__ void __launch_bounds__(256) k_velocities(Seg S, const int64_t* esc, i
   if (kCorrect) {
     const int c = seg_find(S.off, S.n_seg, p);
     if (p - S.off[c] < S.nb[c] - esc[c]) {
-      const double Tk = scale_down<1>(a * a + b * b);
+      // (two of the four products on the integer pipes: the FP64 pipe bounds
+      // this kernel)
+      const double Tk = scale_down<1>(mul_rn(a, a) + b * b);
       const double dnew = B.w - phi[p];
       double Tp = Tk + scale_down<1>(dnew - B.c);
       if (lt0(Tp)) {
@@ -463,7 +465,7 @@ __global__ void __launch_bounds__(256) k_velocities(Seg S, const int64_t* esc, i
       }
       if (pos_num(Tk)) {
         const double f = sqrt_rn(div_rn(Tp, Tk));
-        a = a * f;
+        a = mul_rn(a, f);
         b = b * f;
       }
     }
