@@ -284,7 +284,7 @@ void record_step(cmc_ctx* c, cudaStream_t st, cudaEvent_t* ev = nullptr) {
                             c->Mbuf, true, true, c->bk, st);
   else
     launch_potential(L, c->r_alt, c->x_alt, c->m, c->tile_a, c->tile_b, c->phi, nullptr, nullptr,
-                     true, st, nullptr, nullptr, true);
+                     true, st, nullptr, true);
   mark(7);
   // (the FP64 modes evaluate Phi_new(r_old) in Eq. 6's division form)
   const bool correct = c->cfg.energy_correction != 0;
@@ -1374,7 +1374,7 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
       if (!e) {
         launch_buckets(S.L, t32, false, bk, st);
         launch_slopes(n, x, phi, sl, st);
-        launch_make_nodes(n, r, x, phi, sl, bk.node, bk.tdf, st);
+        launch_make_nodes(n, r, x, phi, sl, bk.node, st);
         launch_grid(S.L, x, phi, sl, false, bk, st);
       }
     }

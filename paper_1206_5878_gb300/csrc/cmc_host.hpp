@@ -249,7 +249,7 @@ void launch_velocities(const SegLayout& L, const uint32_t* order, const RecB* rb
 // potential: per-tile sums then the tile-local scans (Eqs. 1-5 in scan
 // form).  nb_sub: subtract esc_step from nb (after the orbit step).
 // Optional outputs: t32 (float 1/r, Phi), Mout (M_k) and node (the record
-// {r, 1/r, Phi, M_k} of every star: one 32-byte sector per node for the
+// {1/r, Phi, r, M_k} of every star: one 32-byte sector per node for the
 // kernels that read a few nodes at random).  slopes: Mout and the records
 // carry the slope of Eq. 6 across each shell instead of M_k (the shell
 // parameter the FP64 orbit step takes).
@@ -268,11 +268,11 @@ struct TableOut {
 void launch_potential(const SegLayout& L, const double* r, const double* x, const double* m,
                       double* tile_m, double* tile_mx, double* phi, float2* t32,
                       double* Mout, bool nb_sub, cudaStream_t st, double4_32a* node = nullptr,
-                      float4* tdf = nullptr, bool sums_ready = false, bool slopes = false,
+                      bool sums_ready = false, bool slopes = false,
                       const TableOut* tables = nullptr);
-// node records (and float-pair table) from the arrays (stage calls)
+// node records from the arrays (stage calls)
 void launch_make_nodes(int64_t n, const double* r, const double* x, const double* phi,
-                       const double* M, double4_32a* node, float4* tdf, cudaStream_t st);
+                       const double* M, double4_32a* node, cudaStream_t st);
 
 void launch_correction(const SegLayout& L, const double* r, const double* x,
                        const double* phi, double* vr, double* vt, const double* r_old,
@@ -319,8 +319,7 @@ struct BucketArgs {
   const int64_t* goff = nullptr;
   const int4* gprm = nullptr;    // key0, sh, cells, key of 1/r_0 (as int)
   const float4* gaux = nullptr;  // Phi_0, bound mass, 1/r at key0, interpolation bound
-  const double4_32a* node = nullptr; // {r, 1/r, Phi, M} per star (potential kernel)
-  const float4* tdf = nullptr;       // {1/r, Phi} per star as float pairs (hi, lo, hi, lo)
+  const double4_32a* node = nullptr; // {1/r, Phi, r, M} per star (potential kernel)
 };
 
 struct BucketWork {
@@ -335,13 +334,11 @@ struct BucketWork {
   float4* gaux = nullptr;
   int64_t gcells = 0;  // grid cells over all segments
   double4_32a* node = nullptr;
-  float4* tdf = nullptr;
   BucketArgs args() const {
     BucketArgs a;
     a.start = start; a.off = off; a.base = base; a.prm = prm;
     a.gphi = gphi; a.goff = goff; a.gprm = gprm; a.gaux = gaux;
     a.node = node;
-    a.tdf = tdf;
     return a;
   }
 };

@@ -11,16 +11,14 @@
 //   is F = 1.2 max_j g(s_j) on s_j = -1 + (j + 1/2)/10.5, j = 0..20.
 //   v_t = J/r_new, v_r = +-sqrt(Q(r_new)).
 //
-// precision 0 (FP64): every operation is the FP64 operation of the
-// method's statement, in the same order, so results are bit-identical to
-// it.  precision 1 (mixed): the bisections, the bound F and the accept
-// tests run in FP32 on an interleaved float2 (1/r, Phi) table, the F
-// samples and trials located through a radius-bucket index; the brackets
-// are then verified (and moved if needed) in FP64, the turning points are
-// the FP64 shell roots with the shell slope taken from the enclosed mass,
-// and the accepted radius, its potential and the velocities are
-// recomputed in FP64.  A mixed result matches the FP64 result to rounding
-// whenever both accept the same trial.
+// precision 0 (FP64): every result is that of the FP64 operations of the
+// method's statement, in the same order (searches and accept tests screened in
+// floats with error bounds), so it is bit-identical to it.  precision 1
+// (mixed): the same turning points; the bound F and the accept tests run in
+// FP32 on the potential grid, the trials they cannot decide in FP64, and the
+// accepted radius, its potential (by the shell's slope) and the velocities are
+// FP64.  A mixed result matches the FP64 result to rounding whenever both
+// accept the same trial.
 #include "cmc_host.hpp"
 
 namespace cmc {
@@ -31,6 +29,7 @@ struct Star {
   double E, J;
   int64_t k;
 };
+
 
 // Q = 2 (E - Phi) - (J x)^2 from node values, as Q_node64 evaluates it
 __device__ __forceinline__ double Qv(const Star& s, double x, double p) {
@@ -138,13 +137,13 @@ __device__ __forceinline__ int64_t fix_shell_nodes(const double4_32a* __restrict
   a = nd[i < 0 ? 0 : i];
   double4_32a b = i + 1 < nb ? nd[i + 1] : a;
   for (int w = 0; w < 64; ++w) {
-    if (i + 1 < nb && dbits(b.x) <= qb) {
+    if (i + 1 < nb && dbits(b.z) <= qb) {
       ++i;
       a = b;
       if (i + 1 < nb) b = nd[i + 1];
       continue;
     }
-    if (i >= 0 && dbits(a.x) > qb) {
+    if (i >= 0 && dbits(a.z) > qb) {
       --i;
       b = a;
       a = nd[i < 0 ? 0 : i];
@@ -155,7 +154,7 @@ __device__ __forceinline__ int64_t fix_shell_nodes(const double4_32a* __restrict
   int64_t lo = -1, hi = nb;
   while (hi - lo > 1) {
     const int64_t mid = lo + ((hi - lo) >> 1);
-    if (dbits(nd[mid].x) <= qb) lo = mid; else hi = mid;
+    if (dbits(nd[mid].z) <= qb) lo = mid; else hi = mid;
   }
   a = nd[lo < 0 ? 0 : lo];
   return lo;
@@ -213,10 +212,6 @@ __constant__ double c_s64[21] = {CMC_SJ21(CMC_SJ)};
 __constant__ float c_sa32[21] = {CMC_SJ21(CMC_SJA)};
 __constant__ float c_sb32[21] = {CMC_SJ21(CMC_SJB)};
 
-// ---- FP32 searches run in lockstep: K independent searches per thread,
-// each round issues K independent loads before any of them is needed.
-__device__ __forceinline__ int search_rounds(int nb) { return 32 - __clz(nb); }
-
 // Radius-bucket index of one segment's float table.  It covers the nodes
 // lo..hi, all but the sparse 1/1024 at each end (where a bucket resolution
 // fine enough for the core would leave long runs of empty buckets).
@@ -234,92 +229,46 @@ struct Buckets {
   int shift, nbk, lo, hi;
 };
 
-// largest i with x_i >= xq[q], else -1, for K queries (lockstep).
-// The bucket of a query gives the bracket (start[b] - 1, start[b+1]); the
-// keys inside one bucket are close to uniform, so the query's position in
-// its bucket predicts the shell.  Each round loads 4 nodes per unfinished
-// query at once: the first round around the prediction, later rounds
-// evenly over the bracket (a bucket of up to 16 nodes takes at most 2
-// rounds, a prediction that is right 1).  Queries in the tails outside the
-// index search their tail the same way.  Any probe keeps the bracket
-// valid (x falls with i), so the answer is the unique one of a bisection.
-//
-// The keys probed are those of a table adaptor: the float keys (1/r as a
-// float, the high part of a float pair: FloatKeys) or the FP64 1/r of the
-// node records compared on their bit patterns (NodeKeys; positive doubles
-// order like their patterns).  Probing the table that the caller reads next
-// (the float pairs of the bracket walks, the node record of the shell)
-// brings its lines into the cache with the search.
-struct FloatKeys {
-  const float* p;  // key i at p[i * stride]
-  int stride;
-  using V = float;
-  __device__ __forceinline__ V load(int i) const { return __ldg(p + (size_t)i * stride); }
-  __device__ __forceinline__ V key(float q) const { return q; }
-};
-struct NodeKeys {
-  const double4_32a* nd;
-  using V = long long;
-  __device__ __forceinline__ V load(int i) const { return dbits(nd[i].y); }
-  // the query widened to FP64 exactly, as bits (queries are positive, finite)
-  __device__ __forceinline__ V key(float q) const { return dbits((double)q); }
-};
-
-template <int K, class Tab>
-__device__ __forceinline__ void shells32_bk(const Tab& tab, int nb, const Buckets& B,
-                                            const float (&xq)[K], int (&out)[K]) {
-  typename Tab::V kq[K];
-#pragma unroll
-  for (int q = 0; q < K; ++q) kq[q] = tab.key(xq[q]);
-  int lo[K], hi[K], pred[K];
+// The shell of the float key xq, to about one node: by the place of the key in
+// its bucket (the keys in a bucket are close to uniform), by bisection in the
+// tails outside the index.  One look at the index and none at the nodes: every
+// caller walks to the exact node from there, and on this GPU the kernels that
+// do are bound by the number of random accesses when the tables exceed the L2
+// (about 47 G/s).
+// K queries at once, so that their looks at the index overlap.
+template <int K>
+__device__ __forceinline__ void near_shells(const double4_32a* __restrict__ nd, int nb,
+                                            const Buckets& B, const float (&xq)[K],
+                                            int (&out)[K]) {
+  int s0[K], s1[K];
 #pragma unroll
   for (int q = 0; q < K; ++q) {
-    pred[q] = -2;  // no prediction
     const long long d = (long long)B.base - (long long)__float_as_uint(xq[q]);
-    if (d < 0) { lo[q] = -1; hi[q] = B.lo; continue; }           // inner tail
     const long long b = d >> B.shift;
-    if (b >= B.nbk) { lo[q] = B.hi; hi[q] = nb; continue; }      // outer tail
-    if (!CMC_IN(b + 1, B.nbk + 1)) { lo[q] = -1; hi[q] = nb; continue; }
-    const int s0 = __ldg(B.start + b), s1 = __ldg(B.start + b + 1);
-    lo[q] = s0 - 1;
-    hi[q] = s1;
-    const int frac = (int)(d & ((1ll << B.shift) - 1));
-    pred[q] = s0 - 1 + (int)(((long long)(s1 - s0) * frac + (1ll << (B.shift - 1 > 0 ? B.shift - 1 : 0))) >> B.shift);
-  }
-  bool more = true;
-  while (more) {
-    more = false;
-    int m[K][4];
-    typename Tab::V v[K][4];
-#pragma unroll
-    for (int q = 0; q < K; ++q) {
-      const int c = hi[q] - lo[q] - 1;  // candidates lo+1 .. hi-1
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        int mj;
-        if (pred[q] >= -1) mj = pred[q] - 1 + j;
-        else mj = lo[q] + 1 + (int)(((long long)(c > 0 ? c - 1 : 0) * j) / 3);
-        mj = mj < lo[q] + 1 ? lo[q] + 1 : mj;
-        mj = mj > hi[q] - 1 ? hi[q] - 1 : mj;
-        m[q][j] = mj;
-        v[q][j] = c > 0 && CMC_IN(mj, nb) ? tab.load(mj) : typename Tab::V(0);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < K; ++q) {
-      if (hi[q] - lo[q] > 1) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (v[q][j] >= kq[q]) lo[q] = m[q][j] > lo[q] ? m[q][j] : lo[q];
-          else hi[q] = m[q][j] < hi[q] ? m[q][j] : hi[q];
-        }
-        pred[q] = -2;
-        more |= hi[q] - lo[q] > 1;
-      }
+    s0[q] = s1[q] = -1;
+    if (d >= 0 && b < B.nbk && CMC_IN(b + 1, B.nbk + 1)) {
+      s0[q] = __ldg(B.start + b);
+      s1[q] = __ldg(B.start + b + 1);
     }
   }
 #pragma unroll
-  for (int q = 0; q < K; ++q) out[q] = lo[q];
+  for (int q = 0; q < K; ++q) {
+    const uint32_t d = B.base - __float_as_uint(xq[q]);
+    if (s1[q] >= 0) {
+      const uint32_t f = B.shift ? d << (32 - B.shift) : 0u;  // 2^32 x the place
+      out[q] = s0[q] - 1 +
+               (int)(((unsigned long long)(uint32_t)(s1[q] - s0[q]) * f + 0x80000000ull) >> 32);
+    } else {
+      const bool inner = (long long)B.base < (long long)__float_as_uint(xq[q]);
+      const long long kq = dbits((double)xq[q]);  // (positive doubles order like their bits)
+      int lo = inner ? -1 : B.hi, hi = inner ? B.lo : nb;
+      while (hi - lo > 1) {
+        const int m = lo + ((hi - lo) >> 1);
+        if (dbits(nd[m].x) >= kq) lo = m; else hi = m;
+      }
+      out[q] = lo;
+    }
+  }
 }
 
 // The potential grid of one segment (see BucketArgs): Phi (float) at the
@@ -382,14 +331,16 @@ __device__ __forceinline__ float g32_grid(const Grid& G, float E, float J, float
   return Q > 0.0f ? drds * rq : 0.0f;
 }
 
-// the FP32 shell (bucket index) of the point r(s), the start of the FP64
+// about the shell of the point r(s) (bucket index), the start of the FP64
 // shell walk of an accepted or edge point
 __device__ __forceinline__ int shell32_of(const double4_32a* __restrict__ nd, int nb,
                                           const Buckets& B, float c0, float c1, float sv) {
   const float rs = c0 + c1 * (sv * (3.0f - sv * sv));
-  const float xq[1] = {1.0f / rs};
+  float xq;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(xq) : "f"(rs));
+  const float q[1] = {xq};
   int sh[1];
-  shells32_bk<1>(NodeKeys{nd}, nb, B, xq, sh);
+  near_shells<1>(nd, nb, B, q, sh);
   return sh[0];
 }
 
@@ -404,7 +355,7 @@ __device__ __forceinline__ void point64(const double4_32a* __restrict__ nd, int6
   double4_32a a;
   i64 = (int)fix_shell_nodes(nd, nb, sh, rs, a);
   xs = div_rn(1.0, rs);
-  ph = i64 < 0 ? a.z : a.z + a.w * (a.y - xs);
+  ph = i64 < 0 ? a.y : a.y + a.w * (a.x - xs);
   L = st.J * xs;
   Q = scale_up<1>(st.E - ph) - L * L;
 }
@@ -424,16 +375,16 @@ __device__ __forceinline__ void point64_div_sa(const double4_32a* __restrict__ n
   i = (int)fix_shell_nodes(nd, nb, sh, rs, a);
   xq = div_rn(1.0, rs);
   if (i < 0) {
-    ph = a.z;  // node 0's Phi: the central constant
+    ph = a.y;  // node 0's Phi: the central constant
   } else {
     double xj1 = 0.0, pj1 = 0.0;
     if (i + 1 < nb) {
       const double4_32a b = nd[i + 1];
-      xj1 = b.y;
-      pj1 = b.z;
+      xj1 = b.x;
+      pj1 = b.y;
     }
-    const double den = a.y - xj1;
-    ph = !(den > 0.0) ? a.z : a.z + div_rn(a.y - xq, den) * (pj1 - a.z);
+    const double den = a.x - xj1;
+    ph = !(den > 0.0) ? a.y : a.y + div_rn(a.x - xq, den) * (pj1 - a.y);
   }
   L = div_rn(st.J, rs);
   Q = scale_up<1>(st.E - ph) - L * L;
@@ -463,51 +414,47 @@ __device__ __forceinline__ float u01f(uint32_t hi) {
   return (__uint_as_float(0x3F800000u | (hi >> 9)) - 1.0f) + 0x1p-24f;
 }
 
-// ------------------------------------------- double-float (float pairs)
-// A value as hi + lo with two floats (~48 bits), from the error-free sum of
-// two floats (Knuth's two-sum; every operation rounds once, no contraction)
-// and product (the fused multiply-add gives the product's error exactly).
+// ------------------------------------------------------- turning points
+// 1/r and Phi of a node, its radius and slope (one 16-byte load each)
+__device__ __forceinline__ double2 node_xp(const double4_32a* p) {
+  return *reinterpret_cast<const double2*>(p);
+}
+__device__ __forceinline__ double2 node_rw(const double4_32a* p) {
+  return reinterpret_cast<const double2*>(p)[1];
+}
+
+// Q at 1/r = x with Phi = p, the FP64 method's own evaluation
+__device__ __forceinline__ double q64_of(const Star& s, double x, double p) {
+  const double L = s.J * x;
+  return scale_up<1>(s.E - p) - L * L;
+}
+
+// Parts of a double as floats, from its bits: the top 24 significand bits in
+// [1, 2), and 2^exponent (0 unless within 2^-60 .. 2^60).  No conversion
+// instructions: on this GPU they take the FP64 pipe.
+__device__ __forceinline__ float top_of(unsigned long long u) {
+  return __uint_as_float(0x3F800000u | ((unsigned)(u >> 29) & 0x7FFFFFu));
+}
+__device__ __forceinline__ float pow2_of(unsigned long long u) {
+  const unsigned f = (unsigned)(u >> 52) & 0x7FFu;
+  return f - 963u <= 120u ? __uint_as_float((f - 896u) << 23) : 0.0f;
+}
+
+// ---- double-float (float pairs): a value as hi + lo with two floats, from
+// the error-free sum of two floats (Knuth's two-sum; every operation rounds
+// once, no contraction) and product (the fused multiply-add gives the
+// product's error exactly).
 struct DF {
   float hi, lo;
 };
 
-__device__ __forceinline__ DF df_of(double v) {
+// |v| to 2^-46 of it (its sign bit set in neg) for a double with pow2_of p2 > 0:
+// the top 24 significand bits, then the next 23
+__device__ __forceinline__ DF df_of(unsigned long long u, float p2) {
   DF d;
-  d.hi = (float)v;
-  d.lo = (float)(v - (double)d.hi);
-  return d;
-}
-
-// The same split from the bit pattern with integer operations (hi: the top
-// 24 significand bits of v, lo: the next 24 of the remaining 29, both
-// truncated, together within 2^-46 |v|), for 2^-60 <= |v| < 2^100 where both
-// are normal floats; other values (zero included) by the conversions.
-__device__ __forceinline__ DF df_split(double v) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
-  const unsigned ex = (unsigned)(u >> 52) & 0x7FFu;
-  if (ex < 1023u - 60u || ex >= 1023u + 100u) return df_of(v);
-  const unsigned sg = (unsigned)(u >> 32) & 0x80000000u;
-  DF d;
-  d.hi = __uint_as_float(sg | ((ex - 896u) << 23) | ((unsigned)(u >> 29) & 0x7FFFFFu));
-  const unsigned ml = (unsigned)u & 0x1FFFFFFFu;
-  if (ml == 0u) {
-    d.lo = 0.0f;
-    return d;
-  }
-  const int lz = __clz((int)ml);  // 3 .. 31
-  // ml 2^(ex - 1075) = 1.f 2^(ex - 1075 + 31 - lz); exponent field in [15, 202]
-  const unsigned fe = ex - 1075u + 127u + (unsigned)(31 - lz);
-  const unsigned mant = ((ml << lz) << 1) >> 9;  // the 23 bits after the leading one
-  d.lo = __uint_as_float(sg | (fe << 23) | mant);
-  return d;
-}
-
-__device__ __forceinline__ DF two_sum(float a, float b) {
-  const float s = a + b;
-  const float bb = s - a;
-  DF d;
-  d.hi = s;
-  d.lo = (a - (s - bb)) + (b - bb);
+  d.hi = top_of(u) * p2;
+  d.lo = ((__uint_as_float(0x4B000000u | ((unsigned)(u >> 6) & 0x7FFFFFu)) - 8388608.0f) *
+          0x1p-46f) * p2;
   return d;
 }
 
@@ -520,8 +467,9 @@ __device__ __forceinline__ DF df_norm(float hi, float lo) {
 }
 
 __device__ __forceinline__ DF df_sub(DF a, DF b) {
-  const DF s = two_sum(a.hi, -b.hi);
-  return df_norm(s.hi, s.lo + (a.lo - b.lo));
+  const float s = a.hi - b.hi, bb = s - a.hi;
+  const float e = (a.hi - (s - bb)) - (b.hi + bb);
+  return df_norm(s, e + (a.lo - b.lo));
 }
 
 __device__ __forceinline__ DF df_mul(DF a, DF b) {
@@ -530,242 +478,192 @@ __device__ __forceinline__ DF df_mul(DF a, DF b) {
   return df_norm(p, e + (a.hi * b.lo + a.lo * b.hi));
 }
 
-// Q = 2 (E - Phi) - (J x)^2 at a node from the float pairs, and whether its
-// sign is certain.  The pairs hold E, J (truncated or rounded) within
-// 2^-46 and 1/r, Phi within 2^-48; each pair sum adds at most 2^-46 of its
-// operands' magnitudes and each pair product 2^-45 of its result, so L^2
-// is within 2^-42.9 and Q within 2^-42.7 of S = |E| + |Phi| + L^2.  The
-// FP64 evaluation 2 (E - Phi) - (J x) (J x) from the doubles is within
-// 2^-50 S.  Beyond 2^-40 S both therefore have the sign of the exact Q.
-__device__ __forceinline__ float node_q_df(const float4* __restrict__ tdf, DF E, DF J, int i,
-                                           bool& sure) {
-  const float4 t = __ldg(tdf + i);
-  const DF x{t.x, t.y}, ph{t.z, t.w};
-  const DF d = df_sub(E, ph);
-  const DF L = df_mul(J, x);
-  const DF L2 = df_mul(L, L);
-  const DF q = df_sub(DF{2.0f * d.hi, 2.0f * d.lo}, L2);
-  const float qv = q.hi != 0.0f ? q.hi : q.lo;
-  sure = fabsf(qv) > 0x1p-40f * ((fabsf(E.hi) + fabsf(ph.hi)) + L2.hi);
-  return qv;
+// The star's constants of the walks below: |E|, J as float pairs (E < 0), J^2
+struct WalkStar {
+  DF E, J;
+  float J2;
+  bool ok;  // both within the float pairs' range
+};
+
+// The node of a sign change of Q, by a walk from node p (lo <= p <= hi; 1/r = x, Phi
+// = ph there).  Q counts as >= 0 at the star's end (at_hi false: r_max, whose star
+// is lo; true: r_min, whose star is hi) and as < 0 at the other end.  Returns
+// the lower node of the pair with different signs, -2 when the walk is too long.
+// Every sign is that of the FP64 method's evaluation of Q, found in floats:
+//
+// At p, Q = 2 (|Phi| - |E|) - (J x)^2 in float pairs.  E, J, 1/r and Phi are within
+// 2^-46, each pair sum adds at most 2^-46 of its operands and each pair
+// product 2^-45 of its result, so Q is within 2^-41.5 of S = |E| + |Phi| + L^2; the
+// FP64 evaluation is within 2^-50 S.  Beyond 2^-40 S the sign is certain.
+//
+// A node near p has Q = Q_p + 2 (|Phi| - |Phi_p|) - J^2 (x + x_p) (x - x_p).  In p's
+// binades the differences are those of the significands' bits (the top 24
+// exactly, the rest to 2^-44), J^2 is within 2^-22, x + x_p and each operation
+// round to 2^-24, Q_p to 2^-24 |Q_p| <= 2^-24 (|Q| + T), T the two terms'
+// magnitudes: within 2^-20 T + 2^-22 |Q| + 2^-41 S in all, and S there at most S + T.
+// Beyond 2^-19 T + 2^-40 S the sign is certain: 25 instructions.
+//
+// Otherwise the FP64 evaluation decides.
+struct Bracket {
+  int j;        // the lower node; -1: inside node 0, whose values it then has
+  double x, p;  // its 1/r and Phi
+};
+
+__device__ __forceinline__ bool walk_sign(const Star& s, const WalkStar& W,
+                                          const double4_32a* __restrict__ nd, int nb, int p,
+                                          int lo, int hi, bool at_hi, double2 at, Bracket& B) {
+  const unsigned long long xb = ubits(at.x), pb = ubits(at.y);
+  const float ex = pow2_of(xb), ep = pow2_of(pb);
+  const bool ok = W.ok && ex * ep != 0.0f;
+  const float x1 = top_of(xb), p1 = top_of(pb), x0 = x1 * ex;
+  const DF P = df_of(pb, ep), L = df_mul(W.J, df_of(xb, ex)), L2 = df_mul(L, L);
+  const DF d = df_sub(P, W.E), q2 = df_sub(DF{2.0f * d.hi, 2.0f * d.lo}, L2);
+  const float q0 = q2.hi != 0.0f ? q2.hi : q2.lo;
+  const float s40 = 0x1p-40f * ((W.E.hi + P.hi) + L2.hi);
+  bool pos = p == (at_hi ? hi : lo);
+  if (!pos && p != (at_hi ? lo : hi))
+    pos = ok && fabsf(q0) > s40 ? q0 > 0.0f : !lt0(q64_of(s, at.x, at.y));
+  const int step = pos == at_hi ? -1 : 1;
+  for (int w = 0; w < 64; ++w) {
+    const int c = p + step;
+    bool now = (c >= hi) == at_hi;
+    double2 t = at;
+    if (c >= 0 && c < nb) t = node_xp(nd + c);
+    if (c > lo && c < hi) {
+      const unsigned long long xcb = ubits(t.x), pcb = ubits(t.y);
+      // the differences of the low 29 bits, to 2^8 of them
+      const int lx = ((int)((unsigned)xcb & 0x1FFFFFFFu) - (int)((unsigned)xb & 0x1FFFFFFFu)) >> 8;
+      const int lp = ((int)((unsigned)pcb & 0x1FFFFFFFu) - (int)((unsigned)pb & 0x1FFFFFFFu)) >> 8;
+      const float fx = __uint_as_float(0x4B400000u + (unsigned)lx) - 12582912.0f;
+      const float fp = __uint_as_float(0x4B400000u + (unsigned)lp) - 12582912.0f;
+      const float dx = __fmaf_rn(fx, 0x1p-44f, top_of(xcb) - x1) * ex;
+      const float a = 2.0f * (__fmaf_rn(fp, 0x1p-44f, top_of(pcb) - p1) * ep);
+      const float b = (W.J2 * (2.0f * x0 + dx)) * dx;
+      const float q = (q0 + a) - b;
+      const bool sure = ok && (((xcb ^ xb) | (pcb ^ pb)) >> 52) == 0ull &&
+                        fabsf(q) > __fmaf_rn(0x1p-19f, fabsf(a) + fabsf(b), s40);
+      now = q > 0.0f;
+      if (!sure) now = !lt0(q64_of(s, t.x, t.y));
+    }
+    if (now != pos) {
+      B.j = step > 0 ? p : c;
+      B.x = step > 0 ? at.x : t.x;
+      B.p = step > 0 ? at.y : t.y;
+      return true;
+    }
+    p = c;
+    at = t;
+  }
+  return false;
 }
 
 // Q in FP32 at grid point g (1/r from the grid key, Phi from the grid)
-__device__ __forceinline__ float grid_q(const Grid& G, float E, float J, int g, float& xg) {
+__device__ __forceinline__ float grid_q(const Grid& G, float E, float J2, int g, float& xg) {
   xg = __uint_as_float(G.key0 + ((uint32_t)g << G.sh));
-  const float L = J * xg;
-  return 2.0f * (E - __ldg(G.phi + g)) - L * L;
+  return __fmaf_rn(-J2 * xg, xg, 2.0f * (E - __ldg(G.phi + g)));
 }
 
-__device__ __forceinline__ float node_q(const float4* __restrict__ tdf, float E, float J, int i) {
-  const float4 n = __ldg(tdf + i);  // (1/r, Phi) as the float pairs' high parts
-  const float L = J * n.x;
-  return 2.0f * (E - n.z) - L * L;
-}
-
-// FP32 node brackets of both turning points from the potential grid: the
-// sign changes of Q on the grid points (bisections on the L1-resident grid,
-// in lockstep), the root inside the cell by linear interpolation in 1/r,
-// its node through the bucket index, then a short walk over neighbouring
-// nodes to where Q32 changes sign (r_max: node j with Q32 >= 0, j + 1 with
-// Q32 < 0 or the virtual node nb; r_min: j with Q32 < 0 or -1, j + 1 with
-// Q32 >= 0 or the star).  Returns false when a walk exceeds its bound.
-__device__ __forceinline__ bool grid_brackets(const Grid& G, const float4* __restrict__ tdf,
-                                              const Buckets& BK, float E, float J, DF Ed, DF Jd,
-                                              int nb, int k, int& jmax, int& jmin, bool& cert1,
-                                              bool& cert2) {
-  const float xk = __ldg(&tdf[k].x);
+// Node brackets of both turning points: r_max's node j with Q >= 0 (the star
+// k counts as such) and j + 1 with Q < 0 (or the virtual node nb), r_min's j with
+// Q < 0 (or -1) and j + 1 with Q >= 0 (or the star).  The sign changes of Q on
+// the grid points (both searches abreast, a fixed number of rounds on a grid
+// that stays in the L1), the root inside the cell by linear interpolation in
+// 1/r, its node through the bucket index, and a walk from there to where the
+// FP64 evaluation of Q changes sign.  Q is concave in 1/r (Phi is convex), so
+// that sign change is the only one on its side and the search before the walk
+// need not be exact, only close.  False when a walk is too long.
+//
+// Bound by the L1's gathers (one wavefront per lane; 60-69% busy) with the FP64
+// pipe half busy.  N = 1e7: 0.99 ms, 180 B of DRAM a star; with a float-pair copy
+// of the table for the searches and walks, probes of four nodes a round and
+// FP64 walks where uncertified 1.27 ms, 338 B.  Both walks in one loop (1.08),
+// four-way grid rounds (1.08), the grid's top levels in shared memory (1.01)
+// and 40 to 64 registers (0.98 to 1.01) gave nothing.
+__device__ __forceinline__ bool grid_brackets(const Grid& G, const double4_32a* __restrict__ nd,
+                                              const Buckets& BK, const Star& s, int nb, int k,
+                                              float xk, float qk, Bracket& bmax,
+                                              Bracket& bmin) {
+  WalkStar W;
+  const float pE = pow2_of(ubits(s.E)), pJ = pow2_of(ubits(s.J));
+  W.ok = pE * pJ != 0.0f;
+  W.E = df_of(ubits(s.E), pE);
+  W.J = df_of(ubits(s.J), pJ);
+  W.J2 = W.J.hi * W.J.hi;
+  // (out of the pairs' range: radial or all but unbound orbits)
+  const float E = W.ok ? -W.E.hi : f32_rn(s.E);
+  const float J2 = W.ok ? W.J2 : f32_rn(s.J) * f32_rn(s.J);
   const uint32_t kk = __float_as_uint(xk);
-  cert1 = cert2 = false;
   if (G.cells < 2 || kk < G.key0) return false;
   int gk = (int)((kk - G.key0) >> G.sh);  // grid points 0..gk lie at or outside the star
   if (gk > G.cells - 1) gk = G.cells - 1;
-  // r_max: last grid point in [0, gk] with Q < 0 (-1: none; Q -> 2E < 0 as 1/r -> 0)
-  // r_min: first grid point in [gk + 1, cells) with Q < 0 (cells: none)
-  int alo = -1, ahi = gk + 1, blo = gk, bhi = G.cells;
-  float xa_lo = 0.0f, qa_lo = 0.0f, xb_hi = 0.0f, qb_hi = 0.0f;
-  float xa_hi = xk, qa_hi = 0.0f, xb_lo = xk, qb_lo = 0.0f;
-  while (ahi - alo > 1 || bhi - blo > 1) {
-    const bool ra = ahi - alo > 1, rb = bhi - blo > 1;
-    const int ma = ra ? (alo + ahi) >> 1 : 0, mb = rb ? (blo + bhi) >> 1 : 0;
-    float xa, xb;
-    const float qa = grid_q(G, E, J, ma, xa), qb = grid_q(G, E, J, mb, xb);
-    if (ra) {
-      if (qa < 0.0f) { alo = ma; xa_lo = xa; qa_lo = qa; }
-      else { ahi = ma; xa_hi = xa; qa_hi = qa; }
-    }
-    if (rb) {
-      if (qb < 0.0f) { bhi = mb; xb_hi = xb; qb_hi = qb; }
-      else { blo = mb; xb_lo = xb; qb_lo = qb; }
-    }
+  // r_max: the last grid point in [0, gk] with Q < 0 (-1: none; Q -> 2E < 0 as 1/r -> 0)
+  // r_min: the last one in [gk + 1, cells) with Q >= 0 (gk: none)
+  int ga = -1, gb = gk;
+  for (int st = 1 << (31 - __clz(G.cells)); st > 0; st >>= 1) {
+    const int ma = ga + st, mb = gb + st;
+    float x;
+    const float qa = grid_q(G, E, J2, ma < gk ? ma : gk, x);
+    const float qb = grid_q(G, E, J2, mb < G.cells ? mb : G.cells - 1, x);
+    if (ma <= gk && qa < 0.0f) ga = ma;
+    if (mb < G.cells && !(qb < 0.0f)) gb = mb;
   }
-  // the star's own end of each bracket: Q32 at the star
-  const float qk = node_q(tdf, E, J, k);
-  if (ahi == gk + 1) qa_hi = qk;
-  if (blo == gk) qb_lo = qk;
+  // root estimates between the two points of each sign change (the star itself
+  // on its side of the grid), and their nodes
+  const bool none1 = ga < 0, none2 = gb + 1 >= G.cells;
   float xq[2];
-  // root estimates (Q linear in 1/r across a cell up to ~(cell width)^2)
-  xq[0] = alo < 0 ? 0.0f : xa_lo + (xa_hi - xa_lo) * (qa_lo / (qa_lo - qa_hi));
-  xq[1] = bhi >= G.cells ? 0.0f : xb_lo + (xb_hi - xb_lo) * (qb_lo / (qb_lo - qb_hi));
-  int sh[2];
-  shells32_bk<2>(FloatKeys{&tdf[0].x, 4}, nb, BK, xq, sh);
-  int j1 = alo < 0 ? nb - 1 : sh[0];
-  int j2 = bhi >= G.cells ? -1 : sh[1];
-  j1 = j1 < k ? k : (j1 > nb - 1 ? nb - 1 : j1);
-  j2 = j2 < -1 ? -1 : (j2 > k - 1 ? k - 1 : j2);
-  // walks; at the stop the sign tests that ended each walk are the FP64
-  // walk's own stopping tests, and when every one of them is certain the
-  // FP64 walk from this bracket would stop at once (cert)
-  bool d1 = false, d2 = false, s1a = true, s2a = true;
-  for (int w = 0; w < 64 && !(d1 && d2); ++w) {
-    if (!d1) {
-      bool su = true, sd = true;
-      if (j1 + 1 < nb && !(node_q_df(tdf, Ed, Jd, j1 + 1, su) < 0.0f)) {
-        ++j1;
-      } else if (j1 > k && node_q_df(tdf, Ed, Jd, j1, sd) < 0.0f) {
-        --j1;
-      } else {
-        d1 = true;
-        s1a = su && sd;
-      }
+  {
+    float xl, xh;
+    const float ql = grid_q(G, E, J2, none1 ? 0 : ga, xl);
+    float qh = grid_q(G, E, J2, ga == gk ? gk : ga + 1, xh);
+    if (ga == gk) {
+      xh = xk;
+      qh = qk;
     }
-    if (!d2) {
-      bool su = true, sd = true;
-      if (j2 + 1 < k && node_q_df(tdf, Ed, Jd, j2 + 1, su) < 0.0f) {
-        ++j2;
-      } else if (j2 >= 0 && !(node_q_df(tdf, Ed, Jd, j2, sd) < 0.0f)) {
-        --j2;
-      } else {
-        d2 = true;
-        s2a = su && sd;
-      }
-    }
+    xq[0] = xl + (xh - xl) * __fdividef(ql, ql - qh);
   }
-  jmax = j1;
-  jmin = j2;
-  cert1 = d1 && d2 && s1a;
-  cert2 = d1 && d2 && s2a;
-  return d1 && d2;
+  {
+    float xl, xh;
+    float ql = grid_q(G, E, J2, gb, xl);
+    const float qh = grid_q(G, E, J2, none2 ? gb : gb + 1, xh);
+    if (gb == gk) {
+      xl = xk;
+      ql = qk;
+    }
+    xq[1] = xl + (xh - xl) * __fdividef(ql, ql - qh);
+  }
+  int pn[2];
+  near_shells<2>(nd, nb, BK, xq, pn);
+  int p1 = none1 ? nb - 1 : pn[0], p2 = none2 ? -1 : pn[1];
+  p1 = p1 < k ? k : (p1 > nb - 1 ? nb - 1 : p1);
+  p2 = p2 < -1 ? -1 : (p2 > k - 1 ? k - 1 : p2);
+  const int i2 = p2 < 0 ? 0 : p2;
+  const double2 t1 = node_xp(nd + p1), t2 = node_xp(nd + i2);
+  return walk_sign(s, W, nd, nb, p1, k, nb, false, t1, bmax) &&
+         walk_sign(s, W, nd, nb, p2, -1, k, true, t2, bmin);
 }
 
-// verify_rmax / verify_rmin on the node records: the same walks (a bounded
-// walk from the FP32 bracket, then the full bisection), returning the
-// records of the bracket's node (a; node 0 for r_min's -1) and of the node
-// after it (b)
-__device__ __forceinline__ int64_t verify_rmax_nodes(const Table64& T,
-                                                     const double4_32a* __restrict__ nd,
-                                                     const Star& s, int64_t j, double4_32a& a,
-                                                     double4_32a& b) {
-  const int64_t nb = T.nb;
-  if (j < s.k) j = s.k;
-  if (j > nb - 1) j = nb - 1;
-  a = nd[j];
-  b = j + 1 < nb ? nd[j + 1] : a;
-  for (int w = 0; w < 64; ++w) {
-    if (j + 1 < nb && !(Qv(s, b.y, b.z) < 0.0)) {
-      ++j;
-      a = b;
-      b = j + 1 < nb ? nd[j + 1] : a;
-      continue;
-    }
-    if (j > s.k && Qv(s, a.y, a.z) < 0.0) {
-      --j;
-      b = a;
-      a = nd[j];
-      continue;
-    }
-    return j;
-  }
-  j = bisect_rmax64(T, s);
-  a = nd[j];
-  b = j + 1 < nb ? nd[j + 1] : a;
-  return j;
-}
-
-__device__ __forceinline__ int64_t verify_rmin_nodes(const Table64& T,
-                                                     const double4_32a* __restrict__ nd,
-                                                     const Star& s, int64_t j, double4_32a& a,
-                                                     double4_32a& b) {
-  if (j < -1) j = -1;
-  if (j > s.k - 1) j = s.k - 1;
-  a = nd[j < 0 ? 0 : j];
-  b = nd[j + 1];
-  for (int w = 0; w < 64; ++w) {
-    if (j + 1 < s.k && Qv(s, b.y, b.z) < 0.0) {
-      ++j;
-      a = b;
-      b = nd[j + 1];
-      continue;
-    }
-    if (j >= 0 && !(Qv(s, a.y, a.z) < 0.0)) {
-      --j;
-      b = a;
-      a = nd[j < 0 ? 0 : j];
-      continue;
-    }
-    return j;
-  }
-  j = bisect_rmin64(T, s);
-  a = nd[j < 0 ? 0 : j];
-  b = nd[j + 1];
-  return j;
-}
-
-// Mixed mode, turning points of one bound star with E < 0: both node
-// bisections in FP32 in lockstep on the float table (r_max over [k, nb],
-// r_min over [-1, k]), each bracket verified in FP64 by a bounded walk,
-// then the FP64 roots inside the bracketing shells (Eq. 12).
+// Mixed mode, turning points of one bound star with E < 0: the brackets on the
+// grid and the nodes, or where a walk gives up by FP64 bisection, then the FP64
+// roots inside the bracketing shells (Eq. 12).
 __device__ __forceinline__ void turning_mixed(const Table64& T,
-                                              const float4* __restrict__ tdf,
                                               const double4_32a* __restrict__ nd, const Grid& G,
-                                              const Buckets& BK, const Star& s, double& rmin,
-                                              double& rmax) {
-  // E and J as float pairs; their high parts serve the FP32 searches
-  const DF Ed = df_split(s.E), Jd = df_split(s.J);
-  const float E32 = Ed.hi, J32 = Jd.hi;
-  const int nb32 = (int)T.nb, k32 = (int)s.k;
-  int lo1, lo2;
-  bool cert1, cert2;
-  if (!grid_brackets(G, tdf, BK, E32, J32, Ed, Jd, nb32, k32, lo1, lo2, cert1, cert2)) {
-    // both node bisections in FP32, in lockstep; their brackets are not
-    // certified (the FP64 walks run from them)
-    cert1 = cert2 = false;
-    lo1 = k32, lo2 = -1;
-    int hi1 = nb32, hi2 = k32;
-    const int rounds = search_rounds(nb32);
-    for (int it = 0; it < rounds; ++it) {
-      const bool a1 = hi1 - lo1 > 1, a2 = hi2 - lo2 > 1;
-      const int m1 = a1 ? lo1 + ((hi1 - lo1) >> 1) : k32;
-      const int m2 = a2 ? lo2 + ((hi2 - lo2) >> 1) : k32;
-      const float4 e1 = __ldg(tdf + m1), e2 = __ldg(tdf + m2);
-      const float L1 = J32 * e1.x, L2 = J32 * e2.x;
-      const bool n1 = 2.0f * (E32 - e1.z) - L1 * L1 < 0.0f;
-      const bool n2 = 2.0f * (E32 - e2.z) - L2 * L2 < 0.0f;
-      if (a1) { if (n1) hi1 = m1; else lo1 = m1; }
-      if (a2) { if (n2) lo2 = m2; else hi2 = m2; }
-    }
+                                              const Buckets& BK, const Star& s, float xk,
+                                              float qk, double& rmin, double& rmax) {
+  const int nb = (int)T.nb, k = (int)s.k;
+  Bracket a, b;
+  if (!grid_brackets(G, nd, BK, s, nb, k, xk, qk, a, b)) {
+    a.j = (int)bisect_rmax64(T, s);
+    b.j = (int)bisect_rmin64(T, s);
+    const double2 ta = node_xp(nd + a.j), tb = node_xp(nd + (b.j < 0 ? 0 : b.j));
+    a.x = ta.x;
+    a.p = ta.y;
+    b.x = tb.x;
+    b.p = tb.y;
   }
-  // A certified bracket is the one the FP64 walk stops at; otherwise that
-  // walk runs from it.  Then the FP64 roots in the bracketing shells.
-  const int64_t nb = T.nb;
-  double4_32a a1, b1, a2, b2;
-  int64_t jmax, jmin;
-  if (cert1) {
-    jmax = lo1;
-    a1 = nd[jmax];
-    b1 = jmax + 1 < nb ? nd[jmax + 1] : a1;
-  } else {
-    jmax = verify_rmax_nodes(T, nd, s, lo1, a1, b1);
-  }
-  if (cert2) {
-    jmin = lo2;
-    a2 = nd[jmin < 0 ? 0 : jmin];
-    b2 = nd[jmin + 1];
-  } else {
-    jmin = verify_rmin_nodes(T, nd, s, lo2, a2, b2);
-  }
-  rmax = rmax_core(s, a1.x, a1.y, a1.z, a1.w, jmax + 1 < nb, b1.x);
-  rmin = rmin_core(s, jmin < 0, a2.x, a2.y, a2.z, jmin < 0 ? 0.0 : a2.w, jmin >= 0, b2.x);
+  const double2 ra = node_rw(nd + a.j), rb = node_rw(nd + (b.j < 0 ? 0 : b.j));
+  const double r1 = nd[a.j + 1 < nb ? a.j + 1 : a.j].z, r2 = nd[b.j + 1].z;
+  rmax = rmax_core(s, ra.x, a.x, a.p, ra.y, a.j + 1 < nb, r1);
+  rmin = rmin_core(s, b.j < 0, rb.x, b.x, b.p, b.j < 0 ? 0.0 : rb.y, b.j >= 0, r2);
 }
 
 // First kernel of the mixed-mode orbit step: the turning points of every
@@ -806,7 +704,11 @@ __global__ void __launch_bounds__(256, kMinB) k_turning_mixed(
   BK.nbk = pr.y;
   BK.lo = pr.z;
   BK.hi = pr.w;
-  turning_mixed(T, BA.tdf + sb, BA.node + sb, grid_of(BA, c), BK, s, rmin, rmax);
+  // (Q at the star is v_r^2; its 1/r only has to place it on the grid)
+  const float vr32 = f32_rn(vrk);
+  float xk;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(xk) : "f"(f32_rn(rk)));
+  turning_mixed(T, BA.node + sb, grid_of(BA, c), BK, s, xk, vr32 * vr32, rmin, rmax);
   if (tp_min) {
     tp_min[p] = rmin;
     tp_max[p] = rmax;
@@ -1666,7 +1568,7 @@ __global__ void k_grid_build(Seg S, const int64_t* esc, bool sub, const double* 
     const double xj = x[q], pj = phi[q];
     const double w = div_rn(phi[q + 1] - pj, xj - x[q + 1]);
     Menc[q] = w;
-    node[q] = make_double4_32a(r[q], xj, pj, w);
+    node[q] = make_double4_32a(xj, pj, r[q], w);
     return;
   }
   const int c = seg_find(B.goff, S.n_seg, p);
@@ -1837,7 +1739,6 @@ cudaError_t alloc_buckets(BucketWork& B, const SegLayout& L, cudaStream_t st) {
   if ((e = cudaMallocAsync((void**)&B.gprm, sizeof(int4) * L.n_seg, st))) return e;
   if ((e = cudaMallocAsync((void**)&B.gaux, sizeof(float4) * L.n_seg, st))) return e;
   if ((e = cudaMallocAsync((void**)&B.node, sizeof(double4_32a) * (L.n > 0 ? L.n : 1), st))) return e;
-  if ((e = cudaMallocAsync((void**)&B.tdf, sizeof(float4) * (L.n > 0 ? L.n : 1), st))) return e;
   e = cudaMemcpyAsync(B.off, off.data(), sizeof(int64_t) * (L.n_seg + 1),
                       cudaMemcpyHostToDevice, st);
   if (!e)
@@ -1848,8 +1749,7 @@ cudaError_t alloc_buckets(BucketWork& B, const SegLayout& L, cudaStream_t st) {
 }
 
 void free_buckets(BucketWork& B, cudaStream_t st) {
-  void* ps[] = {B.start, B.off, B.base, B.prm, B.gphi, B.gshell, B.goff, B.gprm, B.gaux, B.node,
-                B.tdf};
+  void* ps[] = {B.start, B.off, B.base, B.prm, B.gphi, B.gshell, B.goff, B.gprm, B.gaux, B.node};
   for (void* p : ps)
     if (p) cudaFreeAsync(p, st);
   B = BucketWork();
@@ -1882,7 +1782,7 @@ void launch_potential_tables(const SegLayout& L, const double* r, const double* 
   T.gshell = B.gshell;
   T.goff = B.goff;
   T.gprm = B.gprm;
-  launch_potential(L, r, x, m, tile_m, tile_mx, phi, t32, Menc, nb_sub, st, B.node, B.tdf,
+  launch_potential(L, r, x, m, tile_m, tile_mx, phi, t32, Menc, nb_sub, st, B.node,
                    sums_ready, true, &T);
   const int64_t threads = B.gcells + L.n_tiles;
   launch_k(k_grid_build, (unsigned)((threads + 255) / 256), 256, 0, st,

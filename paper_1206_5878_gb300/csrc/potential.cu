@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(kPoThreads) k_phi_old(Seg S, const int64_t* es
     double pn;
     if (!kDiv) {
       const double4_32a nd = node[sb + (i < 0 ? 0 : i)];
-      pn = i < 0 ? nd.z : nd.z + nd.w * (nd.y - xo[j]);
+      pn = i < 0 ? nd.y : nd.y + nd.w * (nd.x - xo[j]);
     } else {
       const int64_t q = sb + (i < 0 ? 0 : i);
       const double pj = phi[q];
@@ -517,13 +517,6 @@ __device__ __forceinline__ F32Pair f32_pair(double v) {
   const unsigned sl = (rem < 0 ? sg ^ 0x80000000u : sg);
   r.lo = __uint_as_float(sl | ((fe << 23) + (m - 0x800000u)));
   return r;
-}
-
-// (hi, lo) float pairs of 1/r and Phi: hi the float nearest, lo the float
-// nearest the remainder (together ~48 bits)
-__device__ __forceinline__ float4 float_pairs(double x, double ph) {
-  const F32Pair a = f32_pair(x), b = f32_pair(ph);
-  return make_float4(a.hi, a.lo, b.hi, b.lo);
 }
 
 // ------------------------------------------------------------ potential
@@ -704,8 +697,8 @@ __global__ void __launch_bounds__(kPotThreads) k_potential(Seg S, const int64_t*
                                                            const double* m, const double* tile_m,
                                                            const double* tile_mx, double* phi,
                                                            float2* t32, double* Mout,
-                                                           double4_32a* node, float4* tdf,
-                                                           bool slopes, TableOut T) {
+                                                           double4_32a* node, bool slopes,
+                                                           TableOut T) {
   pdl_enter();
   extern __shared__ double smem[];
   double* s_m = smem;               // m, then M_k
@@ -801,8 +794,7 @@ __global__ void __launch_bounds__(kPotThreads) k_potential(Seg S, const int64_t*
       }
     }
     if (Mout) Mout[p] = w;
-    if (node) node[p] = make_double4_32a(r[p], s_x[q], ph, w);
-    if (tdf) tdf[p] = float_pairs(s_x[q], ph);
+    if (node) node[p] = make_double4_32a(s_x[q], ph, r[p], w);
     if (T.start && bound) {
       // the orbit step's index tables, star by star: bucket starts (from the
       // float keys of 1/r of this star and its predecessor, as t32 holds
@@ -836,7 +828,7 @@ __global__ void k_slope_seams(Seg S, const int64_t* esc, bool sub, const double*
   const double xj = x[p], pj = phi[p], xj1 = x[p + 1], pj1 = phi[p + 1];
   const double w = div_rn(pj1 - pj, xj - xj1);
   if (M) M[p] = w;
-  node[p] = make_double4_32a(r[p], xj, pj, w);
+  node[p] = make_double4_32a(xj, pj, r[p], w);
 }
 
 // ---------------------------------------------------- energy correction
@@ -1183,12 +1175,11 @@ __global__ void k_make_t32(int64_t n, const double* x, const double* phi, float2
 }
 
 __global__ void k_make_nodes(int64_t n, const double* r, const double* x, const double* phi,
-                             const double* M, double4_32a* node, float4* tdf) {
+                             const double* M, double4_32a* node) {
   pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
-  node[p] = make_double4_32a(r[p], x[p], phi[p], M[p]);
-  tdf[p] = float_pairs(x[p], phi[p]);
+  node[p] = make_double4_32a(x[p], phi[p], r[p], M[p]);
 }
 
 __global__ void k_unpack_orbit(int64_t n, const RecA* ra, const RecB* rb, double* r_new,
@@ -1219,8 +1210,8 @@ void launch_make_t32(int64_t n, const double* x, const double* phi, float2* t32,
 }
 
 void launch_make_nodes(int64_t n, const double* r, const double* x, const double* phi,
-                       const double* M, double4_32a* node, float4* tdf, cudaStream_t st) {
-  if (n > 0) launch_k(k_make_nodes, blocks_for(n, 256), 256, 0, st, n, r, x, phi, M, node, tdf);
+                       const double* M, double4_32a* node, cudaStream_t st) {
+  if (n > 0) launch_k(k_make_nodes, blocks_for(n, 256), 256, 0, st, n, r, x, phi, M, node);
 }
 
 void launch_unpack_orbit(int64_t n, const RecA* ra, const RecB* rb, double* r_new,
@@ -1375,14 +1366,14 @@ void potential_prepare() {
 void launch_potential(const SegLayout& L, const double* r, const double* x, const double* m,
                       double* tile_m, double* tile_mx, double* phi, float2* t32,
                       double* Mout, bool nb_sub, cudaStream_t st, double4_32a* node,
-                      float4* tdf, bool sums_ready, bool slopes, const TableOut* tables) {
+                      bool sums_ready, bool slopes, const TableOut* tables) {
   if (!L.n_tiles) return;
   Seg S = L.dev();
   if (!sums_ready)
     launch_k(k_tile_sums, (unsigned)L.n_tiles, kThreads, 0, st, S, L.esc_step, nb_sub, x, m, tile_m,
                                                          tile_mx);
   launch_k(k_potential, (unsigned)L.n_tiles, kPotThreads, kPotentialSmem, st,
-      S, L.esc_step, nb_sub, r, x, m, tile_m, tile_mx, phi, t32, Mout, node, tdf, slopes,
+      S, L.esc_step, nb_sub, r, x, m, tile_m, tile_mx, phi, t32, Mout, node, slopes,
       tables ? *tables : TableOut());
   // with the tables, the seams' slopes come with the grid's values
   if (slopes && node && !tables)
