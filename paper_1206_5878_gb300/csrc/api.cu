@@ -33,7 +33,6 @@ struct cmc_ctx {
   double *r_alt = nullptr, *x_alt = nullptr;
   int side = 0;
   uint32_t* id = nullptr;
-  float2* t32 = nullptr;
   // scratch
   uint64_t* keys = nullptr;
   uint32_t* vals = nullptr;
@@ -43,7 +42,7 @@ struct cmc_ctx {
   BinWork bins;                // the timestep's counting sort (cfg.sort_packed)
   std::vector<unsigned int> max_id;  // per segment, as the bins have it
   double *r_old = nullptr, *cc = nullptr, *nbin = nullptr;
-  double *tile_a = nullptr, *tile_b = nullptr, *tile_c = nullptr, *Mbuf = nullptr,
+  double *tile_a = nullptr, *tile_b = nullptr, *tile_c = nullptr,
          *out3 = nullptr, *fr = nullptr, *lag = nullptr;
   uint32_t* err = nullptr;
   uint32_t* step = nullptr;
@@ -192,11 +191,10 @@ void finish_order(cmc_ctx* c, cudaStream_t st) {
   // the float tables, node records and indexes of the sampled orbit step
   // (precision 0 and 1)
   if (c->cfg.precision != 2)
-    launch_potential_tables(L, c->r, c->x, c->m, c->tile_a, c->tile_b, c->phi, c->t32, c->Mbuf,
-                            false, false, c->bk, st);
+    launch_potential_tables(L, c->r, c->x, c->m, c->tile_a, c->tile_b, c->phi, false, false, c->bk,
+                            st);
   else
-    launch_potential(L, c->r, c->x, c->m, c->tile_a, c->tile_b, c->phi, nullptr, nullptr, false,
-                     st);
+    launch_potential(L, c->r, c->x, c->m, c->tile_a, c->tile_b, c->phi, nullptr, false, st);
 }
 
 void order_state(cmc_ctx* c, cudaStream_t st) {
@@ -247,13 +245,12 @@ void record_step(cmc_ctx* c, cudaStream_t st, cudaEvent_t* ev = nullptr) {
   mark(2);
   // the turning points (as the orbit records), then sampling
   if (tab)
-    launch_turning(L, c->r, c->x, c->phi, c->Mbuf, c->vr, c->vt, c->bk.args(), nullptr,
+    launch_turning(L, c->r, c->x, c->phi, c->vr, c->vt, c->bk.args(), nullptr,
                    nullptr, c->orb, c->cfg.orbit_block, st);
   mark(3);
   const bool binned = c->cfg.sort_packed != 0;
   const bool counted = L.n <= kCountInOrbit;
-  launch_orbit(L, c->cfg.precision, c->cfg.max_trials, c->r, c->x, c->phi,
-               tab ? c->Mbuf : nullptr, c->vr, c->vt, c->m, c->id,
+  launch_orbit(L, c->cfg.precision, c->cfg.max_trials, c->r, c->x, c->phi, c->vr, c->vt, c->m, c->id,
                c->step, c->keys, c->ra, c->rb, nullptr, c->cfg.orbit_block, c->orbit_variant,
                c->bk.args(), c->r_old, c->cc, c->vals, c->pcount, st, false, c->R, c->Rp,
                c->cfg.precision == 0 ? &c->env : nullptr, c->A, c->Ap, c->orb,
@@ -280,11 +277,11 @@ void record_step(cmc_ctx* c, cudaStream_t st, cudaEvent_t* ev = nullptr) {
   // scan's enclosed masses): the sampled step's turning points and points
   // are then FP64 mode's
   if (tab)
-    launch_potential_tables(L, c->r_alt, c->x_alt, c->m, c->tile_a, c->tile_b, c->phi, c->t32,
-                            c->Mbuf, true, true, c->bk, st);
+    launch_potential_tables(L, c->r_alt, c->x_alt, c->m, c->tile_a, c->tile_b, c->phi, true, true,
+                            c->bk, st);
   else
-    launch_potential(L, c->r_alt, c->x_alt, c->m, c->tile_a, c->tile_b, c->phi, nullptr, nullptr,
-                     true, st, nullptr, true);
+    launch_potential(L, c->r_alt, c->x_alt, c->m, c->tile_a, c->tile_b, c->phi, nullptr, true, st,
+                     true);
   mark(7);
   // (the FP64 modes evaluate Phi_new(r_old) in Eq. 6's division form)
   const bool correct = c->cfg.energy_correction != 0;
@@ -313,13 +310,12 @@ int count_step_kernels(const cmc_ctx* c) {
   // bins, relax, orbit, gather with the tile sums, potential, velocities, step
   // end; the sort: scan, scatter, long runs [count], or upsweep (with the
   // histograms' scans), 5 passes, tie fix; [precision 0 and 1: turning points,
-  // FP32 sampler, FP64 continuation, the tables' parameters, the grid's values
-  // with the seams' slopes; precision 0: the envelope's screen and
-  // evaluation], [Phi_new(r_old)]
+  // FP32 sampler, FP64 continuation, the grid's values with the seams' slopes;
+  // precision 0: the envelope's screen and evaluation], [Phi_new(r_old)]
   const int p = c->cfg.precision;
   const int sort = c->cfg.sort_packed ? (c->L.n <= kCountInOrbit ? 3 : 4) : 7;
   return 7 + sort + ((c->R || c->A) ? 1 : 0) + (c->ring ? 4 : 0) +
-         (p == 1 ? 5 : p == 0 ? 7 : 0) + (c->cfg.energy_correction ? 1 : 0);
+         (p == 1 ? 4 : p == 0 ? 6 : 0) + (c->cfg.energy_correction ? 1 : 0);
 }
 
 void free_ctx(cmc_ctx* c) {
@@ -329,14 +325,13 @@ void free_ctx(cmc_ctx* c) {
   for (cudaGraphExec_t e : c->exec)
     if (e) cudaGraphExecDestroy(e);
   double** ds[] = {&c->r_alt, &c->x_alt, &c->r, &c->x, &c->vr, &c->vt, &c->m, &c->phi, &c->r_old, &c->cc, &c->nbin,
-                   &c->tile_a, &c->tile_b, &c->tile_c, &c->Mbuf, &c->out3, &c->fr, &c->lag};
+                   &c->tile_a, &c->tile_b, &c->tile_c, &c->out3, &c->fr, &c->lag};
   for (double** p : ds) dfree(*p, st);
   dfree(c->id, st);
   dfree(c->R, st);
   dfree(c->Rp, st);
   dfree(c->A, st);
   dfree(c->Ap, st);
-  dfree(c->t32, st);
   dfree(c->keys, st);
   dfree(c->vals, st);
   dfree(c->ra, st);
@@ -546,8 +541,7 @@ cmc_status autotune(cmc_ctx* c) {
     if (es) return cuda_fail(c, es, "autotune");
   }
   auto run_orbit = [&](int blk, int var) {
-    launch_orbit(L, c->cfg.precision, c->cfg.max_trials, c->r, c->x, c->phi,
-                 tab ? c->Mbuf : nullptr, c->vr, c->vt, c->m,
+    launch_orbit(L, c->cfg.precision, c->cfg.max_trials, c->r, c->x, c->phi, c->vr, c->vt, c->m,
                  c->id, c->step, c->keys, c->ra, c->rb, nullptr, blk, var, c->bk.args(), c->r_old,
                  c->cc, c->vals, c->pcount, st, true, nullptr, nullptr,
                  c->cfg.precision == 0 ? &c->env : nullptr, nullptr, nullptr, c->orb);
@@ -760,7 +754,6 @@ cmc_status cmc_init(cmc_ctx** out, const cmc_config* cfg_in, int32_t n_clusters,
   CMC_ALLOC(c->m, n);
   CMC_ALLOC(c->phi, n);
   CMC_ALLOC(c->id, n);
-  if (cfg.precision != 2) CMC_ALLOC(c->t32, n);
   if (!e && cfg.precision == 0) e = alloc_env(c->env, (int64_t)n, st);
   if (cfg.precision != 2) CMC_ALLOC(c->orb, n);
   if (cfg.diag_ring > 0) {
@@ -777,7 +770,6 @@ cmc_status cmc_init(cmc_ctx** out, const cmc_config* cfg_in, int32_t n_clusters,
   CMC_ALLOC(c->x_alt, n);
   CMC_ALLOC(c->r_old, n);
   CMC_ALLOC(c->cc, n);
-  CMC_ALLOC(c->Mbuf, n);
   CMC_ALLOC(c->nbin, (size_t)L.n_bins);
   CMC_ALLOC(c->tile_a, (size_t)L.n_tiles);
   CMC_ALLOC(c->tile_b, (size_t)L.n_tiles);
@@ -1283,7 +1275,7 @@ cmc_status cmc_potential(int64_t n, const double* r, const double* m, double* ph
   if (!e) {
     potential_prepare();
     launch_recip(n, r, x, st);
-    launch_potential(S.L, r, x, m, ta, tb, phi, nullptr, M, false, st);
+    launch_potential(S.L, r, x, m, ta, tb, phi, M, false, st);
     e = cudaGetLastError();
   }
   dfree(x, st);
@@ -1375,7 +1367,7 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
         launch_buckets(S.L, t32, false, bk, st);
         launch_slopes(n, x, phi, sl, st);
         launch_make_nodes(n, r, x, phi, sl, bk.node, st);
-        launch_grid(S.L, x, phi, sl, false, bk, st);
+        launch_grid(S.L, x, phi, false, bk, st);
       }
     }
     OrbitStageOut d;
@@ -1391,7 +1383,7 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
     if (!e && tab) e = dalloc(pcnt, 1, st);
     if (!e && precision == 0) e = alloc_env(env, n, st);
     if (!e)
-      launch_orbit(S.L, precision, max_trials, r, x, phi, sl, vr, vt, mm, id, dstep, keys,
+      launch_orbit(S.L, precision, max_trials, r, x, phi, vr, vt, mm, id, dstep, keys,
                    ra, rb, &d, 0, 0, bk.args(), tmin, tmax, plist, pcnt, st, true, nullptr,
                    nullptr, precision == 0 ? &env : nullptr, nullptr, nullptr, orb);
     free_buckets(bk, st);

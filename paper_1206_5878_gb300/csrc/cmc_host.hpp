@@ -248,27 +248,26 @@ void launch_velocities(const SegLayout& L, const uint32_t* order, const RecB* rb
 
 // potential: per-tile sums then the tile-local scans (Eqs. 1-5 in scan
 // form).  nb_sub: subtract esc_step from nb (after the orbit step).
-// Optional outputs: t32 (float 1/r, Phi), Mout (M_k) and node (the record
-// {1/r, Phi, r, M_k} of every star: one 32-byte sector per node for the
-// kernels that read a few nodes at random).  slopes: Mout and the records
-// carry the slope of Eq. 6 across each shell instead of M_k (the shell
-// parameter the FP64 orbit step takes).
+// Optional output: Mout (M_k); with tables instead the record {1/r, Phi, r,
+// slope} of every star (node: one 32-byte sector per node for the kernels that
+// read a few nodes at random; the slope of Eq. 6 across the shell is the FP64
+// orbit step's parameter) and the orbit step's index tables.
 // The orbit step's index tables as the potential kernel writes them beside
 // Phi: the bucket starts and the grid's key shells (their per-segment
 // parameters computed before it, from 1/r).
 struct TableOut {
   int* start = nullptr;
   const int64_t* boff = nullptr;
-  const uint32_t* base = nullptr;
-  const int4* prm = nullptr;
+  uint32_t* base = nullptr;  // per segment (also read by the orbit step's kernels)
+  int4* prm = nullptr;
   int* gshell = nullptr;
   const int64_t* goff = nullptr;
-  const int4* gprm = nullptr;
+  int4* gprm = nullptr;
+  float4* gaux = nullptr;
 };
 void launch_potential(const SegLayout& L, const double* r, const double* x, const double* m,
-                      double* tile_m, double* tile_mx, double* phi, float2* t32,
-                      double* Mout, bool nb_sub, cudaStream_t st, double4_32a* node = nullptr,
-                      bool sums_ready = false, bool slopes = false,
+                      double* tile_m, double* tile_mx, double* phi, double* Mout, bool nb_sub,
+                      cudaStream_t st, bool sums_ready = false, double4_32a* node = nullptr,
                       const TableOut* tables = nullptr);
 // node records from the arrays (stage calls)
 void launch_make_nodes(int64_t n, const double* r, const double* x, const double* phi,
@@ -348,20 +347,18 @@ void free_buckets(BucketWork& B, cudaStream_t st);
 // build the index from t32 over the bound stars (nb - esc_step when nb_sub)
 void launch_buckets(const SegLayout& L, const float2* t32, bool nb_sub, BucketWork& B,
                     cudaStream_t st);
-// build the potential grid from the FP64 table (x, Phi, enclosed masses)
-void launch_grid(const SegLayout& L, const double* x, const double* phi, const double* Menc,
-                 bool nb_sub, BucketWork& B, cudaStream_t st);
-// The potential with the orbit step's tables in three kernels: the
-// segments' bucket and grid parameters (from 1/r), the potential writing Phi,
-// the slopes, node records, float tables, bucket starts and grid key shells,
-// then the grid's values with the slopes at the tile seams.  The same tables
-// as launch_potential + launch_buckets + launch_grid (slopes mode).
+// build the potential grid from the FP64 table (x, Phi, the node records)
+void launch_grid(const SegLayout& L, const double* x, const double* phi, bool nb_sub,
+                 BucketWork& B, cudaStream_t st);
+// The potential with the orbit step's tables in two kernels: the potential
+// writing Phi, the node records, bucket starts and grid key shells with the
+// segments' parameters, then the grid's values with the slopes at the tile
+// seams.  The same tables as launch_potential + launch_make_nodes +
+// launch_buckets + launch_grid.
 void launch_potential_tables(const SegLayout& L, const double* r, const double* x,
                              const double* m, double* tile_m, double* tile_mx, double* phi,
-                             float2* t32, double* Menc, bool nb_sub, bool sums_ready,
-                             BucketWork& B, cudaStream_t st);
+                             bool nb_sub, bool sums_ready, BucketWork& B, cudaStream_t st);
 
-// Menc (precision 0 and 1): the slope of Phi in 1/r across shell k.
 // launch_orbit writes the stars' records, and with bins their sort bins (count:
 // counted too) or else their sort keys.  precision 1 (mixed): it runs four kernels (turning points,
 // FP32 sampler, FP64 continuation of the pending stars, finishing) and
@@ -396,8 +393,7 @@ cudaError_t alloc_env(EnvWork& W, int64_t n, cudaStream_t st);
 void free_env(EnvWork& W, cudaStream_t st);
 
 void launch_orbit(const SegLayout& L, int precision, int max_trials, const double* r,
-                  const double* x, const double* phi, const double* Menc,
-                  const double* vr,
+                  const double* x, const double* phi, const double* vr,
                   const double* vt, const double* m, const uint32_t* id, const uint32_t* step,
                   uint64_t* keys, RecA* ra, RecB* rb, const OrbitStageOut* dbg, int block,
                   int variant, const BucketArgs& ba, double* tp_min, double* tp_max,
@@ -409,7 +405,7 @@ void launch_orbit(const SegLayout& L, int precision, int max_trials, const doubl
 // the turning-point kernel alone (mixed mode; launch_orbit(..., false)
 // then runs the sampling kernel only)
 void launch_turning(const SegLayout& L, const double* r, const double* x, const double* phi,
-                    const double* Menc, const double* vr, const double* vt,
+                    const double* vr, const double* vt,
                     const BucketArgs& ba, double* tp_min, double* tp_max, double4_32a* orb,
                     int block, cudaStream_t st);
 // mixed-mode orbit variants: register caps for 1 (none), 2, 3, 4, 5, 6 and

@@ -672,7 +672,7 @@ __device__ __forceinline__ void turning_mixed(const Table64& T,
 template <int kMinB>
 __global__ void __launch_bounds__(256, kMinB) k_turning_mixed(
     Seg S, const double* r, const double* x, const double* phi,
-    const double* Menc, const double* vr, const double* vt, BucketArgs BA, double* tp_min,
+    const double* vr, const double* vt, BucketArgs BA, double* tp_min,
     double* tp_max, double4_32a* orb, int64_t n) {
   pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1259,8 +1259,8 @@ __device__ __forceinline__ void put_star(const Seg& S, const BinOut& O, uint64_t
 template <int kPrec, int kMinB, bool kTaus>
 __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, const double* r,
                                                const double* x, const double* phi,
-                                               const double* Menc, const double* vr,
-                                               const double* vt, const double* m,
+                                               const double* vr, const double* vt,
+                                               const double* m,
                                                const uint32_t* id, const uint32_t* step_p,
                                                uint64_t* keys, RecA* ra, RecB* rb,
                                                int64_t* esc, OrbitStageOut dbg, BucketArgs BA,
@@ -1506,7 +1506,7 @@ int64_t grid_capacity(int64_t nc) {
 // mass (Phi = Phi_0 inside the first star; outside the last one Phi falls
 // by M_bound per unit of 1/r)
 __global__ void k_grid_params(Seg S, const int64_t* esc, bool sub, const double* x,
-                              const double* phi, const double* Menc, const int64_t* goff,
+                              const double* phi, const double4_32a* node, const int64_t* goff,
                               int4* gprm, float4* gaux) {
   pdl_enter();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1524,7 +1524,7 @@ __global__ void k_grid_params(Seg S, const int64_t* esc, bool sub, const double*
   const uint32_t key0 = (klo >> sh) << sh;
   const int cells = (int)((khi - key0) >> sh) + 2;
   gprm[c] = make_int4((int)key0, sh, cells, (int)khi);
-  gaux[c] = make_float4((float)phi[sb], (float)Menc[sb + nb - 1], __uint_as_float(key0), 0.f);
+  gaux[c] = make_float4((float)phi[sb], (float)node[sb + nb - 1].w, __uint_as_float(key0), 0.f);
 }
 
 // The shell of every grid key, largest i with 1/r_i >= key (-1 when none),
@@ -1533,14 +1533,18 @@ __global__ void k_grid_shells(Seg S, const int64_t* esc, bool sub, const double*
                               BucketArgs B, int* gshell, int64_t n) {
   pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned mask = __ballot_sync(0xFFFFFFFFu, p < n);
   if (p >= n) return;
   const int c = seg_find(S.off, S.n_seg, p);
   int64_t nb = S.nb[c];
   if (sub) nb -= esc[c];
   const int64_t sb = S.off[c], k = p - sb;
-  if (k >= nb) return;
-  grid_shells_of(k, nb, __ldg(x + p), k + 1 < nb ? __ldg(x + p + 1) : 0.0, B.gprm[c],
+  const int4 pr = B.gprm[c];
+  const bool live = k < nb;
+  grid_shells_of(mask, live, (int)k, (int)nb, live ? grid_last_cell(__ldg(x + p), pr) : -1,
+                 live && k + 1 < nb ? grid_last_cell(__ldg(x + p + 1), pr) : -1, pr,
                  gshell + B.goff[c]);
+  if (live && k == 0) grid_close(grid_last_cell(__ldg(x + p), pr), pr, gshell + B.goff[c], 0, 1);
 }
 
 // Phi at every grid key from the FP64 table: Phi = Phi_i + M_i (1/r_i - 1/r)
@@ -1551,9 +1555,9 @@ __global__ void k_grid_shells(Seg S, const int64_t* esc, bool sub, const double*
 // locally where a cell needs one), and each segment's cell 0 fills Phi_0 and
 // the bound mass into gaux
 __global__ void k_grid_build(Seg S, const int64_t* esc, bool sub, const double* x,
-                             const double* phi, double* Menc, BucketArgs B,
+                             const double* phi, BucketArgs B,
                              const int* gshell, float* gphi, float4* gaux, int64_t total,
-                             bool fused, const double* r, double4_32a* node, int64_t n_tiles) {
+                             bool fused, double4_32a* node, int64_t n_tiles) {
   pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned am = __ballot_sync(0xFFFFFFFFu, p < total);
@@ -1565,10 +1569,8 @@ __global__ void k_grid_build(Seg S, const int64_t* esc, bool sub, const double* 
     const int64_t k = (t - S.tile_off[cs]) * kTile + kTile - 1;  // the tile's last star
     if (k + 1 >= nbs) return;
     const int64_t q = sbs + k;
-    const double xj = x[q], pj = phi[q];
-    const double w = div_rn(phi[q + 1] - pj, xj - x[q + 1]);
-    Menc[q] = w;
-    node[q] = make_double4_32a(xj, pj, r[q], w);
+    // (only the slope: other threads read the record's 1/r and Phi)
+    node[q].w = div_rn(phi[q + 1] - phi[q], x[q] - x[q + 1]);
     return;
   }
   const int c = seg_find(B.goff, S.n_seg, p);
@@ -1578,22 +1580,26 @@ __global__ void k_grid_build(Seg S, const int64_t* esc, bool sub, const double* 
   const int64_t nb = S.nb[c] - (sub ? esc[c] : 0);
   // shell i's slope (a seam's computed as the seam threads do)
   auto slope = [&](int64_t i) {
-    if (fused && i % kTile == kTile - 1 && i + 1 < nb)
-      return div_rn(__ldg(phi + sb + i + 1) - __ldg(phi + sb + i),
-                    __ldg(x + sb + i) - __ldg(x + sb + i + 1));
-    return __ldg(Menc + sb + i);
+    if (fused && i % kTile == kTile - 1 && i + 1 < nb) {
+      const double2 a = node_xp(node + sb + i), b = node_xp(node + sb + i + 1);
+      return div_rn(b.y - a.y, a.x - b.x);
+    }
+    return node[sb + i].w;
   };
   float rel = 0.0f;
   if (g < pr.z) {
     if (fused && g == 0) {
       gaux[c].x = (float)__ldg(phi + sb);
-      gaux[c].y = (float)__ldg(Menc + sb + nb - 1);
+      gaux[c].y = (float)node[sb + nb - 1].w;
     }
     const double xg = (double)__uint_as_float((uint32_t)pr.x + ((uint32_t)g << pr.y));
     const double xn = (double)__uint_as_float((uint32_t)pr.x + ((uint32_t)(g + 1) << pr.y));
     const int64_t lo = gshell[p];
-    const double ph = lo < 0 ? __ldg(phi + sb)
-                             : __ldg(phi + sb + lo) + slope(lo) * (__ldg(x + sb + lo) - xg);
+    double ph = __ldg(phi + sb);
+    if (lo >= 0) {
+      const double2 a = node_xp(node + sb + lo);
+      ph = a.y + slope(lo) * (a.x - xg);
+    }
     gphi[p] = (float)ph;
     // Phi is convex in 1/r (its slope -M(1/r) rises with 1/r), so inside the
     // cell [xg, xn] it lies below the chord by at most (xn - xg) dM / 4, dM
@@ -1613,50 +1619,6 @@ __global__ void k_grid_build(Seg S, const int64_t* esc, bool sub, const double* 
   const unsigned mx = __reduce_max_sync(grp, __float_as_uint(rel));
   if ((threadIdx.x & 31) == (unsigned)(__ffs(grp) - 1) && mx)
     atomicMax(reinterpret_cast<unsigned int*>(&gaux[c].w), mx);
-}
-
-// Both tables' per-segment parameters from 1/r alone (before the potential
-// kernel writes the tables): as k_bucket_params (its float keys are the
-// floats nearest 1/r, as t32 holds them) and k_grid_params, with Phi_0 and
-// the bound mass left to k_grid_build (fused)
-__global__ void k_table_params(Seg S, const int64_t* esc, bool sub, const double* x,
-                               const int64_t* boff, uint32_t* base, int4* prm,
-                               const int64_t* goff, int4* gprm, float4* gaux) {
-  pdl_enter();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= S.n_seg) return;
-  int64_t nb = S.nb[c];
-  if (sub) nb -= esc[c];
-  if (nb <= 0) {
-    base[c] = 0;
-    prm[c] = make_int4(0, 0, 0, -1);
-    gprm[c] = make_int4(0, 0, 0, 0);
-    gaux[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-    return;
-  }
-  const int64_t sb = S.off[c];
-  // buckets
-  const int tail = nb >= 4096 ? (int)(nb >> 10) : 0;
-  const int lo = tail, hi = (int)nb - 1 - tail;
-  const uint32_t b0 = __float_as_uint(f32_rn(x[sb + lo]));
-  const uint32_t b1 = __float_as_uint(f32_rn(x[sb + hi]));
-  const uint32_t span = b0 >= b1 ? b0 - b1 : 0u;
-  const int64_t bcap = boff[c + 1] - boff[c] - 1;
-  int bs = 0;
-  while ((int64_t)(span >> bs) + 1 > bcap) ++bs;
-  base[c] = b0;
-  prm[c] = make_int4(bs, (int)((span >> bs) + 1), lo, hi);
-  // grid
-  const uint32_t klo = __float_as_uint((float)x[sb + nb - 1]);
-  const uint32_t khi = __float_as_uint((float)x[sb]);
-  const int64_t gcap = goff[c + 1] - goff[c];
-  int gp = 10;
-  while (gp > 0 && (int64_t)((khi >> (23 - gp)) - (klo >> (23 - gp))) + 2 > gcap) --gp;
-  const int sh = 23 - gp;
-  const uint32_t key0 = (klo >> sh) << sh;
-  const int cells = (int)((khi - key0) >> sh) + 2;
-  gprm[c] = make_int4((int)key0, sh, cells, (int)khi);
-  gaux[c] = make_float4(0.f, 0.f, __uint_as_float(key0), 0.f);
 }
 
 // per segment: the indexed node range lo..hi, base = bits(x_lo), the
@@ -1689,16 +1651,18 @@ __global__ void k_bucket_build(Seg S, const int64_t* esc, bool sub, const float2
                                BucketArgs B, int* start, int64_t n) {
   pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned mask = __ballot_sync(0xFFFFFFFFu, p < n);
   if (p >= n) return;
   const int c = seg_find(S.off, S.n_seg, p);
   int64_t nb = S.nb[c];
   if (sub) nb -= esc[c];
-  const int4 pr = B.prm[c];
   const int64_t k = p - S.off[c];
-  if (k < pr.z || k > pr.w) return;
-  bucket_starts_of(k, nb, pr, B.base[c], __float_as_uint(t32[p].x),
-                   k == pr.z ? 0u : __float_as_uint(t32[p - 1].x), start + B.off[c],
+  bucket_starts_of(mask, k < nb, (int)k, B.prm[c], B.base[c], __float_as_uint(t32[p].x),
+                   k > 0 ? __float_as_uint(t32[p - 1].x) : 0u, start + B.off[c],
                    B.off[c + 1] - B.off[c]);
+  if (k == B.prm[c].w)
+    bucket_close((int)nb, B.prm[c], B.base[c], __float_as_uint(t32[p].x), start + B.off[c],
+                 B.off[c + 1] - B.off[c], 0, 1);
 }
 
 // slope of Phi in 1/r across each shell of one table, for callers that
@@ -1724,7 +1688,12 @@ cudaError_t alloc_buckets(BucketWork& B, const SegLayout& L, cudaStream_t st) {
   std::vector<int64_t> off(L.n_seg + 1, 0), goff(L.n_seg + 1, 0);
   for (int c = 0; c < L.n_seg; ++c) {
     const int64_t nc = L.h_off[c + 1] - L.h_off[c];
-    off[c + 1] = off[c] + nc / 2 + 2;  // about two stars per bucket
+    // a bucket per star on average over the key range.  With half as many the walks
+    // at the ends of a bucket are longer (turning points of 10^6 stars 124 us
+    // against 109, of 64 x 10^5 stars 616 against 599; the fill costs 7 and 2 us
+    // less); with twice as many the table no longer stays in the L2 (the orbit
+    // stage of 10^7 stars 1354 us against 1242).
+    off[c + 1] = off[c] + nc + 2;
     goff[c + 1] = goff[c] + grid_capacity(nc);
   }
   B.gcells = goff[L.n_seg];
@@ -1755,25 +1724,22 @@ void free_buckets(BucketWork& B, cudaStream_t st) {
   B = BucketWork();
 }
 
-void launch_grid(const SegLayout& L, const double* x, const double* phi, const double* Menc,
-                 bool nb_sub, BucketWork& B, cudaStream_t st) {
+void launch_grid(const SegLayout& L, const double* x, const double* phi, bool nb_sub,
+                 BucketWork& B, cudaStream_t st) {
   if (!L.n || !B.gcells) return;
-  launch_k(k_grid_params, (unsigned)((L.n_seg + 127) / 128), 128, 0, st,
-      L.dev(), L.esc_step, nb_sub, x, phi, Menc, B.goff, B.gprm, B.gaux);
+  launch_k(k_grid_params, (unsigned)((L.n_seg + 127) / 128), 128, 0, st, L.dev(), L.esc_step,
+           nb_sub, x, phi, B.node, B.goff, B.gprm, B.gaux);
   launch_k(k_grid_shells, (unsigned)((L.n + 255) / 256), 256, 0, st, L.dev(), L.esc_step, nb_sub, x,
-                                                              B.args(), B.gshell, L.n);
-  launch_k(k_grid_build, (unsigned)((B.gcells + 255) / 256), 256, 0, st,
-      L.dev(), L.esc_step, nb_sub, x, phi, const_cast<double*>(Menc), B.args(), B.gshell,
-      B.gphi, B.gaux, B.gcells, false, nullptr, nullptr, 0);
+           B.args(), B.gshell, L.n);
+  launch_k(k_grid_build, (unsigned)((B.gcells + 255) / 256), 256, 0, st, L.dev(), L.esc_step,
+           nb_sub, x, phi, B.args(), B.gshell, B.gphi, B.gaux, B.gcells, false, B.node,
+           (int64_t)0);
 }
 
 void launch_potential_tables(const SegLayout& L, const double* r, const double* x,
                              const double* m, double* tile_m, double* tile_mx, double* phi,
-                             float2* t32, double* Menc, bool nb_sub, bool sums_ready,
-                             BucketWork& B, cudaStream_t st) {
+                             bool nb_sub, bool sums_ready, BucketWork& B, cudaStream_t st) {
   if (!L.n) return;
-  launch_k(k_table_params, (unsigned)((L.n_seg + 127) / 128), 128, 0, st,
-      L.dev(), L.esc_step, nb_sub, x, B.off, B.base, B.prm, B.goff, B.gprm, B.gaux);
   TableOut T;
   T.start = B.start;
   T.boff = B.off;
@@ -1782,12 +1748,11 @@ void launch_potential_tables(const SegLayout& L, const double* r, const double* 
   T.gshell = B.gshell;
   T.goff = B.goff;
   T.gprm = B.gprm;
-  launch_potential(L, r, x, m, tile_m, tile_mx, phi, t32, Menc, nb_sub, st, B.node,
-                   sums_ready, true, &T);
+  T.gaux = B.gaux;
+  launch_potential(L, r, x, m, tile_m, tile_mx, phi, nullptr, nb_sub, st, sums_ready, B.node, &T);
   const int64_t threads = B.gcells + L.n_tiles;
-  launch_k(k_grid_build, (unsigned)((threads + 255) / 256), 256, 0, st,
-      L.dev(), L.esc_step, nb_sub, x, phi, Menc, B.args(), B.gshell, B.gphi, B.gaux, B.gcells,
-      true, r, B.node, L.n_tiles);
+  launch_k(k_grid_build, (unsigned)((threads + 255) / 256), 256, 0, st, L.dev(), L.esc_step,
+           nb_sub, x, phi, B.args(), B.gshell, B.gphi, B.gaux, B.gcells, true, B.node, L.n_tiles);
 }
 
 void launch_buckets(const SegLayout& L, const float2* t32, bool nb_sub, BucketWork& B,
@@ -1822,18 +1787,18 @@ void free_env(EnvWork& W, cudaStream_t st) {
 }
 
 void launch_turning(const SegLayout& L, const double* r, const double* x, const double* phi,
-                    const double* Menc, const double* vr, const double* vt,
+                    const double* vr, const double* vt,
                     const BucketArgs& ba, double* tp_min, double* tp_max, double4_32a* orb,
                     int block, cudaStream_t st) {
   if (!L.n) return;
   if (block <= 0) block = 64;
   const unsigned grid = (unsigned)((L.n + block - 1) / block);
-  launch_k(k_turning_mixed<5>, grid, block, 0, st, L.dev(), r, x, phi, Menc, vr, vt, ba, tp_min,
+  launch_k(k_turning_mixed<5>, grid, block, 0, st, L.dev(), r, x, phi, vr, vt, ba, tp_min,
                                              tp_max, orb, L.n);
 }
 
 void launch_orbit(const SegLayout& L, int precision, int max_trials, const double* r,
-                  const double* x, const double* phi, const double* Menc,
+                  const double* x, const double* phi,
                   const double* vr, const double* vt, const double* m, const uint32_t* id,
                   const uint32_t* step,
                   uint64_t* keys, RecA* ra, RecB* rb, const OrbitStageOut* dbg, int block,
@@ -1865,10 +1830,10 @@ void launch_orbit(const SegLayout& L, int precision, int max_trials, const doubl
   // by bisection (kPrec 0)
   const bool exact = precision == 0;
 #define CMC_TURN(B)                                                                          \
-  launch_k(k_turning_mixed<5>, grid, block, 0, st, L.dev(), r, x, phi, Menc, vr, vt, ba,      \
+  launch_k(k_turning_mixed<5>, grid, block, 0, st, L.dev(), r, x, phi, vr, vt, ba,      \
                                              tp_min, tp_max, orb, L.n)
 #define CMC_ORBIT(P, B, T)                                                                  \
-  launch_k(k_orbit<P, B, T>, grid, block, 0, st, L.dev(), max_trials, r, x, phi, Menc, vr, vt, \
+  launch_k(k_orbit<P, B, T>, grid, block, 0, st, L.dev(), max_trials, r, x, phi, vr, vt, \
            m, id, step, keys, ra, rb, L.esc_step, d, ba, tp_min, tp_max, orb, L.n, Rv, Rp, Fx, \
            Av, Ap, bo)
 #define CMC_SAMPLED(B, T, X)                                                                \

@@ -555,30 +555,43 @@ __global__ void __launch_bounds__(kThreads) k_tile_sums(Seg S, const int64_t* es
 // each, so that two tiles' worth of warps (32) share an SM; its shared
 // arrays pad one double per 8 (a thread's run of 8 sits 9 words from its
 // neighbour's, free of bank conflicts within each half-warp).
+// With few tiles the blocks share a tile, up to 16 to one: each takes the tile's
+// integer sums by itself (they are exact, so the same in every block) and
+// finishes its part of the stars.  Up to two blocks per SM that way: one block
+// per tile leaves most SMs idle (the potential stage of 10^4, 10^5 stars 42, 42 us
+// against 26, 29; at 245 tiles and more a second block per tile only adds the
+// sums' work, 70.2 us against 71.7).
+constexpr int kPotParts = 4;    // log2
+constexpr int kPotBlocks = 304;
 constexpr int kPotThreads = 512;
 constexpr int kPotPer = kTile / kPotThreads;
 constexpr int kPotWarps = kPotThreads / 32;
 __device__ __forceinline__ int pad8(int e) { return e + (e >> 3); }
 constexpr int kPad8N = kTile + kTile / 8;
 
-// fixed-order block sum over kPotThreads threads: a tree in each warp, then
-// a tree over the warp totals in the first warp (w17: kPotWarps + 1 slots)
-__device__ __forceinline__ double block_sum_pot(double v, double* w17) {
+// fixed-order block sums of two values over kPotThreads threads: a tree in each
+// warp, then a tree over the warp totals in the first warp (a, b: kPotWarps + 1
+// slots each).  A warp of zeros skips its tree, so a few tiles cost few FP64
+// additions (16 cycles each on one SM's pipe).
+__device__ __forceinline__ double tree_sum_pot(double v, int o) {
+  if (!__any_sync(0xFFFFFFFFu, (ubits(v) << 1) != 0ull)) return 0.0;
+  for (; o > 0; o >>= 1) v = v + __shfl_down_sync(0xFFFFFFFFu, v, o);
+  return v;
+}
+__device__ __forceinline__ void block_sums_pot(double& u, double& v, double* a, double* b) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = v + __shfl_down_sync(0xFFFFFFFFu, v, o);
-  if (lane == 0) w17[w] = v;
+  u = tree_sum_pot(u, 16);
+  v = tree_sum_pot(v, 16);
+  if (lane == 0) a[w] = u, b[w] = v;
   __syncthreads();
-  if (w == 0) {
-    double u = lane < kPotWarps ? w17[lane] : 0.0;
-#pragma unroll
-    for (int o = kPotWarps / 2; o > 0; o >>= 1) u = u + __shfl_down_sync(0xFFFFFFFFu, u, o);
-    if (lane == 0) w17[kPotWarps] = u;
+  if (w < 2) {
+    double* q = w ? b : a;
+    const double z = tree_sum_pot(lane < kPotWarps ? q[lane] : 0.0, kPotWarps / 2);
+    if (lane == 0) q[kPotWarps] = z;
   }
   __syncthreads();
-  const double r = w17[kPotWarps];
-  __syncthreads();
-  return r;
+  u = a[kPotWarps];
+  v = b[kPotWarps];
 }
 
 // Fixed point for the sums inside a tile: v >= 0 as round(v 2^S) in 64
@@ -597,13 +610,11 @@ __device__ __forceinline__ long long fix_of(double v, int S) {
   if (e == 0) return 0;  // zero (and subnormals, far below any sum here)
   const unsigned long long mant = (u & 0xFFFFFFFFFFFFFull) | (1ull << 52);
   const int sh = e - 1075 + S;  // v = mant 2^(e - 1075); sh <= -3 for the largest
-  if (sh >= 0) return (long long)(mant << sh);
   if (sh < -60) return 0;
   const int d = -sh;
-  // round to nearest, ties to even
-  const unsigned long long q = mant >> d, rem = mant & ((1ull << d) - 1ull),
-                           half = 1ull << (d - 1);
-  return (long long)(q + ((rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull));
+  // round to nearest, ties to even (d in [3, 60]; the rest in the top bits)
+  const unsigned long long q = mant >> d, rem = (mant << (64 - d)) | (q & 1ull);
+  return (long long)(q + (rem > (1ull << 63) ? 1ull : 0ull));
 }
 
 // V 2^-S (V >= 0) as the nearest double, ties to even
@@ -617,8 +628,8 @@ __device__ __forceinline__ double dbl_of_fix(long long V, int S) {
   } else {
     const int d = top - 52;
     m = a >> d;
-    const unsigned long long rem = a & ((1ull << d) - 1ull), half = 1ull << (d - 1);
-    if (rem > half || (rem == half && (m & 1ull))) ++m;
+    const unsigned long long rem = (a << (64 - d)) | (m & 1ull);
+    if (rem > (1ull << 63)) ++m;
     if (m >> 53) {
       m >>= 1;
       ++top;
@@ -686,38 +697,101 @@ __device__ __forceinline__ void block_scans_fix(long long vm, long long vs, long
   __syncthreads();
 }
 
+// The index tables' parameters of a segment of nb bound stars (x: its 1/r, from
+// the innermost star out).  Buckets: the indexed node range, the smallest shift
+// that fits its range of float keys into cap buckets, their count; base = the
+// key of the first indexed node.  Grid: the finest 2^p cells per binade (p <= 10)
+// that fit cap.
+__device__ __forceinline__ int4 bucket_params_of(const double* x, int64_t nb, int64_t cap,
+                                                 uint32_t& base) {
+  base = 0;
+  if (nb <= 0) return make_int4(0, 0, 0, -1);
+  const int tail = nb >= 4096 ? (int)(nb >> 10) : 0;
+  const int lo = tail, hi = (int)nb - 1 - tail;
+  const uint32_t b0 = __float_as_uint(f32_rn(x[lo])), b1 = __float_as_uint(f32_rn(x[hi]));
+  const uint32_t span = b0 >= b1 ? b0 - b1 : 0u;
+  int bs = 0;
+  while ((int64_t)(span >> bs) + 1 > cap) ++bs;
+  base = b0;
+  return make_int4(bs, (int)((span >> bs) + 1), lo, hi);
+}
+__device__ __forceinline__ int4 grid_params_of(const double* x, int64_t nb, int64_t cap) {
+  if (nb <= 0) return make_int4(0, 0, 0, 0);
+  const uint32_t klo = __float_as_uint(f32_rn(x[nb - 1])), khi = __float_as_uint(f32_rn(x[0]));
+  int gp = 10;
+  while (gp > 0 && (int64_t)((khi >> (23 - gp)) - (klo >> (23 - gp))) + 2 > cap) --gp;
+  const int sh = 23 - gp;
+  const uint32_t key0 = (klo >> sh) << sh;
+  return make_int4((int)key0, sh, (int)((khi - key0) >> sh) + 2, (int)khi);
+}
+
 // Phi_k = -(M_k x_k + S_k) over one tile.  The tile's m and x are staged in
 // shared memory with coalesced loads; each thread scans its 8 consecutive
 // elements (local suffix sums of m x kept in registers), the per-thread
-// totals are scanned across the block, and the results (Phi, M_k, the
-// float tables, the node records) leave through shared memory with
-// coalesced stores.
-__global__ void __launch_bounds__(kPotThreads) k_potential(Seg S, const int64_t* esc, bool sub,
-                                                           const double* r, const double* x,
-                                                           const double* m, const double* tile_m,
-                                                           const double* tile_mx, double* phi,
-                                                           float2* t32, double* Mout,
-                                                           double4_32a* node, bool slopes,
-                                                           TableOut T) {
+// totals are scanned across the block, and the results leave through shared
+// memory with coalesced stores.  kTables: with the orbit step's tables (node
+// records, bucket starts, the grid's key shells, their parameters), else Phi
+// and, if wanted, M_k.
+// Bound with the tables by instruction issue (about 600 a star: three roundings
+// to fixed point, two back, a quotient, two fills) and two thirds of the FP64
+// pipe; the memory traffic of 76 B a star would take a third of the time.  4 x
+// 10^6 stars 154 us, with Phi over M_k in shared memory and 40 registers for
+// three blocks an SM (two blocks of 64 registers and no spill: 171).  What the
+// tables' readers do not use is not written (float pairs, M_k), neighbours'
+// keys and cells come by shuffle, and the tables' parameters are found here by
+// two threads of each block while the tile loads (a kernel of one thread per
+// segment before took 4.4 us): the stage of 10^7 stars 457 us to 367, of 64 x
+// 10^5 stars 328 to 287, of 1021 stars 33 to 20.5.
+template <bool kTables>
+__global__ void __launch_bounds__(kPotThreads, kTables ? 3 : 2) k_potential(
+    Seg S, const int64_t* esc, bool sub, const double* r, const double* x, const double* m,
+    const double* tile_m, const double* tile_mx, double* phi, double* Mout, double4_32a* node,
+    TableOut T, int lp) {
   pdl_enter();
   extern __shared__ double smem[];
   double* s_m = smem;               // m, then M_k
   double* s_x = smem + kPad8N;      // x
-  double* s_p = smem + 2 * kPad8N;  // Phi
-  __shared__ double wm[kPotWarps + 1], ws[kPotWarps];
+  double* s_p = kTables ? s_m : smem + 2 * kPad8N;  // Phi (over M_k, unless that is wanted)
+  __shared__ double wm[kPotWarps + 1], ws[kPotWarps + 1];
   __shared__ long long wq[kPotWarps], wr[kPotWarps];
   __shared__ int we[kPotWarps];
-  TR R = tile_of(S, esc, blockIdx.x, sub);
-  const int64_t t0 = blockIdx.x - R.lt;
+  const int64_t tile = blockIdx.x >> lp;
+  TR R = tile_of(S, esc, tile, sub);
+  const int64_t t0 = tile - R.lt;
   const int t = threadIdx.x;
+  // this block's part of the tile: elements c0 .. c1 - 1
+  const int c0 = (int)(blockIdx.x & ((1u << lp) - 1u)) * (kTile >> lp), c1 = c0 + (kTile >> lp);
+  if (R.begin + c0 >= R.end) return;
+  // (uniform: the last tile's parts beyond the segment)
+  __shared__ int4 s_prm[2];
+  __shared__ uint32_t s_base;
+  const int64_t nbk = R.bound_end - R.seg_begin;
+  if (kTables) {
+    const bool out = R.lt == 0 && c0 == 0;  // for the kernels that follow
+    if (t == 0) {
+      uint32_t base;
+      s_prm[0] = bucket_params_of(x + R.seg_begin, nbk, T.boff[R.seg + 1] - T.boff[R.seg] - 1, base);
+      s_base = base;
+      if (out) {
+        T.prm[R.seg] = s_prm[0];
+        T.base[R.seg] = base;
+      }
+    } else if (t == 32) {
+      s_prm[1] = grid_params_of(x + R.seg_begin, nbk, T.goff[R.seg + 1] - T.goff[R.seg]);
+      if (out) {
+        T.gprm[R.seg] = s_prm[1];
+        T.gaux[R.seg] = make_float4(0.f, 0.f, __uint_as_float((uint32_t)s_prm[1].x), 0.f);
+      }
+    }
+  }
   // tiles before (M) and after (S) this one, in a fixed order
   double pm = 0.0, ps = 0.0;
   for (int64_t j = t; j < R.nt; j += kPotThreads) {
     if (j < R.lt) pm = pm + tile_m[t0 + j];
     if (j > R.lt) ps = ps + tile_mx[t0 + j];
   }
-  const double Mbefore = block_sum_pot(pm, wm);
-  const double Safter = block_sum_pot(ps, wm);
+  block_sums_pot(pm, ps, wm, ws);
+  const double Mbefore = pm, Safter = ps;
 #pragma unroll
   for (int i = 0; i < kPotPer; ++i) {
     const int e = i * kPotThreads + t;
@@ -755,80 +829,84 @@ __global__ void __launch_bounds__(kPotThreads) k_potential(Seg S, const int64_t*
   for (int i = 0; i < kPotPer; ++i) am = am + fix_of(s_m[pad8(e0 + i)], Sm);
   long long pre_m, suf_s;
   block_scans_fix(am, ax, wq, wr, pre_m, suf_s);
+  // the part's own elements, and the next one (for the last slope)
   long long run = pre_m;
+  const bool own = e0 <= c1 && e0 + kPotPer > c0;
 #pragma unroll
   for (int i = 0; i < kPotPer; ++i) {
+    if (!own) break;
     const int q = pad8(e0 + i);
     run = run + fix_of(s_m[q], Sm);
     const double Mk = Mbefore + dbl_of_fix(run, Sm);
     const double Sk = Safter + dbl_of_fix(suf_s + suf[i], Sx);
     const double ph = -(Mk * s_x[q] + Sk);
-    s_m[q] = Mk;
+    if (!kTables) s_m[q] = Mk;
     s_p[q] = ph;
   }
   __syncthreads();
+  if (!kTables) {
 #pragma unroll 4
-  for (int i = 0; i < kPotPer; ++i) {
-    const int e = i * kPotThreads + t;
-    const int64_t p = R.begin + e;
-    if (p >= R.end) break;
-    const bool bound = p < R.bound_end;
-    const int q = pad8(e);
-    const double ph = bound ? s_p[q] : 0.0;
-    phi[p] = ph;
-    if (t32) t32[p] = make_float2(f32_pair(s_x[q]).hi, f32_pair(ph).hi);
-    // the enclosed mass M_k, or with `slopes` the slope of Eq. 6 in 1/r
-    // across shell k, (Phi_{k+1} - Phi_k) / (x_k - x_{k+1}) with Phi = 0 at
-    // 1/r = 0 beyond the last bound star (the FP64 orbit step's shell
-    // parameter); a tile's last star, whose neighbour is in the next tile,
-    // gets its slope from k_slope_seams
-    double w = bound ? s_m[q] : 0.0;
-    if (slopes) {
-      w = 0.0;
-      if (bound) {
-        if (p + 1 >= R.bound_end) w = div_rn(0.0 - ph, s_x[q] - 0.0);
-        else if (e + 1 < kTile) {
-          const int q1 = pad8(e + 1);
-          w = div_rn(s_p[q1] - ph, s_x[q] - s_x[q1]);
-        }
-      }
+    for (int e = c0 + t; e < c1; e += kPotThreads) {
+      const int64_t p = R.begin + e;
+      if (p >= R.end) break;
+      const bool bound = p < R.bound_end;
+      phi[p] = bound ? s_p[pad8(e)] : 0.0;
+      if (Mout) Mout[p] = bound ? s_m[pad8(e)] : 0.0;
     }
-    if (Mout) Mout[p] = w;
-    if (node) node[p] = make_double4_32a(s_x[q], ph, r[p], w);
-    if (T.start && bound) {
-      // the orbit step's index tables, star by star: bucket starts (from the
-      // float keys of 1/r of this star and its predecessor, as t32 holds
-      // them) and the grid cells between 1/r of this star and the next
-      const int c = R.seg;
-      const int64_t k = p - R.seg_begin, nb = R.bound_end - R.seg_begin;
-      const int4 pr = T.prm[c];
-      if (k >= pr.z && k <= pr.w) {
-        const double xm1 = e > 0 ? s_x[pad8(e - 1)] : (k > 0 ? __ldg(x + p - 1) : 0.0);
-        bucket_starts_of(k, nb, pr, T.base[c], __float_as_uint(f32_pair(s_x[q]).hi),
-                         k > pr.z ? __float_as_uint(f32_pair(xm1).hi) : 0u,
-                         T.start + T.boff[c], T.boff[c + 1] - T.boff[c]);
-      }
-      const double xk1 = k + 1 < nb ? (e + 1 < kTile ? s_x[pad8(e + 1)] : __ldg(x + p + 1)) : 0.0;
-      grid_shells_of(k, nb, s_x[q], xk1, T.gprm[c], T.gshell + T.goff[c]);
-    }
+    return;
   }
-}
-
-// The slopes k_potential leaves to the seams between tiles: the last star
-// of every tile whose next star (in the next tile) is bound.
-__global__ void k_slope_seams(Seg S, const int64_t* esc, bool sub, const double* r,
-                              const double* x, const double* phi, double* M,
-                              double4_32a* node, int64_t n_tiles) {
-  pdl_enter();
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_tiles) return;
-  TR R = tile_of(S, esc, t, sub);
-  const int64_t p = R.end - 1;
-  if (p < R.begin || p + 1 >= R.bound_end) return;
-  const double xj = x[p], pj = phi[p], xj1 = x[p + 1], pj1 = phi[p + 1];
-  const double w = div_rn(pj1 - pj, xj - xj1);
-  if (M) M[p] = w;
-  node[p] = make_double4_32a(xj, pj, r[p], w);
+  // Phi, the node records and the orbit step's index tables
+  const int c = R.seg;
+  const int4 prm = s_prm[0], gpr = s_prm[1];
+  const uint32_t base = s_base;
+  int* start = T.start + T.boff[c];
+  const int64_t cap = T.boff[c + 1] - T.boff[c];
+  int* gsh = T.gshell + T.goff[c];
+  const int nb = (int)nbk;
+  const int lane = t & 31;
+#pragma unroll 2
+  for (int e = c0 + t; e < c1; e += kPotThreads) {  // (whole warps)
+    const int64_t p = R.begin + e;
+    const bool bound = p < R.end && p < R.bound_end;
+    const int q = pad8(e);
+    const double ph = bound ? s_p[q] : 0.0, xk = s_x[q];
+    if (p < R.end) {
+      phi[p] = ph;
+      // the slope of Eq. 6 in 1/r across shell k, (Phi_{k+1} - Phi_k) / (x_k -
+      // x_{k+1}) with Phi = 0 at 1/r = 0 beyond the last bound star (the FP64
+      // orbit step's shell parameter); a tile's last star, whose neighbour is
+      // in the next tile, gets its slope from k_grid_build
+      double w = 0.0;
+      if (bound && (p + 1 >= R.bound_end || e + 1 < kTile)) {
+        const bool last = p + 1 >= R.bound_end;
+        const int q1 = pad8(e + 1 < kTile ? e + 1 : e);
+        w = div_rn((last ? 0.0 : s_p[q1]) - ph, xk - (last ? 0.0 : s_x[q1]));
+      }
+      node[p] = make_double4_32a(xk, ph, r[p], w);
+    }
+    // the index tables, star by star: bucket starts from the float keys of 1/r
+    // of this star and its predecessor, and the grid cells between 1/r of
+    // this star and the next (the neighbours' by shuffle)
+    const int64_t k = p - R.seg_begin;
+    const uint32_t key = __float_as_uint(f32_rn(xk));
+    const int cell = grid_last_cell(xk, gpr);
+    uint32_t before = __shfl_up_sync(0xFFFFFFFFu, key, 1);
+    int after = __shfl_down_sync(0xFFFFFFFFu, cell, 1);
+    if (lane == 0)
+      before = __float_as_uint(f32_rn(e > 0 ? s_x[pad8(e - 1)] : bound && k > 0 ? x[p - 1] : 0.0));
+    if (lane == 31)
+      after = grid_last_cell(e + 1 < kTile ? s_x[pad8(e + 1)] : bound && k + 1 < nb ? x[p + 1] : 0.0,
+                             gpr);
+    bucket_starts_of(0xFFFFFFFFu, bound, (int)k, prm, base, key, before, start, cap);
+    grid_shells_of(0xFFFFFFFFu, bound, (int)k, nb, cell, after, gpr, gsh);
+  }
+  // the ends of both tables, by the part that has their star
+  const int64_t ew = prm.w - R.lt * kTile;
+  if (nb > 0 && ew >= c0 && ew < c1)
+    bucket_close(nb, prm, base, __float_as_uint(f32_rn(s_x[pad8((int)ew)])), start, cap, t,
+                 kPotThreads);
+  if (nb > 0 && R.lt == 0 && c0 == 0)
+    grid_close(grid_last_cell(s_x[0], gpr), gpr, gsh, t, kPotThreads);
 }
 
 // ---------------------------------------------------- energy correction
@@ -1355,30 +1433,32 @@ void launch_velocities(const SegLayout& L, const uint32_t* order, const RecB* rb
            L.dev(), L.esc_step, L.n, order, rb, phi, m, vr, vt);
 }
 
-constexpr size_t kPotentialSmem = sizeof(double) * 3 * kPad8N;
+constexpr size_t potential_smem(bool tables) {
+  return sizeof(double) * (tables ? 2 : 3) * kPad8N;
+}
 
 void potential_prepare() {
-  cudaFuncSetAttribute(k_potential, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)kPotentialSmem);
+  cudaFuncSetAttribute(k_potential<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)potential_smem(false));
+  cudaFuncSetAttribute(k_potential<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)potential_smem(true));
 }
 
 
 void launch_potential(const SegLayout& L, const double* r, const double* x, const double* m,
-                      double* tile_m, double* tile_mx, double* phi, float2* t32,
-                      double* Mout, bool nb_sub, cudaStream_t st, double4_32a* node,
-                      bool sums_ready, bool slopes, const TableOut* tables) {
+                      double* tile_m, double* tile_mx, double* phi, double* Mout, bool nb_sub,
+                      cudaStream_t st, bool sums_ready, double4_32a* node,
+                      const TableOut* tables) {
   if (!L.n_tiles) return;
   Seg S = L.dev();
   if (!sums_ready)
-    launch_k(k_tile_sums, (unsigned)L.n_tiles, kThreads, 0, st, S, L.esc_step, nb_sub, x, m, tile_m,
-                                                         tile_mx);
-  launch_k(k_potential, (unsigned)L.n_tiles, kPotThreads, kPotentialSmem, st,
-      S, L.esc_step, nb_sub, r, x, m, tile_m, tile_mx, phi, t32, Mout, node, slopes,
-      tables ? *tables : TableOut());
-  // with the tables, the seams' slopes come with the grid's values
-  if (slopes && node && !tables)
-    launch_k(k_slope_seams, blocks_for(L.n_tiles, 128), 128, 0, st, S, L.esc_step, nb_sub, r, x, phi,
-                                                              Mout, node, L.n_tiles);
+    launch_k(k_tile_sums, (unsigned)L.n_tiles, kThreads, 0, st, S, L.esc_step, nb_sub, x, m,
+             tile_m, tile_mx);
+  int lp = 0;
+  while (lp < kPotParts && L.n_tiles << (lp + 1) <= kPotBlocks) ++lp;
+  launch_k(tables ? k_potential<true> : k_potential<false>, (unsigned)(L.n_tiles << lp),
+           kPotThreads, potential_smem(tables != nullptr), st, S, L.esc_step, nb_sub, r, x, m, tile_m, tile_mx, phi, Mout, node,
+           tables ? *tables : TableOut(), lp);
 }
 
 void launch_correction(const SegLayout& L, const double* r, const double* x,

@@ -1,0 +1,78 @@
+"""The orbit step's tables where the potential kernel's blocks share a tile or fill
+long ranges together: FP64 mode with the tables (precision 0) against bisection
+on the FP64 table (precision 2), two timesteps, bit for bit; Phi against exact
+sums.  No tolerance for the states: both modes compute the same FP64 operations.
+M and
+Phi: each term is rounded to a unit of at most 2^-49 of its tile's largest (half
+of it off, 4096 terms at most), the sums over the tile are exact, and fewer than
+32 roundings of 2^-53 follow (the trees over the tiles, the product, the sums),
+for the outer sum one more per product."""
+import math
+
+import numpy as np
+import pytest
+
+import initial_conditions as ic
+from gpu_util import dev, host
+
+pytestmark = pytest.mark.gpu
+
+
+def _model(n, seed, kind="plummer"):
+    d = ic.plummer(n, seed=seed, masses="salpeter")
+    if kind == "gap":  # two thin shells a factor 10^3 apart: a thousand cells in one range
+        r = np.where(np.arange(n) < n // 2, 1e-2, 10.0) * (1.0 + 1e-7 * np.arange(n))
+        d["vr"], d["vt"] = np.zeros(n), np.sqrt((np.arange(n) + 1.0) / n / r) * 0.9
+        d["r"] = r
+    elif kind == "halo":  # stars out to 10^6 radii: most cells belong to few stars
+        k = max(n // 50, 1)
+        d["r"][:k] = np.geomspace(50.0, 1e6, k)
+        d["vr"][:k], d["vt"][:k] = 0.0, 0.5 / np.sqrt(d["r"][:k])
+    return d
+
+
+def _agree(g, d, sizes=None):
+    S = []
+    for p in (0, 2):
+        seeds = [5] if sizes is None else list(range(5, 5 + len(sizes)))
+        c = g.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, seeds, precision=p, sizes=sizes)
+        c.step(2)
+        S.append(c.get_state())
+    for k in ("r", "vr", "vt", "m", "id", "phi"):
+        np.testing.assert_array_equal(S[0][k], S[1][k], err_msg=k)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 255, 256, 257, 511, 513, 2047, 2049, 4095, 4096, 4097,
+                               8193, 19 * 4096 + 257, 38 * 4096 - 1, 38 * 4096 + 1,
+                               77 * 4096 + 4095, 153 * 4096 + 1])
+def test_parts_of_tiles(g_stage, n):
+    _agree(g_stage, _model(n, n))
+
+
+@pytest.mark.parametrize("kind", ["gap", "halo"])
+@pytest.mark.parametrize("n", [64, 5000, 200_000])
+def test_long_ranges(g_stage, n, kind):
+    _agree(g_stage, _model(n, 3, kind))
+
+
+def test_ragged_ensemble(g_stage):
+    sizes = [1, 300, 4096, 256, 9001, 33, 4097, 2]
+    parts = [_model(n, 40 + i) for i, n in enumerate(sizes)]
+    _agree(g_stage, {k: np.concatenate([q[k] for q in parts]) for k in parts[0]}, sizes)
+
+
+@pytest.mark.parametrize("n", [1, 256, 257, 4097, 38 * 4096 + 1])
+def test_phi_of_parts(g_stage, n):
+    d = _model(n, 9)
+    p = np.argsort(d["r"], kind="stable")
+    r, m = d["r"][p], d["m"][p]
+    phi, M = (host(v) for v in g_stage.stage_potential(dev(r), dev(m), want_M=True))
+    x = 1.0 / r
+    mx = m * x
+    t, u = min(n, 4096) * 2.0 ** -50, 32 * 2.0 ** -53
+    for k in np.unique(np.linspace(0, n - 1, 40).astype(int)):
+        Mk, Sk = math.fsum(m[: k + 1]), math.fsum(mx[k + 1:])
+        dM, dS = t * m.max() + u * Mk, t * mx.max() + u * Sk
+        assert abs(M[k] - Mk) <= dM
+        want = math.fsum([Mk * x[k], Sk])
+        assert abs(phi[k] + want) <= dM * x[k] + dS + u * want
