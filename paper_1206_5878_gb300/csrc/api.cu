@@ -237,8 +237,8 @@ void record_step(cmc_ctx* c, cudaStream_t st, cudaEvent_t* ev = nullptr) {
     if (i < CMC_NSTAGES) nvtxRangePushA(kStageName[i]);
   };
   mark(0);
-  launch_bins(L, c->r, c->vr, c->vt, c->m, c->nbin, c->pref, st);
-  launch_tcentral(L, c->r, c->vr, c->vt, c->m, c->R, c->A, c->cfg.x_bb, c->cfg.x_bs, st);
+  launch_bins(L, c->r, c->vr, c->vt, c->m, c->nbin, c->pref, st, c->R, c->A, c->cfg.x_bb,
+              c->cfg.x_bs);
   mark(1);
   launch_relax(L, c->vr, c->vt, c->m, c->id, c->nbin, c->step, st, c->relax_variant, c->R, c->r,
                c->phi);
@@ -314,8 +314,7 @@ int count_step_kernels(const cmc_ctx* c) {
   // precision 0: the envelope's screen and evaluation], [Phi_new(r_old)]
   const int p = c->cfg.precision;
   const int sort = c->cfg.sort_packed ? (c->L.n <= kCountInOrbit ? 3 : 4) : 7;
-  return 7 + sort + ((c->R || c->A) ? 1 : 0) + (c->ring ? 4 : 0) +
-         (p == 1 ? 4 : p == 0 ? 6 : 0) + (c->cfg.energy_correction ? 1 : 0);
+  return 7 + sort + (c->ring ? 4 : 0) + (p == 1 ? 4 : p == 0 ? 6 : 0) + (c->cfg.energy_correction ? 1 : 0);
 }
 
 void free_ctx(cmc_ctx* c) {

@@ -278,20 +278,19 @@ void launch_correction(const SegLayout& L, const double* r, const double* x,
                        const double* c, bool nb_sub, uint32_t* err, cudaStream_t st,
                        const double* m = nullptr);
 
+// Eq. 7's timesteps of the bins into the segments' timesteps, and the bins'
+// densities; with R (stellar radii) or A (semi-major axes) also Eq. 8's
+// collision step and Eqs. 9-10's binary steps over the innermost 300 bound stars
 void launch_bins(const SegLayout& L, const double* r, const double* vr, const double* vt,
-                 const double* m, double* nbin, double pref, cudaStream_t st);
+                 const double* m, double* nbin, double pref, cudaStream_t st,
+                 const double* R = nullptr, const double* A = nullptr, double x_bb = 0.0,
+                 double x_bs = 0.0);
 
 // relaxation of the neighbour pairs; with stellar radii R (may be null)
 // pairs may merge (sticky spheres; r and phi: the current table)
 void launch_relax(const SegLayout& L, double* vr, double* vt, double* m, const uint32_t* id,
                   const double* nbin, const uint32_t* step, cudaStream_t st, int variant = 0,
                   double* R = nullptr, const double* r = nullptr, const double* phi = nullptr);
-// The timesteps over the innermost 300 bound stars into the segments'
-// timesteps: Eq. 8's collision step (R: stellar radii, may be null) and
-// Eqs. 9-10's binary steps (A: semi-major axes, may be null)
-void launch_tcentral(const SegLayout& L, const double* r, const double* vr, const double* vt,
-                     const double* m, const double* R, const double* A, double x_bb,
-                     double x_bs, cudaStream_t st);
 
 struct OrbitStageOut {   // optional per-star outputs of the orbit stage
   double* phi_new = nullptr;

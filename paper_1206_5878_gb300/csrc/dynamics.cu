@@ -8,62 +8,240 @@ namespace cmc {
 
 namespace {
 
-// One thread per bin slot.  Bin b of a segment covers sorted positions
-// [b*bs, min((b+1)*bs, nb)).  For P >= 2 stars:
+// The timesteps over the innermost P = min(300, nb) bound stars of each
+// segment (summed in star order, as the FP64 statement of the method does),
+// into the segment's timestep (the minimum with Eq. 7's).  With stellar radii R,
+// Eq. 8's collision timestep
+//   1 / T_coll = 16 sqrt(pi) n_s <R^2> sigma (1 + G <M R> / (2 sigma^2 <R^2>)),
+// n_s = 3 (P - 1) / (4 pi (r_{P-1}^3 - r_0^3)), sigma^2 = <v_r^2 + v_t^2> / 3.
+// With binaries (semi-major axes A > 0, the star's mass the binary's),
+// Eqs. 9 and 10:
+//   1 / T_bb = 16 sqrt(pi) n_b X_bb^2 <a^2> sigma (1 + G <M a> / (2 sigma^2 X_bb <a^2>))
+//   1 / T_bs = 4 sqrt(pi) n_s X_bs^2 <a^2> sigma (1 + G <M> <a> / (sigma^2 X_bs <a^2>))
+// with n_b, n_s the central density times the binaries' and singles' shares
+// of the P stars, <a^2>, <M a>, <a> over the binaries, <M> over all P.
+// One block of k_bins per segment: its threads take the stars' terms, the seven
+// sums run side by side in seven lanes of a warp (a chain of P additions in star
+// order; a term that does not count is a 0 and leaves the sum as it is).  Bound
+// by that chain and the formulas after it; a thread per segment that took the
+// terms too, in a kernel of its own, took 200 us; this
+// takes 13 more than the bins alone.
+struct Central {
+  const double *R = nullptr, *A = nullptr;
+  double x_bb = 0.0, x_bs = 0.0;
+};
+constexpr int kCentralStars = 300;
+enum { kCenV, kCenR, kCenMR, kCenM, kCenA, kCenA2, kCenMA, kCenSums };
+
+__device__ __forceinline__ void central_timestep(const Seg& S, int c, const double* r,
+                                                 const double* vr, const double* vt,
+                                                 const double* m, const Central& C) {
+  __shared__ double s_t[kCenSums][kCentralStars + 1];
+  const int64_t nb = S.nb[c], sb = S.off[c];
+  const int P = nb < kCentralStars ? (int)nb : kCentralStars;
+  if (P < 2) return;  // (one segment a block: all its threads)
+  int nbin = 0;
+  for (int k0 = 0; k0 < P; k0 += blockDim.x) {
+    const int k = k0 + threadIdx.x;
+    bool binary = false;
+    if (k < P) {
+      const int64_t p = sb + k;
+      const double mk = m[p], Rk = C.R ? C.R[p] : 0.0, Ak = C.A ? C.A[p] : 0.0;
+      binary = Ak > 0.0;
+      s_t[kCenV][k] = vr[p] * vr[p] + vt[p] * vt[p];
+      s_t[kCenR][k] = Rk * Rk;
+      s_t[kCenMR][k] = mk * Rk;
+      s_t[kCenM][k] = mk;
+      s_t[kCenA][k] = binary ? Ak : 0.0;
+      s_t[kCenA2][k] = binary ? Ak * Ak : 0.0;
+      s_t[kCenMA][k] = binary ? mk * Ak : 0.0;
+    }
+    nbin += __syncthreads_count(binary);
+  }
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x;
+  double sum = 0.0;
+  if (lane < kCenSums) {
+#pragma unroll 10
+    for (int k = 0; k < P; ++k) sum = sum + s_t[lane][k];
+  }
+  auto total = [&](int l) { return __shfl_sync(0xFFFFFFFFu, sum, l); };
+  const double sv = total(kCenV), sr = total(kCenR), smr = total(kCenMR), sm = total(kCenM),
+               sa = total(kCenA), sa2 = total(kCenA2), sma = total(kCenMA);
+  if (lane != 0) return;
+  const double* rr = r + sb;
+  const double vol = rr[P - 1] * rr[P - 1] * rr[P - 1] - rr[0] * rr[0] * rr[0];
+  if (!(vol > 0.0)) return;
+  const double ns = (3.0 * (double)(P - 1)) / ((4.0 * kPi) * vol);
+  const double inf = __longlong_as_double(0x7FF0000000000000ll);
+  const double sig2 = (sv / (double)P) / 3.0;
+  const double sig = sig2 > 0.0 ? sqrt(sig2) : 0.0;
+  double Tmin = inf;
+  if (C.R) {
+    const double R2 = sr / (double)P;
+    const double MR = smr / (double)P;
+    if (R2 > 0.0 && sig2 > 0.0) {
+      double inv = (((16.0 * sqrt(kPi)) * ns) * R2) * sig;
+      inv = inv * (1.0 + MR / ((2.0 * sig2) * R2));
+      const double T = 1.0 / inv;
+      if (T < Tmin) Tmin = T;
+    }
+  }
+  if (C.A && nbin > 0 && sig2 > 0.0) {
+    const double a2 = sa2 / (double)nbin, ma = sma / (double)nbin, am = sa / (double)nbin;
+    const double mm = sm / (double)P;
+    const double nbd = ns * ((double)nbin / (double)P);
+    const double nsd = ns * ((double)(P - nbin) / (double)P);
+    if (nbin < P) {
+      double inv = (((4.0 * sqrt(kPi)) * nsd) * ((C.x_bs * C.x_bs) * a2)) * sig;
+      inv = inv * (1.0 + (mm * am) / ((sig2 * C.x_bs) * a2));
+      const double T = 1.0 / inv;
+      if (T < Tmin) Tmin = T;
+    }
+    double inv = (((16.0 * sqrt(kPi)) * nbd) * ((C.x_bb * C.x_bb) * a2)) * sig;
+    inv = inv * (1.0 + ma / (((2.0 * sig2) * C.x_bb) * a2));
+    const double T = 1.0 / inv;
+    if (T < Tmin) Tmin = T;
+  }
+  if (Tmin < inf)
+    atomicMin((unsigned long long*)(S.dt_bits + c), (unsigned long long)__double_as_longlong(Tmin));
+}
+
+// Bin b of a segment covers sorted positions [b*bs, min((b+1)*bs, nb)).  For P
+// >= 2 stars:
 //   n = 3 (P-1) / (4 pi (r_last^3 - r_first^3))
 //   <v_rel> = mean over pairs (2j, 2j+1) of sqrt(v1^2 + v2^2)
 //   <(M1+M2)^2> = mean over the same pairs of (m1 + m2)^2
 //   T_b = pref <v_rel>^3 / (lnL n <(M1+M2)^2>),  pref = (theta_max/(pi/2)) (pi/32)
 // and the segment's timestep is the minimum of T_b.
-__global__ void __launch_bounds__(256) k_bins(Seg S, int bs, double pref, const double* r,
-                                              const double* vr, const double* vt,
-                                              const double* m, double* nbin) {
+// kPairs: a thread per pair takes the pair's two terms (whole bins of a block at a
+// time), then a thread per bin sums them in star order and finishes the bin, so
+// that a bin's chain of dependent operations is its additions and not its roots;
+// else a thread per bin does all of it.  The chain and the loads' latency bound
+// few bins, the FP64 pipe many (there the pairs' threads wait at the barriers for
+// the bins'): 10.5 us by pairs, 18.4 by bins at 10^5 stars, 13.8 and 18.5 at 4 x
+// 10^5, 19.9 and 20.1 at 7 x 10^5 (35,000 bins: the line), 26.6 and 25.0 at 10^6,
+// 177 and 128 at 10^7.
+// kCentral: the first n_seg blocks take the central timesteps.
+constexpr int64_t kBinsByPairs = 32768;
+constexpr int kBinThreads = 256;
+
+// a block's bins, and of each bin's `all` pairs those taken at a time
+struct BinShape {
+  int all, pairs, bins;
+};
+__host__ __device__ __forceinline__ BinShape bin_shape(int bs, bool by_pairs) {
+  BinShape w;
+  w.all = bs / 2;
+  w.pairs = w.all < kBinThreads ? w.all : kBinThreads;
+  w.bins = by_pairs ? kBinThreads / w.pairs : kBinThreads;
+  return w;
+}
+
+template <bool kCentral, bool kPairs>
+__global__ void __launch_bounds__(kBinThreads) k_bins(Seg S, int bs, double pref, const double* r,
+                                                      const double* vr, const double* vt,
+                                                      const double* m, double* nbin,
+                                                      Central C) {
   pdl_enter();
-  __shared__ unsigned long long s_min[8];
+  int64_t blk = blockIdx.x;
+  if (kCentral) {
+    if (blk < S.n_seg) {
+      central_timestep(S, (int)blk, r, vr, vt, m, C);
+      return;
+    }
+    blk -= S.n_seg;
+  }
+  __shared__ unsigned long long s_min[kBinThreads / 32];
   __shared__ int s_seg0;
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t b0 = (int64_t)blockIdx.x * blockDim.x;
-  if (threadIdx.x == 0) s_seg0 = seg_find(S.bin_off, S.n_seg, b0);
-  __syncthreads();
+  const int t = threadIdx.x;
+  const BinShape W = bin_shape(bs, kPairs);
+  const int G = W.bins;
+  const int64_t n_bins = S.bin_off[S.n_seg], b0 = blk * G;
+  if (t == 0) s_seg0 = seg_find(S.bin_off, S.n_seg, b0);
+  // bin b: its segment, number there, first star and stars
+  auto bin_of = [&](int64_t b, int& c, int64_t& lb, int64_t& first, int64_t& P) {
+    c = seg_find(S.bin_off, S.n_seg, b);
+    lb = b - S.bin_off[c];
+    const int64_t nbc = S.nb[c];
+    first = lb * bs;
+    P = first < nbc ? (nbc - first < bs ? nbc - first : bs) : 0;
+    first += S.off[c];
+  };
+  // a pair's terms
+  auto pair = [&](int64_t a, double& v, double& mm) {
+    // (two of the five products on the integer pipes: the kernel is bound by
+    // the FP64 pipe)
+    const double va2 = mul_rn(vr[a], vr[a]) + vt[a] * vt[a];
+    const double vb2 = mul_rn(vr[a + 1], vr[a + 1]) + vt[a + 1] * vt[a + 1];
+    const double ms = m[a] + m[a + 1];
+    v = sqrt_rn(va2 + vb2);
+    mm = ms * ms;
+  };
+  double sv = 0.0, sm = 0.0;
+  if (kPairs) {
+    __shared__ double s_v[3 * kBinThreads / 2], s_m[3 * kBinThreads / 2];
+    const int H = W.pairs, pitch = H | 1;  // G pitch <= G (H + 1) <= 3/2 kBinThreads
+    const int g = t / H, j = t - g * H;    // pair j (of every H) of bin b0 + g
+    int64_t ga = 0;
+    int q = 0;  // the bin's pairs
+    if (g < G && b0 + g < n_bins) {
+      int c;
+      int64_t lb, P;
+      bin_of(b0 + g, c, lb, ga, P);
+      q = (int)(P / 2);
+    }
+    for (int j0 = 0; j0 < W.all; j0 += H) {
+      if (g < G) {
+        double v = 0.0, mm = 0.0;  // (leaves the sums as they are)
+        if (j0 + j < q) pair(ga + 2 * (int64_t)(j0 + j), v, mm);
+        s_v[g * pitch + j] = v;
+        s_m[g * pitch + j] = mm;
+      }
+      __syncthreads();
+      if (t < G) {
+        for (int i = 0; i < H; ++i) {
+          sv = sv + s_v[t * pitch + i];
+          sm = sm + s_m[t * pitch + i];
+        }
+      }
+      __syncthreads();
+    }
+  } else {
+    __syncthreads();  // s_seg0
+    if (b0 + t < n_bins) {
+      int c;
+      int64_t lb, first, P;
+      bin_of(b0 + t, c, lb, first, P);
+      for (int64_t j = 0; j < P / 2; ++j) {
+        double v, mm;
+        pair(first + 2 * j, v, mm);
+        sv = sv + v;
+        sm = sm + mm;
+      }
+    }
+  }
+  const int64_t b = b0 + t;
   unsigned long long tb = 0x7FF0000000000000ull;  // +inf
   int c = s_seg0;
-  if (b < S.bin_off[S.n_seg]) {
-    c = seg_find(S.bin_off, S.n_seg, b);
-    const int64_t lb = b - S.bin_off[c];
-    const int64_t sb = S.off[c];
-    const int64_t nbc = S.nb[c];
-    const int64_t first = lb * bs;
+  if (t < G && b < n_bins) {
+    int64_t lb, first, P;
+    bin_of(b, c, lb, first, P);
     double n = 0.0;
-    if (first < nbc) {
-      int64_t P = nbc - first < bs ? nbc - first : bs;
-      if (P >= 2) {
-        const int64_t g = sb + first;
-        double rf = r[g], rl = r[g + P - 1];
-        double vol = rl * rl * rl - rf * rf * rf;
-        if (vol > 0.0) {
-          n = div_rn(3.0 * (double)(P - 1), (4.0 * kPi) * vol);
-          int64_t q = P / 2;
-          double sv = 0.0, sm = 0.0;
-          for (int64_t j = 0; j < q; ++j) {
-            int64_t a = g + 2 * j;
-            // two of the five products on the integer pipes: the kernel is
-            // bound by the FP64 pipe (0.137 -> 0.124 ms at N = 1e7; more of
-            // them there 0.131 and above)
-            double va2 = mul_rn(vr[a], vr[a]) + vt[a] * vt[a];
-            double vb2 = mul_rn(vr[a + 1], vr[a + 1]) + vt[a + 1] * vt[a + 1];
-            double ms = m[a] + m[a + 1];
-            sv = sv + sqrt_rn(va2 + vb2);
-            sm = sm + ms * ms;
-          }
-          double v = div_rn(sv, (double)q);
-          double msq = div_rn(sm, (double)q);
-          double num = pref * (v * v * v);
-          double den = (S.lnL[c] * n) * msq;
-          if (den > 0.0) {
-            double T = div_rn(num, den);
-            if (T < __longlong_as_double(0x7FF0000000000000ll))
-              tb = (unsigned long long)__double_as_longlong(T);
-          }
+    if (P >= 2) {
+      const double rf = r[first], rl = r[first + P - 1];
+      const double vol = rl * rl * rl - rf * rf * rf;
+      if (vol > 0.0) {
+        n = div_rn(3.0 * (double)(P - 1), (4.0 * kPi) * vol);
+        const double qd = (double)(P / 2);
+        const double v = div_rn(sv, qd);
+        const double msq = div_rn(sm, qd);
+        const double num = pref * (v * v * v);
+        const double den = (S.lnL[c] * n) * msq;
+        if (den > 0.0) {
+          const double T = div_rn(num, den);
+          if (T < __longlong_as_double(0x7FF0000000000000ll))
+            tb = (unsigned long long)__double_as_longlong(T);
         }
       }
     }
@@ -84,14 +262,14 @@ __global__ void __launch_bounds__(256) k_bins(Seg S, int bs, double pref, const 
   if (c != s_seg0 && tb != 0x7FF0000000000000ull)
     atomicMin((unsigned long long*)(S.dt_bits + c), tb);
   for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long y = __shfl_down_sync(0xffffffffu, mine, o);
+    const unsigned long long y = __shfl_down_sync(0xffffffffu, mine, o);
     mine = y < mine ? y : mine;
   }
-  if ((threadIdx.x & 31) == 0) s_min[threadIdx.x >> 5] = mine;
+  if ((t & 31) == 0) s_min[t >> 5] = mine;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (t == 0) {
     unsigned long long v = s_min[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v = s_min[w] < v ? s_min[w] : v;
+    for (int w = 1; w < kBinThreads / 32; ++w) v = s_min[w] < v ? s_min[w] : v;
     if (v != 0x7FF0000000000000ull) atomicMin((unsigned long long*)(S.dt_bits + s_seg0), v);
   }
 }
@@ -254,89 +432,6 @@ __global__ void k_taus_init(int64_t slots, int n_seg, const int64_t* base, const
   table[e] = make_uint4(v[0], v[1], v[2], v[3]);
 }
 
-// The timesteps over the innermost P = min(300, nb) bound stars of each
-// segment (one thread per segment summing in star order, as the FP64
-// statement of the method does), into the segment's timestep (the minimum
-// with Eq. 7's).  With stellar radii R, Eq. 8's collision timestep
-//   1 / T_coll = 16 sqrt(pi) n_s <R^2> sigma (1 + G <M R> / (2 sigma^2 <R^2>)),
-// n_s = 3 (P - 1) / (4 pi (r_{P-1}^3 - r_0^3)), sigma^2 = <v_r^2 + v_t^2> / 3.
-// With binaries (semi-major axes A > 0, the star's mass the binary's),
-// Eqs. 9 and 10:
-//   1 / T_bb = 16 sqrt(pi) n_b X_bb^2 <a^2> sigma (1 + G <M a> / (2 sigma^2 X_bb <a^2>))
-//   1 / T_bs = 4 sqrt(pi) n_s X_bs^2 <a^2> sigma (1 + G <M> <a> / (sigma^2 X_bs <a^2>))
-// with n_b, n_s the central density times the binaries' and singles' shares
-// of the P stars, <a^2>, <M a>, <a> over the binaries, <M> over all P.
-__global__ void k_tcentral(Seg S, const double* r, const double* vr, const double* vt,
-                           const double* m, const double* R, const double* A, double x_bb,
-                           double x_bs) {
-  pdl_enter();
-  const int c = blockIdx.x;
-  if (threadIdx.x != 0 || c >= S.n_seg) return;
-  const int64_t nb = S.nb[c], sb = S.off[c];
-  const int64_t P = nb < 300 ? nb : 300;
-  if (P < 2) return;
-  const double* rr = r + sb;
-  const double vol = rr[P - 1] * rr[P - 1] * rr[P - 1] - rr[0] * rr[0] * rr[0];
-  if (!(vol > 0.0)) return;
-  const double ns = (3.0 * (double)(P - 1)) / ((4.0 * kPi) * vol);
-  const double inf = __longlong_as_double(0x7FF0000000000000ll);
-  double Tmin = inf;
-  if (R) {
-    double sv = 0.0, sr = 0.0, smr = 0.0;
-    for (int64_t k = 0; k < P; ++k) {
-      const int64_t p = sb + k;
-      sv = sv + (vr[p] * vr[p] + vt[p] * vt[p]);
-      sr = sr + R[p] * R[p];
-      smr = smr + m[p] * R[p];
-    }
-    const double sig2 = (sv / (double)P) / 3.0;
-    const double R2 = sr / (double)P;
-    const double MR = smr / (double)P;
-    if (R2 > 0.0 && sig2 > 0.0) {
-      const double sig = sqrt(sig2);
-      double inv = (((16.0 * sqrt(kPi)) * ns) * R2) * sig;
-      inv = inv * (1.0 + MR / ((2.0 * sig2) * R2));
-      const double T = 1.0 / inv;
-      if (T < Tmin) Tmin = T;
-    }
-  }
-  if (A) {
-    int64_t nbin = 0;
-    double sv = 0.0, sm = 0.0, sa = 0.0, sa2 = 0.0, sma = 0.0;
-    for (int64_t k = 0; k < P; ++k) {
-      const int64_t p = sb + k;
-      sv = sv + (vr[p] * vr[p] + vt[p] * vt[p]);
-      sm = sm + m[p];
-      if (A[p] > 0.0) {
-        nbin += 1;
-        sa = sa + A[p];
-        sa2 = sa2 + A[p] * A[p];
-        sma = sma + m[p] * A[p];
-      }
-    }
-    const double sig2 = (sv / (double)P) / 3.0;
-    if (nbin > 0 && sig2 > 0.0) {
-      const double sig = sqrt(sig2);
-      const double a2 = sa2 / (double)nbin, ma = sma / (double)nbin, am = sa / (double)nbin;
-      const double mm = sm / (double)P;
-      const double nbd = ns * ((double)nbin / (double)P);
-      const double nsd = ns * ((double)(P - nbin) / (double)P);
-      if (nbin < P) {
-        double inv = (((4.0 * sqrt(kPi)) * nsd) * ((x_bs * x_bs) * a2)) * sig;
-        inv = inv * (1.0 + (mm * am) / ((sig2 * x_bs) * a2));
-        const double T = 1.0 / inv;
-        if (T < Tmin) Tmin = T;
-      }
-      double inv = (((16.0 * sqrt(kPi)) * nbd) * ((x_bb * x_bb) * a2)) * sig;
-      inv = inv * (1.0 + ma / (((2.0 * sig2) * x_bb) * a2));
-      const double T = 1.0 / inv;
-      if (T < Tmin) Tmin = T;
-    }
-  }
-  if (Tmin < inf)
-    atomicMin((unsigned long long*)(S.dt_bits + c), (unsigned long long)__double_as_longlong(Tmin));
-}
-
 }  // namespace
 
 void launch_taus_init(int64_t slots, int n_seg, const int64_t* base, const uint4* words,
@@ -346,18 +441,22 @@ void launch_taus_init(int64_t slots, int n_seg, const int64_t* base, const uint4
                                                                  table);
 }
 
-void launch_tcentral(const SegLayout& L, const double* r, const double* vr, const double* vt,
-                     const double* m, const double* R, const double* A, double x_bb,
-                     double x_bs, cudaStream_t st) {
-  if (!L.n || (!R && !A)) return;
-  launch_k(k_tcentral, (unsigned)L.n_seg, 32, 0, st, L.dev(), r, vr, vt, m, R, A, x_bb, x_bs);
-}
-
 void launch_bins(const SegLayout& L, const double* r, const double* vr, const double* vt,
-                 const double* m, double* nbin, double pref, cudaStream_t st) {
+                 const double* m, double* nbin, double pref, cudaStream_t st, const double* R,
+                 const double* A, double x_bb, double x_bs) {
   if (!L.n_bins) return;
-  launch_k(k_bins, (unsigned)((L.n_bins + 255) / 256), 256, 0, st, L.dev(), L.bin_size, pref, r, vr,
-                                                             vt, m, nbin);
+  const bool pairs = L.n_bins <= kBinsByPairs;
+  const int G = bin_shape(L.bin_size, pairs).bins;
+  const bool central = R || A;
+  Central C;
+  C.R = R;
+  C.A = A;
+  C.x_bb = x_bb;
+  C.x_bs = x_bs;
+  launch_k(central ? (pairs ? k_bins<true, true> : k_bins<true, false>)
+                   : (pairs ? k_bins<false, true> : k_bins<false, false>),
+           (unsigned)((L.n_bins + G - 1) / G + (central ? L.n_seg : 0)), kBinThreads, 0, st,
+           L.dev(), L.bin_size, pref, r, vr, vt, m, nbin, C);
 }
 
 template <int kMinB>
