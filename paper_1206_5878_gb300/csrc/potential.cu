@@ -313,12 +313,15 @@ __global__ void __launch_bounds__(kGatThreads, kGatThreads == 512 ? 3 : 1) k_gat
 // abreast) and reads one node next to its neighbours'.  Where the stretch is
 // too long to stage, the search runs on the table.  With the velocities'
 // kernel 0.42 ms at N = 1e7, 18 us at 1e5; the one kernel before them, in the new
-// order with a random search through the bucket index per star, 0.44 ms.
+// order with a random search through the bucket index per star, 0.44 ms.  With one
+// star a thread there are four times the blocks: faster while they find idle
+// SMs (both kernels at 10^4, 10^5, 2 x 10^5 stars 12.3, 14.3, 17.7 us against
+// 16.4, 18.4, 20.5), slower above (7 x 10^5: 39.3 against 37.5).
 constexpr int kPoThreads = 256;
-constexpr int kPoPer = 4;
-constexpr int kPoChunk = kPoThreads * kPoPer;  // stars per block
-constexpr int kPoWin = 2048;                   // staged radii at most
-static_assert(kTile % kPoChunk == 0, "whole chunks in a tile");
+constexpr int kPoPer = 4;     // stars per thread, 1 while there are few tiles
+constexpr int64_t kPoFewTiles = 76;
+constexpr int kPoWin = 2048;  // staged radii at most
+static_assert(kTile % (kPoThreads * kPoPer) == 0, "whole chunks in a tile");
 
 // largest i in [0, nb) with r[i] <= q, else -1, by one warp
 __device__ __forceinline__ int64_t warp_shell(const double* r, int64_t nb, double q) {
@@ -339,7 +342,7 @@ __device__ __forceinline__ int64_t warp_shell(const double* r, int64_t nb, doubl
   return lo;
 }
 
-template <bool kDiv>
+template <bool kDiv, int kPer>
 __global__ void __launch_bounds__(kPoThreads) k_phi_old(Seg S, const int64_t* esc,
                                                         const double* r_in, const double* x_in,
                                                         const double* r, const double* x,
@@ -349,6 +352,7 @@ __global__ void __launch_bounds__(kPoThreads) k_phi_old(Seg S, const int64_t* es
   __shared__ long long po_r[kPoWin];
   __shared__ int64_t s_lo, s_hi;
   const int t = threadIdx.x;
+  constexpr int kPoChunk = kPoThreads * kPer;  // the block's stars
   constexpr int kSub = kTile / kPoChunk;
   TR R = tile_of(S, esc, blockIdx.x / kSub, false);
   // the old order's bound stars in this chunk; the new table
@@ -358,9 +362,9 @@ __global__ void __launch_bounds__(kPoThreads) k_phi_old(Seg S, const int64_t* es
   if (begin >= end) return;
   const int64_t sb = R.seg_begin, nb = S.nb[R.seg] - esc[R.seg];
   if (nb <= 0) return;
-  double ro[kPoPer], xo[kPoPer];
+  double ro[kPer], xo[kPer];
 #pragma unroll
-  for (int j = 0; j < kPoPer; ++j) {
+  for (int j = 0; j < kPer; ++j) {
     const int64_t p = begin + j * kPoThreads + t;
     ro[j] = p < end ? r_in[p] : 0.0;
     xo[j] = p < end ? x_in[p] : 0.0;
@@ -374,20 +378,20 @@ __global__ void __launch_bounds__(kPoThreads) k_phi_old(Seg S, const int64_t* es
   const int64_t lo0 = s_lo, hi0 = s_hi + 1;  // shells lo0 .. hi0 - 1
   const int64_t first = lo0 < 0 ? 0 : lo0;
   const int staged = (int)(hi0 - first < kPoWin ? hi0 - first : kPoWin + 1);
-  int64_t at[kPoPer];
+  int64_t at[kPer];
   if (staged <= kPoWin) {
     for (int i = t; i < staged; i += kPoThreads) po_r[i] = dbits(r[sb + first + i]);
     __syncthreads();
-    int lo[kPoPer], hi[kPoPer];
+    int lo[kPer], hi[kPer];
 #pragma unroll
-    for (int j = 0; j < kPoPer; ++j) {
+    for (int j = 0; j < kPer; ++j) {
       lo[j] = lo0 < 0 ? -1 : 0;  // (r[lo0] is not above the chunk's first star)
       hi[j] = staged;
     }
     // every star's bracket shrinks alike: staged or staged + 1 candidates
     for (int width = staged + 1; width > 1; width = (width + 1) >> 1) {
 #pragma unroll
-      for (int j = 0; j < kPoPer; ++j) {
+      for (int j = 0; j < kPer; ++j) {
         const int mid = (lo[j] + hi[j]) >> 1;
         if (mid > lo[j]) {
           if (po_r[mid] <= dbits(ro[j])) lo[j] = mid; else hi[j] = mid;
@@ -395,10 +399,10 @@ __global__ void __launch_bounds__(kPoThreads) k_phi_old(Seg S, const int64_t* es
       }
     }
 #pragma unroll
-    for (int j = 0; j < kPoPer; ++j) at[j] = first + lo[j];
+    for (int j = 0; j < kPer; ++j) at[j] = first + lo[j];
   } else {
 #pragma unroll
-    for (int j = 0; j < kPoPer; ++j) {
+    for (int j = 0; j < kPer; ++j) {
       int64_t lo = lo0, hi = hi0;
       while (hi - lo > 1) {
         const int64_t mid = lo + ((hi - lo) >> 1);
@@ -408,7 +412,7 @@ __global__ void __launch_bounds__(kPoThreads) k_phi_old(Seg S, const int64_t* es
     }
   }
 #pragma unroll
-  for (int j = 0; j < kPoPer; ++j) {
+  for (int j = 0; j < kPer; ++j) {
     const int64_t p = begin + j * kPoThreads + t;
     if (p >= end) continue;
     const int64_t i = at[j];
@@ -472,51 +476,6 @@ __global__ void __launch_bounds__(256) k_velocities(Seg S, const int64_t* esc, i
   }
   vr[p] = a;
   vt[p] = b;
-}
-
-// Double -> float rounding to nearest even with integer operations: the
-// conversion instruction runs on the FP64 pipe, which the potential kernel
-// otherwise keeps busy with its scans.  For 2^-60 <= |v| < 2^126 (both
-// parts below normal floats) the top 24 significand bits are rounded by the
-// 29 bits below them; the remainder v - hi is then exact in those 29 bits
-// and rounded the same way.  Other values take the conversions.
-struct F32Pair {
-  float hi, lo;
-};
-
-__device__ __forceinline__ F32Pair f32_pair(double v) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
-  const unsigned ex = (unsigned)(u >> 52) & 0x7FFu;
-  F32Pair r;
-  if (ex - 963u > 186u) {  // outside [963, 1149]
-    r.hi = (float)v;
-    r.lo = (float)(v - (double)r.hi);
-    return r;
-  }
-  const unsigned sg = (unsigned)(u >> 32) & 0x80000000u;
-  const unsigned top = ((ex - 896u) << 23) | ((unsigned)(u >> 29) & 0x7FFFFFu);
-  const unsigned rest = (unsigned)u & 0x1FFFFFFFu;  // the 29 bits below
-  const bool up = rest > 0x10000000u || (rest == 0x10000000u && (top & 1u));
-  r.hi = __uint_as_float(sg | (top + (up ? 1u : 0u)));  // a carry moves the exponent
-  // v - hi = (rest - (up ? 2^29 : 0)) 2^(ex - 1075), |.| <= 2^28
-  const int rem = (int)rest - (up ? (1 << 29) : 0);
-  if (rem == 0) {
-    r.lo = 0.0f;
-    return r;
-  }
-  const unsigned a = (unsigned)(rem < 0 ? -rem : rem);
-  const int lz = __clz((int)a);            // >= 3
-  const int pb = 31 - lz;                  // top bit of a
-  const unsigned n = a << lz;              // top bit at 31
-  unsigned m = n >> 8;                     // 24 bits with the leading one
-  const unsigned low = n & 0xFFu;
-  m += (low > 0x80u || (low == 0x80u && (m & 1u))) ? 1u : 0u;
-  // a 2^(ex - 1075) = (m / 2^23) 2^(ex - 1075 + pb); a carry to 2^24 bumps
-  // the exponent through the addition below
-  const unsigned fe = ex - 1075u + 127u + (unsigned)pb;  // in [15, 229]
-  const unsigned sl = (rem < 0 ? sg ^ 0x80000000u : sg);
-  r.lo = __uint_as_float(sl | ((fe << 23) + (m - 0x800000u)));
-  return r;
 }
 
 // ------------------------------------------------------------ potential
@@ -1421,8 +1380,11 @@ void launch_phi_old(const SegLayout& L, const double* r_in, const double* x_in, 
                     const double* x, const double* phi, const double4_32a* node, RecB* rb,
                     bool div_form, cudaStream_t st) {
   if (!L.n_tiles) return;
-  launch_k(div_form ? k_phi_old<true> : k_phi_old<false>,
-           (unsigned)(L.n_tiles * (kTile / kPoChunk)), kPoThreads, 0, st, L.dev(), L.esc_step, r_in, x_in, r, x, phi, node, rb);
+  const int per = L.n_tiles <= kPoFewTiles ? 1 : kPoPer;
+  launch_k(per == 1 ? (div_form ? k_phi_old<true, 1> : k_phi_old<false, 1>)
+                    : (div_form ? k_phi_old<true, kPoPer> : k_phi_old<false, kPoPer>),
+           (unsigned)(L.n_tiles * (kTile / (kPoThreads * per))), kPoThreads, 0, st, L.dev(),
+           L.esc_step, r_in, x_in, r, x, phi, node, rb);
 }
 
 void launch_velocities(const SegLayout& L, const uint32_t* order, const RecB* rb,
