@@ -59,6 +59,7 @@ struct SegLayout {
   double* dt_cap = nullptr;         // outside bounds on the timestep (cmc_set_dt_cap; 0: none)
   unsigned long long* stats = nullptr;
   double* esc_me = nullptr;         // [n_seg][2]: mass, energy carried off by escapers
+  uint32_t* tile_done = nullptr;    // blocks of a tile that have finished; zero between kernels
   uint4* taus = nullptr;            // combined-Tausworthe streams (stream mode only)
   int64_t* taus_base = nullptr;     // per segment: first stream slot
   int64_t taus_slots = 0;

@@ -132,12 +132,13 @@ __global__ void k_gather(int64_t n, const uint32_t* perm, const RecA* ra, const 
   r[p] = A.r; x[p] = A.x; vr[p] = B.vr; vt[p] = B.vt; m[p] = A.m; id[p] = A.id;
 }
 
-// The timestep's gather, one block per tile of kTile new positions.  Each star
+// The timestep's gather, a block per tile of kTile new positions or (kSpan <
+// kTile) per part of one.  Each star
 // counts the members of its bin's run that come before it in (r, id) order --
 // runs hold one or two stars, so a few neighbours -- and writes its record to
-// its place.  A star belongs to the tile its place falls in, so the block walks
-// the tile and kRunMax positions on each side: a run of up to kRunMax stars
-// across the tile's edge is seen whole.  Longer runs are in order already
+// its place.  A star belongs to the block its place falls in, so the block walks
+// its span and kRunMax positions on each side: a run of up to kRunMax stars
+// across its edge is seen whole.  Longer runs are in order already
 // (k_long_runs).
 //
 // Bound by the random 32-byte reads of the records (0.215 ms at N = 1e7 for
@@ -150,12 +151,16 @@ __global__ void k_gather(int64_t n, const uint32_t* perm, const RecA* ra, const 
 // The potential's per-tile sums of m and m x (k_tile_sums over the bound stars
 // after the orbit step) come from the values just written, in the same
 // striped element order and tree, so they are the same sums: half the block
-// sums m, the other half m x.
+// sums m, the other half m x.  Of a tile in parts, the block that finishes last
+// (a counter per tile) takes them.
 // Blocks of 512 threads, three to an SM (40 registers: a spill would miss the
 // L1 under the random reads, which made the kernel twice as slow); while there
-// are fewer tiles than SMs blocks of 1024, whose walk is half as long.
-constexpr int kGatWin = kTile + 2 * kRunMax;
-constexpr int kGatFewTiles = 152;
+// are fewer tiles than SMs blocks of 1024, whose walk is half as long; with few
+// tiles a tile in eight parts whose walk is one sub-tile (the stage at 10^4, 10^5,
+// 2 x 10^5, 3 x 10^5, 6 x 10^5 stars 19.1, 20.4, 25.8, 31.4, 46.4 us against 30.9,
+// 32.1, 32.6, 32.6, 33.0; in sixteen parts 18.6, 24.4, 30.6, 37.6, 61.4).
+constexpr int64_t kGatFewTiles = 152, kGatPartTiles = 64;
+constexpr int kGatSpan = 512;
 
 struct GatherOut {
   double *r, *x, *m;
@@ -166,24 +171,33 @@ struct GatherOut {
   double *R, *A;
 };
 
-template <bool kExact, int kGatThreads>
-__global__ void __launch_bounds__(kGatThreads, kGatThreads == 512 ? 3 : 1) k_gather_step(
+template <bool kExact, int kSpan, int kGatThreads>
+__global__ void __launch_bounds__(kGatThreads, kGatThreads == 512 ? 3 : kGatThreads == 1024 ? 1 : 2)
+    k_gather_step(
     Seg S, const int64_t* esc, int64_t n, const uint32_t* order, const RecA* ra, const RecB* rb,
     const double* r_in, GatherOut O, uint32_t* cnt, int64_t n_bins, unsigned long long* desc,
-    int64_t n_desc, uint32_t* ctl) {
+    int64_t n_desc, uint32_t* ctl, uint32_t* done) {
   pdl_enter();
+  constexpr int kParts = kTile / kSpan;
+  constexpr int kGatWin = kSpan + 2 * kRunMax;
   constexpr int kGatSub = (kGatWin + kGatThreads - 1) / kGatThreads;  // the last one partial
-  constexpr int kGatRing = 4 * kGatThreads;
+  constexpr int kGatRing = kParts > 1 ? 2048 : 4 * kGatThreads;
+  static_assert(kParts == 1 || (kGatSub + 1) * kGatThreads <= kGatRing, "the ring does not wrap");
   static_assert(kRunMax < kGatThreads, "a run's reach is the next sub-tile");
-  static_assert(kGatThreads >= 2 * kThreads, "two trees of kThreads");
+  static_assert(kGatThreads >= 2 * kThreads && kGatThreads <= 1024, "two trees of kThreads");
   __shared__ unsigned long long s_r[kGatRing];
   __shared__ uint32_t s_bin[kGatRing];
   __shared__ double s_red[2 * kThreads];
   const int t = threadIdx.x;
-  TR R = tile_of(S, esc, blockIdx.x, true);
-  const int len = (int)(R.end - R.begin);
-  // window element w = local position w - kRunMax, within the segment
-  const int64_t w0 = R.begin - kRunMax;
+  const int64_t tile = blockIdx.x / kParts;
+  TR R = tile_of(S, esc, tile, true);
+  const int tlen = (int)(R.end - R.begin);
+  // this block's part of the tile; window element w = its position w - kRunMax,
+  // within the segment
+  const int c0 = (int)(blockIdx.x % kParts) * kSpan;
+  const int len = tlen - c0 < kSpan ? tlen - c0 : kSpan;  // (<= 0 in a last tile's empty parts)
+  const int64_t pb = R.begin + c0;
+  const int64_t w0 = pb - kRunMax;
   const int wa = w0 < R.seg_begin ? (int)(R.seg_begin - w0) : 0;
   const int64_t we = S.off[R.seg + 1] - w0;
   const int wb = we < kGatWin ? (int)we : kGatWin;
@@ -236,7 +250,7 @@ __global__ void __launch_bounds__(kGatThreads, kGatThreads == 512 ? 3 : 1) k_gat
       }
       f -= kRunMax;
       if (f >= 0 && f < len) {
-        const int64_t p = R.begin + f;
+        const int64_t p = pb + f;
         O.r[p] = __longlong_as_double((long long)r);
         O.x[p] = px;
         O.m[p] = pm;
@@ -262,37 +276,62 @@ __global__ void __launch_bounds__(kGatThreads, kGatThreads == 512 ? 3 : 1) k_gat
     v = v1;
     v1 = v2;
   }
-  __syncthreads();
-  // the tile's sums
-  const int h = t & (kThreads - 1);
-  const bool sums = t < 2 * kThreads, second = t >= kThreads;
-  const int64_t bl = R.bound_end - R.begin;
-  const int lb = bl < len ? (int)(bl < 0 ? 0 : bl) : len;
-  const double* tm = O.m + R.begin;
-  const double* tx = O.x + R.begin;
-  double a = 0.0;
-  if (sums) {
-#pragma unroll 8
-    for (int i = 0; i < kPer; ++i) {
-      const int e = i * kThreads + h;
-      if (e < lb) a = a + (second ? tm[e] * tx[e] : tm[e]);
+  // the tile's sums, by its last block
+  bool last = true;
+  if (kParts > 1) {
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (t == 0) {
+      s_last = atomicAdd(done + tile, 1u) == kParts - 1u;
+      if (s_last) done[tile] = 0u;
+      __threadfence();
     }
-    s_red[t] = a;
+    __syncthreads();
+    last = s_last;
+  } else {
+    __syncthreads();
   }
-  __syncthreads();
-  // block_sum's tree, its last levels in a warp's registers
-#pragma unroll
-  for (int w = kThreads / 2; w >= 32; w >>= 1) {
-    if (sums && h < w) {
-      a = a + s_red[t + w];
+  if (last) {
+    const int h = t & (kThreads - 1);
+    const bool sums = t < 2 * kThreads, second = t >= kThreads;
+    const int64_t bl = R.bound_end - R.begin;
+    const int lb = bl < tlen ? (int)(bl < 0 ? 0 : bl) : tlen;
+    const double* tm = O.m + R.begin;
+    const double* tx = O.x + R.begin;
+    double a = 0.0;
+    if (sums) {
+#pragma unroll(kParts > 1 ? kPer : 8)
+      for (int i = 0; i < kPer; ++i) {
+        const int e = i * kThreads + h;
+        if (e < lb) {
+          if (kParts > 1) {
+            // (past the L1: other blocks wrote them; one block at work: the
+            // products on the integer pipes)
+            const double me = __ldcg(tm + e);
+            a = a + (second ? mul_rn(me, __ldcg(tx + e)) : me);
+          } else {
+            a = a + (second ? tm[e] * tx[e] : tm[e]);
+          }
+        }
+      }
       s_red[t] = a;
     }
     __syncthreads();
-  }
-  if (sums && h < 32) {
+    // block_sum's tree, its last levels in a warp's registers
 #pragma unroll
-    for (int w = 16; w > 0; w >>= 1) a = a + __shfl_down_sync(0xFFFFFFFFu, a, w);
-    if (h == 0) (second ? O.tile_mx : O.tile_m)[blockIdx.x] = a;
+    for (int w = kThreads / 2; w >= 32; w >>= 1) {
+      if (sums && h < w) {
+        a = a + s_red[t + w];
+        s_red[t] = a;
+      }
+      __syncthreads();
+    }
+    if (sums && h < 32) {
+#pragma unroll
+      for (int w = 16; w > 0; w >>= 1) a = a + __shfl_down_sync(0xFFFFFFFFu, a, w);
+      if (h == 0) (second ? O.tile_mx : O.tile_m)[tile] = a;
+    }
   }
   // the bins' counts and the scan's words, zero again for the next step
   if (cnt) {
@@ -1298,6 +1337,7 @@ cudaError_t alloc_layout(SegLayout& L, const std::vector<int64_t>& sizes,
   CMC_A(L.stats, sizeof(unsigned long long) * kStStride * L.n_seg);
   CMC_A(L.esc_me, sizeof(double) * 2 * L.n_seg);
   CMC_A(L.dt_cap, sizeof(double) * L.n_seg);
+  CMC_A(L.tile_done, sizeof(uint32_t) * (L.n_tiles + 1));
 #undef CMC_A
   cudaMemcpyAsync(L.off, L.h_off.data(), s1, cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(L.tile_off, L.h_tile_off.data(), s1, cudaMemcpyHostToDevice, st);
@@ -1314,13 +1354,14 @@ cudaError_t alloc_layout(SegLayout& L, const std::vector<int64_t>& sizes,
   cudaMemsetAsync(L.stats, 0, sizeof(unsigned long long) * kStStride * L.n_seg, st);
   cudaMemsetAsync(L.esc_me, 0, sizeof(double) * 2 * L.n_seg, st);
   cudaMemsetAsync(L.dt_cap, 0, sizeof(double) * L.n_seg, st);
+  cudaMemsetAsync(L.tile_done, 0, sizeof(uint32_t) * (L.n_tiles + 1), st);
   // the host vectors above must outlive the copies
   return cudaStreamSynchronize(st);
 }
 
 void free_layout(SegLayout& L, cudaStream_t st) {
   void* ps[] = {L.off, L.tile_off, L.pair_off, L.bin_off, L.seed, L.lnL,
-                L.nb, L.esc_step, L.dt_bits, L.dt_last, L.stats, L.esc_me, L.dt_cap};
+                L.nb, L.esc_step, L.dt_bits, L.dt_last, L.stats, L.esc_me, L.dt_cap, L.tile_done};
   for (void* p : ps)
     if (p) cudaFreeAsync(p, st);
   L = SegLayout();
@@ -1368,12 +1409,18 @@ void launch_gather_step(const SegLayout& L, BinWork* B, const uint32_t* order_in
   O.tile_m = tile_m; O.tile_mx = tile_mx;
   O.Rp = Rp; O.Ap = Ap;
   O.R = Rout; O.A = Aout;
-  const bool few = L.n_tiles <= kGatFewTiles;
-  launch_k(exact ? (few ? k_gather_step<true, 1024> : k_gather_step<true, 512>)
-                 : (few ? k_gather_step<false, 1024> : k_gather_step<false, 512>),
-           (unsigned)L.n_tiles, few ? 1024 : 512, 0, st, L.dev(), L.esc_step, L.n, order_in, ra, rb, r_in, O,
-           B ? B->cnt : nullptr, B ? B->n_bins : 0, B ? B->desc : nullptr, B ? B->n_tiles : 0,
-           B ? B->ctl : nullptr);
+  constexpr int kPart = kGatSpan + 2 * kRunMax;  // threads
+  const bool part = L.n_tiles <= kGatPartTiles, few = L.n_tiles <= kGatFewTiles;
+  launch_k(exact ? (part  ? k_gather_step<true, kGatSpan, kPart>
+                    : few ? k_gather_step<true, kTile, 1024>
+                          : k_gather_step<true, kTile, 512>)
+                 : (part  ? k_gather_step<false, kGatSpan, kPart>
+                    : few ? k_gather_step<false, kTile, 1024>
+                          : k_gather_step<false, kTile, 512>),
+           (unsigned)(part ? L.n_tiles * (kTile / kGatSpan) : L.n_tiles),
+           part ? kPart : few ? 1024 : 512, 0, st, L.dev(), L.esc_step, L.n, order_in, ra, rb, r_in,
+           O, B ? B->cnt : nullptr, B ? B->n_bins : 0, B ? B->desc : nullptr, B ? B->n_tiles : 0,
+           B ? B->ctl : nullptr, L.tile_done);
 }
 
 void launch_phi_old(const SegLayout& L, const double* r_in, const double* x_in, const double* r,

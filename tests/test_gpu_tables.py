@@ -76,3 +76,20 @@ def test_phi_of_parts(g_stage, n):
         assert abs(M[k] - Mk) <= dM
         want = math.fsum([Mk * x[k], Sk])
         assert abs(phi[k] + want) <= dM * x[k] + dS + u * want
+
+
+@pytest.mark.parametrize("n", [511, 512, 513, 543, 545, 4095, 4097, 9 * 512 + 31, 64 * 4096,
+                               64 * 4096 + 1, 152 * 4096, 152 * 4096 + 513])
+def test_gather_in_parts(g_stage, n):
+    """Stars gathered by parts of a tile, the tiles' sums by their last block: the
+    step's Phi is the potential entry point's, whose sums are a kernel's of their
+    own, bit for bit, and nothing is lost."""
+    d = _model(n, n % 89)
+    d["vr"][:: 3] *= 1.6  # some escape
+    c = g_stage.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, [3], precision=1)
+    c.step(3)
+    st = c.get_state()
+    nb = int(np.isfinite(st["r"]).sum())
+    assert nb < n and np.array_equal(np.sort(st["id"]), np.sort(d["id"]))
+    phi = host(g_stage.stage_potential(dev(st["r"][:nb]), dev(st["m"][:nb]), want_M=True)[0])
+    np.testing.assert_array_equal(st["phi"][:nb], phi)
