@@ -665,9 +665,11 @@ __device__ __forceinline__ void fill_range(unsigned mask, int* a, int from, int 
   }
 }
 
+// (in the table whatever the key: after a reported sort failure the radii need not
+// be in order)
 __device__ __forceinline__ int bucket_of(uint32_t key, uint32_t base, int4 prm) {
-  const int b = (int)((base - key) >> prm.x);
-  return b < prm.y ? b : prm.y - 1;
+  const uint32_t b = (base - key) >> prm.x;
+  return b < (uint32_t)prm.y ? (int)b : prm.y - 1;
 }
 // star k's buckets (key_k, key_km1: float bits of 1/r of stars k and k - 1);
 // every lane of mask calls it, live false where there is nothing to write

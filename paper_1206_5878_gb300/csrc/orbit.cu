@@ -1534,7 +1534,7 @@ __global__ void k_grid_params(Seg S, const int64_t* esc, bool sub, const double*
   const int sh = 23 - p;
   const uint32_t key0 = (klo >> sh) << sh;
   const int cells = (int)((khi - key0) >> sh) + 2;
-  gprm[c] = make_int4((int)key0, sh, cells, (int)khi);
+  gprm[c] = make_int4((int)key0, sh, cells < cap ? cells : (int)cap, (int)khi);
   gaux[c] = make_float4((float)phi[sb], (float)node[sb + nb - 1].w, __uint_as_float(key0), 0.f);
 }
 

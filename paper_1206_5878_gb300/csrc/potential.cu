@@ -116,7 +116,8 @@ __global__ void k_rekey_radius(int64_t n, const uint32_t* perm, const double* r,
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   uint32_t q = perm[p];
-  keys[p] = radius_key(r[q], id[q]);
+  // (out of range only after a reported sort failure)
+  keys[p] = (int64_t)q < n ? radius_key(r[q], id[q]) : ~0ull;
 }
 
 __global__ void k_gather(int64_t n, const uint32_t* perm, const RecA* ra, const RecB* rb,
@@ -720,7 +721,8 @@ __device__ __forceinline__ int4 grid_params_of(const double* x, int64_t nb, int6
   while (gp > 0 && (int64_t)((khi >> (23 - gp)) - (klo >> (23 - gp))) + 2 > cap) --gp;
   const int sh = 23 - gp;
   const uint32_t key0 = (klo >> sh) << sh;
-  return make_int4((int)key0, sh, (int)((khi - key0) >> sh) + 2, (int)khi);
+  const int cells = (int)((khi - key0) >> sh) + 2;
+  return make_int4((int)key0, sh, cells < cap ? cells : (int)cap, (int)khi);  // (as bucket_of)
 }
 
 // Phi_k = -(M_k x_k + S_k) over one tile.  The tile's m and x are staged in

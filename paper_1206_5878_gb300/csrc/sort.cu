@@ -323,6 +323,10 @@ __global__ void k_tiefix(const int64_t* off, int n_seg, int64_t n, uint64_t* key
   pdl_enter();
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
+  if (*err & kErrTimeout) {
+    vals[p] = (uint32_t)p;  // as k_long_runs: no order that was not written
+    return;
+  }
   int c = seg_find(off, n_seg, p);
   int64_t sb = __ldg(off + c), se = __ldg(off + c + 1);
   const uint64_t kp = keys[p], hp = kp >> shift;
@@ -330,11 +334,6 @@ __global__ void k_tiefix(const int64_t* off, int n_seg, int64_t n, uint64_t* key
   if (p > sb && (keys[p - 1] >> shift) == hp) return;  // not the start of the run
   int64_t e = p + 2;
   while (e < se && (keys[e] >> shift) == hp) ++e;
-  for (int64_t i = p; i < e; ++i)
-    if ((int64_t)vals[i] >= n) {
-      set_err(err, kErrTimeout);
-      return;
-    }
   // insertion sort of the run by (key, id)
   const long long move_cap = g_tie_move_cap;
   long long moves = 0;
@@ -486,8 +485,17 @@ __global__ void __launch_bounds__(256) k_bin_scatter(int64_t n, const uint32_t* 
 constexpr int kRunItems = 8;  // indices per thread and chunk
 __global__ void __launch_bounds__(kThreads) k_long_runs(int64_t n, const uint32_t* ctl,
                                                         const uint2* runs, const RecA* rec,
-                                                        uint32_t* order, uint32_t* scratch) {
+                                                        uint32_t* order, uint32_t* scratch,
+                                                        const uint32_t* err) {
   pdl_enter();
+  if (*err & kErrTimeout) {
+    // After a timed-out look-back the order is not a permutation: the stars stay
+    // where they are, so that what follows up to the report reads stars only.
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
+         p += (int64_t)gridDim.x * blockDim.x)
+      order[p] = (uint32_t)p;
+    return;
+  }
   __shared__ uint32_t whist[kWarps][kBins];
   __shared__ uint32_t base[kBins], s_warp[kWarps];
   __shared__ unsigned long long s_dr;
@@ -802,7 +810,7 @@ void launch_bin_sort(const SegLayout& L, BinWork& B, const uint32_t* bin, const 
   launch_k(k_bin_scatter, grid, 256, 0, st, L.n, bin, B.cnt, order, err);
   const int64_t most = L.n / kRunMax + 1;  // listed runs at most
   launch_k(k_long_runs, (unsigned)(most < 152 ? most : 152), kThreads, 0, st, L.n, B.ctl, B.runs,
-           rec, order, scratch);
+           rec, order, scratch, err);
 }
 
 void launch_philox(int64_t n, const uint32_t* ctr, uint64_t seed, uint32_t* out,

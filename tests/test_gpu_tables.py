@@ -93,3 +93,28 @@ def test_gather_in_parts(g_stage, n):
     assert nb < n and np.array_equal(np.sort(st["id"]), np.sort(d["id"]))
     phi = host(g_stage.stage_potential(dev(st["r"][:nb]), dev(st["m"][:nb]), want_M=True)[0])
     np.testing.assert_array_equal(st["phi"][:nb], phi)
+
+
+@pytest.mark.parametrize("n", [300_000, 700_000])
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("packed", [0, 1])
+def test_steps_after_a_sort_that_timed_out(g_stage, n, precision, packed):
+    """A look-back that gives up is reported after the call; the steps until then
+    run on stars only (no order that was never written), and another context is
+    as before."""
+    d = _model(n, 5)
+    other = g_stage.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, [5], autotune=0)
+    c = g_stage.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, [5], autotune=0,
+                        precision=precision, sort_packed=packed)
+    g_stage.set_wait_limits(lookback_polls=1)
+    try:
+        c.step(3)
+    except g_stage.CMCError as e:
+        assert e.status == 5  # CMC_ETIMEOUT (whether a poll finds its word is a race)
+    finally:
+        g_stage.set_wait_limits()
+        c.close()
+    other.step(1)
+    r = other.get_state()["r"]
+    r = r[np.isfinite(r)]
+    assert np.all(np.diff(r) >= 0)
