@@ -1226,11 +1226,13 @@ cmc_status cmc_sort_radius(int64_t n, const double* r, const uint32_t* id, uint3
   uint32_t* err = nullptr;
   cudaError_t e = alloc_sort(W, S.L, 8, st);
   uint32_t he = 0;
-  if (!e) e = dalloc(keys, n, st);
-  if (!e) e = dalloc(err, 1, st);
+  void* block = nullptr;
+  Carve C;
+  C.zero(err, 1);
+  C.add(keys, n);
+  if (!e) e = C.alloc(block, st);
   if (!e) {
     sort_prepare();
-    cudaMemsetAsync(err, 0, sizeof(uint32_t), st);
     launch_make_keys(S.L, r, id, keys, st);
     // as in the timestep: passes over bits 24-63, then runs equal in those
     // bits in (r, id) order
@@ -1250,8 +1252,7 @@ cmc_status cmc_sort_radius(int64_t n, const double* r, const uint32_t* id, uint3
     }
     if (!e) e = cudaGetLastError();
   }
-  dfree(keys, st);
-  dfree(err, st);
+  dfree(block, st);
   free_sort(W, st);
   if (e) return cuda_fail(nullptr, e, "cmc_sort_radius");
   if (he & kErrTimeout)
@@ -1268,18 +1269,19 @@ cmc_status cmc_potential(int64_t n, const double* r, const double* m, double* ph
   Stage S(n, 0, 0.0, 20, st);
   if (S.e) return cuda_fail(nullptr, S.e, "cmc_potential");
   double *x = nullptr, *ta = nullptr, *tb = nullptr;
-  cudaError_t e = dalloc(x, n, st);
-  if (!e) e = dalloc(ta, (size_t)S.L.n_tiles, st);
-  if (!e) e = dalloc(tb, (size_t)S.L.n_tiles, st);
+  void* block = nullptr;
+  Carve C;
+  C.add(x, n);
+  C.add(ta, (size_t)S.L.n_tiles);
+  C.add(tb, (size_t)S.L.n_tiles);
+  cudaError_t e = C.alloc(block, st);
   if (!e) {
     potential_prepare();
     launch_recip(n, r, x, st);
     launch_potential(S.L, r, x, m, ta, tb, phi, M, false, st);
     e = cudaGetLastError();
   }
-  dfree(x, st);
-  dfree(ta, st);
-  dfree(tb, st);
+  dfree(block, st);
   return e ? cuda_fail(nullptr, e, "cmc_potential") : CMC_OK;
 }
 
@@ -1344,25 +1346,35 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
   RecA* ra = nullptr;
   RecB* rb = nullptr;
   uint32_t* dstep = nullptr;
-  cudaError_t e = dalloc(x, n, st);
-  if (!e) e = dalloc(mm, n, st);
-  if (!e) e = dalloc(t32, n, st);
-  if (!e) e = dalloc(keys, n, st);
-  if (!e) e = dalloc(ra, n, st);
-  if (!e) e = dalloc(rb, n, st);
-  if (!e) e = dalloc(dstep, 1, st);
-  if (!e) e = cudaMemsetAsync(mm, 0, sizeof(double) * n, st);
-  if (!e) e = cudaMemcpyAsync(dstep, &step, sizeof(uint32_t), cudaMemcpyHostToDevice, st);
+  double *sl = nullptr, *tmin = nullptr, *tmax = nullptr;  // sl: the shells' slopes
+  double4_32a* orb = nullptr;
+  uint32_t *plist = nullptr, *pcnt = nullptr;
+  const bool tab = precision != 2;
+  void* block = nullptr;
+  Carve C;
+  C.put(dstep, &step, 1);
+  C.zero(mm, n);
+  C.add(x, n);
+  C.add(keys, n);
+  C.add(ra, n);
+  C.add(rb, n);
+  if (tab) {
+    C.add(t32, n);
+    C.add(sl, n);
+    C.add(tmin, n);
+    C.add(tmax, n);
+    C.add(orb, n);
+    C.add(plist, n);
+    C.add(pcnt, 1);
+  }
+  cudaError_t e = C.alloc(block, st);
   if (!e) {
     launch_recip(n, r, x, st);
-    launch_make_t32(n, x, phi, t32, st);
     BucketWork bk;
-    double* sl = nullptr;  // shell slopes (enclosed masses) from the potential
-    const bool tab = precision != 2;
     if (tab) {
       e = alloc_buckets(bk, S.L, st);
-      if (!e) e = dalloc(sl, n, st);
       if (!e) {
+        launch_make_t32(n, x, phi, t32, st);
         launch_buckets(S.L, t32, false, bk, st);
         launch_slopes(n, x, phi, sl, st);
         launch_make_nodes(n, r, x, phi, sl, bk.node, st);
@@ -1371,15 +1383,7 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
     }
     OrbitStageOut d;
     d.phi_new = phi_new; d.rmin = rmin; d.rmax = rmax; d.F = F; d.code = code;
-    double *tmin = nullptr, *tmax = nullptr;
-    double4_32a* orb = nullptr;
     EnvWork env;
-    uint32_t *plist = nullptr, *pcnt = nullptr;
-    if (!e && tab) e = dalloc(tmin, n, st);
-    if (!e && tab) e = dalloc(tmax, n, st);
-    if (!e && tab) e = dalloc(orb, n, st);
-    if (!e && tab) e = dalloc(plist, n, st);
-    if (!e && tab) e = dalloc(pcnt, 1, st);
     if (!e && precision == 0) e = alloc_env(env, n, st);
     if (!e)
       launch_orbit(S.L, precision, max_trials, r, x, phi, vr, vt, mm, id, dstep, keys,
@@ -1387,23 +1391,11 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
                    nullptr, precision == 0 ? &env : nullptr, nullptr, nullptr, orb);
     free_buckets(bk, st);
     free_env(env, st);
-    dfree(sl, st);
-    dfree(tmin, st);
-    dfree(tmax, st);
-    dfree(orb, st);
-    dfree(plist, st);
-    dfree(pcnt, st);
     launch_unpack_orbit(n, ra, rb, r_new, vr_new, vt_new, st);
     e = cudaGetLastError();
   }
   if (!e) e = cudaStreamSynchronize(st);
-  dfree(x, st);
-  dfree(mm, st);
-  dfree(t32, st);
-  dfree(keys, st);
-  dfree(ra, st);
-  dfree(rb, st);
-  dfree(dstep, st);
+  dfree(block, st);
   return e ? cuda_fail(nullptr, e, "cmc_orbit") : CMC_OK;
 }
 

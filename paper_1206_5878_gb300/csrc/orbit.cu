@@ -1708,30 +1708,23 @@ cudaError_t alloc_buckets(BucketWork& B, const SegLayout& L, cudaStream_t st) {
     goff[c + 1] = goff[c] + grid_capacity(nc);
   }
   B.gcells = goff[L.n_seg];
-  cudaError_t e;
-  if ((e = cudaMallocAsync((void**)&B.start, sizeof(int) * off[L.n_seg], st))) return e;
-  if ((e = cudaMallocAsync((void**)&B.off, sizeof(int64_t) * (L.n_seg + 1), st))) return e;
-  if ((e = cudaMallocAsync((void**)&B.base, sizeof(uint32_t) * L.n_seg, st))) return e;
-  if ((e = cudaMallocAsync((void**)&B.prm, sizeof(int4) * L.n_seg, st))) return e;
-  if ((e = cudaMallocAsync((void**)&B.gphi, sizeof(float) * B.gcells, st))) return e;
-  if ((e = cudaMallocAsync((void**)&B.gshell, sizeof(int) * B.gcells, st))) return e;
-  if ((e = cudaMallocAsync((void**)&B.goff, sizeof(int64_t) * (L.n_seg + 1), st))) return e;
-  if ((e = cudaMallocAsync((void**)&B.gprm, sizeof(int4) * L.n_seg, st))) return e;
-  if ((e = cudaMallocAsync((void**)&B.gaux, sizeof(float4) * L.n_seg, st))) return e;
-  if ((e = cudaMallocAsync((void**)&B.node, sizeof(double4_32a) * (L.n > 0 ? L.n : 1), st))) return e;
-  e = cudaMemcpyAsync(B.off, off.data(), sizeof(int64_t) * (L.n_seg + 1),
-                      cudaMemcpyHostToDevice, st);
-  if (!e)
-    e = cudaMemcpyAsync(B.goff, goff.data(), sizeof(int64_t) * (L.n_seg + 1),
-                        cudaMemcpyHostToDevice, st);
-  if (e) return e;
-  return cudaStreamSynchronize(st);  // off, goff live on this stack
+  const size_t seg = (size_t)L.n_seg;
+  Carve C;
+  C.put(B.off, off.data(), seg + 1);
+  C.put(B.goff, goff.data(), seg + 1);
+  C.add(B.start, (size_t)off[seg]);
+  C.add(B.base, seg);
+  C.add(B.prm, seg);
+  C.add(B.gphi, (size_t)B.gcells);
+  C.add(B.gshell, (size_t)B.gcells);
+  C.add(B.gprm, seg);
+  C.add(B.gaux, seg);
+  C.add(B.node, (size_t)L.n);
+  return C.alloc(B.block, st);
 }
 
 void free_buckets(BucketWork& B, cudaStream_t st) {
-  void* ps[] = {B.start, B.off, B.base, B.prm, B.gphi, B.gshell, B.goff, B.gprm, B.gaux, B.node};
-  for (void* p : ps)
-    if (p) cudaFreeAsync(p, st);
+  if (B.block) cudaFreeAsync(B.block, st);
   B = BucketWork();
 }
 
@@ -1778,11 +1771,13 @@ void launch_buckets(const SegLayout& L, const float2* t32, bool nb_sub, BucketWo
 cudaError_t alloc_env(EnvWork& W, int64_t n, cudaStream_t st) {
   const int64_t m = n > 0 ? n : 1;
   W.cap = 2 * m + 1024;  // the pairs: 1.1 per star measured on Plummer models
-  cudaError_t e = cudaMallocAsync((void**)&W.gmax, sizeof(double) * m, st);
-  if (!e) e = cudaMallocAsync((void**)&W.star, sizeof(double4_32a) * m, st);
-  if (!e) e = cudaMallocAsync((void**)&W.list, sizeof(uint64_t) * W.cap, st);
-  if (!e) e = cudaMallocAsync((void**)&W.spill, sizeof(uint64_t) * m, st);
-  if (!e) e = cudaMallocAsync((void**)&W.cnt, 2 * sizeof(unsigned long long), st);
+  Carve C;
+  C.add(W.gmax, (size_t)m);
+  C.add(W.star, (size_t)m);
+  C.add(W.list, (size_t)W.cap);
+  C.add(W.spill, (size_t)m);
+  C.add(W.cnt, 2);
+  cudaError_t e = C.alloc(W.block, st);
   if (!e) {
     launch_k(k_env_tables, 1, 32, 0, st);
     e = cudaGetLastError();
@@ -1791,9 +1786,7 @@ cudaError_t alloc_env(EnvWork& W, int64_t n, cudaStream_t st) {
 }
 
 void free_env(EnvWork& W, cudaStream_t st) {
-  void* ps[] = {W.gmax, W.star, W.list, W.spill, W.cnt};
-  for (void* q : ps)
-    if (q) cudaFreeAsync(q, st);
+  if (W.block) cudaFreeAsync(W.block, st);
   W = EnvWork();
 }
 

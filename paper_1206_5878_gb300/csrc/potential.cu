@@ -11,6 +11,7 @@
 // run, so a cluster gives the same bits whether it is advanced alone or in
 // an ensemble, and a resumed run repeats an uninterrupted one exactly.
 #include <cmath>
+#include <cstring>
 
 #include "cmc_host.hpp"
 
@@ -1272,6 +1273,16 @@ __global__ void k_unpack_orbit(int64_t n, const RecA* ra, const RecB* rb, double
 
 inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
+// the first words of a Carve's block from its image, zero up to `words`
+struct CarveImage {
+  uint4 w[128];
+};
+__global__ void k_carve(uint4* dst, int64_t words, int image, CarveImage im) {
+  pdl_enter();
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < words) dst[i] = i < image ? im.w[i] : make_uint4(0u, 0u, 0u, 0u);
+}
+
 }  // namespace
 
 void launch_nb_from_keys(const SegLayout& L, const uint64_t* keys, cudaStream_t st) {
@@ -1299,6 +1310,29 @@ void launch_unpack_orbit(int64_t n, const RecA* ra, const RecB* rb, double* r_ne
 }
 
 // ------------------------------------------------------------------ host
+void Carve::copy(unsigned char* to, const void* from, size_t n) { memcpy(to, from, n); }
+
+cudaError_t Carve::alloc(void*& block, cudaStream_t st) {
+  cudaError_t e = cudaMallocAsync(&block, bytes_ ? bytes_ : 1, st);
+  if (e) return e;
+  for (const Part& q : parts_) *q.ptr = (unsigned char*)block + q.at;
+  if (zero_ == 0) return cudaSuccess;
+  if (image_.size() <= sizeof(CarveImage)) {
+    CarveImage im;
+    memset(&im, 0, sizeof(im));
+    if (!image_.empty()) memcpy(&im, image_.data(), image_.size());
+    const int64_t words = (int64_t)(zero_ / 16);
+    launch_k(k_carve, blocks_for(words, 256), 256, 0, st, (uint4*)block, words,
+             (int)(image_.size() / 16), im);
+    return cudaGetLastError();
+  }
+  e = cudaMemcpyAsync(block, image_.data(), image_.size(), cudaMemcpyHostToDevice, st);
+  if (!e && zero_ > image_.size())
+    e = cudaMemsetAsync((unsigned char*)block + image_.size(), 0, zero_ - image_.size(), st);
+  if (!e) e = cudaStreamSynchronize(st);  // the image lives on the caller's stack
+  return e;
+}
+
 cudaError_t alloc_layout(SegLayout& L, const std::vector<int64_t>& sizes,
                          const std::vector<uint64_t>& seeds, const std::vector<double>& lnL,
                          int bin_size, cudaStream_t st) {
@@ -1322,50 +1356,28 @@ cudaError_t alloc_layout(SegLayout& L, const std::vector<int64_t>& sizes,
   L.n_tiles = L.h_tile_off[L.n_seg];
   L.n_pairs = L.h_pair_off[L.n_seg];
   L.n_bins = L.h_bin_off[L.n_seg];
-  size_t s1 = sizeof(int64_t) * (L.n_seg + 1);
-  cudaError_t e;
-#define CMC_A(ptr, bytes) \
-  if ((e = cudaMallocAsync((void**)&(ptr), (bytes), st))) return e;
-  CMC_A(L.off, s1);
-  CMC_A(L.tile_off, s1);
-  CMC_A(L.pair_off, s1);
-  CMC_A(L.bin_off, s1);
-  CMC_A(L.seed, sizeof(uint64_t) * L.n_seg);
-  CMC_A(L.lnL, sizeof(double) * L.n_seg);
-  CMC_A(L.nb, sizeof(int64_t) * L.n_seg);
-  CMC_A(L.esc_step, sizeof(int64_t) * L.n_seg);
-  CMC_A(L.dt_bits, sizeof(uint64_t) * L.n_seg);
-  CMC_A(L.dt_last, sizeof(uint64_t) * L.n_seg);
-  CMC_A(L.stats, sizeof(unsigned long long) * kStStride * L.n_seg);
-  CMC_A(L.esc_me, sizeof(double) * 2 * L.n_seg);
-  CMC_A(L.dt_cap, sizeof(double) * L.n_seg);
-  CMC_A(L.tile_done, sizeof(uint32_t) * (L.n_tiles + 1));
-#undef CMC_A
-  cudaMemcpyAsync(L.off, L.h_off.data(), s1, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(L.tile_off, L.h_tile_off.data(), s1, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(L.pair_off, L.h_pair_off.data(), s1, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(L.bin_off, L.h_bin_off.data(), s1, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(L.seed, seeds.data(), sizeof(uint64_t) * L.n_seg, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(L.lnL, lnL.data(), sizeof(double) * L.n_seg, cudaMemcpyHostToDevice, st);
-  std::vector<int64_t> nb(sizes.begin(), sizes.end());
-  cudaMemcpyAsync(L.nb, nb.data(), sizeof(int64_t) * L.n_seg, cudaMemcpyHostToDevice, st);
-  cudaMemsetAsync(L.esc_step, 0, sizeof(int64_t) * L.n_seg, st);
-  std::vector<uint64_t> inf(L.n_seg, 0x7FF0000000000000ull);
-  cudaMemcpyAsync(L.dt_bits, inf.data(), sizeof(uint64_t) * L.n_seg, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(L.dt_last, inf.data(), sizeof(uint64_t) * L.n_seg, cudaMemcpyHostToDevice, st);
-  cudaMemsetAsync(L.stats, 0, sizeof(unsigned long long) * kStStride * L.n_seg, st);
-  cudaMemsetAsync(L.esc_me, 0, sizeof(double) * 2 * L.n_seg, st);
-  cudaMemsetAsync(L.dt_cap, 0, sizeof(double) * L.n_seg, st);
-  cudaMemsetAsync(L.tile_done, 0, sizeof(uint32_t) * (L.n_tiles + 1), st);
-  // the host vectors above must outlive the copies
-  return cudaStreamSynchronize(st);
+  const size_t seg = (size_t)L.n_seg, s1 = seg + 1;
+  const std::vector<uint64_t> inf(seg, 0x7FF0000000000000ull);
+  Carve C;
+  C.put(L.off, L.h_off.data(), s1);
+  C.put(L.tile_off, L.h_tile_off.data(), s1);
+  C.put(L.pair_off, L.h_pair_off.data(), s1);
+  C.put(L.bin_off, L.h_bin_off.data(), s1);
+  C.put(L.seed, seeds.data(), seg);
+  C.put(L.lnL, lnL.data(), seg);
+  C.put(L.nb, sizes.data(), seg);
+  C.put(L.dt_bits, inf.data(), seg);
+  C.put(L.dt_last, inf.data(), seg);
+  C.zero(L.esc_step, seg);
+  C.zero(L.stats, kStStride * seg);
+  C.zero(L.esc_me, 2 * seg);
+  C.zero(L.dt_cap, seg);
+  C.zero(L.tile_done, (size_t)L.n_tiles + 1);
+  return C.alloc(L.block, st);
 }
 
 void free_layout(SegLayout& L, cudaStream_t st) {
-  void* ps[] = {L.off, L.tile_off, L.pair_off, L.bin_off, L.seed, L.lnL,
-                L.nb, L.esc_step, L.dt_bits, L.dt_last, L.stats, L.esc_me, L.dt_cap, L.tile_done};
-  for (void* p : ps)
-    if (p) cudaFreeAsync(p, st);
+  if (L.block) cudaFreeAsync(L.block, st);
   L = SegLayout();
 }
 

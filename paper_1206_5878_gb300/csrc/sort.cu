@@ -670,11 +670,6 @@ cudaError_t sort_set_shape(const SegLayout& L, SortWork& W, int ipt, int rank,
 cudaError_t alloc_sort(SortWork& W, const SegLayout& L, int max_passes, cudaStream_t st) {
   W.max_passes = max_passes;
   size_t n = (size_t)L.n;
-  cudaError_t e;
-  if ((e = cudaMallocAsync((void**)&W.keys_alt, sizeof(uint64_t) * (n ? n : 1), st))) return e;
-  if ((e = cudaMallocAsync((void**)&W.vals_alt, sizeof(uint32_t) * (n ? n : 1), st))) return e;
-  if ((e = cudaMallocAsync((void**)&W.stile_off, sizeof(int64_t) * (L.n_seg + 1), st)))
-    return e;
   // look-back words for the smallest tiles (the most tiles)
   const int64_t max_tiles = sort_tile_offsets(L, kThreads * 8)[L.n_seg];
   size_t desc_b = sizeof(unsigned long long) * (size_t)max_passes * max_tiles * kBins;
@@ -686,19 +681,28 @@ cudaError_t alloc_sort(SortWork& W, const SegLayout& L, int max_passes, cudaStre
   const size_t head_b = (hist_b + tick_b + done_b + 255) / 256 * 256;
   W.zero_bytes = head_b + desc_b;
   W.zero_head = head_b;
-  if ((e = cudaMallocAsync(&W.zero_base, W.zero_bytes, st))) return e;
+  W.ipt = 16;
+  W.rank = 0;
+  const std::vector<int64_t> o = sort_tile_offsets(L, kThreads * W.ipt);
+  W.n_stiles = o[L.n_seg];
+  unsigned char* zeroed = nullptr;
+  Carve C;
+  C.put(W.stile_off, o.data(), o.size());
+  C.add(W.keys_alt, n);
+  C.add(W.vals_alt, n);
+  C.add(zeroed, W.zero_bytes);
+  const cudaError_t e = C.alloc(W.block, st);
+  if (e) return e;
+  W.zero_base = zeroed;
   W.hist = (uint32_t*)W.zero_base;
   W.tickets = (uint32_t*)((char*)W.zero_base + hist_b);
   W.done = (uint32_t*)((char*)W.zero_base + hist_b + tick_b);
   W.desc = (unsigned long long*)((char*)W.zero_base + head_b);
-  return sort_set_shape(L, W, 16, 0, st);
+  return cudaSuccess;
 }
 
 void free_sort(SortWork& W, cudaStream_t st) {
-  if (W.keys_alt) cudaFreeAsync(W.keys_alt, st);
-  if (W.vals_alt) cudaFreeAsync(W.vals_alt, st);
-  if (W.stile_off) cudaFreeAsync(W.stile_off, st);
-  if (W.zero_base) cudaFreeAsync(W.zero_base, st);
+  if (W.block) cudaFreeAsync(W.block, st);
   W = SortWork();
 }
 
