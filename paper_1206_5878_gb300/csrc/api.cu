@@ -292,8 +292,7 @@ void record_step(cmc_ctx* c, cudaStream_t st, cudaEvent_t* ev = nullptr) {
   launch_step_end(L, c->step, c->r_old, c->cc, c->m, st);
   if (c->ring) {
     // K and W of the new state (r_old is free scratch now), then the record
-    launch_energy(L, c->r_alt, c->vr, c->vt, c->m, c->tile_a, c->tile_b, c->tile_c, c->r_old,
-                  c->out3, st);
+    launch_energy(L, c->r_alt, c->vr, c->vt, c->m, c->tile_a, c->tile_b, c->tile_c, c->out3, st);
     launch_diag_ring(L, c->out3, c->step, c->err, c->ring, c->cfg.diag_ring, st);
   }
   mark(9);
@@ -794,6 +793,7 @@ cmc_status cmc_init(cmc_ctx** out, const cmc_config* cfg_in, int32_t n_clusters,
   if (e) { cmc_status s = cuda_fail(nullptr, e, "cmc_init: allocation"); free_ctx(c); return s; }
   sort_prepare();
   potential_prepare();
+  diag_prepare();
   cmc_status s = load_state(c, r, vr, vt, m, id, ptr_kind, false, 0);
   if (s != CMC_OK) {
     g_err = c->last_error;
@@ -895,8 +895,7 @@ cmc_status cmc_energy(cmc_ctx* c, double* out) {
   if (!c || !out) return fail(c, CMC_EINVAL, "cmc_energy: bad arguments");
   if (c->poisoned) return fail(c, CMC_EPOISONED, c->last_error);
   DeviceGuard g(c->device);
-  launch_energy(c->L, c->r, c->vr, c->vt, c->m, c->tile_a, c->tile_b, c->tile_c, c->r_old,
-                c->out3, c->stream);
+  launch_energy(c->L, c->r, c->vr, c->vt, c->m, c->tile_a, c->tile_b, c->tile_c, c->out3, c->stream);
   cudaError_t e = cudaMemcpyAsync(out, c->out3, sizeof(double) * 3 * c->L.n_seg,
                                   cudaMemcpyDeviceToHost, c->stream);
   if (!e) e = cudaStreamSynchronize(c->stream);
@@ -965,8 +964,7 @@ cmc_status cmc_lagrange_radii(cmc_ctx* c, const double* fracs, int32_t nf, doubl
   if (!e) e = dalloc(dout, (size_t)nf * c->L.n_seg, st);
   if (!e) e = cudaMemcpyAsync(dfr, fracs, sizeof(double) * nf, cudaMemcpyHostToDevice, st);
   if (!e) {
-    launch_energy(c->L, c->r, c->vr, c->vt, c->m, c->tile_a, c->tile_b, c->tile_c, c->r_old,
-                  c->out3, st);
+    launch_masses(c->L, c->m, c->tile_a, c->r_old, st);
     launch_lagrange(c->L, c->r, c->r_old, dfr, nf, dout, st);
     e = cudaMemcpyAsync(out, dout, sizeof(double) * nf * c->L.n_seg, cudaMemcpyDeviceToHost,
                         st);
@@ -1277,8 +1275,7 @@ cmc_status cmc_potential(int64_t n, const double* r, const double* m, double* ph
   cudaError_t e = C.alloc(block, st);
   if (!e) {
     potential_prepare();
-    launch_recip(n, r, x, st);
-    launch_potential(S.L, r, x, m, ta, tb, phi, M, false, st);
+    launch_potential(S.L, r, x, m, ta, tb, phi, M, false, st, false, nullptr, nullptr, x);
     e = cudaGetLastError();
   }
   dfree(block, st);

@@ -294,6 +294,7 @@ void launch_velocities(const SegLayout& L, const uint32_t* order, const RecB* rb
 
 // potential: per-tile sums then the tile-local scans (Eqs. 1-5 in scan
 // form).  nb_sub: subtract esc_step from nb (after the orbit step).
+// With recip (= x), x = 1/r is computed too, with the tiles' sums.
 // Optional output: Mout (M_k); with tables instead the record {1/r, Phi, r,
 // slope} of every star (node: one 32-byte sector per node for the kernels that
 // read a few nodes at random; the slope of Eq. 6 across the shell is the FP64
@@ -314,7 +315,7 @@ struct TableOut {
 void launch_potential(const SegLayout& L, const double* r, const double* x, const double* m,
                       double* tile_m, double* tile_mx, double* phi, double* Mout, bool nb_sub,
                       cudaStream_t st, bool sums_ready = false, double4_32a* node = nullptr,
-                      const TableOut* tables = nullptr);
+                      const TableOut* tables = nullptr, double* recip = nullptr);
 // node records from the arrays (stage calls)
 void launch_make_nodes(int64_t n, const double* r, const double* x, const double* phi,
                        const double* M, double4_32a* node, cudaStream_t st);
@@ -467,10 +468,13 @@ constexpr int kRelaxVariants = 3;  // relaxation kernel register caps (launch_re
 void launch_step_end(const SegLayout& L, uint32_t* step, const double* r_old, const double* c,
                      const double* m, cudaStream_t st);
 
-// energy diagnostics: per-segment K, W_pair (Mbuf receives M_k)
+// energy diagnostics: per-segment K, W_pair
 void launch_energy(const SegLayout& L, const double* r, const double* vr, const double* vt,
                    const double* m, double* tile_m, double* tile_k, double* tile_w,
-                   double* Mbuf, double* out3, cudaStream_t st);
+                   double* out3, cudaStream_t st);
+// the mass up to and including every bound star
+void launch_masses(const SegLayout& L, const double* m, double* tile_m, double* Mout,
+                   cudaStream_t st);
 
 // core diagnostics (Eq. 19) per cluster: out3 = {rho_c, r_c, estimates};
 // tiles4: 4 * n_tiles doubles of scratch
@@ -494,6 +498,7 @@ void sort_prepare();
 // look-back polls and tie-fix moves before the sort's waits give up (<= 0:
 // the defaults), on the current device
 cudaError_t set_wait_limits(int spin_polls, long long tie_moves);
+void diag_prepare();
 void potential_prepare();  // shared-memory limit of the potential kernel
 
 // (r, id) order of staged stars (flag bit 0 set when not) and the largest id

@@ -42,29 +42,6 @@ __device__ __forceinline__ double block_sum(double v, double* s) {
   return r;
 }
 
-// fixed-shape inclusive scans of one double per thread (Hillis-Steele on
-// shared memory): forward for vm, backward for vs; returns the exclusive
-// values (sum over lower threads, sum over higher threads)
-__device__ __forceinline__ void block_scans(double vm, double vs, double* s1, double* s2,
-                                            double& pre_m, double& suf_s) {
-  // inclusive forward scan of vm, inclusive backward scan of vs
-  const int t = threadIdx.x;
-  s1[t] = vm;
-  s2[t] = vs;
-  __syncthreads();
-  for (int o = 1; o < kThreads; o <<= 1) {
-    double a = t >= o ? s1[t - o] : 0.0;
-    double b = t + o < kThreads ? s2[t + o] : 0.0;
-    __syncthreads();
-    if (t >= o) s1[t] = a + s1[t];
-    if (t + o < kThreads) s2[t] = s2[t] + b;
-    __syncthreads();
-  }
-  pre_m = t > 0 ? s1[t - 1] : 0.0;
-  suf_s = t + 1 < kThreads ? s2[t + 1] : 0.0;
-  __syncthreads();
-}
-
 struct TR {
   int seg;
   int64_t lt, nt, seg_begin, begin, end, bound_end;
@@ -520,35 +497,79 @@ __global__ void __launch_bounds__(256) k_velocities(Seg S, const int64_t* esc, i
 }
 
 // ------------------------------------------------------------ potential
-// per-tile sums of m and m x (striped, coalesced loads; fixed tree)
-__global__ void __launch_bounds__(kThreads) k_tile_sums(Seg S, const int64_t* esc, bool sub,
-                                                        const double* x, const double* m,
-                                                        double* tile_m, double* tile_mx) {
+// per-tile sums of m and m x (striped, coalesced loads; fixed tree).
+// kSumsRecip: x = 1/r of every star is computed here too, from r in x's place.
+// kSumsMass: of m alone.  The products and quotients are taken by all threads, on
+// the integer pipes; the sums run from shared memory, m's by one half of the
+// block, m x's by the other.  Two blocks of 64 registers an SM (three spill).
+// cmc_potential on 4 x 10^6 stars: reciprocals and sums in two kernels, the sums
+// by one thread for both, took 76 us, this kernel half of it.
+enum { kSumsOfX, kSumsRecip, kSumsMass };
+constexpr int kSumsThreads = 2 * kThreads;
+template <int kKind>
+__global__ void __launch_bounds__(kSumsThreads, 2) k_tile_sums(Seg S, const int64_t* esc, bool sub,
+                                                            const double* x, const double* m,
+                                                            double* tile_m, double* tile_mx,
+                                                            double* x_out) {
   pdl_enter();
-  __shared__ double s[kThreads];
+  constexpr bool kBoth = kKind != kSumsMass;
+  extern __shared__ double smem[];
+  double* s_m = smem;
+  double* s_mx = smem + (kBoth ? kTile : 0);
+  __shared__ double s_red[kSumsThreads];
   TR R = tile_of(S, esc, blockIdx.x, sub);
-  // all 32 loads issued before the sums, which still run in element order
-  double mv[kPer], xv[kPer];
-  unsigned ok = 0;
+  const int t = threadIdx.x, h = t & (kThreads - 1);
+  const bool second = t >= kThreads;
+  double mv[kTile / kSumsThreads], xv[kTile / kSumsThreads];
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    const int64_t p = R.begin + (int64_t)i * kThreads + threadIdx.x;
+  for (int j = 0; j < kTile / kSumsThreads; ++j) {
+    const int64_t p = R.begin + j * kSumsThreads + t;
     const bool in = p < R.end && p < R.bound_end;
-    ok |= (unsigned)in << i;
-    mv[i] = in ? __ldg(m + p) : 0.0;
-    xv[i] = in ? __ldg(x + p) : 0.0;
+    mv[j] = in ? __ldg(m + p) : 0.0;
+    if (kBoth) xv[j] = (kKind == kSumsRecip ? p < R.end : in) ? __ldg(x + p) : 1.0;
   }
-  double am = 0.0, ax = 0.0;
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    if ((ok >> i) & 1u) {
-      am = am + mv[i];
-      ax = ax + mv[i] * xv[i];
+  for (int j = 0; j < kTile / kSumsThreads; ++j) {
+    const int e = j * kSumsThreads + t;
+    if (kKind == kSumsRecip) {
+      xv[j] = div_rn(1.0, xv[j]);
+      if (R.begin + e < R.end) x_out[R.begin + e] = xv[j];
     }
+    s_m[e] = mv[j];  // (0 where there is no bound star: the sums stay as they are)
+    if (kBoth) s_mx[e] = R.begin + e < R.bound_end ? mul_rn(mv[j], xv[j]) : 0.0;
   }
-  double tm = block_sum(am, s);
-  double tx = block_sum(ax, s);
-  if (threadIdx.x == 0) { tile_m[blockIdx.x] = tm; tile_mx[blockIdx.x] = tx; }
+  __syncthreads();
+  // half the block sums m, the other half m x: 16 striped elements a thread,
+  // then a tree
+  double a = 0.0;
+  if (kBoth || !second) {
+    const double* q = second ? s_mx : s_m;
+#pragma unroll 4
+    for (int i = 0; i < kPer; ++i) a = a + q[i * kThreads + h];
+  }
+  s_red[t] = a;
+  __syncthreads();
+#pragma unroll
+  for (int w = kThreads / 2; w >= 32; w >>= 1) {
+    if (h < w) {
+      a = a + s_red[t + w];
+      s_red[t] = a;
+    }
+    __syncthreads();
+  }
+  if (h < 32) {
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) a = a + __shfl_down_sync(0xFFFFFFFFu, a, w);
+    if (h == 0 && (kBoth || !second)) (second ? tile_mx : tile_m)[blockIdx.x] = a;
+  }
+}
+
+template <int kKind>
+void launch_tile_sums(const SegLayout& L, bool nb_sub, const double* x, const double* m,
+                      double* tile_m, double* tile_mx, double* x_out, cudaStream_t st) {
+  launch_k(k_tile_sums<kKind>, (unsigned)L.n_tiles, kSumsThreads,
+           sizeof(double) * kTile * (kKind == kSumsMass ? 1 : 2), st, L.dev(), L.esc_step, nb_sub,
+           x, m, tile_m, tile_mx, x_out);
 }
 
 // The potential kernel runs 512 threads on a tile, 8 consecutive elements
@@ -744,7 +765,7 @@ __device__ __forceinline__ int4 grid_params_of(const double* x, int64_t nb, int6
 // segment before took 4.4 us): the stage of 10^7 stars 457 us to 367, of 64 x
 // 10^5 stars 328 to 287, of 1021 stars 33 to 20.5.
 template <bool kTables>
-__global__ void __launch_bounds__(kPotThreads, kTables ? 3 : 2) k_potential(
+__global__ void __launch_bounds__(kPotThreads, 3) k_potential(
     Seg S, const int64_t* esc, bool sub, const double* r, const double* x, const double* m,
     const double* tile_m, const double* tile_mx, double* phi, double* Mout, double4_32a* node,
     TableOut T, int lp) {
@@ -752,7 +773,7 @@ __global__ void __launch_bounds__(kPotThreads, kTables ? 3 : 2) k_potential(
   extern __shared__ double smem[];
   double* s_m = smem;               // m, then M_k
   double* s_x = smem + kPad8N;      // x
-  double* s_p = kTables ? s_m : smem + 2 * kPad8N;  // Phi (over M_k, unless that is wanted)
+  double* s_p = kTables ? s_m : s_x;  // Phi, over what is not needed any more
   __shared__ double wm[kPotWarps + 1], ws[kPotWarps + 1];
   __shared__ long long wq[kPotWarps], wr[kPotWarps];
   __shared__ int we[kPotWarps];
@@ -951,48 +972,121 @@ __global__ void k_correction(Seg S, const int64_t* esc, bool sub, const double* 
 }
 
 // ---------------------------------------------------------- diagnostics
-__global__ void __launch_bounds__(kThreads) k_energy_tiles(Seg S, const double* r,
-                                                           const double* vr, const double* vt,
-                                                           const double* m,
-                                                           const double* tile_m,
-                                                           double* tile_k, double* tile_w,
-                                                           double* Mout) {
+// Both kernels sum runs of 16 consecutive stars per thread and then a tree over
+// 256 threads.  512 threads stage the tile with coalesced loads and take the
+// stars' terms (products and quotients on the integer pipes); 256 of them sum the
+// runs from shared memory (a run of 16 + 1 padded doubles each, free of bank
+// conflicts).  Bound by the FP64 pipe (two thirds of the time: the sums) and, at
+// 10^6 stars, by the SMs that have two of the 245 tiles; three blocks an SM.
+// 42.9 and 46.8 us at 10^6 stars, the masses alone 19.2; with a thread per run
+// taking everything, loads of 128 B strides and FP64 divisions, 56.6 and 65.2.
+constexpr int kDiagThreads = 512;
+constexpr int kDiagPer = kTile / kDiagThreads;
+__device__ __forceinline__ int pad16(int e) { return e + (e >> 4); }
+constexpr int kPad16N = kTile + kTile / 16;
+
+// block_sum of the first kThreads threads' values in a block of kDiagThreads
+__device__ __forceinline__ double diag_sum(double v, double* s) {
+  const int t = threadIdx.x;
+  if (t < kThreads) s[t] = v;
+  __syncthreads();
+  for (int w = kThreads / 2; w > 0; w >>= 1) {
+    if (t < w) s[t] = s[t] + s[t + w];
+    __syncthreads();
+  }
+  const double r = s[0];
+  __syncthreads();
+  return r;
+}
+
+// kMass: only M_k, the mass up to and including star k, into Mout; else the
+// tile's sums of m v^2 and m_k M_{k-1} / r_k.
+template <bool kMass>
+__global__ void __launch_bounds__(kDiagThreads, 3) k_energy_tiles(Seg S, const double* r,
+                                                               const double* vr, const double* vt,
+                                                               const double* m,
+                                                               const double* tile_m,
+                                                               double* tile_k, double* tile_w,
+                                                               double* Mout) {
   pdl_enter();
-  __shared__ double s1[kThreads], s2[kThreads];
+  extern __shared__ double smem[];
+  double* s_m = smem;            // m, then the mass inside, then m M / r
+  double* s_k = smem + kPad16N;  // m v^2
+  __shared__ double s1[kThreads];
   TR R = tile_of(S, nullptr, blockIdx.x, false);
   const int64_t t0 = blockIdx.x - R.lt;
-  double pm = 0.0;
-  for (int64_t j = threadIdx.x; j < R.lt; j += kThreads) pm = pm + tile_m[t0 + j];
-  double Mbefore = block_sum(pm, s1);
-  const int64_t b = R.begin + (int64_t)threadIdx.x * kPer;
-  double mm[kPer];
-  double am = 0.0;
+  const int t = threadIdx.x;
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    int64_t p = b + i;
-    mm[i] = (p < R.end && p < R.bound_end) ? m[p] : 0.0;
-    am = am + mm[i];
-  }
-  double pre_m, dummy;
-  block_scans(am, 0.0, s1, s2, pre_m, dummy);
-  double run = 0.0, ak = 0.0, aw = 0.0;
-#pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    int64_t p = b + i;
-    if (p < R.end && p < R.bound_end) {
-      double Mex = (Mbefore + pre_m) + run;  // mass strictly inside star p
-      double a = vr[p], bb = vt[p];
-      ak = ak + mm[i] * (a * a + bb * bb);
-      aw = aw + mm[i] * Mex / r[p];
-      run = run + mm[i];
-      if (Mout) Mout[p] = (Mbefore + pre_m) + run;
-    } else if (p < R.end && Mout) {
-      Mout[p] = 0.0;
+  for (int j = 0; j < kDiagPer; ++j) {
+    const int e = j * kDiagThreads + t;
+    const int64_t p = R.begin + e;
+    const bool in = p < R.end && p < R.bound_end;
+    const double me = in ? m[p] : 0.0;
+    s_m[pad16(e)] = me;
+    if (!kMass) {
+      const double a = in ? vr[p] : 0.0, b = in ? vt[p] : 0.0;
+      s_k[pad16(e)] = mul_rn(me, mul_rn(a, a) + mul_rn(b, b));
     }
   }
-  double tk = block_sum(ak, s1);
-  double tw = block_sum(aw, s1);
-  if (threadIdx.x == 0) { tile_k[blockIdx.x] = tk; tile_w[blockIdx.x] = tw; }
+  double pm = 0.0;
+  if (t < kThreads)
+    for (int64_t j = t; j < R.lt; j += kThreads) pm = pm + tile_m[t0 + j];
+  const double Mbefore = diag_sum(pm, s1);
+  if (t < kThreads) {
+    double am = 0.0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) am = am + s_m[pad16(t * kPer + i)];
+    s1[t] = am;
+  }
+  __syncthreads();
+  // inclusive scan of the runs (fixed shape: doubling steps)
+  for (int o = 1; o < kThreads; o <<= 1) {
+    const double a = t >= o && t < kThreads ? s1[t - o] : 0.0;
+    __syncthreads();
+    if (t >= o && t < kThreads) s1[t] = a + s1[t];
+    __syncthreads();
+  }
+  if (t < kThreads) {
+    const double base = Mbefore + (t > 0 ? s1[t - 1] : 0.0);
+    double run = 0.0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const int q = pad16(t * kPer + i);
+      const double mi = s_m[q];
+      if (!kMass) s_m[q] = base + run;  // the mass strictly inside
+      run = run + mi;
+      if (kMass) s_m[q] = base + run;
+    }
+  }
+  __syncthreads();
+  if (kMass) {
+#pragma unroll
+    for (int j = 0; j < kDiagPer; ++j) {
+      const int e = j * kDiagThreads + t;
+      const int64_t p = R.begin + e;
+      if (p < R.end) Mout[p] = p < R.bound_end ? s_m[pad16(e)] : 0.0;
+    }
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < kDiagPer; ++j) {
+    const int e = j * kDiagThreads + t, q = pad16(e);
+    const int64_t p = R.begin + e;
+    if (p < R.end && p < R.bound_end) s_m[q] = div_rn(mul_rn(m[p], s_m[q]), r[p]);
+    else s_m[q] = 0.0;
+  }
+  __syncthreads();
+  double ak = 0.0, aw = 0.0;
+  if (t < kThreads) {
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      ak = ak + s_k[pad16(t * kPer + i)];
+      aw = aw + s_m[pad16(t * kPer + i)];
+    }
+  }
+  const double tk = diag_sum(ak, s1);
+  const double tw = diag_sum(aw, s1);
+  if (t == 0) { tile_k[blockIdx.x] = tk; tile_w[blockIdx.x] = tw; }
 }
 
 // Core diagnostics (section 4.2, Eq. 19): per bound star k with three
@@ -1000,38 +1094,70 @@ __global__ void __launch_bounds__(kThreads) k_energy_tiles(Seg S, const double* 
 // order, rho_k = (m_{k-2} + ... + m_{k+2}) / (4 pi / 3 (r_{k+3}^3 - r_{k-3}^3));
 // per tile the sums of rho, rho^2, rho r and the number of estimates, each
 // in a fixed order (runs of 16 per thread, then a fixed tree).
-__global__ void __launch_bounds__(kThreads) k_core_tiles(Seg S, const double* r, const double* m,
-                                                         double* tile_s1, double* tile_s2,
-                                                         double* tile_sr, double* tile_n) {
+__global__ void __launch_bounds__(kDiagThreads, 3) k_core_tiles(Seg S, const double* r,
+                                                             const double* m, double* tile_s1,
+                                                             double* tile_s2, double* tile_sr,
+                                                             double* tile_n) {
   pdl_enter();
+  extern __shared__ double smem[];
+  double* s_c = smem;                // r^3 of the tile and 3 stars on each side, then rho
+  double* s_m = smem + kPad16N + 8;  // m, likewise, then r
   __shared__ double s[kThreads];
   TR R = tile_of(S, nullptr, blockIdx.x, false);
-  const int64_t b = R.begin + (int64_t)threadIdx.x * kPer;
-  const double c43 = (4.0 * kPi) / 3.0;
-  double a1 = 0.0, a2 = 0.0, ar = 0.0, an = 0.0;
-  for (int i = 0; i < kPer; ++i) {
-    const int64_t p = b + i;
-    const int64_t k = p - R.seg_begin;
-    if (p >= R.end || k < 3 || p + 3 >= R.bound_end) continue;
-    const double ro = r[p + 3], ri = r[p - 3];
-    const double vol = c43 * (ro * ro * ro - ri * ri * ri);
-    if (!pos_num(vol)) continue;
-    const double mass = (((m[p - 2] + m[p - 1]) + m[p]) + m[p + 1]) + m[p + 2];
-    const double rho = mass / vol;
-    a1 = a1 + rho;
-    a2 = a2 + rho * rho;
-    ar = ar + rho * r[p];
-    an = an + 1.0;
+  const int t = threadIdx.x;
+  for (int e = t; e < kTile + 6; e += kDiagThreads) {
+    const int64_t p = R.begin + e - 3;
+    const bool in = p >= R.seg_begin && p < R.bound_end;
+    const double re = in ? r[p] : 0.0;
+    s_c[e] = mul_rn(re * re, re);
+    s_m[e] = in ? m[p] : 0.0;
   }
-  const double t1 = block_sum(a1, s), t2 = block_sum(a2, s), tr = block_sum(ar, s),
-               tn = block_sum(an, s);
-  if (threadIdx.x == 0) {
+  __syncthreads();
+  const double c43 = (4.0 * kPi) / 3.0;
+  double rho[kDiagPer];
+  unsigned ok = 0;
+#pragma unroll
+  for (int j = 0; j < kDiagPer; ++j) {
+    const int e = j * kDiagThreads + t;
+    const int64_t p = R.begin + e;
+    rho[j] = 0.0;
+    if (p >= R.end || p - R.seg_begin < 3 || p + 3 >= R.bound_end) continue;
+    const double vol = mul_rn(c43, s_c[e + 6] - s_c[e]);
+    if (!pos_num(vol)) continue;
+    const double mass = (((s_m[e + 1] + s_m[e + 2]) + s_m[e + 3]) + s_m[e + 4]) + s_m[e + 5];
+    rho[j] = div_rn(mass, vol);
+    ok |= 1u << j;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kDiagPer; ++j) {
+    const int e = j * kDiagThreads + t;
+    s_c[pad16(e)] = rho[j];
+    s_m[pad16(e)] = (ok >> j) & 1u ? r[R.begin + e] : 0.0;
+  }
+  // (an estimate that is not there is a 0 and leaves the sums as they are)
+  int count = 0;
+#pragma unroll
+  for (int j = 0; j < kDiagPer; ++j) count += __syncthreads_count((ok >> j) & 1u);
+  double a1 = 0.0, a2 = 0.0, ar = 0.0;
+  if (t < kThreads) {
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const double q = s_c[pad16(t * kPer + i)];
+      a1 = a1 + q;
+      a2 = a2 + mul_rn(q, q);
+      ar = ar + mul_rn(q, s_m[pad16(t * kPer + i)]);
+    }
+  }
+  const double t1 = diag_sum(a1, s), t2 = diag_sum(a2, s), tr = diag_sum(ar, s);
+  if (t == 0) {
     tile_s1[blockIdx.x] = t1;
     tile_s2[blockIdx.x] = t2;
     tile_sr[blockIdx.x] = tr;
-    tile_n[blockIdx.x] = tn;
+    tile_n[blockIdx.x] = (double)count;
   }
 }
+constexpr size_t kDiagSmem = sizeof(double) * 2 * (kPad16N + 8);
 
 // per cluster: rho_c = sum rho^2 / sum rho, r_c = sum rho r / sum rho and the
 // number of estimates (3 doubles per cluster)
@@ -1080,21 +1206,45 @@ __global__ void __launch_bounds__(kThreads) k_energy_final(Seg S, const double* 
   }
 }
 
+// The first star whose enclosed mass reaches each fraction: a warp per search.  A
+// round takes five halvings: lane l (1 to 31) probes node l of the tree of the
+// next five midpoints, the answers pick the path (same midpoints and result as
+// one halving at a time, which took 13.7 us at 10^6 stars; 8.0).
 __global__ void k_lagrange(Seg S, const double* r, const double* M, const double* fracs,
                            int nf, double* out) {
   pdl_enter();
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
   if (i >= S.n_seg * nf) return;
-  int c = i / nf, q = i % nf;
-  int64_t sb = S.off[c], nbc = S.nb[c];
-  if (nbc <= 0) { out[i] = 0.0; return; }
-  double target = fracs[q] * M[sb + nbc - 1];
+  const int c = i / nf, q = i % nf;
+  const int64_t sb = S.off[c], nbc = S.nb[c];
+  if (nbc <= 0) {
+    if (lane == 0) out[i] = 0.0;
+    return;
+  }
+  const double target = fracs[q] * M[sb + nbc - 1];
   int64_t lo = -1, hi = nbc - 1;  // first k with M_k >= target (M[nb-1] qualifies)
   while (hi - lo > 1) {
-    int64_t mid = lo + ((hi - lo) >> 1);
-    if (M[sb + mid] >= target) hi = mid; else lo = mid;
+    int64_t a = lo, b = hi;
+    for (int bit = 30 - __clz(lane | 1); bit >= 0; --bit) {
+      if (b - a <= 1) break;
+      const int64_t mid = a + ((b - a) >> 1);
+      if ((lane >> bit) & 1) b = mid; else a = mid;
+    }
+    const bool ge = lane > 0 && b - a > 1 && M[sb + a + ((b - a) >> 1)] >= target;
+    const unsigned pick = __ballot_sync(0xFFFFFFFFu, ge);
+    for (int node = 1; node < 32 && hi - lo > 1;) {
+      const int64_t mid = lo + ((hi - lo) >> 1);
+      if ((pick >> node) & 1u) {
+        hi = mid;
+        node = 2 * node + 1;
+      } else {
+        lo = mid;
+        node = 2 * node;
+      }
+    }
   }
-  out[i] = r[sb + hi];
+  if (lane == 0) out[i] = r[sb + hi];
 }
 
 __global__ void k_validate(int64_t n, const double* r, const double* vr, const double* vt,
@@ -1456,31 +1606,46 @@ void launch_velocities(const SegLayout& L, const uint32_t* order, const RecB* rb
            L.dev(), L.esc_step, L.n, order, rb, phi, m, vr, vt);
 }
 
-constexpr size_t potential_smem(bool tables) {
-  return sizeof(double) * (tables ? 2 : 3) * kPad8N;
+constexpr size_t kPotentialSmem = sizeof(double) * 2 * kPad8N;
+
+template <int kKind>
+void tile_sums_prepare() {
+  cudaFuncSetAttribute(k_tile_sums<kKind>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)(sizeof(double) * kTile * 2));
+}
+
+void diag_prepare() {
+  cudaFuncSetAttribute(k_energy_tiles<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)kDiagSmem);
+  cudaFuncSetAttribute(k_energy_tiles<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)kDiagSmem);
+  cudaFuncSetAttribute(k_core_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDiagSmem);
 }
 
 void potential_prepare() {
   cudaFuncSetAttribute(k_potential<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)potential_smem(false));
+                       (int)kPotentialSmem);
   cudaFuncSetAttribute(k_potential<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)potential_smem(true));
+                       (int)kPotentialSmem);
+  tile_sums_prepare<kSumsOfX>();
+  tile_sums_prepare<kSumsRecip>();
 }
 
 
 void launch_potential(const SegLayout& L, const double* r, const double* x, const double* m,
                       double* tile_m, double* tile_mx, double* phi, double* Mout, bool nb_sub,
                       cudaStream_t st, bool sums_ready, double4_32a* node,
-                      const TableOut* tables) {
+                      const TableOut* tables, double* recip) {
   if (!L.n_tiles) return;
   Seg S = L.dev();
-  if (!sums_ready)
-    launch_k(k_tile_sums, (unsigned)L.n_tiles, kThreads, 0, st, S, L.esc_step, nb_sub, x, m,
-             tile_m, tile_mx);
+  if (recip)
+    launch_tile_sums<kSumsRecip>(L, nb_sub, r, m, tile_m, tile_mx, recip, st);
+  else if (!sums_ready)
+    launch_tile_sums<kSumsOfX>(L, nb_sub, x, m, tile_m, tile_mx, nullptr, st);
   int lp = 0;
   while (lp < kPotParts && L.n_tiles << (lp + 1) <= kPotBlocks) ++lp;
   launch_k(tables ? k_potential<true> : k_potential<false>, (unsigned)(L.n_tiles << lp),
-           kPotThreads, potential_smem(tables != nullptr), st, S, L.esc_step, nb_sub, r, x, m, tile_m, tile_mx, phi, Mout, node,
+           kPotThreads, kPotentialSmem, st, S, L.esc_step, nb_sub, r, x, m, tile_m, tile_mx, phi, Mout, node,
            tables ? *tables : TableOut(), lp);
 }
 
@@ -1496,14 +1661,22 @@ void launch_correction(const SegLayout& L, const double* r, const double* x,
 
 void launch_energy(const SegLayout& L, const double* r, const double* vr, const double* vt,
                    const double* m, double* tile_m, double* tile_k, double* tile_w,
-                   double* Mbuf, double* out3, cudaStream_t st) {
+                   double* out3, cudaStream_t st) {
   if (!L.n_tiles) return;
   Seg S = L.dev();
-  launch_k(k_tile_sums, (unsigned)L.n_tiles, kThreads, 0, st, S, L.esc_step, false, r, m, tile_m,
-                                                       tile_k);
-  launch_k(k_energy_tiles, (unsigned)L.n_tiles, kThreads, 0, st, S, r, vr, vt, m, tile_m, tile_k,
-                                                          tile_w, Mbuf);
+  launch_tile_sums<kSumsMass>(L, false, nullptr, m, tile_m, nullptr, nullptr, st);
+  launch_k(k_energy_tiles<false>, (unsigned)L.n_tiles, kDiagThreads, kDiagSmem, st, S, r, vr, vt, m,
+           tile_m, tile_k, tile_w, nullptr);
   launch_k(k_energy_final, (unsigned)L.n_seg, kThreads, 0, st, S, tile_k, tile_w, out3);
+}
+
+void launch_masses(const SegLayout& L, const double* m, double* tile_m, double* Mout,
+                   cudaStream_t st) {
+  if (!L.n_tiles) return;
+  Seg S = L.dev();
+  launch_tile_sums<kSumsMass>(L, false, nullptr, m, tile_m, nullptr, nullptr, st);
+  launch_k(k_energy_tiles<true>, (unsigned)L.n_tiles, kDiagThreads, kDiagSmem, st, S, nullptr,
+           nullptr, nullptr, m, tile_m, nullptr, nullptr, Mout);
 }
 
 void launch_diag_ring(const SegLayout& L, const double* out3, const uint32_t* step,
@@ -1518,8 +1691,8 @@ void launch_core(const SegLayout& L, const double* r, const double* m, double* t
   if (!L.n_tiles) return;
   Seg S = L.dev();
   const int64_t t = L.n_tiles;
-  launch_k(k_core_tiles, (unsigned)t, kThreads, 0, st, S, r, m, tiles4, tiles4 + t, tiles4 + 2 * t,
-                                                  tiles4 + 3 * t);
+  launch_k(k_core_tiles, (unsigned)t, kDiagThreads, kDiagSmem, st, S, r, m, tiles4, tiles4 + t,
+           tiles4 + 2 * t, tiles4 + 3 * t);
   launch_k(k_core_final, (unsigned)L.n_seg, kThreads, 0, st, S, tiles4, tiles4 + t, tiles4 + 2 * t,
                                                        tiles4 + 3 * t, out3);
 }
@@ -1527,7 +1700,7 @@ void launch_core(const SegLayout& L, const double* r, const double* m, double* t
 void launch_lagrange(const SegLayout& L, const double* r, const double* M,
                      const double* fracs, int nf, double* out, cudaStream_t st) {
   int n = L.n_seg * nf;
-  if (n) launch_k(k_lagrange, blocks_for(n, 128), 128, 0, st, L.dev(), r, M, fracs, nf, out);
+  if (n) launch_k(k_lagrange, blocks_for(n, 4), 128, 0, st, L.dev(), r, M, fracs, nf, out);
 }
 
 void launch_validate(const SegLayout& L, const double* r, const double* vr,
