@@ -1135,11 +1135,12 @@ __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
 // pending star and leave at once.
 // one pending star (p = n: an idle lane); counts go to the statistics
 // kExact (FP64 mode): F = 1.2 Fx, the points and g as FP64 mode's
-template <bool kTaus, bool kExact>
+template <bool kTaus, bool kExact, bool kAhead>
 __device__ __forceinline__ void pending_star(Seg S, int max_trials, const uint32_t* id,
                                              const uint32_t* step_p, BucketArgs BA,
                                              const double4_32a* orb, uint64_t* keys, int64_t p,
-                                             int64_t n, const double* Fx) {
+                                             int64_t n, const double* Fx, int lanes_each) {
+  const int G = kAhead ? lanes_each : 1;
   unsigned long long viol = 0;
   unsigned int n64 = 0;
   int c = -1;
@@ -1171,30 +1172,49 @@ __device__ __forceinline__ void pending_star(Seg S, int max_trials, const uint32
         // stream mode: the blocks of trials 0 .. t-1 were the FP32 sampler's
         Draws<kTaus> g = draws_of<kTaus>(S, c, id[p], *step_p);
         g.skip((uint32_t)t);
-        for (; t < max_trials; ++t) {
-          const U4 w = g.block(kTagRej, (uint32_t)t);
-          const double sv = sym_double(sym_int(w.x, w.y));
-          const int guess =
-              shell32_of(BA.node + sb, (int)nbc, BK, c0f, c1f, 2.0f * u01f(w.y) - 1.0f);
-          double g64v;
-          if (kExact) {
-            double rs, ph, Q, L, xq;
-            int i;
-            point64_div(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, ph, Q, L, xq, i);
-            g64v = g_of_point(c1, sv, Q);
-          } else {
-            double rs, xs, ph, L, Q;
-            int i;
-            point64(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, xs, ph, L, Q, i);
-            g64v = pos_num(Q) ? div_rn((3.0 * c1) * (1.0 - sv * sv), sqrt_rn(Q)) : 0.0;
+        // G lanes take G trials at a time; the first accepted one counts, as do
+        // the trials up to it
+        const int lane = threadIdx.x & 31, sub = lane & (G - 1);
+        const unsigned group = (G == 32 ? 0u : 1u << G) - 1u, at = lane - sub;
+        for (; t < max_trials; t += G) {
+          const int mine = t + sub;
+          bool over = false, take = false;
+          if (mine < max_trials) {
+            const U4 w = g.block(kTagRej, (uint32_t)mine);
+            const double sv = sym_double(sym_int(w.x, w.y));
+            const int guess =
+                shell32_of(BA.node + sb, (int)nbc, BK, c0f, c1f, 2.0f * u01f(w.y) - 1.0f);
+            double g64v;
+            if (kExact) {
+              double rs, ph, Q, L, xq;
+              int i;
+              point64_div(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, ph, Q, L, xq, i);
+              g64v = g_of_point(c1, sv, Q);
+            } else {
+              double rs, xs, ph, L, Q;
+              int i;
+              point64(BA.node + sb, nbc, s, c0, c1, sv, guess, rs, xs, ph, L, Q, i);
+              g64v = pos_num(Q) ? div_rn((3.0 * c1) * (1.0 - sv * sv), sqrt_rn(Q)) : 0.0;
+            }
+            over = g64v > F;
+            take = F * u01(w.z, w.w) < g64v;
           }
-          ++n64;
-          if (g64v > F) ++viol;
-          if (F * u01(w.z, w.w) < g64v) { st = kSmpAccepted; break; }
+          const unsigned acc = kAhead ? (__ballot_sync(group << at, take) >> at) & group : take;
+          const int last = acc ? __ffs(acc) - 1 : G - 1;
+          if (mine < max_trials && sub <= last) {
+            ++n64;
+            viol += over;
+          }
+          if (acc) {
+            st = kSmpAccepted;
+            t += last;
+            break;
+          }
         }
         if (t >= max_trials) t = max_trials;
-        keys[p] = (res & 0xFFFFFFFF00000000ull) | ((uint64_t)st << 30) |
-                  (uint64_t)(t & 0x3FFFFFFF);
+        if (sub == 0)
+          keys[p] = (res & 0xFFFFFFFF00000000ull) | ((uint64_t)st << 30) |
+                    (uint64_t)(t & 0x3FFFFFFF);
       }
     }
   }
@@ -1208,7 +1228,7 @@ __device__ __forceinline__ void pending_star(Seg S, int max_trials, const uint32
   }
 }
 
-constexpr uint32_t kPendingWarps = 4 * 152;
+constexpr uint32_t kPendingWarps = 16 * 152;
 
 template <bool kTaus, bool kExact>
 __global__ void __launch_bounds__(128) k_pending64(Seg S, int max_trials, const uint32_t* id,
@@ -1219,19 +1239,32 @@ __global__ void __launch_bounds__(128) k_pending64(Seg S, int max_trials, const 
                                                    const double* Fx) {
   pdl_enter();
   const uint32_t np = *pcount;
-  // A short list goes over more warps, `lanes` stars to each: a warp's walks and
-  // trials last as long as its slowest star's, and FP64 instructions of up to
-  // four warps per SM run side by side (the orbit stage of 10^3, 10^4, 10^5 stars
-  // 44.0, 58.1, 56.0 us with full warps, 42.2, 56.5, 53.5 this way, 42.5, 57.2,
-  // 54.9 with one warp per SM, 42.9, 56.6, 53.7 with sixteen).
+  // A short list goes over more warps, `lanes` stars to each (a warp's walks and
+  // trials last as long as its slowest star's), and the lanes left over take
+  // trials ahead, which costs no instructions: the orbit stage of 10^3, 10^4 (FP64
+  // mode), 10^5, 10^6 stars 42.2, 56.1, 52.7, 165.7 us with one lane a star over four
+  // warps per SM, 26.1, 46.3, 37.9, 166.5 with trials ahead, 26.5, 46.3, 35.5, 149.8
+  // over sixteen warps per SM (eight: 25.8, 46.3, 35.5, 158.6; 32: 26.4, 45.6, 36.3,
+  // 148.7); full warps 44.0, 58.1, 56.0.
   const uint32_t warps = gridDim.x * (blockDim.x / 32), lane = threadIdx.x & 31;
   uint32_t lanes = (np + kPendingWarps - 1) / kPendingWarps;
   lanes = lanes < 32u ? lanes : 32u;
   if (lanes * warps < np) lanes = 32u;
+  // ... and the lanes left over take trials ahead
+  const int G = kTaus || lanes > 16u ? 1
+                : lanes > 8u             ? 2
+                : lanes > 4u             ? 4
+                : lanes > 2u             ? 8
+                : lanes > 1u             ? 16
+                                         : 32;
+  const uint32_t slot = lane / G;
   for (uint32_t w = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; w * lanes < np; w += warps) {
-    const uint32_t i = w * lanes + lane;
-    pending_star<kTaus, kExact>(S, max_trials, id, step_p, BA, orb, keys,
-                                lane < lanes && i < np ? (int64_t)plist[i] : n, n, Fx);
+    const uint32_t i = w * lanes + slot;
+    const int64_t p = slot < lanes && i < np ? (int64_t)plist[i] : n;
+    if (!kTaus && G > 1)
+      pending_star<kTaus, kExact, true>(S, max_trials, id, step_p, BA, orb, keys, p, n, Fx, G);
+    else
+      pending_star<kTaus, kExact, false>(S, max_trials, id, step_p, BA, orb, keys, p, n, Fx, 1);
   }
 }
 
