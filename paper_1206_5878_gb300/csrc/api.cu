@@ -776,6 +776,7 @@ cmc_status cmc_init(cmc_ctx** out, const cmc_config* cfg_in, int32_t n_clusters,
   CMC_ALLOC(c->err, 1);
   CMC_ALLOC(c->step, 1);
   CMC_ALLOC(c->pcount, 1);
+  if (!e) e = cudaMemsetAsync(c->pcount, 0, sizeof(uint32_t), st);
   if (cfg.collisions) {
     CMC_ALLOC(c->R, n);
     CMC_ALLOC(c->Rp, n);
@@ -1351,6 +1352,7 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
   Carve C;
   C.put(dstep, &step, 1);
   C.zero(mm, n);
+  if (tab) C.zero(pcnt, 1);
   C.add(x, n);
   C.add(keys, n);
   C.add(ra, n);
@@ -1362,7 +1364,6 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
     C.add(tmax, n);
     C.add(orb, n);
     C.add(plist, n);
-    C.add(pcnt, 1);
   }
   cudaError_t e = C.alloc(block, st);
   if (!e) {

@@ -411,7 +411,8 @@ void launch_potential_tables(const SegLayout& L, const double* r, const double* 
 // FP32 sampler, FP64 continuation of the pending stars, finishing) and
 // needs n records orb (E, J, c0 = (r_max + r_min) / 2, c1 = (r_max -
 // r_min) / 4, from the turning-point kernel, for the sampling kernels), a
-// list of n uint32 (the pending stars) and one uint32 counter; tp_min,
+// list of n uint32 (the pending stars) and one uint32 counter, zero before
+// and after (as EnvWork's); tp_min,
 // tp_max (n doubles each: the turning points) only with the stage outputs
 // of dbg (rmin, rmax).
 // precision 0 (FP64): the same kernels with FP64 mode's envelope (two more

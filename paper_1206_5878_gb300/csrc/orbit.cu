@@ -894,20 +894,25 @@ __device__ __forceinline__ bool env_star(const Seg& S, const double4_32a* orb, i
   return lt0(E) && gt_pos(c1, 0.0);
 }
 
+// kG > 1 (few stars, as k_sample32): kG lanes a star share the samples.  FP64 mode's
+// orbit stage of 10^3, 10^4, 3 x 10^4 stars 43.0, 45.4, 47.9 us with a lane a star here,
+// 33.9, 34.3, 40.3 so (2 to 3 us of it two fills less).
+template <int kG>
 __global__ void __launch_bounds__(kEnvThreads) k_env_screen(Seg S, BucketArgs BA,
                                                             const double4_32a* orb, EnvWork W,
                                                             int64_t n) {
   pdl_enter();
   __shared__ float s_hi[21][kEnvThreads];  // upper bounds of the samples
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
+  const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kG;
+  const int lane = threadIdx.x & 31, sub = lane & (kG - 1);
+  const unsigned group = ((kG == 32 ? 0u : 1u << kG) - 1u) << (lane - sub);
   int c = -1;
   unsigned cand = 0u;
   if (p < n) {
     double E, J, c0, c1;
     if (env_star(S, orb, p, c, E, J, c0, c1)) {
       // the star's values for the evaluation of its pairs
-      W.star[p] = make_double4_32a(E, J, c0, c1);
+      if (sub == 0) W.star[p] = make_double4_32a(E, J, c0, c1);
       const float c0f = f32_rn(c0), c1f = f32_rn(c1), E32 = f32_rn(E), J32 = f32_rn(J);
       const Grid GD = grid_of(BA, c);
       unsigned pos = 0u;
@@ -915,7 +920,7 @@ __global__ void __launch_bounds__(kEnvThreads) k_env_screen(Seg S, BucketArgs BA
       // one copy of the sample code (not unrolled: code size), the upper
       // bounds kept in shared memory
 #pragma unroll 1
-      for (int jj = 0; jj < 21; ++jj) {
+      for (int jj = sub; jj < 21; jj += kG) {
         float g = 0.0f, eg = 0.0f;
         const int st = g32_bounded(GD, E32, J32, c0f, c1f, c_s32[jj], g, eg);
         float h = 0.0f;
@@ -929,11 +934,17 @@ __global__ void __launch_bounds__(kEnvThreads) k_env_screen(Seg S, BucketArgs BA
         }
         s_hi[jj][threadIdx.x] = h;
       }
+      // (bits of floats >= 0 order like them)
+      if (kG > 1) lo_max = __uint_as_float(__reduce_max_sync(group, __float_as_uint(lo_max)));
 #pragma unroll 1
-      for (int jj = 0; jj < 21; ++jj)
+      for (int jj = sub; jj < 21; jj += kG)
         if (((pos >> jj) & 1u) && s_hi[jj][threadIdx.x] >= lo_max) cand |= 1u << jj;
+      if (kG > 1) {
+        cand = __reduce_or_sync(group, cand);
+        if (sub != 0) cand = 0u;  // the star's pairs are its first lane's
+      }
     }
-    W.gmax[p] = 0.0;
+    if (sub == 0) W.gmax[p] = 0.0;
   }
   // the warp's pairs go to the list in lane order, with one atomic
   const unsigned cnt = (unsigned)__popc(cand);
@@ -1053,7 +1064,13 @@ enum : uint32_t { kSmpAccepted = 0, kSmpPending = 1, kSmpDegenerate = 2, kSmpCap
 // kExact (FP64 mode): F is FP64 mode's envelope, 1.2 Fx (Fx from k_env_eval),
 // and a trial is decided here only where the FP64 decision and violation
 // count are certain.
-template <int kMinB, bool kTaus, bool kExact>
+// kG > 1 (few stars, chip idle): kG lanes a star share the envelope's samples and
+// take kG trials at a time, the first one that is accepted or undecided counts.
+// Orbit stage of 10^3, 10^4, 3 x 10^4, 6 x 10^4 stars 24.9, 29.1, 30.8, 32.9 us with a
+// lane, 22.4, 23.8, 26.7, 32.9 with four, 20.4, 22.8, 28.6, 36.3 with eight.
+constexpr int64_t kSample8 = 16384, kSample4 = 49152;
+
+template <int kMinB, bool kTaus, bool kExact, int kG>
 __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
                                                   const uint32_t* id,
                                                   const uint32_t* step_p, BucketArgs BA,
@@ -1061,7 +1078,10 @@ __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
                                                   uint64_t* keys, uint32_t* plist,
                                                   uint32_t* pcount, int64_t n, const double* Fx) {
   pdl_enter();
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kG;
+  // (kG > 1: the star's lanes)
+  const int lane = threadIdx.x & 31, sub = lane & (kG - 1), at = lane - sub;
+  const unsigned group = (kG == 32 ? 0u : 1u << kG) - 1u;
   unsigned long long viol = 0;
   bool pend = false;
   int c = -1;  // lanes past the end form their own group below
@@ -1084,10 +1104,13 @@ __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
       } else {
         float gmax = 0.0f;
 #pragma unroll 3
-        for (int j = 0; j < 21; ++j) {
+        for (int j = sub; j < 21; j += kG) {
           const float g = g32_grid(GD, E32, J32, c0f, c1f, c_sa32[j], c_sb32[j]);
           gmax = g > gmax ? g : gmax;
         }
+        // (bits of floats >= 0 order like them)
+        if (kG > 1)
+          gmax = __uint_as_float(__reduce_max_sync(group << at, __float_as_uint(gmax)));
         F32 = 1.2f * gmax;
         degenerate = !gt_pos(c1, 0.0) || !(F32 > 0.0f);
       }
@@ -1097,24 +1120,43 @@ __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
         st = kSmpDegenerate;
       } else {
         Draws<kTaus> g = draws_of<kTaus>(S, c, id[p], *step_p);
-        for (; t < max_trials; ++t) {
-          const U4 w = g.block(kTagRej, (uint32_t)t);
-          const int d = accept32<kExact>(GD, E32, J32, c0f, c1f, F32, 2.0f * u01f(w.y) - 1.0f,
-                                 u01f(w.w), viol);
-          if (d == 0) continue;
-          st = d > 0 ? kSmpAccepted : kSmpPending;
-          break;
+        for (; t < max_trials; t += kG) {
+          const int mine = t + sub;
+          unsigned long long over = 0;
+          int d = 0;
+          if (kG == 1 || mine < max_trials) {
+            const U4 w = g.block(kTagRej, (uint32_t)mine);
+            d = accept32<kExact>(GD, E32, J32, c0f, c1f, F32, 2.0f * u01f(w.y) - 1.0f, u01f(w.w),
+                                 over);
+          }
+          if (kG == 1) {
+            viol += over;
+            if (d == 0) continue;
+            st = d > 0 ? kSmpAccepted : kSmpPending;
+            break;
+          }
+          const unsigned acc = (__ballot_sync(group << at, d > 0) >> at) & group;
+          const unsigned any = acc | ((__ballot_sync(group << at, d < 0) >> at) & group);
+          const int last = any ? __ffs(any) - 1 : kG - 1;
+          if (sub <= last) viol += over;
+          if (any) {
+            st = (acc >> last) & 1u ? kSmpAccepted : kSmpPending;
+            t += last;
+            break;
+          }
         }
+        if (kG > 1 && t > max_trials) t = max_trials;
       }
-      keys[p] = ((uint64_t)__float_as_uint(F32) << 32) | ((uint64_t)st << 30) |
-                (uint64_t)(t & 0x3FFFFFFF);
-      pend = st == kSmpPending;
+      if (sub == 0) {
+        keys[p] = ((uint64_t)__float_as_uint(F32) << 32) | ((uint64_t)st << 30) |
+                  (uint64_t)(t & 0x3FFFFFFF);
+        pend = st == kSmpPending;
+      }
     }
   }
   // pending stars onto the list of k_pending64 (one atomic per warp)
   const unsigned pm = __ballot_sync(__activemask(), pend);
   if (pm) {
-    const int lane = threadIdx.x & 31;
     uint32_t base = 0;
     if (lane == __ffs(pm) - 1) base = atomicAdd(pcount, (uint32_t)__popc(pm));
     base = __shfl_sync(__activemask(), base, __ffs(pm) - 1);
@@ -1312,8 +1354,15 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
                                                const double4_32a* orb,
                                                int64_t n, const double* Rv, double* Rp,
                                                const double* Fx, const double* Av,
-                                               double* Ap, BinOut bo) {
+                                               double* Ap, BinOut bo, uint32_t* pcount,
+                                               unsigned long long* ecount) {
   pdl_enter();
+  // the lists' counters, read by the kernels before this one, zero for the next
+  // orbit step (two fills less between its kernels)
+  if (kPrec != 0 && blockIdx.x == 0 && threadIdx.x == 0) {
+    *pcount = 0u;
+    if (kPrec == 2) ecount[0] = ecount[1] = 0ull;
+  }
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const int c = seg_find(S.off, S.n_seg, p);
@@ -1805,11 +1854,11 @@ cudaError_t alloc_env(EnvWork& W, int64_t n, cudaStream_t st) {
   const int64_t m = n > 0 ? n : 1;
   W.cap = 2 * m + 1024;  // the pairs: 1.1 per star measured on Plummer models
   Carve C;
+  C.zero(W.cnt, 2);
   C.add(W.gmax, (size_t)m);
   C.add(W.star, (size_t)m);
   C.add(W.list, (size_t)W.cap);
   C.add(W.spill, (size_t)m);
-  C.add(W.cnt, 2);
   cudaError_t e = C.alloc(W.block, st);
   if (!e) {
     launch_k(k_env_tables, 1, 32, 0, st);
@@ -1872,19 +1921,26 @@ void launch_orbit(const SegLayout& L, int precision, int max_trials, const doubl
 #define CMC_ORBIT(P, B, T)                                                                  \
   launch_k(k_orbit<P, B, T>, grid, block, 0, st, L.dev(), max_trials, r, x, phi, vr, vt, \
            m, id, step, keys, ra, rb, L.esc_step, d, ba, tp_min, tp_max, orb, L.n, Rv, Rp, Fx, \
-           Av, Ap, bo)
+           Av, Ap, bo, pcount, W.cnt)
 #define CMC_SAMPLED(B, T, X)                                                                \
   do {                                                                                      \
     if (with_turning) CMC_TURN(B);                                                          \
     if (X) {                                                                                \
-      cudaMemsetAsync(W.cnt, 0, 2 * sizeof(unsigned long long), st);                        \
-      launch_k(k_env_screen, (unsigned)((L.n + kEnvThreads - 1) / kEnvThreads), kEnvThreads, 0, st,  \
-          L.dev(), ba, orb, W, L.n);                                                         \
+      const int g = L.n <= kSample8 ? 8 : L.n <= kSample4 ? 4 : 1;                          \
+      launch_k(g == 8   ? k_env_screen<8>                                                   \
+               : g == 4 ? k_env_screen<4>                                                   \
+                        : k_env_screen<1>,                                                  \
+               (unsigned)((L.n * g + kEnvThreads - 1) / kEnvThreads), kEnvThreads, 0, st,   \
+               L.dev(), ba, orb, W, L.n);                                                   \
       launch_k(k_env_eval, egrid, kEnvThreads, 0, st, L.dev(), ba, W);                             \
     }                                                                                       \
-    cudaMemsetAsync(pcount, 0, sizeof(uint32_t), st);                                      \
-    launch_k(k_sample32<B, T, X>, grid, block, 0, st, L.dev(), max_trials, id, step, ba, orb, keys, \
-                                                plist, pcount, L.n, Fx);                    \
+    const int ahead = T ? 1 : L.n <= kSample8 ? 8 : L.n <= kSample4 ? 4 : 1;                 \
+    launch_k(ahead == 8   ? k_sample32<4, false, X, 8>                                      \
+             : ahead == 4 ? k_sample32<4, false, X, 4>                                      \
+                          : k_sample32<B, T, X, 1>,                                         \
+             ahead > 1 ? (unsigned)((L.n * ahead + 127) / 128) : grid,                      \
+             ahead > 1 ? 128 : block, 0, st, L.dev(), max_trials, id, step, ba, orb, keys,  \
+             plist, pcount, L.n, Fx);                                                       \
     launch_k(k_pending64<T, X>, pgrid, 128, 0, st, L.dev(), max_trials, id, step, ba, orb, keys,  \
                                              plist, pcount, L.n, Fx);                       \
     CMC_ORBIT(X ? 2 : 1, 5, T);                                                             \
