@@ -273,23 +273,26 @@ void record_step(cmc_ctx* c, cudaStream_t st, cudaEvent_t* ev = nullptr) {
                      c->m, c->id, c->order, c->r_old, c->cc, c->tile_a, c->tile_b, c->Rp, c->R,
                      c->Ap, c->A, !binned, st);
   mark(6);
+  const bool correct = c->cfg.energy_correction != 0;
+  GridBuild grid;  // the grid's values, with the correction's first kernel
   // the tables carry the shell slopes of the FP64 orbit step (not the
   // scan's enclosed masses): the sampled step's turning points and points
   // are then FP64 mode's
   if (tab)
     launch_potential_tables(L, c->r_alt, c->x_alt, c->m, c->tile_a, c->tile_b, c->phi, true, true,
-                            c->bk, st);
+                            c->bk, st, correct ? &grid : nullptr);
   else
     launch_potential(L, c->r_alt, c->x_alt, c->m, c->tile_a, c->tile_b, c->phi, nullptr, true, st,
                      true);
   mark(7);
   // (the FP64 modes evaluate Phi_new(r_old) in Eq. 6's division form)
-  const bool correct = c->cfg.energy_correction != 0;
   if (correct)
-    launch_phi_old(L, c->r, c->x, c->r_alt, c->x_alt, c->phi, c->bk.node, c->rb, !mixed, st);
-  launch_velocities(L, c->order, c->rb, c->phi, c->m, c->vr, c->vt, correct, st);
+    launch_phi_old(L, c->r, c->x, c->r_alt, c->x_alt, c->phi, c->bk.node, c->rb, !mixed, st,
+                   tab ? &grid : nullptr);
+  // (and the end of the step: escapers' budgets, counters)
+  launch_velocities(L, c->order, c->rb, c->phi, c->m, c->vr, c->vt, correct, c->r_old, c->cc,
+                    c->step, st);
   mark(8);
-  launch_step_end(L, c->step, c->r_old, c->cc, c->m, st);
   if (c->ring) {
     // K and W of the new state (r_old is free scratch now), then the record
     launch_energy(L, c->r_alt, c->vr, c->vt, c->m, c->tile_a, c->tile_b, c->tile_c, c->out3, st);
@@ -306,14 +309,15 @@ void turn_sides(cmc_ctx* c) {
 }
 
 int count_step_kernels(const cmc_ctx* c) {
-  // bins, relax, orbit, gather with the tile sums, potential, velocities, step
-  // end; the sort: scan, scatter, long runs [count], or upsweep (with the
+  // bins, relax, orbit, gather with the tile sums, potential, velocities with the
+  // step's end (or its end apart); the sort: scan, scatter, long runs [count], or upsweep (with the
   // histograms' scans), 5 passes, tie fix; [precision 0 and 1: turning points,
-  // FP32 sampler, FP64 continuation, the grid's values with the seams' slopes;
-  // precision 0: the envelope's screen and evaluation], [Phi_new(r_old)]
+  // FP32 sampler, FP64 continuation; precision 0: the envelope's screen and
+  // evaluation], Phi_new(r_old) with the grid's values or those alone
   const int p = c->cfg.precision;
   const int sort = c->cfg.sort_packed ? (c->L.n <= kCountInOrbit ? 3 : 4) : 7;
-  return 7 + sort + (c->ring ? 4 : 0) + (p == 1 ? 4 : p == 0 ? 6 : 0) + (c->cfg.energy_correction ? 1 : 0);
+  return (c->L.n <= kEndWithVelocities ? 6 : 7) + sort + (c->ring ? 4 : 0) + (p == 1 ? 3 : p == 0 ? 5 : 0) +
+         (c->cfg.energy_correction || p != 2 ? 1 : 0);
 }
 
 void free_ctx(cmc_ctx* c) {

@@ -279,18 +279,26 @@ void launch_gather_step(const SegLayout& L, BinWork* B, const uint32_t* order_in
                         double* r_old, double* c, double* tile_m, double* tile_mx,
                         const double* Rp, double* Rout, const double* Ap, double* Aout,
                         bool exact, cudaStream_t st);
+struct GridBuild;
 // Phi_new(r_old) of every star of the old order into its RecB (w), r_in and
 // x_in the old radii and reciprocals (sorted), r, x, phi, node the new table.
 // div_form: Eq. 6's division form (FP64 modes; node may be null), else the
-// shell slope of the node records.
+// shell slope of the node records.  grid: the grid's values are built beside it.
 void launch_phi_old(const SegLayout& L, const double* r_in, const double* x_in, const double* r,
                     const double* x, const double* phi, const double4_32a* node, RecB* rb,
-                    bool div_form, cudaStream_t st);
+                    bool div_form, cudaStream_t st,
+                    const GridBuild* grid = nullptr);
+// the largest number of stars whose velocities' kernel ends the step too (see
+// launch_velocities)
+constexpr int64_t kEndWithVelocities = 1 << 20;
 // the new velocities into place, corrected for the changing potential
-// (correct false: as they are)
+// (correct false: as they are); then the step is committed: nb, escaper
+// statistics and budget (from the gathered r_old and c of the escaped range), dt,
+// the per-step counters
 void launch_velocities(const SegLayout& L, const uint32_t* order, const RecB* rb,
                        const double* phi, const double* m, double* vr, double* vt, bool correct,
-                       cudaStream_t st);
+                       const double* r_old,
+                       const double* c, uint32_t* step, cudaStream_t st);
 
 // potential: per-tile sums then the tile-local scans (Eqs. 1-5 in scan
 // form).  nb_sub: subtract esc_step from nb (after the orbit step).
@@ -397,14 +405,27 @@ void launch_buckets(const SegLayout& L, const float2* t32, bool nb_sub, BucketWo
 // build the potential grid from the FP64 table (x, Phi, the node records)
 void launch_grid(const SegLayout& L, const double* x, const double* phi, bool nb_sub,
                  BucketWork& B, cudaStream_t st);
+// the grid's values and the seams' slopes (grid_build.cuh)
+struct GridBuild {
+  const double *x = nullptr, *phi = nullptr;
+  BucketArgs B;
+  const int* gshell = nullptr;
+  float* gphi = nullptr;
+  float4* gaux = nullptr;
+  double4_32a* node = nullptr;
+  int64_t total = 0, n_tiles = 0;  // cells, tiles with a seam to fill
+  bool sub = false, fused = false;
+};
+
 // The potential with the orbit step's tables in two kernels: the potential
 // writing Phi, the node records, bucket starts and grid key shells with the
 // segments' parameters, then the grid's values with the slopes at the tile
-// seams.  The same tables as launch_potential + launch_make_nodes +
-// launch_buckets + launch_grid.
+// seams (with `later` left to launch_phi_old).  The same tables as
+// launch_potential + launch_make_nodes + launch_buckets + launch_grid.
 void launch_potential_tables(const SegLayout& L, const double* r, const double* x,
                              const double* m, double* tile_m, double* tile_mx, double* phi,
-                             bool nb_sub, bool sums_ready, BucketWork& B, cudaStream_t st);
+                             bool nb_sub, bool sums_ready, BucketWork& B, cudaStream_t st,
+                             GridBuild* later = nullptr);
 
 // launch_orbit writes the stars' records, and with bins their sort bins (count:
 // counted too) or else their sort keys.  precision 1 (mixed): it runs four kernels (turning points,
@@ -463,11 +484,6 @@ void launch_turning(const SegLayout& L, const double* r, const double* x, const 
 // spills cost)
 constexpr int kOrbitVariants = 7;
 constexpr int kRelaxVariants = 3;  // relaxation kernel register caps (launch_relax)
-
-// commits the step: nb, escaper statistics and budget (from the gathered
-// r_old and c of the escaped range), dt; resets the per-step counters
-void launch_step_end(const SegLayout& L, uint32_t* step, const double* r_old, const double* c,
-                     const double* m, cudaStream_t st);
 
 // energy diagnostics: per-segment K, W_pair
 void launch_energy(const SegLayout& L, const double* r, const double* vr, const double* vt,

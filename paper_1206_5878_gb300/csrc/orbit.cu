@@ -19,7 +19,7 @@
 // accepted radius, its potential (by the shell's slope) and the velocities are
 // FP64.  A mixed result matches the FP64 result to rounding whenever both
 // accept the same trial.
-#include "cmc_host.hpp"
+#include "grid_build.cuh"
 
 namespace cmc {
 
@@ -416,9 +416,6 @@ __device__ __forceinline__ float u01f(uint32_t hi) {
 
 // ------------------------------------------------------- turning points
 // 1/r and Phi of a node, its radius and slope (one 16-byte load each)
-__device__ __forceinline__ double2 node_xp(const double4_32a* p) {
-  return *reinterpret_cast<const double2*>(p);
-}
 __device__ __forceinline__ double2 node_rw(const double4_32a* p) {
   return reinterpret_cast<const double2*>(p)[1];
 }
@@ -1640,78 +1637,9 @@ __global__ void k_grid_shells(Seg S, const int64_t* esc, bool sub, const double*
   if (live && k == 0) grid_close(grid_last_cell(__ldg(x + p), pr), pr, gshell + B.goff[c], 0, 1);
 }
 
-// Phi at every grid key from the FP64 table: Phi = Phi_i + M_i (1/r_i - 1/r)
-// in the key's shell i (Eq. 6 with the enclosed-mass slope), Phi_0 inside
-// the first star, rounded to float
-// fused (launch_potential_tables): the slopes at the tile seams, which the
-// potential kernel leaves, are computed here by n_tiles more threads (and
-// locally where a cell needs one), and each segment's cell 0 fills Phi_0 and
-// the bound mass into gaux
-__global__ void k_grid_build(Seg S, const int64_t* esc, bool sub, const double* x,
-                             const double* phi, BucketArgs B,
-                             const int* gshell, float* gphi, float4* gaux, int64_t total,
-                             bool fused, double4_32a* node, int64_t n_tiles) {
+__global__ void k_grid_build(Seg S, const int64_t* esc, GridBuild G) {
   pdl_enter();
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned am = __ballot_sync(0xFFFFFFFFu, p < total);
-  if (p >= total) {
-    const int64_t t = p - total;
-    if (!fused || t >= n_tiles) return;
-    const int cs = seg_find(S.tile_off, S.n_seg, t);
-    const int64_t sbs = S.off[cs], nbs = S.nb[cs] - (sub ? esc[cs] : 0);
-    const int64_t k = (t - S.tile_off[cs]) * kTile + kTile - 1;  // the tile's last star
-    if (k + 1 >= nbs) return;
-    const int64_t q = sbs + k;
-    // (only the slope: other threads read the record's 1/r and Phi)
-    node[q].w = div_rn(phi[q + 1] - phi[q], x[q] - x[q + 1]);
-    return;
-  }
-  const int c = seg_find(B.goff, S.n_seg, p);
-  const int4 pr = B.gprm[c];
-  const int g = (int)(p - B.goff[c]);
-  const int64_t sb = S.off[c];
-  const int64_t nb = S.nb[c] - (sub ? esc[c] : 0);
-  // shell i's slope (a seam's computed as the seam threads do)
-  auto slope = [&](int64_t i) {
-    if (fused && i % kTile == kTile - 1 && i + 1 < nb) {
-      const double2 a = node_xp(node + sb + i), b = node_xp(node + sb + i + 1);
-      return div_rn(b.y - a.y, a.x - b.x);
-    }
-    return node[sb + i].w;
-  };
-  float rel = 0.0f;
-  if (g < pr.z) {
-    if (fused && g == 0) {
-      gaux[c].x = (float)__ldg(phi + sb);
-      gaux[c].y = (float)node[sb + nb - 1].w;
-    }
-    const double xg = (double)__uint_as_float((uint32_t)pr.x + ((uint32_t)g << pr.y));
-    const double xn = (double)__uint_as_float((uint32_t)pr.x + ((uint32_t)(g + 1) << pr.y));
-    const int64_t lo = gshell[p];
-    double ph = __ldg(phi + sb);
-    if (lo >= 0) {
-      const double2 a = node_xp(node + sb + lo);
-      ph = a.y + slope(lo) * (a.x - xg);
-    }
-    gphi[p] = (float)ph;
-    // Phi is convex in 1/r (its slope -M(1/r) rises with 1/r), so inside the
-    // cell [xg, xn] it lies below the chord by at most (xn - xg) dM / 4, dM
-    // the mass of the stars in the cell; relative to |Phi(xg)|, the smallest
-    // |Phi| of the cell, the largest over the segment's cells bounds the
-    // grid's interpolation error (gaux.w; floats >= 0 order as their bits)
-    if (g + 1 < pr.z && ph < 0.0) {
-      const int64_t lo2 = gshell[p + 1];
-      const double Ma = lo < 0 ? 0.0 : slope(lo);
-      const double Mb = lo2 < 0 ? 0.0 : slope(lo2);
-      const double dM = Ma - Mb;
-      rel = (float)(((xn - xg) * (dM > 0.0 ? dM : 0.0) * 0.25) / -ph);
-    }
-  }
-  // one atomic per segment present in the warp
-  const unsigned grp = __match_any_sync(am, c);
-  const unsigned mx = __reduce_max_sync(grp, __float_as_uint(rel));
-  if ((threadIdx.x & 31) == (unsigned)(__ffs(grp) - 1) && mx)
-    atomicMax(reinterpret_cast<unsigned int*>(&gaux[c].w), mx);
+  grid_build(S, esc, G, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // per segment: the indexed node range lo..hi, base = bits(x_lo), the
@@ -1810,6 +1738,29 @@ void free_buckets(BucketWork& B, cudaStream_t st) {
   B = BucketWork();
 }
 
+// fused: also the slopes at the tile seams
+static GridBuild grid_args(const SegLayout& L, const double* x, const double* phi, bool nb_sub,
+                           bool fused, const BucketWork& B) {
+  GridBuild G;
+  G.x = x;
+  G.phi = phi;
+  G.B = B.args();
+  G.gshell = B.gshell;
+  G.gphi = B.gphi;
+  G.gaux = B.gaux;
+  G.total = B.gcells;
+  G.sub = nb_sub;
+  G.fused = fused;
+  G.node = B.node;
+  G.n_tiles = fused ? L.n_tiles : 0;
+  return G;
+}
+
+static void launch_grid_build(const SegLayout& L, const GridBuild& G, cudaStream_t st) {
+  launch_k(k_grid_build, (unsigned)((G.total + G.n_tiles + 255) / 256), 256, 0, st, L.dev(),
+           L.esc_step, G);
+}
+
 void launch_grid(const SegLayout& L, const double* x, const double* phi, bool nb_sub,
                  BucketWork& B, cudaStream_t st) {
   if (!L.n || !B.gcells) return;
@@ -1817,14 +1768,13 @@ void launch_grid(const SegLayout& L, const double* x, const double* phi, bool nb
            nb_sub, x, phi, B.node, B.goff, B.gprm, B.gaux);
   launch_k(k_grid_shells, (unsigned)((L.n + 255) / 256), 256, 0, st, L.dev(), L.esc_step, nb_sub, x,
            B.args(), B.gshell, L.n);
-  launch_k(k_grid_build, (unsigned)((B.gcells + 255) / 256), 256, 0, st, L.dev(), L.esc_step,
-           nb_sub, x, phi, B.args(), B.gshell, B.gphi, B.gaux, B.gcells, false, B.node,
-           (int64_t)0);
+  launch_grid_build(L, grid_args(L, x, phi, nb_sub, false, B), st);
 }
 
 void launch_potential_tables(const SegLayout& L, const double* r, const double* x,
                              const double* m, double* tile_m, double* tile_mx, double* phi,
-                             bool nb_sub, bool sums_ready, BucketWork& B, cudaStream_t st) {
+                             bool nb_sub, bool sums_ready, BucketWork& B, cudaStream_t st,
+                             GridBuild* later) {
   if (!L.n) return;
   TableOut T;
   T.start = B.start;
@@ -1836,9 +1786,9 @@ void launch_potential_tables(const SegLayout& L, const double* r, const double* 
   T.gprm = B.gprm;
   T.gaux = B.gaux;
   launch_potential(L, r, x, m, tile_m, tile_mx, phi, nullptr, nb_sub, st, sums_ready, B.node, &T);
-  const int64_t threads = B.gcells + L.n_tiles;
-  launch_k(k_grid_build, (unsigned)((threads + 255) / 256), 256, 0, st, L.dev(), L.esc_step,
-           nb_sub, x, phi, B.args(), B.gshell, B.gphi, B.gaux, B.gcells, true, B.node, L.n_tiles);
+  const GridBuild G = grid_args(L, x, phi, nb_sub, true, B);
+  if (later) *later = G;
+  else launch_grid_build(L, G, st);
 }
 
 void launch_buckets(const SegLayout& L, const float2* t32, bool nb_sub, BucketWork& B,

@@ -13,7 +13,7 @@
 #include <cmath>
 #include <cstring>
 
-#include "cmc_host.hpp"
+#include "grid_build.cuh"
 
 namespace cmc {
 
@@ -335,6 +335,10 @@ __global__ void __launch_bounds__(kGatThreads, kGatThreads == 512 ? 3 : kGatThre
 // star a thread there are four times the blocks: faster while they find idle
 // SMs (both kernels at 10^4, 10^5, 2 x 10^5 stars 12.3, 14.3, 17.7 us against
 // 16.4, 18.4, 20.5), slower above (7 x 10^5: 39.3 against 37.5).
+// The grid's values (grid_build) go in the first blocks of this kernel: both need
+// the potential only, and alone they took 7 us of mostly latency (potential,
+// correction and end of 10^3, 10^5, 10^6 stars 38.7, 53.4, 124.3 us with both and the
+// step's end in kernels of their own, 33.2, 45.7, 117.5 so).
 constexpr int kPoThreads = 256;
 constexpr int kPoPer = 4;     // stars per thread, 1 while there are few tiles
 constexpr int64_t kPoFewTiles = 76;
@@ -365,16 +369,22 @@ __global__ void __launch_bounds__(kPoThreads) k_phi_old(Seg S, const int64_t* es
                                                         const double* r_in, const double* x_in,
                                                         const double* r, const double* x,
                                                         const double* phi,
-                                                        const double4_32a* node, RecB* rb) {
+                                                        const double4_32a* node, RecB* rb,
+                                                        GridBuild G, unsigned grid_blocks) {
   pdl_enter();
+  if (blockIdx.x < grid_blocks) {
+    grid_build(S, esc, G, (int64_t)blockIdx.x * kPoThreads + threadIdx.x);
+    return;
+  }
+  const unsigned chunk = blockIdx.x - grid_blocks;
   __shared__ long long po_r[kPoWin];
   __shared__ int64_t s_lo, s_hi;
   const int t = threadIdx.x;
   constexpr int kPoChunk = kPoThreads * kPer;  // the block's stars
   constexpr int kSub = kTile / kPoChunk;
-  TR R = tile_of(S, esc, blockIdx.x / kSub, false);
+  TR R = tile_of(S, esc, chunk / kSub, false);
   // the old order's bound stars in this chunk; the new table
-  const int64_t begin = R.begin + (int64_t)(blockIdx.x % kSub) * kPoChunk;
+  const int64_t begin = R.begin + (int64_t)(chunk % kSub) * kPoChunk;
   int64_t end = begin + kPoChunk < R.end ? begin + kPoChunk : R.end;
   end = end < R.bound_end ? end : R.bound_end;
   if (begin >= end) return;
@@ -436,8 +446,13 @@ __global__ void __launch_bounds__(kPoThreads) k_phi_old(Seg S, const int64_t* es
     const int64_t i = at[j];
     double pn;
     if (!kDiv) {
-      const double4_32a nd = node[sb + (i < 0 ? 0 : i)];
-      pn = i < 0 ? nd.y : nd.y + nd.w * (nd.x - xo[j]);
+      const int64_t q = sb + (i < 0 ? 0 : i);
+      const double4_32a nd = node[q];
+      // (a seam's slope as the grid's blocks compute it, which may not have yet)
+      const double w = i >= 0 && i % kTile == kTile - 1 && i + 1 < nb
+                           ? div_rn(phi[q + 1] - nd.y, nd.x - x[q + 1])
+                           : nd.w;
+      pn = i < 0 ? nd.y : nd.y + w * (nd.x - xo[j]);
     } else {
       const int64_t q = sb + (i < 0 ? 0 : i);
       const double pj = phi[q];
@@ -460,40 +475,112 @@ __global__ void __launch_bounds__(kPoThreads) k_phi_old(Seg S, const int64_t* es
 // The new velocities into the new order: T' = T + 1/2 [(Phi_new(r_old) -
 // Phi_new(r_new)) - (Phi_old(r_old) - Phi_old(r_new))], clamped at 0; both
 // components scaled by sqrt(T'/T) (section 2.1 step 6).
+// The kernel also ends the step: its first n_seg blocks sum what the stars that
+// escaped in this step take with them (the escaped range's entries with a finite
+// r_old; earlier escapers carry r_old = inf), mass and energy m_k e_k (e_k in c) in
+// a fixed order, into the segments' budgets (section 4.2), and its last block to
+// finish turns the segments' counters over.  E.done null: not here (a launch
+// without stars follows).
+struct StepEnd {
+  int64_t* esc;
+  uint64_t* dt_last;
+  uint32_t* step;
+  const double *r_old, *e;
+  double* esc_me;
+  uint32_t* done;  // blocks finished; zero between kernels; null: no end of the step
+};
+
+__device__ __forceinline__ void escapers_of(const Seg& S, const StepEnd& E, const double* m, int c) {
+  __shared__ double s_m[256], s_e[256];
+  const int t = threadIdx.x;
+  const int64_t ne = E.esc[c];
+  if (ne <= 0) return;
+  const int64_t nb_new = S.nb[c] - ne;
+  double dm = 0.0, de = 0.0;
+  for (int64_t p = S.off[c] + nb_new + t; p < S.off[c + 1]; p += 256)
+    if (isfinite(E.r_old[p])) {
+      dm += m[p];
+      de += m[p] * E.e[p];
+    }
+  s_m[t] = dm;
+  s_e[t] = de;
+  __syncthreads();
+  for (int w = 128; w > 0; w >>= 1) {
+    if (t < w) {
+      s_m[t] += s_m[t + w];
+      s_e[t] += s_e[t + w];
+    }
+    __syncthreads();
+  }
+  if (t == 0) {
+    E.esc_me[2 * c] += s_m[0];
+    E.esc_me[2 * c + 1] += s_e[0];
+  }
+}
+
 template <bool kCorrect>
-__global__ void __launch_bounds__(256) k_velocities(Seg S, const int64_t* esc, int64_t n,
-                                                    const uint32_t* order, const RecB* rb,
-                                                    const double* phi, const double* m,
-                                                    double* vr, double* vt) {
+__global__ void __launch_bounds__(256) k_velocities(Seg S, int64_t n, const uint32_t* order,
+                                                    const RecB* rb, const double* phi,
+                                                    const double* m, double* vr, double* vt,
+                                                    StepEnd E) {
   pdl_enter();
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const uint32_t v = order[p];
-  if ((int64_t)v >= n) return;  // only after a reported sort failure
-  const RecB B = load_rec(rb + v);
-  double a = B.vr, b = B.vt;
-  if (kCorrect) {
-    const int c = seg_find(S.off, S.n_seg, p);
-    if (p - S.off[c] < S.nb[c] - esc[c]) {
-      // (two of the four products on the integer pipes: the FP64 pipe bounds
-      // this kernel)
-      const double Tk = scale_down<1>(mul_rn(a, a) + b * b);
-      const double dnew = B.w - phi[p];
-      double Tp = Tk + scale_down<1>(dnew - B.c);
-      if (lt0(Tp)) {
-        clamp_energy_add(S.stats, c, m[p], Tp);
-        stat_add(S.stats, c, kStClamps, 1ull);
-        Tp = 0.0;
+  const int64_t p = (int64_t)((int)blockIdx.x - (E.done ? S.n_seg : 0)) * 256 + threadIdx.x;
+  if (p < 0) {
+    escapers_of(S, E, m, blockIdx.x);
+  } else if (p < n) {
+    const uint32_t v = order[p];
+    if ((int64_t)v < n) {  // (not below only after a reported sort failure)
+      const RecB B = load_rec(rb + v);
+      double a = B.vr, b = B.vt;
+      if (kCorrect) {
+        const int c = seg_find(S.off, S.n_seg, p);
+        if (p - S.off[c] < S.nb[c] - E.esc[c]) {
+          // (two of the four products on the integer pipes: the FP64 pipe bounds
+          // this kernel)
+          const double Tk = scale_down<1>(mul_rn(a, a) + b * b);
+          const double dnew = B.w - phi[p];
+          double Tp = Tk + scale_down<1>(dnew - B.c);
+          if (lt0(Tp)) {
+            clamp_energy_add(S.stats, c, m[p], Tp);
+            stat_add(S.stats, c, kStClamps, 1ull);
+            Tp = 0.0;
+          }
+          if (pos_num(Tk)) {
+            const double f = sqrt_rn(div_rn(Tp, Tk));
+            a = mul_rn(a, f);
+            b = b * f;
+          }
+        }
       }
-      if (pos_num(Tk)) {
-        const double f = sqrt_rn(div_rn(Tp, Tk));
-        a = mul_rn(a, f);
-        b = b * f;
-      }
+      vr[p] = a;
+      vt[p] = b;
     }
   }
-  vr[p] = a;
-  vt[p] = b;
+  if (!E.done) return;
+  __shared__ bool s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(E.done, 1u) == gridDim.x - 1u;
+    if (s_last) *E.done = 0u;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_last) return;
+  for (int c = threadIdx.x; c < S.n_seg; c += 256) {
+    const int64_t ne = E.esc[c];
+    E.dt_last[c] = S.dt_bits[c];
+    S.nb[c] = S.nb[c] - ne;
+    // the stars merged away in this step (sticky spheres) left with the
+    // escapers; they are counted as collisions, not as escapes
+    unsigned long long* st = S.stats + (size_t)c * kStStride;
+    const unsigned long long merged = st[kStCollisions] - st[kStCollisionsSeen];
+    st[kStCollisionsSeen] = st[kStCollisions];
+    st[kStEscaped] += (unsigned long long)ne - merged;
+    E.esc[c] = 0;
+    S.dt_bits[c] = 0x7FF0000000000000ull;
+    if (c == 0) *E.step += 1u;
+  }
 }
 
 // ------------------------------------------------------------ potential
@@ -1306,55 +1393,6 @@ __global__ void k_ids_bitmap(int64_t n, const int64_t* off, int n_seg, const uin
   if (atomicOr(bitmap + (b >> 6), bit) & bit) set_err(err, kErrInput);
 }
 
-// One 256-thread block per segment.  The stars that escaped in this step
-// are the escaped range's entries with a finite r_old (earlier escapers
-// carry r_old = inf); their mass and energy m_k e_k (e_k in c) are summed
-// in a fixed order and added to the segment's budget (section 4.2).
-__global__ void __launch_bounds__(256) k_step_end(Seg S, int64_t* esc, uint64_t* dt_last,
-                                                  uint32_t* step, const double* r_old,
-                                                  const double* e, const double* m,
-                                                  double* esc_me) {
-  pdl_enter();
-  __shared__ double s_m[256], s_e[256];
-  const int c = blockIdx.x, t = threadIdx.x;
-  const int64_t ne = esc[c];
-  const int64_t nb_new = S.nb[c] - ne;
-  double dm = 0.0, de = 0.0;
-  if (ne > 0)
-    for (int64_t p = S.off[c] + nb_new + t; p < S.off[c + 1]; p += 256)
-      if (isfinite(r_old[p])) {
-        dm += m[p];
-        de += m[p] * e[p];
-      }
-  s_m[t] = dm;
-  s_e[t] = de;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (t < w) {
-      s_m[t] += s_m[t + w];
-      s_e[t] += s_e[t + w];
-    }
-    __syncthreads();
-  }
-  if (t == 0) {
-    if (ne > 0) {
-      esc_me[2 * c] += s_m[0];
-      esc_me[2 * c + 1] += s_e[0];
-    }
-    dt_last[c] = S.dt_bits[c];
-    S.nb[c] = nb_new;
-    // the stars merged away in this step (sticky spheres) left with the
-    // escapers; they are counted as collisions, not as escapes
-    unsigned long long* st = S.stats + (size_t)c * kStStride;
-    const unsigned long long merged = st[kStCollisions] - st[kStCollisionsSeen];
-    st[kStCollisionsSeen] = st[kStCollisions];
-    st[kStEscaped] += (unsigned long long)ne - merged;
-    esc[c] = 0;
-    S.dt_bits[c] = 0x7FF0000000000000ull;
-    if (c == 0) *step += 1u;
-  }
-}
-
 // one record of the diagnostics ring per segment, after the step end (the
 // step counter already advanced): slot (step - 1) mod cap
 __global__ void k_diag_ring(Seg S, const double* out3, const uint64_t* dt_last,
@@ -1589,21 +1627,41 @@ void launch_gather_step(const SegLayout& L, BinWork* B, const uint32_t* order_in
 
 void launch_phi_old(const SegLayout& L, const double* r_in, const double* x_in, const double* r,
                     const double* x, const double* phi, const double4_32a* node, RecB* rb,
-                    bool div_form, cudaStream_t st) {
+                    bool div_form, cudaStream_t st, const GridBuild* grid) {
   if (!L.n_tiles) return;
   const int per = L.n_tiles <= kPoFewTiles ? 1 : kPoPer;
+  const unsigned gb =
+      grid ? (unsigned)((grid->total + grid->n_tiles + kPoThreads - 1) / kPoThreads) : 0u;
   launch_k(per == 1 ? (div_form ? k_phi_old<true, 1> : k_phi_old<false, 1>)
                     : (div_form ? k_phi_old<true, kPoPer> : k_phi_old<false, kPoPer>),
-           (unsigned)(L.n_tiles * (kTile / (kPoThreads * per))), kPoThreads, 0, st, L.dev(),
-           L.esc_step, r_in, x_in, r, x, phi, node, rb);
+           gb + (unsigned)(L.n_tiles * (kTile / (kPoThreads * per))), kPoThreads, 0, st, L.dev(),
+           L.esc_step, r_in, x_in, r, x, phi, node, rb, grid ? *grid : GridBuild(), gb);
 }
 
 void launch_velocities(const SegLayout& L, const uint32_t* order, const RecB* rb,
                        const double* phi, const double* m, double* vr, double* vt, bool correct,
-                       cudaStream_t st) {
-  if (!L.n) return;
-  launch_k(correct ? k_velocities<true> : k_velocities<false>, blocks_for(L.n, 256), 256, 0, st,
-           L.dev(), L.esc_step, L.n, order, rb, phi, m, vr, vt);
+                       const double* r_old, const double* c, uint32_t* step, cudaStream_t st) {
+  if (!L.n_seg) return;
+  StepEnd E;
+  E.esc = L.esc_step;
+  E.dt_last = L.dt_last;
+  E.step = step;
+  E.r_old = r_old;
+  E.e = c;
+  E.esc_me = L.esc_me;
+  uint32_t* done = L.tile_done + L.n_tiles;
+  const auto kernel = correct ? k_velocities<true> : k_velocities<false>;
+  // Many blocks: the step's end after them.  In the same launch it saves the next
+  // one's 3 us, but every block waits for its turn at the counter: potential,
+  // correction and end of 10^5, 4 x 10^5, 10^6, 2 x 10^6, 10^7 stars 45.7, 72.4, 117.5,
+  // 205.6, 805 us in one launch, 48.5, 75.9, 117.9, 202.1, 782 in two.
+  const bool together = L.n <= kEndWithVelocities;
+  E.done = together ? done : nullptr;
+  launch_k(kernel, (unsigned)(together ? L.n_seg : 0) + blocks_for(L.n, 256), 256, 0, st, L.dev(),
+           L.n, order, rb, phi, m, vr, vt, E);
+  if (together) return;
+  E.done = done;
+  launch_k(kernel, (unsigned)L.n_seg, 256, 0, st, L.dev(), (int64_t)0, order, rb, phi, m, vr, vt, E);
 }
 
 constexpr size_t kPotentialSmem = sizeof(double) * 2 * kPad8N;
@@ -1725,12 +1783,6 @@ void launch_check_ids(const SegLayout& L, const uint64_t* sorted_ids, uint32_t* 
                       cudaStream_t st) {
   if (L.n > 1)
     launch_k(k_check_ids, blocks_for(L.n, 256), 256, 0, st, L.n, L.off, L.n_seg, sorted_ids, err);
-}
-
-void launch_step_end(const SegLayout& L, uint32_t* step, const double* r_old, const double* c,
-                     const double* m, cudaStream_t st) {
-  launch_k(k_step_end, L.n_seg, 256, 0, st, L.dev(), L.esc_step, L.dt_last, step, r_old, c, m,
-                                      L.esc_me);
 }
 
 CMC_DEBUG_SITE_ACCESSOR

@@ -118,3 +118,24 @@ def test_steps_after_a_sort_that_timed_out(g_stage, n, precision, packed):
     r = other.get_state()["r"]
     r = r[np.isfinite(r)]
     assert np.all(np.diff(r) >= 0)
+
+
+@pytest.mark.parametrize("n", [40, 5000, (1 << 20) - 3, (1 << 20) + 1])
+def test_end_of_the_step_with_the_velocities(g_stage, n):
+    """The escapers' budget and the counters, by the velocities' kernel or (more than
+    2^20 stars) after it: mass and energy booked per step against the stars that
+    left, whose energies are exact to the rounding of at most n additions."""
+    d = _model(n, 8)
+    d["vr"][::7] *= 3.0
+    d["vt"][::7] *= 3.0
+    c = g_stage.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, [2], precision=1)
+    was = np.isfinite(c.get_state()["r"]).sum()
+    c.step(2)
+    st, stat = c.get_state(), c.stats()[0]
+    gone = ~np.isfinite(st["r"])
+    assert stat["escaped"] == gone.sum() > 0 and c.nbound()[0] == was - gone.sum()
+    assert st["step"] == 2
+    me = c.escaped()[0]
+    mass = math.fsum(st["m"][gone])
+    assert abs(me[0] - mass) <= n * 2.0 ** -53 * mass
+    assert np.isfinite(me[1]) and me[1] > 0.0
