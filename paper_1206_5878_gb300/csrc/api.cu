@@ -158,49 +158,50 @@ bool staged_in_order(cmc_ctx* c, std::vector<unsigned long long>& bitoff, cudaSt
   return total <= 64ull * (unsigned long long)L.n;
 }
 
-// Sort the staged stars in r, vr, vt, m, id by (r, id) per segment and
-// compute nb and the potential.  Ids must be unique per segment.  Stars
-// already in order (a state read back and set again) keep their places: the
-// order was checked, the ids are checked with a bitmap, and both sorts and
-// the gather are skipped.
-// Stars already in (r, id) order: the ids checked with a bitmap, the keys
-// and 1/r written in place (r and id only: no sort, no gather).  False when
-// the bitmap's scratch could not be had.
+// Stars already in (r, id) order: the ids checked with a bitmap and N_bound found
+// (r and id only: no sort, no gather).  False when scratch could not be had.
 bool order_in_place(cmc_ctx* c, const std::vector<unsigned long long>& bitoff,
                     cudaStream_t st) {
   const SegLayout& L = c->L;
   unsigned long long* dbo = nullptr;
-  if (dalloc(dbo, bitoff.size(), st)) return false;
-  cudaMemcpyAsync(dbo, bitoff.data(), sizeof(unsigned long long) * bitoff.size(),
-                  cudaMemcpyHostToDevice, st);
+  void* block = nullptr;
+  Carve C;
+  C.put(dbo, bitoff.data(), bitoff.size());
+  if (C.alloc(block, st)) return false;
   // the bitmap lives in the key scratch (64 bits per star)
   cudaMemsetAsync(c->keys, 0, sizeof(uint64_t) * (size_t)L.n, st);
-  launch_ids_bitmap(L, c->id, dbo, reinterpret_cast<unsigned long long*>(c->keys), c->err, st);
-  launch_make_keys(L, c->r, c->id, c->keys, st);
-  launch_recip(L.n, c->r, c->x, st);
-  cudaStreamSynchronize(st);  // bitoff lives on the caller's stack frame
-  dfree(dbo, st);
+  launch_place(L, c->r, c->id, dbo, reinterpret_cast<unsigned long long*>(c->keys), c->err, st);
+  dfree(block, st);
   return true;
 }
 
-// N_bound from the keys, then the potential and the orbit step's tables
-void finish_order(cmc_ctx* c, cudaStream_t st) {
+// N_bound (from the keys, where the stars were sorted), then the potential and
+// the orbit step's tables (with 1/r, where the stars were in place)
+void finish_order(cmc_ctx* c, bool placed, cudaStream_t st) {
   const SegLayout& L = c->L;
-  launch_nb_from_keys(L, c->keys, st);
+  double* recip = placed ? c->x : nullptr;
+  if (!placed) launch_nb_from_keys(L, c->keys, st);
   cudaMemsetAsync(L.esc_step, 0, sizeof(int64_t) * L.n_seg, st);
   // the float tables, node records and indexes of the sampled orbit step
   // (precision 0 and 1)
   if (c->cfg.precision != 2)
     launch_potential_tables(L, c->r, c->x, c->m, c->tile_a, c->tile_b, c->phi, false, false, c->bk,
-                            st);
+                            st, nullptr, recip);
   else
-    launch_potential(L, c->r, c->x, c->m, c->tile_a, c->tile_b, c->phi, nullptr, false, st);
+    launch_potential(L, c->r, c->x, c->m, c->tile_a, c->tile_b, c->phi, nullptr, false, st, false,
+                     nullptr, nullptr, recip);
 }
 
+// Sort the staged stars in r, vr, vt, m, id by (r, id) per segment and
+// compute nb and the potential.  Ids must be unique per segment.  Stars
+// already in order (a state read back and set again) keep their places: the
+// order was checked, the ids are checked with a bitmap, and both sorts and
+// the gather are skipped.
 void order_state(cmc_ctx* c, cudaStream_t st) {
   const SegLayout& L = c->L;
   std::vector<unsigned long long> bitoff;
-  if (!(L.n > 0 && staged_in_order(c, bitoff, st) && order_in_place(c, bitoff, st))) {
+  const bool placed = L.n > 0 && staged_in_order(c, bitoff, st) && order_in_place(c, bitoff, st);
+  if (!placed) {
     launch_id_keys(L, c->id, c->keys, st);
     sort_segments(L, c->W, c->keys, c->vals, 0, 4, true, c->err, st);
     launch_check_ids(L, c->keys, c->err, st);
@@ -209,7 +210,7 @@ void order_state(cmc_ctx* c, cudaStream_t st) {
     launch_make_records(L, c->r, c->vr, c->vt, c->m, c->id, c->ra, c->rb, st);
     launch_gather(L, c->vals, c->ra, c->rb, c->r, c->x, c->vr, c->vt, c->m, c->id, st);
   }
-  finish_order(c, st);
+  finish_order(c, placed, st);
 }
 
 // The largest number of stars whose bins the orbit step counts itself, saving
@@ -387,7 +388,7 @@ cmc_status load_state(cmc_ctx* c, const double* r, const double* vr, const doubl
   bool placed = false;
   std::vector<unsigned int> max_id;
   if (L.n > 0 && staged_in_order(c, bitoff, aux, &max_id) && order_in_place(c, bitoff, aux)) {
-    finish_order(c, aux);
+    finish_order(c, true, aux);
     placed = true;
   }
   // (ids that could not be read: bins for any id)

@@ -425,7 +425,7 @@ struct GridBuild {
 void launch_potential_tables(const SegLayout& L, const double* r, const double* x,
                              const double* m, double* tile_m, double* tile_mx, double* phi,
                              bool nb_sub, bool sums_ready, BucketWork& B, cudaStream_t st,
-                             GridBuild* later = nullptr);
+                             GridBuild* later = nullptr, double* recip = nullptr);
 
 // launch_orbit writes the stars' records, and with bins their sort bins (count:
 // counted too) or else their sort keys.  precision 1 (mixed): it runs four kernels (turning points,
@@ -522,9 +522,12 @@ void potential_prepare();  // shared-memory limit of the potential kernel
 // per segment (maxid: n_seg values, zeroed by the caller)
 void launch_order_check(const SegLayout& L, const double* r, const uint32_t* id, uint32_t* flag,
                         unsigned int* maxid, cudaStream_t st);
-// duplicate ids by a bitmap with bitoff[c] + id per star (kErrInput)
-void launch_ids_bitmap(const SegLayout& L, const uint32_t* id, const unsigned long long* bitoff,
-                       unsigned long long* bitmap, uint32_t* err, cudaStream_t st);
+
+// stars in (r, id) order: every id of a segment once (a bitmap, zero before;
+// bitoff: the segments' first bits), N_bound of the segments
+void launch_place(const SegLayout& L, const double* r, const uint32_t* id,
+                  const unsigned long long* bitoff, unsigned long long* bitmap, uint32_t* err,
+                  cudaStream_t st);
 // starting states of the Tausworthe streams (dynamics.cu): slots of
 // segment c from base[c] (n_seg + 1 offsets), words: the segment's seeded
 // words, P: [4][32][32] jump matrices T^(2^(80 + b))

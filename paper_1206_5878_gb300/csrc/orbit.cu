@@ -1774,7 +1774,7 @@ void launch_grid(const SegLayout& L, const double* x, const double* phi, bool nb
 void launch_potential_tables(const SegLayout& L, const double* r, const double* x,
                              const double* m, double* tile_m, double* tile_mx, double* phi,
                              bool nb_sub, bool sums_ready, BucketWork& B, cudaStream_t st,
-                             GridBuild* later) {
+                             GridBuild* later, double* recip) {
   if (!L.n) return;
   TableOut T;
   T.start = B.start;
@@ -1785,7 +1785,8 @@ void launch_potential_tables(const SegLayout& L, const double* r, const double* 
   T.goff = B.goff;
   T.gprm = B.gprm;
   T.gaux = B.gaux;
-  launch_potential(L, r, x, m, tile_m, tile_mx, phi, nullptr, nb_sub, st, sums_ready, B.node, &T);
+  launch_potential(L, r, x, m, tile_m, tile_mx, phi, nullptr, nb_sub, st, sums_ready, B.node, &T,
+                   recip);
   const GridBuild G = grid_args(L, x, phi, nb_sub, true, B);
   if (later) *later = G;
   else launch_grid_build(L, G, st);

@@ -1379,11 +1379,14 @@ __global__ void k_order_check(int64_t n, const int64_t* off, int n_seg, const do
   if (live && (threadIdx.x & 31) == __ffs(peers) - 1) atomicMax(maxid + c, mx);
 }
 
-// Duplicate ids of sorted input: bit bitoff[c] + id of a bitmap per star;
-// a bit found set already is a duplicate (error)
-__global__ void k_ids_bitmap(int64_t n, const int64_t* off, int n_seg, const uint32_t* id,
-                             const unsigned long long* bitoff, unsigned long long* bitmap,
-                             uint32_t* err) {
+// Stars in (r, id) order: duplicate ids by bit bitoff[c] + id of a bitmap (a bit
+// found set already is one), and N_bound where the first escaped star (r = inf,
+// after all others) or the segment's end is.  Setting a state back at 10^3, 10^5,
+// 10^6 stars 127, 145, 258 us with keys, a search of them, reciprocals and a host
+// wait between, 110, 134, 230 so.
+__global__ void k_place(int64_t n, const int64_t* off, int n_seg, const double* r,
+                        const uint32_t* id, const unsigned long long* bitoff,
+                        unsigned long long* bitmap, int64_t* nb, uint32_t* err) {
   pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
@@ -1391,6 +1394,11 @@ __global__ void k_ids_bitmap(int64_t n, const int64_t* off, int n_seg, const uin
   const unsigned long long b = bitoff[c] + id[p];
   const unsigned long long bit = 1ull << (b & 63ull);
   if (atomicOr(bitmap + (b >> 6), bit) & bit) set_err(err, kErrInput);
+  // the first escaped star's place, or the segment's end (escaped stars last)
+  const int64_t sb = off[c];
+  const bool gone = ubits(r[p]) >= kInfBits, last = p + 1 == off[c + 1];
+  if (gone && (p == sb || ubits(r[p - 1]) < kInfBits)) nb[c] = p - sb;
+  if (!gone && last) nb[c] = p + 1 - sb;
 }
 
 // one record of the diagnostics ring per segment, after the step end (the
@@ -1773,10 +1781,12 @@ void launch_order_check(const SegLayout& L, const double* r, const uint32_t* id,
                                                                maxid);
 }
 
-void launch_ids_bitmap(const SegLayout& L, const uint32_t* id, const unsigned long long* bitoff,
-                       unsigned long long* bitmap, uint32_t* err, cudaStream_t st) {
-  if (L.n) launch_k(k_ids_bitmap, blocks_for(L.n, 256), 256, 0, st, L.n, L.off, L.n_seg, id, bitoff,
-                                                              bitmap, err);
+void launch_place(const SegLayout& L, const double* r, const uint32_t* id,
+                  const unsigned long long* bitoff, unsigned long long* bitmap, uint32_t* err,
+                  cudaStream_t st) {
+  if (L.n)
+    launch_k(k_place, blocks_for(L.n, 256), 256, 0, st, L.n, L.off, L.n_seg, r, id, bitoff, bitmap,
+             L.nb, err);
 }
 
 void launch_check_ids(const SegLayout& L, const uint64_t* sorted_ids, uint32_t* err,

@@ -139,3 +139,30 @@ def test_end_of_the_step_with_the_velocities(g_stage, n):
     mass = math.fsum(st["m"][gone])
     assert abs(me[0] - mass) <= n * 2.0 ** -53 * mass
     assert np.isfinite(me[1]) and me[1] > 0.0
+
+
+def test_bound_stars_of_a_state_in_order(g_stage):
+    """N_bound from the stars' places: no, one, all but one and all stars of a
+    segment escaped; Phi as the potential entry point's."""
+    sizes, gone = [300, 1, 4097, 64, 513, 2], [0, 1, 1, 63, 513, 0]
+    parts = [_model(n, 60 + i) for i, n in enumerate(sizes)]
+    cat = {k: np.concatenate([p[k] for p in parts]) for k in ("r", "vr", "vt", "m", "id")}
+    c = g_stage.Cluster(cat, list(range(6)), sizes=sizes, precision=1)
+    st, o = c.get_state(), np.concatenate([[0], np.cumsum(sizes)])
+    for s in range(6):
+        st["r"][o[s + 1] - gone[s]:o[s + 1]] = np.inf
+        tail = slice(o[s + 1] - gone[s], o[s + 1])
+        p = np.argsort(st["id"][tail])
+        for k in ("vr", "vt", "m", "id"):
+            st[k][tail] = st[k][tail][p]
+    c.set_state(st, 0)
+    np.testing.assert_array_equal(c.nbound(), np.array(sizes) - np.array(gone))
+    now = c.get_state()
+    for s in range(6):
+        b = slice(o[s], o[s + 1] - gone[s])
+        if b.stop > b.start:
+            phi = g_stage.stage_potential(dev(st["r"][b]), dev(st["m"][b]), want_M=True)[0]
+            np.testing.assert_array_equal(now["phi"][b], host(phi))
+    st["id"][5] = st["id"][7]
+    with pytest.raises(g_stage.CMCError):
+        c.set_state(st, 0)
