@@ -293,13 +293,26 @@ struct Collide {
   const double* phi = nullptr;
 };
 
-template <bool kTaus, int kMinB, bool kCol>
+//
+// kTwo (few pairs, counter draws): two lanes a pair.  Each draws one of the two
+// angles, takes one of each two roots that do not depend on each other, and
+// finishes one of the stars: the stage of 10^3, 10^4, 3 x 10^4 stars 16.3, 17.4, 17.9 us
+// with a lane a pair, 14.5, 14.9, 16.9 with two; 22.4 and 28.9 at 10^5, where the
+// FP64 pipe has work enough.
+constexpr int64_t kTwoLanes = 16384;
+
+template <bool kTaus, int kMinB, bool kCol, bool kTwo>
 __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr, double* vt,
                                                double* m, const uint32_t* id,
                                                const double* nbin, const uint32_t* step_p,
                                                Collide col) {
   pdl_enter();
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / (kTwo ? 2 : 1);
+  const bool second = kTwo && (threadIdx.x & 1u);  // the pair's second lane
+  const unsigned both = 3u << (threadIdx.x & 30u);
+  auto of = [&](int l, double v) {  // lane l's value of the pair's two
+    return __shfl_sync(both, v, (int)(threadIdx.x & 30u) + l);
+  };
   if (p >= S.pair_off[S.n_seg]) return;
   const int c = seg_find(S.pair_off, S.n_seg, p);
   const int64_t j = p - S.pair_off[c];
@@ -317,7 +330,18 @@ __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr,
   Draws<kTaus> g = draws_of<kTaus>(S, c, id[a], *step_p);
   int fails = 0;
   double cpsi, spsi, cphi, sphi;
-  if (!disk_angle(g, kTagPsi, cpsi, spsi)) ++fails;
+  bool got_phi = true;
+  if (kTwo) {
+    double ca, sa;
+    const bool got = disk_angle(g, second ? kTagPhi : kTagPsi, ca, sa);
+    cpsi = of(0, ca), spsi = of(0, sa);
+    cphi = of(1, ca), sphi = of(1, sa);
+    const unsigned ok = __ballot_sync(both, got) >> (threadIdx.x & 30u);
+    if (!(ok & 1u)) ++fails;
+    got_phi = (ok >> 1) & 1u;
+  } else if (!disk_angle(g, kTagPsi, cpsi, spsi)) {
+    ++fails;
+  }
   const double v1x = vr[a], v1y = vt[a], v1z = 0.0;
   const double v2x = vr[b], vtb = vt[b];
   const double v2y = mul_rn(vtb, cpsi), v2z = mul_rn(vtb, spsi);
@@ -326,10 +350,17 @@ __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr,
   const double w2 = (mul_rn(wx, wx) + wyy) + wzz;
   if (!pos_num(w2)) {
     draws_keep(S, c, g);
-    if (fails) stat_add(S.stats, c, kStAngleFails, (unsigned long long)fails);
+    if (fails && !second) stat_add(S.stats, c, kStAngleFails, (unsigned long long)fails);
     return;
   }
-  const double w = sqrt_rn_nl(w2);
+  const double wp2 = wyy + wzz;
+  double w, wp = 0.0;
+  if (kTwo) {
+    const double q = sqrt_rn_nl(second ? wp2 : w2);
+    w = of(0, q), wp = of(1, q);
+  } else {
+    w = sqrt_rn_nl(w2);
+  }
   if (kCol) {
     const double R1 = col.R[a], R2 = col.R[b];
     if (R1 + R2 > 0.0) {
@@ -345,6 +376,8 @@ __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr,
         const double dW = m2 * (col.phi[a] - col.phi[b]) + div_rn_nl(m1 * m2, col.r[a]);
         const double dK = (0.5 * div_rn_nl(m1 * m2, msum)) * w2;
         draws_keep(S, c, g);
+        if (kTwo) __syncwarp(both);  // (both have read the pair)
+        if (second) return;
         vr[a] = vcx;
         vt[a] = sqrt_rn_nl(vcy * vcy + vcz * vcz);
         m[a] = m1 + m2;
@@ -365,24 +398,36 @@ __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr,
   num = num * n;
   num = num * lnL;
   num = num * dt;
-  double s2 = div_rn_nl(num, w2 * w);
+  // e1 = (w x xhat)/|w x xhat| = (0, wz, -wy)/|.| (yhat for radial w);
+  // u = w x e1 has length |w| and completes the frame perpendicular to w
+  double e1y = 1.0, e1z = 0.0, s2;
+  const bool across = pos_num(wp2);
+  if (kTwo) {
+    const double q = div_rn_nl(second ? wz : num, second ? (across ? wp : 1.0) : w2 * w);
+    s2 = of(0, q);
+    if (across) e1y = of(1, q);
+  } else {
+    s2 = div_rn_nl(num, w2 * w);
+  }
   if (!le1(s2)) s2 = 1.0;
   // cos(beta) = 1 - 2 sin^2(beta/2), sin(beta) = 2 sin(beta/2) cos(beta/2)
   const double cosb = 1.0 - scale_up<1>(s2);
-  const double sinb = scale_up<1>(sqrt_rn_nl(s2)) * sqrt_rn_nl(1.0 - s2);
-  if (!disk_angle(g, kTagPhi, cphi, sphi)) ++fails;
-  draws_keep(S, c, g);
-  // e1 = (w x xhat)/|w x xhat| = (0, wz, -wy)/|.| (yhat for radial w);
-  // u = w x e1 has length |w| and completes the frame perpendicular to w
-  const double wp2 = wyy + wzz;
-  double e1y, e1z;
-  if (pos_num(wp2)) {
-    const double wp = sqrt_rn_nl(wp2);
-    e1y = div_rn_nl(wz, wp);
-    e1z = div_rn_nl(-wy, wp);
+  double sinb;
+  if (kTwo) {
+    const double q = sqrt_rn_nl(second ? 1.0 - s2 : s2);
+    sinb = scale_up<1>(of(0, q)) * of(1, q);
+    if (!got_phi) ++fails;
   } else {
-    e1y = 1.0;
-    e1z = 0.0;
+    sinb = scale_up<1>(sqrt_rn_nl(s2)) * sqrt_rn_nl(1.0 - s2);
+    if (!disk_angle(g, kTagPhi, cphi, sphi)) ++fails;
+  }
+  draws_keep(S, c, g);
+  if (across) {
+    if (!kTwo) {
+      wp = sqrt_rn_nl(wp2);
+      e1y = div_rn_nl(wz, wp);
+    }
+    e1z = div_rn_nl(-wy, wp);
   }
   const double ux = wy * e1z - wz * e1y;
   const double uy = -(wx * e1z);
@@ -397,6 +442,19 @@ __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr,
   // angles' in disk_angle: 17 of the pair's 44) balance the FP64 pipe's load
   // against the issue slots: 0.757 ms at N = 1e7, 0.853 with only these six
   // there, 0.77 to 0.80 with other groups, 0.95 with all (shared body).
+  if (kTwo) {
+    const double f = div_rn_nl(second ? m1 : m2, msum);
+    const double tx = mul_rn(f, dwx), ty = mul_rn(f, dwy), tz = mul_rn(f, dwz);
+    const double px = second ? v2x - tx : v1x + tx, py = second ? v2y - ty : v1y + ty,
+                 pz = second ? v2z - tz : v1z + tz;
+    const int64_t at = second ? b : a;
+    const double pt = sqrt_rn_nl(py * py + pz * pz);
+    __syncwarp(both);  // (both have read the pair)
+    vr[at] = px;
+    vt[at] = pt;
+    if (fails && !second) stat_add(S.stats, c, kStAngleFails, (unsigned long long)fails);
+    return;
+  }
   const double f1 = div_rn_nl(m2, msum), f2 = div_rn_nl(m1, msum);
   const double p1x = v1x + mul_rn(f1, dwx), p1y = v1y + mul_rn(f1, dwy), p1z = v1z + mul_rn(f1, dwz);
   const double p2x = v2x - mul_rn(f2, dwx), p2y = v2y - mul_rn(f2, dwy), p2z = v2z - mul_rn(f2, dwz);
@@ -463,21 +521,17 @@ template <int kMinB>
 static void relax_shape(const SegLayout& L, double* vr, double* vt, double* m,
                         const uint32_t* id, const double* nbin, const uint32_t* step,
                         const Collide& col, cudaStream_t st) {
-  const unsigned grid = (unsigned)((L.n_pairs + 127) / 128);
+  const bool two = !L.taus && L.n_pairs <= kTwoLanes;
+  const unsigned grid = (unsigned)((L.n_pairs * (two ? 2 : 1) + 127) / 128);
   // (the collision code only in the kernels that need it: it costs
   // registers)
-  if (L.taus && col.R)
-    launch_k(k_relax<true, kMinB, true>, grid, 128, 0, st, L.dev(), L.bin_size, vr, vt, m, id, nbin,
-                                                     step, col);
-  else if (L.taus)
-    launch_k(k_relax<true, kMinB, false>, grid, 128, 0, st, L.dev(), L.bin_size, vr, vt, m, id, nbin,
-                                                      step, col);
-  else if (col.R)
-    launch_k(k_relax<false, kMinB, true>, grid, 128, 0, st, L.dev(), L.bin_size, vr, vt, m, id, nbin,
-                                                      step, col);
-  else
-    launch_k(k_relax<false, kMinB, false>, grid, 128, 0, st, L.dev(), L.bin_size, vr, vt, m, id,
-                                                       nbin, step, col);
+  const auto kernel = L.taus  ? (col.R ? k_relax<true, kMinB, true, false>
+                                       : k_relax<true, kMinB, false, false>)
+                      : two   ? (col.R ? k_relax<false, 1, true, true>
+                                       : k_relax<false, 1, false, true>)
+                              : (col.R ? k_relax<false, kMinB, true, false>
+                                       : k_relax<false, kMinB, false, false>);
+  launch_k(kernel, grid, 128, 0, st, L.dev(), L.bin_size, vr, vt, m, id, nbin, step, col);
 }
 
 void launch_relax(const SegLayout& L, double* vr, double* vt, double* m, const uint32_t* id,
