@@ -1066,6 +1066,7 @@ enum : uint32_t { kSmpAccepted = 0, kSmpPending = 1, kSmpDegenerate = 2, kSmpCap
 // Orbit stage of 10^3, 10^4, 3 x 10^4, 6 x 10^4 stars 24.9, 29.1, 30.8, 32.9 us with a
 // lane, 22.4, 23.8, 26.7, 32.9 with four, 20.4, 22.8, 28.6, 36.3 with eight.
 constexpr int64_t kSample8 = 16384, kSample4 = 49152;
+constexpr int kOwnTrials = 2;
 
 template <int kMinB, bool kTaus, bool kExact, int kG>
 __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
@@ -1082,6 +1083,12 @@ __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
   unsigned long long viol = 0;
   bool pend = false;
   int c = -1;  // lanes past the end form their own group below
+  // kG == 1, counter draws: the trials by the warp (below)
+  constexpr bool kPool = kG == 1 && !kTaus;
+  bool live = false;
+  float c0f = 0.0f, c1f = 0.0f, E32 = 0.0f, J32 = 0.0f, F32 = 0.0f;
+  uint32_t st = kSmpCap, idv = 0u;
+  int t = 0;
   if (p < n) {
     c = seg_find(S.off, S.n_seg, p);
     const int64_t k = p - S.off[c];
@@ -1090,9 +1097,8 @@ __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
     const double E = o.x;
     if (k < S.nb[c] && lt0(E)) {
       const double J = o.y, c0 = o.z, c1 = o.w;
-      const float c0f = f32_rn(c0), c1f = f32_rn(c1), E32 = f32_rn(E), J32 = f32_rn(J);
+      c0f = f32_rn(c0), c1f = f32_rn(c1), E32 = f32_rn(E), J32 = f32_rn(J);
       const Grid GD = grid_of(BA, c);
-      float F32;
       bool degenerate;
       if (kExact) {
         const double F64 = 1.2 * __ldg(Fx + p);
@@ -1111,10 +1117,24 @@ __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
         F32 = 1.2f * gmax;
         degenerate = !gt_pos(c1, 0.0) || !(F32 > 0.0f);
       }
-      uint32_t st = kSmpCap;
-      int t = 0;
       if (degenerate) {
         st = kSmpDegenerate;
+      } else if (kPool) {
+        idv = id[p];
+        live = true;
+        // the first trials in the star's lane
+        Draws<false> g = draws_of<false>(S, c, idv, *step_p);
+        const int own = max_trials < kOwnTrials ? max_trials : kOwnTrials;
+        for (; t < own; ++t) {
+          const U4 w = g.block(kTagRej, (uint32_t)t);
+          const int d = accept32<kExact>(GD, E32, J32, c0f, c1f, F32, 2.0f * u01f(w.y) - 1.0f,
+                                         u01f(w.w), viol);
+          if (d == 0) continue;
+          st = d > 0 ? kSmpAccepted : kSmpPending;
+          live = false;
+          break;
+        }
+        if (t >= max_trials) live = false;
       } else {
         Draws<kTaus> g = draws_of<kTaus>(S, c, id[p], *step_p);
         for (; t < max_trials; t += kG) {
@@ -1144,11 +1164,100 @@ __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
         }
         if (kG > 1 && t > max_trials) t = max_trials;
       }
-      if (sub == 0) {
+      if (!kPool && sub == 0) {
         keys[p] = ((uint64_t)__float_as_uint(F32) << 32) | ((uint64_t)st << 30) |
                   (uint64_t)(t & 0x3FFFFFFF);
         pend = st == kSmpPending;
       }
+      if (kPool) pend = true;  // (a result to write)
+    }
+  }
+  if (kPool) {
+    // The further trials, by rounds.  While more than half the lanes are undecided
+    // each takes its own star's next one; then the lanes are shared out, G to each
+    // star that is left, for its next G trials (stars of one segment).  A warp ran
+    // as long as its slowest star (22 of 32 lanes busy, now 30): orbit stage of 10^6,
+    // 64 x 10^5, 10^7 stars 148.5, 851, 1246 us, FP64 mode at 10^7 2294; with the
+    // rounds from the first, second, third, fourth trial on 149.5, 841, 1230, 2277;
+    // 147.5, 837, 1223, 2265; 145.4, 827, 1211, 2253; 146.5, 832, 1217, 2270.
+    const bool result = pend;
+    __shared__ uint8_t s_owner[256];
+    uint8_t* owner = s_owner + (threadIdx.x & ~31u);
+    const bool one = __match_any_sync(0xFFFFFFFFu, c) == 0xFFFFFFFFu;
+    const Grid GD = grid_of(BA, c < 0 ? 0 : c);
+    const uint32_t stp = *step_p;
+    for (;;) {
+      const unsigned lm = __ballot_sync(0xFFFFFFFFu, live);
+      if (!lm) break;
+      const int k = __popc(lm), rank = __popc(lm & ((1u << lane) - 1u));
+      // 2^lg lanes a star: the largest with k 2^lg <= 32
+      const int lg = one ? __clz(2 * k - 1) - 26 : 0;
+      const int G = 1 << lg;
+      float e = E32, jj = J32, a0 = c0f, a1 = c1f, ff = F32;
+      uint32_t iv = idv;
+      int mine = t, from = lane;
+      bool go = live;
+      if (G > 1) {
+        if (live) owner[rank] = (uint8_t)lane;
+        __syncwarp();
+        const int slot = lane >> lg;
+        go = slot < k;
+        from = go ? owner[slot] : lane;
+        __syncwarp();
+        e = __shfl_sync(0xFFFFFFFFu, E32, from);
+        jj = __shfl_sync(0xFFFFFFFFu, J32, from);
+        a0 = __shfl_sync(0xFFFFFFFFu, c0f, from);
+        a1 = __shfl_sync(0xFFFFFFFFu, c1f, from);
+        ff = __shfl_sync(0xFFFFFFFFu, F32, from);
+        iv = __shfl_sync(0xFFFFFFFFu, idv, from);
+        mine = __shfl_sync(0xFFFFFFFFu, t, from) + (lane & (G - 1));
+      }
+      int d = 0;
+      unsigned long long over = 0;
+      if (go && mine < max_trials) {
+        Draws<false> g = draws_of<false>(S, c, iv, stp);
+        const U4 w = g.block(kTagRej, (uint32_t)mine);
+        d = accept32<kExact>(GD, e, jj, a0, a1, ff, 2.0f * u01f(w.y) - 1.0f, u01f(w.w), over);
+      }
+      const unsigned acc = __ballot_sync(0xFFFFFFFFu, d > 0);
+      const unsigned any = acc | __ballot_sync(0xFFFFFFFFu, d < 0);
+      if (G == 1) {
+        viol += over;
+        if (live) {
+          if (d != 0) {
+            st = d > 0 ? kSmpAccepted : kSmpPending;
+            live = false;
+          } else if (++t >= max_trials) {
+            live = false;
+          }
+        }
+      } else {
+        const unsigned gm = G == 32 ? 0xFFFFFFFFu : (1u << G) - 1u;
+        // the executing lanes' group, then the owners'
+        const unsigned mg = (any >> (lane & ~(G - 1))) & gm;
+        if (go && (!mg || (lane & (G - 1)) <= __ffs(mg) - 1)) viol += over;
+        if (live) {
+          const unsigned og = (any >> (rank * G)) & gm;
+          if (og) {
+            const int last = __ffs(og) - 1;
+            st = (acc >> (rank * G + last)) & 1u ? kSmpAccepted : kSmpPending;
+            t += last;
+            live = false;
+          } else {
+            t += G;
+            if (t >= max_trials) {
+              t = max_trials;
+              live = false;
+            }
+          }
+        }
+      }
+    }
+    pend = false;
+    if (result) {
+      keys[p] = ((uint64_t)__float_as_uint(F32) << 32) | ((uint64_t)st << 30) |
+                (uint64_t)(t & 0x3FFFFFFF);
+      pend = st == kSmpPending;
     }
   }
   // pending stars onto the list of k_pending64 (one atomic per warp)

@@ -34,7 +34,7 @@ def test_first_accepted_trial(g_stage, precision, beside):
 
 
 @pytest.mark.parametrize("max_trials", [1, 2, 3, 7])
-@pytest.mark.parametrize("n", [300, 40_000])
+@pytest.mark.parametrize("n", [300, 40_000, 60_000])
 def test_trial_cap(g_stage, n, max_trials):
     d = ic.plummer(n, seed=6)
     x, sx = _run(g_stage, [d], [5], precision=0, max_trials=max_trials)
@@ -43,3 +43,17 @@ def test_trial_cap(g_stage, n, max_trials):
         np.testing.assert_array_equal(x[k], y[k], err_msg=k)
     for k in ("trials", "cap_hits", "violations"):
         assert sx[0][k] == sy[0][k], k
+
+
+@pytest.mark.parametrize("sizes", [[25] * 2400, [31, 33, 64, 1, 2, 40_000, 95, 20_000]])
+def test_warps_of_several_segments(g_stage, sizes):
+    """Enough stars for the trials by rounds, in warps that hold stars of one segment
+    and of several."""
+    parts = [ic.plummer(n, seed=i + 1, masses="salpeter") for i, n in enumerate(sizes)]
+    seeds = list(range(len(sizes)))
+    x, sx = _run(g_stage, parts, seeds, precision=0)
+    y, sy = _run(g_stage, parts, seeds, precision=2)
+    for k in KEYS:
+        np.testing.assert_array_equal(x[k], y[k], err_msg=k)
+    for a, b in zip(sx, sy):
+        assert a["trials"] == b["trials"] and a["violations"] == b["violations"]
