@@ -317,7 +317,8 @@ int count_step_kernels(const cmc_ctx* c) {
   // evaluation], Phi_new(r_old) with the grid's values or those alone
   const int p = c->cfg.precision;
   const int sort = c->cfg.sort_packed ? (c->L.n <= kCountInOrbit ? 3 : 4) : 7;
-  return (c->L.n <= kEndWithVelocities ? 6 : 7) + sort + (c->ring ? 4 : 0) + (p == 1 ? 3 : p == 0 ? 5 : 0) +
+  return (c->L.n <= kEndWithVelocities ? 6 : 7) + sort + (c->ring ? 4 : 0) +
+         (p == 1 ? 3 : p == 0 ? 5 : 0) +
          (c->cfg.energy_correction || p != 2 ? 1 : 0);
 }
 
@@ -327,8 +328,9 @@ void free_ctx(cmc_ctx* c) {
   cudaStream_t st = c->stream;
   for (cudaGraphExec_t e : c->exec)
     if (e) cudaGraphExecDestroy(e);
-  double** ds[] = {&c->r_alt, &c->x_alt, &c->r, &c->x, &c->vr, &c->vt, &c->m, &c->phi, &c->r_old, &c->cc, &c->nbin,
-                   &c->tile_a, &c->tile_b, &c->tile_c, &c->out3, &c->fr, &c->lag};
+  double** ds[] = {&c->r_alt, &c->x_alt, &c->r, &c->x, &c->vr, &c->vt, &c->m, &c->phi, &c->r_old,
+                   &c->cc, &c->nbin, &c->tile_a, &c->tile_b, &c->tile_c, &c->out3,
+                   &c->fr, &c->lag};
   for (double** p : ds) dfree(*p, st);
   dfree(c->id, st);
   dfree(c->R, st);

@@ -1711,8 +1711,8 @@ void launch_potential(const SegLayout& L, const double* r, const double* x, cons
   int lp = 0;
   while (lp < kPotParts && L.n_tiles << (lp + 1) <= kPotBlocks) ++lp;
   launch_k(tables ? k_potential<true> : k_potential<false>, (unsigned)(L.n_tiles << lp),
-           kPotThreads, kPotentialSmem, st, S, L.esc_step, nb_sub, r, x, m, tile_m, tile_mx, phi, Mout, node,
-           tables ? *tables : TableOut(), lp);
+           kPotThreads, kPotentialSmem, st, S, L.esc_step, nb_sub, r, x, m, tile_m, tile_mx, phi,
+           Mout, node, tables ? *tables : TableOut(), lp);
 }
 
 void launch_correction(const SegLayout& L, const double* r, const double* x,
