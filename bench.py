@@ -158,19 +158,20 @@ def profiled_fp64_pipe(kernel: str):
 #   timestep:   r, v_r, v_t, m read (32 B)
 #   relax:      v_r, v_t, m (8 B each), id (4 B) read; v_r, v_t written
 #   turning:    r, v_r, v_t, Phi read; r_min, r_max written
-#   orbit:      r, v_r, v_t, Phi, m, id read; sort key and 48-B payload written
-#   sort:       5 passes of key + value read and written
-#   gather:     key, value and payload read; r, 1/r, v_r, v_t, m, id, r_old, c written
+#   orbit:      r, v_r, v_t, Phi, m, id read; two 32-B records and the bin written
+#   sort:       bins counted (read), their counts (1.13 per star) scanned in place,
+#               bins read again and the order written
+#   gather:     order and one record read; r, 1/r, m, id and the order written
 #               (with the potential's per-tile sums of m and m/r)
-#   potential:  1/r, m read; Phi, M, the float table written
-#   correction: r, 1/r, Phi, v_r, v_t, r_old, c read; v_r, v_t written
-STAGE_BYTES = {"timestep": 32, "relax": 44, "turning": 48, "orbit": 5 * 8 + 4 + 8 + 48,
-               "sort": 5 * 24, "gather": 12 + 48 + 60, "potential": 16 + 24,
-               "correction": 56 + 16}
+#   potential:  r, 1/r, m read; Phi, the 32-B node record, a bucket start written
+#   correction: old r and 1/r, new r and node record read, Phi_new(r_old) written;
+#               order, the other record, Phi read; v_r, v_t written
+STAGE_BYTES = {"timestep": 32, "relax": 44, "turning": 48, "orbit": 5 * 8 + 4 + 64 + 4,
+               "sort": 4 + 9 + 8, "gather": 4 + 32 + 32, "potential": 24 + 44,
+               "correction": 16 + 8 + 32 + 8 + 44 + 16}
 STAGE_KERNEL = {"timestep": "k_bins", "relax": "k_relax", "turning": "k_turning_mixed",
-                "orbit": "k_orbit", "sort": "k_pass", "gather": "k_gather",
-                "potential": "k_potential", "correction": "k_correction_mixed"}
-
+                "orbit": "k_orbit", "sort": "k_bin_scatter", "gather": "k_gather_step",
+                "potential": "k_potential", "correction": "k_phi_old"}
 
 
 # FP64 peak derived from the unit counts and clock (nominal 1.25 TFLOP/s)
