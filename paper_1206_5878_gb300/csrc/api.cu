@@ -644,15 +644,26 @@ cmc_status attr_set(cmc_ctx* c, double* dst, const double* src, int32_t ptr_kind
     return fail(c, CMC_EINVAL, who + ": bad arguments");
   if (c->poisoned) return fail(c, CMC_EPOISONED, who + ": context poisoned");
   if (!dst) return fail(c, CMC_EINVAL, who + ": the context has no " + option);
-  if (ptr_kind == 0)
-    for (int64_t i = 0; i < c->L.n; ++i)
-      if (!(src[i] >= 0.0) || !(src[i] < INFINITY))
-        return fail(c, CMC_EINVAL, who + ": values must be finite and >= 0");
   DeviceGuard g(c->device);
-  cudaError_t e = cudaMemcpyAsync(dst, src, sizeof(double) * (size_t)c->L.n,
-                                  ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                                  c->stream);
-  if (!e) e = cudaStreamSynchronize(c->stream);
+  cudaStream_t st = c->stream;
+  const size_t bytes = sizeof(double) * (size_t)c->L.n;
+  cudaError_t e;
+  if (ptr_kind == 0) {
+    // into scratch, checked there, and only then the context's
+    uint32_t bad = 0;
+    e = cudaMemcpyAsync(c->r_old, src, bytes, cudaMemcpyHostToDevice, st);
+    launch_check_attr(c->L.n, c->r_old, c->pcount, st);
+    if (!e) e = cudaMemcpyAsync(&bad, c->pcount, sizeof(bad), cudaMemcpyDeviceToHost, st);
+    if (!e) e = cudaStreamSynchronize(st);
+    if (!e && bad) {
+      cudaMemsetAsync(c->pcount, 0, sizeof(uint32_t), st);
+      return fail(c, CMC_EINVAL, who + ": values must be finite and >= 0");
+    }
+    if (!e) e = cudaMemcpyAsync(dst, c->r_old, bytes, cudaMemcpyDeviceToDevice, st);
+  } else {
+    e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, st);
+    if (!e) e = cudaStreamSynchronize(st);
+  }
   if (e) return cuda_fail(c, e, call);
   return CMC_OK;
 }

@@ -533,6 +533,8 @@ void launch_place(const SegLayout& L, const double* r, const uint32_t* id,
 // words, P: [4][32][32] jump matrices T^(2^(80 + b))
 void launch_taus_init(int64_t slots, int n_seg, const int64_t* base, const uint4* words,
                       const uint32_t* P, uint4* table, cudaStream_t st);
+// flag = 1 if a value is negative, infinite or NaN
+void launch_check_attr(int64_t n, const double* a, uint32_t* flag, cudaStream_t st);
 void launch_check_ids(const SegLayout& L, const uint64_t* sorted_ids, uint32_t* err,
                       cudaStream_t st);
 

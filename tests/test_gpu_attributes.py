@@ -1,0 +1,38 @@
+"""Stellar radii and semi-major axes are checked on the device before they replace the
+context's: a call with one bad value anywhere fails and leaves radii, axes and the
+next steps as they were."""
+import numpy as np
+import pytest
+
+import initial_conditions as ic
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [2, 255, 257, 30_001])
+@pytest.mark.parametrize("bad", [-1e-300, -1.0, np.inf, -np.inf, np.nan])
+def test_bad_values_change_nothing(g_stage, n, bad):
+    d = ic.plummer(n, seed=2, masses="salpeter")
+    rng = np.random.default_rng(n)
+    R, A = 1e-4 * rng.random(n), np.where(rng.random(n) < 0.2, 1e-3, 0.0)
+    R[0] = -0.0  # not negative
+    c, twin = (g_stage.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, [3], precision=1,
+                               collisions=1, binaries=1, autotune=0) for _ in range(2))
+    for x in (c, twin):
+        x.set_radii(R)
+        x.set_binaries(A)
+    for k in (0, n // 2, n - 1):
+        for call, good in ((c.set_radii, R), (c.set_binaries, A)):
+            v = good.copy()
+            v[k] = bad
+            with pytest.raises(g_stage.CMCError) as e:
+                call(v)
+            assert e.value.status == 1
+    np.testing.assert_array_equal(c.radii(), R)
+    c.step(2)
+    twin.step(2)
+    a, b = c.get_state(), twin.get_state()
+    for k in ("r", "vr", "vt", "m", "id", "phi"):
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    np.testing.assert_array_equal(c.radii(), twin.radii())
+    assert c.stats() == twin.stats()
