@@ -125,7 +125,9 @@ typedef struct {
                                    star's draws taken in a fixed order
                                    (relaxation, orbit trials, v_r sign); ids must
                                    then be below 4 N_c + 64 in every cluster
-                                   (stream slots are indexed by id); the mixed
+                                   (stream slots are indexed by id, up to the
+                                   largest one at cmc_init: cmc_set_state
+                                   refuses larger ids and changes nothing); the mixed
                                    sampler runs one launch shape */
     int32_t relax_variant;      /* relaxation kernel variant (listed at
                                    cmc_get_tuning): -1 = the autotuner's choice

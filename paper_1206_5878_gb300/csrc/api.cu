@@ -41,6 +41,7 @@ struct cmc_ctx {
   uint32_t* order = nullptr;   // the stars' old indices at their new positions
   BinWork bins;                // the timestep's counting sort (cfg.sort_packed)
   std::vector<unsigned int> max_id;  // per segment, as the bins have it
+  std::vector<unsigned int> taus_max_id;  // per segment: the last id with a stream (rng 1)
   double *r_old = nullptr, *cc = nullptr, *nbin = nullptr;
   double *tile_a = nullptr, *tile_b = nullptr, *tile_c = nullptr,
          *out3 = nullptr, *fr = nullptr, *lag = nullptr;
@@ -129,31 +130,45 @@ cmc_status check_err_flags(cmc_ctx* ctx) {
   return fail(ctx, CMC_ECUDA, msg);
 }
 
+// Whether stars on the device are in (r, id) order in every segment (ordered),
+// and the largest id of each (max_id); waits for the stream.
+cudaError_t check_order(const SegLayout& L, const double* r, const uint32_t* id, cudaStream_t st,
+                        bool& ordered, std::vector<unsigned int>& max_id) {
+  unsigned int* d = nullptr;  // [0] order flag, [1 + s] largest id of segment s
+  std::vector<unsigned int> h((size_t)L.n_seg + 1, 0u);
+  cudaError_t e = dalloc(d, h.size(), st);
+  if (e) return e;
+  e = cudaMemsetAsync(d, 0, sizeof(unsigned int) * h.size(), st);
+  if (!e) {
+    launch_order_check(L, r, id, d, d + 1, st);
+    e = cudaGetLastError();
+  }
+  if (!e)
+    e = cudaMemcpyAsync(h.data(), d, sizeof(unsigned int) * h.size(), cudaMemcpyDeviceToHost, st);
+  if (!e) e = cudaStreamSynchronize(st);
+  dfree(d, st);
+  if (e) return e;
+  ordered = h[0] == 0u;
+  max_id.assign(h.begin() + 1, h.end());
+  return cudaSuccess;
+}
+
 // Whether the staged stars are already in (r, id) order in every segment
 // with ids that fit a bitmap of the key scratch (64 bits per star): then
 // bitoff receives each segment's first bit.  A state read back with
-// cmc_get_state always qualifies.  max_id (if given) receives the largest
-// id of each segment either way.
+// cmc_get_state always qualifies.  max_id receives the largest id of each
+// segment either way (empty where it could not be read).
 bool staged_in_order(cmc_ctx* c, std::vector<unsigned long long>& bitoff, cudaStream_t st,
-                     std::vector<unsigned int>* max_id = nullptr) {
+                     std::vector<unsigned int>& max_id) {
   const SegLayout& L = c->L;
-  unsigned int* d = nullptr;  // [0] order flag, [1 + s] largest id of segment s
-  if (dalloc(d, (size_t)L.n_seg + 1, st)) return false;
-  std::vector<unsigned int> h((size_t)L.n_seg + 1, 1u);
-  cudaError_t e = cudaMemsetAsync(d, 0, sizeof(unsigned int) * h.size(), st);
-  if (!e) {
-    launch_order_check(L, c->r, c->id, d, d + 1, st);
-    e = cudaMemcpyAsync(h.data(), d, sizeof(unsigned int) * h.size(), cudaMemcpyDeviceToHost, st);
-  }
-  if (!e) e = cudaStreamSynchronize(st);
-  dfree(d, st);
-  if (!e && max_id) max_id->assign(h.begin() + 1, h.end());
-  if (e || h[0] != 0u) return false;
+  bool ordered = false;
+  max_id.clear();
+  if (check_order(L, c->r, c->id, st, ordered, max_id) || !ordered) return false;
   bitoff.assign((size_t)L.n_seg, 0ull);
   unsigned long long total = 0;
   for (int s = 0; s < L.n_seg; ++s) {
     bitoff[s] = total;
-    total += (unsigned long long)h[1 + s] + 1ull;
+    total += (unsigned long long)max_id[s] + 1ull;
   }
   return total <= 64ull * (unsigned long long)L.n;
 }
@@ -200,7 +215,9 @@ void finish_order(cmc_ctx* c, bool placed, cudaStream_t st) {
 void order_state(cmc_ctx* c, cudaStream_t st) {
   const SegLayout& L = c->L;
   std::vector<unsigned long long> bitoff;
-  const bool placed = L.n > 0 && staged_in_order(c, bitoff, st) && order_in_place(c, bitoff, st);
+  std::vector<unsigned int> max_id;
+  const bool placed =
+      L.n > 0 && staged_in_order(c, bitoff, st, max_id) && order_in_place(c, bitoff, st);
   if (!placed) {
     launch_id_keys(L, c->id, c->keys, st);
     sort_segments(L, c->W, c->keys, c->vals, 0, 4, true, c->err, st);
@@ -389,7 +406,7 @@ cmc_status load_state(cmc_ctx* c, const double* r, const double* vr, const doubl
   std::vector<unsigned long long> bitoff;
   bool placed = false;
   std::vector<unsigned int> max_id;
-  if (L.n > 0 && staged_in_order(c, bitoff, aux, &max_id) && order_in_place(c, bitoff, aux)) {
+  if (L.n > 0 && staged_in_order(c, bitoff, aux, max_id) && order_in_place(c, bitoff, aux)) {
     finish_order(c, true, aux);
     placed = true;
   }
@@ -486,30 +503,24 @@ void taus_seed_words(uint64_t seed, uint32_t w[4]) {
 cmc_status init_streams(cmc_ctx* c, const uint64_t* seeds) {
   SegLayout& L = c->L;
   cudaStream_t st = c->stream;
-  unsigned int* d = nullptr;
-  std::vector<unsigned int> h((size_t)L.n_seg + 1, 0u);
-  cudaError_t e = dalloc(d, h.size(), st);
-  if (!e) e = cudaMemsetAsync(d, 0, sizeof(unsigned int) * h.size(), st);
-  if (!e) {
-    launch_order_check(L, c->r, c->id, d, d + 1, st);
-    e = cudaMemcpyAsync(h.data(), d, sizeof(unsigned int) * h.size(), cudaMemcpyDeviceToHost, st);
-  }
-  if (!e) e = cudaStreamSynchronize(st);
-  dfree(d, st);
+  bool ordered = false;
+  std::vector<unsigned int> max_id;
+  cudaError_t e = check_order(L, c->r, c->id, st, ordered, max_id);
   if (e) return cuda_fail(c, e, "cmc_init: streams");
   std::vector<int64_t> base((size_t)L.n_seg + 1, 0);
   std::vector<uint32_t> words((size_t)4 * L.n_seg);
   for (int s = 0; s < L.n_seg; ++s) {
     const int64_t nc = L.h_off[s + 1] - L.h_off[s];
-    if ((int64_t)h[1 + s] >= 4 * nc + 64)
+    if ((int64_t)max_id[s] >= 4 * nc + 64)
       return fail(c, CMC_EINVAL, "cmc_init: the Tausworthe streams need ids below 4 N + 64");
-    base[s + 1] = base[s] + (int64_t)h[1 + s] + 1;
+    base[s + 1] = base[s] + (int64_t)max_id[s] + 1;
     taus_seed_words(seeds[s], &words[4 * (size_t)s]);
   }
   const std::vector<uint32_t> P = taus_jump_matrices();
   uint32_t* dP = nullptr;
   uint4* dw = nullptr;
   L.taus_slots = base[L.n_seg];
+  c->taus_max_id = max_id;
   e = dalloc(L.taus, (size_t)L.taus_slots, st);
   if (!e) e = dalloc(L.taus_base, base.size(), st);
   if (!e) e = dalloc(dP, P.size(), st);
@@ -527,6 +538,26 @@ cmc_status init_streams(cmc_ctx* c, const uint64_t* seeds) {
   dfree(dP, st);
   dfree(dw, st);
   if (e) return cuda_fail(c, e, "cmc_init: streams");
+  return CMC_OK;
+}
+
+// Whether every id of a new state has a stream (slots are indexed by id, up to the
+// largest id at cmc_init): asked before anything of the state is replaced.
+cmc_status check_stream_ids(cmc_ctx* c, const double* r, const uint32_t* id, int32_t ptr_kind) {
+  const SegLayout& L = c->L;
+  std::vector<unsigned int> max_id((size_t)L.n_seg, 0u);
+  if (ptr_kind == 0) {
+    for (int s = 0; s < L.n_seg; ++s)
+      for (int64_t p = L.h_off[s]; p < L.h_off[s + 1]; ++p)
+        if (id[p] > max_id[s]) max_id[s] = id[p];
+  } else {
+    bool ordered = false;
+    const cudaError_t e = check_order(L, r, id, c->stream, ordered, max_id);
+    if (e) return cuda_fail(c, e, "cmc_set_state: streams");
+  }
+  for (int s = 0; s < L.n_seg; ++s)
+    if (max_id[s] > c->taus_max_id[s])
+      return fail(c, CMC_EINVAL, "cmc_set_state: an id above those that have a Tausworthe stream");
   return CMC_OK;
 }
 
@@ -1022,6 +1053,10 @@ cmc_status cmc_set_state(cmc_ctx* c, const double* r, const double* vr, const do
   if (!c || !r || !vr || !vt || !m || !id || step < 0 || (ptr_kind != 0 && ptr_kind != 1))
     return fail(c, CMC_EINVAL, "cmc_set_state: bad arguments");
   DeviceGuard g(c->device);
+  if (c->L.taus) {
+    const cmc_status s = check_stream_ids(c, r, id, ptr_kind);
+    if (s != CMC_OK) return s;
+  }
   c->poisoned = false;
   // a new state drops the stellar radii and semi-major axes (they belong
   // to the old order)

@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 
 import initial_conditions as ic
+from gpu_util import dev
 from test_golden import paper_values
 from test_gpu_step import _compare_states
 
@@ -129,3 +130,34 @@ def test_stream_mode_argument_checks(g):
             c.set_rng_state(np.zeros(3, dtype=np.uint32))
         with pytest.raises(g.CMCError):
             g.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, [1], rng=2)
+
+
+@pytest.mark.parametrize("device", [False, True])
+@pytest.mark.parametrize("cluster", [0, 1])
+def test_states_with_ids_beyond_the_streams_are_refused(g, device, cluster):
+    """A stream slot is an id: a new state with a larger id than at the start, in the
+    first or the last cluster, is refused from its ids alone and the old state
+    goes on as if it had not been offered."""
+    sizes = [300, 500]
+    parts = [ic.plummer(k, seed=k) for k in sizes]
+    d = {k: np.concatenate([p[k] for p in parts]) for k in ("r", "vr", "vt", "m", "id")}
+    a = g.Cluster(d, [1, 2], sizes=sizes, rng="taus113", precision=1)
+    b = g.Cluster(d, [1, 2], sizes=sizes, rng="taus113", precision=1)
+    a.step(1)
+    b.step(1)
+    st = a.get_state()
+    bad = {k: st[k].copy() for k in ("r", "vr", "vt", "m", "id")}
+    at = sizes[0] * cluster + 7
+    bad["id"][at] = sizes[cluster]  # the first id without a stream
+    if device:
+        bad = {k: dev(v) for k, v in bad.items()}
+    with pytest.raises(g.CMCError) as ei:
+        a.set_state(bad, st["step"])
+    assert ei.value.status == 1  # CMC_EINVAL
+    a.step(2)
+    b.step(2)
+    sa, sb = a.get_state(), b.get_state()
+    for k in ("r", "vr", "vt", "m", "id", "phi", "step"):
+        np.testing.assert_array_equal(sa[k], sb[k], err_msg=k)
+    np.testing.assert_array_equal(a.rng_state(), b.rng_state())
+    a.set_state(st, st["step"])  # the same ids are taken
