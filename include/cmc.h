@@ -222,7 +222,9 @@ cmc_status cmc_get_state(cmc_ctx *ctx, double *r, double *vr, double *vt, double
 /* Replace the state of every cluster (same sizes as at cmc_init) and set
  * the step counter; the stars are re-sorted and the potential recomputed.
  * Escaped stars may be passed with r = +inf.  A state obtained from
- * cmc_get_state resumes bit for bit. */
+ * cmc_get_state resumes bit for bit.  The arrays are copied in before they
+ * are checked, so CMC_EINVAL for an invalid state poisons the context (the old
+ * state is gone); setting a valid one clears that and any earlier poisoning. */
 cmc_status cmc_set_state(cmc_ctx *ctx, const double *r, const double *vr, const double *vt,
                          const double *m, const uint32_t *id, int64_t step,
                          int32_t ptr_kind);

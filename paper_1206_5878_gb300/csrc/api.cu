@@ -123,10 +123,7 @@ cmc_status check_err_flags(cmc_ctx* ctx) {
   if (e & kErrInput) msg += " invalid input state;";
   if (e & kErrNonFinite) msg += " non-finite value;";
   if (e & kErrTimeout) return fail(ctx, CMC_ETIMEOUT, msg);
-  if (e & kErrInput) {
-    ctx->poisoned = false;  // nothing was changed on the device state yet
-    return fail(ctx, CMC_EINVAL, msg);
-  }
+  if (e & kErrInput) return fail(ctx, CMC_EINVAL, msg);
   return fail(ctx, CMC_ECUDA, msg);
 }
 
@@ -1057,12 +1054,15 @@ cmc_status cmc_set_state(cmc_ctx* c, const double* r, const double* vr, const do
     const cmc_status s = check_stream_ids(c, r, id, ptr_kind);
     if (s != CMC_OK) return s;
   }
-  c->poisoned = false;
   // a new state drops the stellar radii and semi-major axes (they belong
   // to the old order)
   if (c->R) cudaMemsetAsync(c->R, 0, sizeof(double) * (size_t)c->L.n, c->stream);
   if (c->A) cudaMemsetAsync(c->A, 0, sizeof(double) * (size_t)c->L.n, c->stream);
-  return load_state(c, r, vr, vt, m, id, ptr_kind, true, step);
+  const cmc_status s = load_state(c, r, vr, vt, m, id, ptr_kind, true, step);
+  // (on failure the arrays hold parts of a state that was refused: nothing to go on
+  // with until a valid one is set)
+  c->poisoned = s != CMC_OK;
+  return s;
 }
 
 cmc_status cmc_get_nbound(cmc_ctx* c, int64_t* out) {

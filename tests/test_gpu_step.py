@@ -402,3 +402,37 @@ def test_unsorted_state_after_the_tuned_sort_shape(g):
     assert c.tuning() == tuned
     c.step(2)
     assert np.all(np.isfinite(c.get_state()["r"][: int(c.nbound()[0])]))
+
+
+@pytest.mark.parametrize("fault", ["nan", "vt", "duplicate", "shuffled"])
+def test_rejected_state_poisons(g, fault):
+    """A new state is copied in before it is checked: a rejected one leaves nothing
+    that could be used, and a valid one puts the context right."""
+    d = ic.plummer(5000, seed=2)
+    c, o = _cluster(g, d, 2, autotune=0), _cluster(g, d, 2, autotune=0)
+    c.step(1)
+    o.step(1)
+    st = c.get_state()
+    bad = {k: st[k].copy() for k in ("r", "vr", "vt", "m", "id")}
+    if fault == "nan":
+        bad["vr"][77] = np.nan
+    elif fault == "vt":
+        bad["vt"][4000] = -1.0
+    else:
+        if fault == "shuffled":
+            p = np.random.default_rng(1).permutation(5000)
+            bad = {k: v[p].copy() for k, v in bad.items()}
+        bad["id"][10] = bad["id"][11]
+    with pytest.raises(g.CMCError) as ei:
+        c.set_state(bad, st["step"])
+    assert ei.value.status == 1  # CMC_EINVAL
+    for call in (c.get_state, c.energy, lambda: c.step(1)):
+        with pytest.raises(g.CMCError) as ei:
+            call()
+        assert ei.value.status == 6  # CMC_EPOISONED
+    c.set_state(st, st["step"])
+    c.step(2)
+    o.step(2)
+    sa, sb = c.get_state(), o.get_state()
+    for k in ("r", "vr", "vt", "m", "id", "phi", "step"):
+        np.testing.assert_array_equal(sa[k], sb[k], err_msg=k)
