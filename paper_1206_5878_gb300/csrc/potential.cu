@@ -1299,13 +1299,13 @@ __global__ void __launch_bounds__(kThreads) k_energy_final(Seg S, const double* 
 // round takes five halvings: lane l (1 to 31) probes node l of the tree of the
 // next five midpoints, the answers pick the path (same midpoints and result as
 // one halving at a time, which took 13.7 us at 10^6 stars; 8.0).
-__global__ void k_lagrange(Seg S, const double* r, const double* M, const double* fracs,
-                           int nf, double* out) {
-  pdl_enter();
-  const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (i >= S.n_seg * nf) return;
-  const int c = i / nf, q = i % nf;
+// (The searches, clusters x fractions, can be more than 2^31: counted in 64 bits,
+// the grid strides over those beyond its blocks.)
+constexpr int kLagThreads = 128;
+__device__ __forceinline__ void lagrange_search(const Seg& S, const double* r, const double* M,
+                                                const double* fracs, int nf, double* out,
+                                                int64_t i, int lane) {
+  const int c = (int)(i / nf), q = (int)(i % nf);
   const int64_t sb = S.off[c], nbc = S.nb[c];
   if (nbc <= 0) {
     if (lane == 0) out[i] = 0.0;
@@ -1334,6 +1334,14 @@ __global__ void k_lagrange(Seg S, const double* r, const double* M, const double
     }
   }
   if (lane == 0) out[i] = r[sb + hi];
+}
+__global__ void __launch_bounds__(kLagThreads) k_lagrange(Seg S, const double* r, const double* M,
+                                                          const double* fracs, int nf,
+                                                          double* out) {
+  pdl_enter();
+  const int64_t n = (int64_t)S.n_seg * nf, step = (int64_t)gridDim.x * (kLagThreads / 32);
+  for (int64_t i = (int64_t)blockIdx.x * (kLagThreads / 32) + (threadIdx.x >> 5); i < n; i += step)
+    lagrange_search(S, r, M, fracs, nf, out, i, threadIdx.x & 31);
 }
 
 __global__ void k_validate(int64_t n, const double* r, const double* vr, const double* vt,
@@ -1778,8 +1786,11 @@ void launch_core(const SegLayout& L, const double* r, const double* m, double* t
 
 void launch_lagrange(const SegLayout& L, const double* r, const double* M,
                      const double* fracs, int nf, double* out, cudaStream_t st) {
-  int n = L.n_seg * nf;
-  if (n) launch_k(k_lagrange, blocks_for(n, 4), 128, 0, st, L.dev(), r, M, fracs, nf, out);
+  const int64_t n = (int64_t)L.n_seg * nf;
+  const int64_t blocks = (n + kLagThreads / 32 - 1) / (kLagThreads / 32), most = 1 << 24;
+  if (n)
+    launch_k(k_lagrange, (unsigned)(blocks < most ? blocks : most), kLagThreads, 0, st, L.dev(), r,
+             M, fracs, nf, out);
 }
 
 void launch_validate(const SegLayout& L, const double* r, const double* vr,

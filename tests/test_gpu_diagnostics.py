@@ -111,3 +111,15 @@ def test_ensemble(g_stage):
     st, o = c.get_state(), np.concatenate([[0], np.cumsum(sizes)])
     for i in range(4):
         _check(c, i, *(st[k][o[i]:o[i + 1]] for k in ("r", "vr", "vt", "m")))
+
+
+def test_lagrange_radii_of_very_many_searches(g_stage):
+    """More than 2^27 pairs of a cluster and a fraction (a warp searches for each, so
+    their threads do not fit 32 bits): clusters of one star, whose radii are
+    all the star's."""
+    n, nf = 32769, 4096
+    d = ic.plummer(n, seed=5)
+    c = g_stage.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, list(range(n)),
+                        sizes=[1] * n, autotune=0)
+    got = c.lagrange_radii(np.linspace(0.0, 1.0, nf))
+    assert got.shape == (n, nf) and np.all(got == d["r"][:, None])
