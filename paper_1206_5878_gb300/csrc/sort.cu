@@ -337,7 +337,6 @@ __global__ void k_tiefix(const int64_t* off, int n_seg, int64_t n, uint64_t* key
   // insertion sort of the run by (key, id)
   const long long move_cap = g_tie_move_cap;
   long long moves = 0;
-  bool equal = false;
   for (int64_t i = p + 1; i < e; ++i) {
     const uint64_t kv = keys[i];
     const uint32_t v = vals[i];
@@ -345,7 +344,6 @@ __global__ void k_tiefix(const int64_t* off, int n_seg, int64_t n, uint64_t* key
     int64_t j = i - 1;
     while (j >= p) {
       const uint64_t kj = keys[j];
-      if (kj == kv) equal = true;
       if (!(kj > kv || (kj == kv && ids_by_val[(size_t)vals[j] * id_stride] > idv))) break;
       keys[j + 1] = kj;
       vals[j + 1] = vals[j];
@@ -360,7 +358,12 @@ __global__ void k_tiefix(const int64_t* off, int n_seg, int64_t n, uint64_t* key
     keys[j + 1] = kv;
     vals[j + 1] = v;
   }
-  if (equal && stats) atomicAdd(stats + (size_t)c * kStStride + kStTies, 1ull);
+  // the run's groups of equal radii, each counted at its second star (as the
+  // timestep's gather does; escapers have keys of their own)
+  unsigned long long groups = 0;
+  for (int64_t i = p + 1; i < e; ++i)
+    groups += keys[i] == keys[i - 1] && (i - 1 == p || keys[i - 2] != keys[i]);
+  if (groups && stats) atomicAdd(stats + (size_t)c * kStStride + kStTies, groups);
 }
 
 // ------------------------------------------------------- counting sort

@@ -131,3 +131,23 @@ def test_new_state_with_other_ids_and_one_step_at_a_time(g_stage):
     sa, sb = c.get_state(), o.get_state()
     for k in KEYS:
         np.testing.assert_array_equal(sa[k], sb[k], err_msg=k)
+
+
+@pytest.mark.parametrize("packed", [0, 1])
+def test_groups_of_equal_radii_are_counted(g_stage, packed):
+    """The tie counter: groups of equal radii, several of them within the low bits
+    that the radix passes leave.  One trial a step, so that most stars stay
+    where they are."""
+    n = 4000
+    d = ic.plummer(n, seed=11)
+    d["r"][:600] = 0.7 + np.repeat(np.arange(120), 5) * 2.0 ** -53
+    d["r"][600:640] = 0.9
+    c = g_stage.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, [4], precision=1, autotune=0,
+                        max_trials=1, sort_packed=packed)
+    want = 0
+    for _ in range(3):
+        c.step(1)
+        r = c.get_state()["r"]
+        r, count = np.unique(r[np.isfinite(r)], return_counts=True)
+        want += int((count > 1).sum())
+        assert want > 50 and c.stats()[0]["ties"] == want
