@@ -338,7 +338,8 @@ cmc_status cmc_sort_radius(int64_t n, const double *r, const uint32_t *id, uint3
                            void *stream);
 
 /* Shell potential, Eqs. 1-5 (scan form), of n sorted stars (all bound).
- * phi: n doubles out.  M (may be NULL): enclosed mass M_k out. */
+ * phi: n doubles out.  M (may be NULL): enclosed mass M_k out.  phi or M may
+ * be r or m itself (written in place). */
 cmc_status cmc_potential(int64_t n, const double *r, const double *m, double *phi, double *M,
                          void *stream);
 

@@ -1332,7 +1332,8 @@ cmc_status cmc_potential(int64_t n, const double* r, const double* m, double* ph
   cudaError_t e = C.alloc(block, st);
   if (!e) {
     potential_prepare();
-    launch_potential(S.L, r, x, m, ta, tb, phi, M, false, st, false, nullptr, nullptr, x);
+    launch_potential(S.L, r, x, m, ta, tb, phi, M, false, st, false, nullptr, nullptr, x,
+                     phi == m || M == m);
     e = cudaGetLastError();
   }
   dfree(block, st);

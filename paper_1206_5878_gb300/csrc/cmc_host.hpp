@@ -303,6 +303,7 @@ void launch_velocities(const SegLayout& L, const uint32_t* order, const RecB* rb
 // potential: per-tile sums then the tile-local scans (Eqs. 1-5 in scan
 // form).  nb_sub: subtract esc_step from nb (after the orbit step).
 // With recip (= x), x = 1/r is computed too, with the tiles' sums.
+// over_m: phi or Mout shares memory with m, place for place.
 // Optional output: Mout (M_k); with tables instead the record {1/r, Phi, r,
 // slope} of every star (node: one 32-byte sector per node for the kernels that
 // read a few nodes at random; the slope of Eq. 6 across the shell is the FP64
@@ -323,7 +324,8 @@ struct TableOut {
 void launch_potential(const SegLayout& L, const double* r, const double* x, const double* m,
                       double* tile_m, double* tile_mx, double* phi, double* Mout, bool nb_sub,
                       cudaStream_t st, bool sums_ready = false, double4_32a* node = nullptr,
-                      const TableOut* tables = nullptr, double* recip = nullptr);
+                      const TableOut* tables = nullptr, double* recip = nullptr,
+                      bool over_m = false);
 // node records from the arrays (stage calls)
 void launch_make_nodes(int64_t n, const double* r, const double* x, const double* phi,
                        const double* M, double4_32a* node, cudaStream_t st);

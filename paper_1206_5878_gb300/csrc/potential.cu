@@ -668,7 +668,8 @@ void launch_tile_sums(const SegLayout& L, bool nb_sub, const double* x, const do
 // finishes its part of the stars.  Up to two blocks per SM that way: one block
 // per tile leaves most SMs idle (the potential stage of 10^4, 10^5 stars 42, 42 us
 // against 26, 29; at 245 tiles and more a second block per tile only adds the
-// sums' work, 70.2 us against 71.7).
+// sums' work, 70.2 us against 71.7).  Where the output lies over the masses, one
+// block a tile: another block of the tile may not have read them yet.
 constexpr int kPotParts = 4;    // log2
 constexpr int kPotBlocks = 304;
 constexpr int kPotThreads = 512;
@@ -1722,7 +1723,7 @@ void potential_prepare() {
 void launch_potential(const SegLayout& L, const double* r, const double* x, const double* m,
                       double* tile_m, double* tile_mx, double* phi, double* Mout, bool nb_sub,
                       cudaStream_t st, bool sums_ready, double4_32a* node,
-                      const TableOut* tables, double* recip) {
+                      const TableOut* tables, double* recip, bool over_m) {
   if (!L.n_tiles) return;
   Seg S = L.dev();
   if (recip)
@@ -1730,7 +1731,7 @@ void launch_potential(const SegLayout& L, const double* r, const double* x, cons
   else if (!sums_ready)
     launch_tile_sums<kSumsOfX>(L, nb_sub, x, m, tile_m, tile_mx, nullptr, st);
   int lp = 0;
-  while (lp < kPotParts && L.n_tiles << (lp + 1) <= kPotBlocks) ++lp;
+  while (!over_m && lp < kPotParts && L.n_tiles << (lp + 1) <= kPotBlocks) ++lp;
   launch_k(tables ? k_potential<true> : k_potential<false>, (unsigned)(L.n_tiles << lp),
            kPotThreads, kPotentialSmem, st, S, L.esc_step, nb_sub, r, x, m, tile_m, tile_mx, phi,
            Mout, node, tables ? *tables : TableOut(), lp);

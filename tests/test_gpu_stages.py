@@ -74,6 +74,27 @@ def test_potential_within_1e12(g, orc, n, masses):
     assert np.max(np.abs(host(M) / Mref - 1)) < 1e-12
 
 
+@pytest.mark.parametrize("n", [5, 4096, 3 * 4096 + 17, 100 * 4096 + 5])
+def test_potential_over_its_inputs(g, n):
+    """Phi or M written over the masses or the radii (a caller short of memory): the
+    same bits as into arrays of their own."""
+    import torch
+    s = sorted_plummer(n, seed=3, masses="salpeter")
+    r, m = dev(s["r"]), dev(s["m"])
+    phi, M = g.stage_potential(r, m, want_M=True)
+    lib, spare = g.load(), torch.empty_like(m)
+    for _ in range(20):
+        a, b = m.clone(), m.clone()
+        assert lib.cmc_potential(n, r.data_ptr(), a.data_ptr(), a.data_ptr(), None, None) == 0
+        assert lib.cmc_potential(n, r.data_ptr(), b.data_ptr(), spare.data_ptr(), b.data_ptr(),
+                                 None) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(a, phi) and torch.equal(b, M) and torch.equal(spare, phi)
+    a, b = r.clone(), m.clone()
+    assert lib.cmc_potential(n, a.data_ptr(), b.data_ptr(), a.data_ptr(), b.data_ptr(), None) == 0
+    assert torch.equal(a, phi) and torch.equal(b, M)
+
+
 @pytest.mark.parametrize("n", [2, 3, 20, 21, 41, 4097, 100_003])
 def test_timestep_bit_exact(g, orc, n):
     s = sorted_plummer(n, seed=7, masses="salpeter")
