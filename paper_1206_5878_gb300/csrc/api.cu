@@ -86,6 +86,7 @@ cmc_status fail(cmc_ctx* ctx, cmc_status s, const std::string& msg) {
 }
 
 cmc_status cuda_fail(cmc_ctx* ctx, cudaError_t e, const char* where) {
+  cudaGetLastError();  // reported here: not the next call's
   std::string msg = std::string(where) + ": " + cudaGetErrorString(e);
   if (e == cudaErrorMemoryAllocation) return fail(ctx, CMC_ENOMEM, msg);
   return fail(ctx, CMC_ECUDA, msg);
@@ -160,7 +161,11 @@ bool staged_in_order(cmc_ctx* c, std::vector<unsigned long long>& bitoff, cudaSt
   const SegLayout& L = c->L;
   bool ordered = false;
   max_id.clear();
-  if (check_order(L, c->r, c->id, st, ordered, max_id) || !ordered) return false;
+  if (check_order(L, c->r, c->id, st, ordered, max_id)) {
+    cudaGetLastError();  // (no scratch: the sorted path)
+    return false;
+  }
+  if (!ordered) return false;
   bitoff.assign((size_t)L.n_seg, 0ull);
   unsigned long long total = 0;
   for (int s = 0; s < L.n_seg; ++s) {
@@ -179,7 +184,10 @@ bool order_in_place(cmc_ctx* c, const std::vector<unsigned long long>& bitoff,
   void* block = nullptr;
   Carve C;
   C.put(dbo, bitoff.data(), bitoff.size());
-  if (C.alloc(block, st)) return false;
+  if (C.alloc(block, st)) {
+    cudaGetLastError();
+    return false;
+  }
   // the bitmap lives in the key scratch (64 bits per star)
   cudaMemsetAsync(c->keys, 0, sizeof(uint64_t) * (size_t)L.n, st);
   launch_place(L, c->r, c->id, dbo, reinterpret_cast<unsigned long long*>(c->keys), c->err, st);

@@ -52,7 +52,10 @@ __global__ void k_check_arith(int op, unsigned long long n, unsigned long long s
 cmc_status cmc_check_arith(int32_t op, uint64_t n, uint64_t seed, uint64_t* mismatches) {
   if (op < 0 || op > 2 || !mismatches) return CMC_EINVAL;
   unsigned long long* d = nullptr;
-  if (cudaMalloc(&d, sizeof(unsigned long long)) != cudaSuccess) return CMC_ECUDA;
+  if (cudaMalloc(&d, sizeof(unsigned long long)) != cudaSuccess) {
+    cudaGetLastError();  // reported here: not the next call's
+    return CMC_ECUDA;
+  }
   cudaError_t e = cudaMemset(d, 0, sizeof(unsigned long long));
   if (!e && n) {
     k_check_arith<<<152 * 8, 256>>>(op, (unsigned long long)n, (unsigned long long)seed, d);
@@ -61,7 +64,10 @@ cmc_status cmc_check_arith(int32_t op, uint64_t n, uint64_t seed, uint64_t* mism
   unsigned long long h = 0;
   if (!e) e = cudaMemcpy(&h, d, sizeof h, cudaMemcpyDeviceToHost);
   cudaFree(d);
-  if (e) return CMC_ECUDA;
+  if (e) {
+    cudaGetLastError();
+    return CMC_ECUDA;
+  }
   *mismatches = (uint64_t)h;
   return CMC_OK;
 }

@@ -1532,7 +1532,10 @@ void Carve::copy(unsigned char* to, const void* from, size_t n) { memcpy(to, fro
 
 cudaError_t Carve::alloc(void*& block, cudaStream_t st) {
   cudaError_t e = cudaMallocAsync(&block, bytes_ ? bytes_ : 1, st);
-  if (e) return e;
+  if (e) {
+    block = nullptr;
+    return e;
+  }
   for (const Part& q : parts_) *q.ptr = (unsigned char*)block + q.at;
   if (zero_ == 0) return cudaSuccess;
   if (image_.size() <= sizeof(CarveImage)) {
@@ -1542,12 +1545,17 @@ cudaError_t Carve::alloc(void*& block, cudaStream_t st) {
     const int64_t words = (int64_t)(zero_ / 16);
     launch_k(k_carve, blocks_for(words, 256), 256, 0, st, (uint4*)block, words,
              (int)(image_.size() / 16), im);
-    return cudaGetLastError();
+    e = cudaGetLastError();
+  } else {
+    e = cudaMemcpyAsync(block, image_.data(), image_.size(), cudaMemcpyHostToDevice, st);
+    if (!e && zero_ > image_.size())
+      e = cudaMemsetAsync((unsigned char*)block + image_.size(), 0, zero_ - image_.size(), st);
+    if (!e) e = cudaStreamSynchronize(st);  // the image lives on the caller's stack
   }
-  e = cudaMemcpyAsync(block, image_.data(), image_.size(), cudaMemcpyHostToDevice, st);
-  if (!e && zero_ > image_.size())
-    e = cudaMemsetAsync((unsigned char*)block + image_.size(), 0, zero_ - image_.size(), st);
-  if (!e) e = cudaStreamSynchronize(st);  // the image lives on the caller's stack
+  if (e) {
+    cudaFreeAsync(block, st);
+    block = nullptr;
+  }
   return e;
 }
 

@@ -36,3 +36,29 @@ def test_bad_values_change_nothing(g_stage, n, bad):
         np.testing.assert_array_equal(a[k], b[k], err_msg=k)
     np.testing.assert_array_equal(c.radii(), twin.radii())
     assert c.stats() == twin.stats()
+
+
+def test_a_failed_call_leaves_nothing_to_the_next(g_stage):
+    """A context whose diagnostics ring does not fit (419 GB: one allocation that is
+    refused at once) is CMC_ENOMEM; the calls after it are as if it had not been."""
+    import torch
+    n = 5000
+    d = ic.plummer(n, seed=1)
+    st = {k: d[k] for k in ("r", "vr", "vt", "m", "id")}
+    r = torch.from_numpy(np.sort(d["r"])).cuda()
+    m = torch.from_numpy(d["m"]).cuda()
+    phi = g_stage.stage_potential(r, m)
+
+    def refused():
+        with pytest.raises(g_stage.CMCError) as ei:
+            g_stage.Cluster(st, list(range(n)), sizes=[1] * n, diag_ring=1 << 20)
+        assert ei.value.status == 2  # CMC_ENOMEM
+
+    refused()
+    assert torch.equal(g_stage.stage_potential(r, m), phi)
+    refused()
+    c = g_stage.Cluster(st, [1], collisions=1)
+    refused()
+    c.set_radii(np.full(n, 1e-9))
+    refused()
+    c.step(1)
