@@ -426,6 +426,8 @@ cmc_status load_state(cmc_ctx* c, const double* r, const double* vr, const doubl
   if (!e) e = cudaStreamWaitEvent(st, c->ev_aux, 0);
   if (e) return cuda_fail(c, e, "ordering the state");
   launch_validate(c->L, c->r, c->vr, c->vt, c->m, allow_inf, c->err, st);
+  e = cudaGetLastError();
+  if (e) return cuda_fail(c, e, "setting the state");
   cmc_status s = check_err_flags(c);
   if (s != CMC_OK) return s;
   if (!placed) {
@@ -688,7 +690,10 @@ cmc_status attr_set(cmc_ctx* c, double* dst, const double* src, int32_t ptr_kind
     // into scratch, checked there, and only then the context's
     uint32_t bad = 0;
     e = cudaMemcpyAsync(c->r_old, src, bytes, cudaMemcpyHostToDevice, st);
-    launch_check_attr(c->L.n, c->r_old, c->pcount, st);
+    if (!e) {
+      launch_check_attr(c->L.n, c->r_old, c->pcount, st);
+      e = cudaGetLastError();
+    }
     if (!e) e = cudaMemcpyAsync(&bad, c->pcount, sizeof(bad), cudaMemcpyDeviceToHost, st);
     if (!e) e = cudaStreamSynchronize(st);
     if (!e && bad) {
@@ -896,7 +901,12 @@ cmc_status cmc_step(cmc_ctx* c, int32_t n_steps) {
       e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
       if (!e) {
         record_step(c, c->cap);
+        const cudaError_t el = cudaGetLastError();
         e = cudaStreamEndCapture(c->cap, &graph);
+        if (!e && el) {
+          cudaGraphDestroy(graph);
+          e = el;
+        }
       }
       if (!e) {
         e = cudaGraphInstantiate(&c->exec[side], graph, 0);
@@ -930,7 +940,8 @@ cmc_status cmc_step_profiled(cmc_ctx* c, int32_t n_steps, double* stage_ms) {
     record_step(c, c->stream, &ev[(size_t)i * (CMC_NSTAGES + 1)]);
     turn_sides(c);
   }
-  cudaError_t e = cudaStreamSynchronize(c->stream);
+  cudaError_t e = cudaGetLastError();
+  if (!e) e = cudaStreamSynchronize(c->stream);
   if (!e) {
     for (int32_t i = 0; i < n_steps; ++i)
       for (int sidx = 0; sidx < CMC_NSTAGES; ++sidx) {
@@ -941,7 +952,10 @@ cmc_status cmc_step_profiled(cmc_ctx* c, int32_t n_steps, double* stage_ms) {
       }
   }
   for (auto& x : ev) cudaEventDestroy(x);
-  if (e) return cuda_fail(c, e, "cmc_step_profiled");
+  if (e) {
+    c->poisoned = true;  // (a step in part)
+    return cuda_fail(c, e, "cmc_step_profiled");
+  }
   c->steps_taken += n_steps;
   return check_err_flags(c);
 }
@@ -951,8 +965,10 @@ cmc_status cmc_energy(cmc_ctx* c, double* out) {
   if (c->poisoned) return fail(c, CMC_EPOISONED, c->last_error);
   DeviceGuard g(c->device);
   launch_energy(c->L, c->r, c->vr, c->vt, c->m, c->tile_a, c->tile_b, c->tile_c, c->out3, c->stream);
-  cudaError_t e = cudaMemcpyAsync(out, c->out3, sizeof(double) * 3 * c->L.n_seg,
-                                  cudaMemcpyDeviceToHost, c->stream);
+  cudaError_t e = cudaGetLastError();
+  if (!e)
+    e = cudaMemcpyAsync(out, c->out3, sizeof(double) * 3 * c->L.n_seg, cudaMemcpyDeviceToHost,
+                        c->stream);
   if (!e) e = cudaStreamSynchronize(c->stream);
   if (e) return cuda_fail(c, e, "cmc_energy");
   return CMC_OK;
@@ -1021,9 +1037,10 @@ cmc_status cmc_lagrange_radii(cmc_ctx* c, const double* fracs, int32_t nf, doubl
   if (!e) {
     launch_masses(c->L, c->m, c->tile_a, c->r_old, st);
     launch_lagrange(c->L, c->r, c->r_old, dfr, nf, dout, st);
-    e = cudaMemcpyAsync(out, dout, sizeof(double) * nf * c->L.n_seg, cudaMemcpyDeviceToHost,
-                        st);
+    e = cudaGetLastError();
   }
+  if (!e)
+    e = cudaMemcpyAsync(out, dout, sizeof(double) * nf * c->L.n_seg, cudaMemcpyDeviceToHost, st);
   if (!e) e = cudaStreamSynchronize(st);
   dfree(dfr, st);
   dfree(dout, st);
@@ -1454,8 +1471,10 @@ cmc_status cmc_orbit(int64_t n, const double* r, const double* phi, const double
                    nullptr, precision == 0 ? &env : nullptr, nullptr, nullptr, orb);
     free_buckets(bk, st);
     free_env(env, st);
-    launch_unpack_orbit(n, ra, rb, r_new, vr_new, vt_new, st);
-    e = cudaGetLastError();
+    if (!e) {
+      launch_unpack_orbit(n, ra, rb, r_new, vr_new, vt_new, st);
+      e = cudaGetLastError();
+    }
   }
   if (!e) e = cudaStreamSynchronize(st);
   dfree(block, st);

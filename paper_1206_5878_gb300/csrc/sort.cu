@@ -751,7 +751,7 @@ cudaError_t sort_segments(const SegLayout& L, SortWork& W, uint64_t* keys, uint3
                         st);
     }
   }
-  return cudaGetLastError();
+  return cudaPeekAtLastError();  // (left for the caller's own look)
 }
 
 void launch_tiefix(const SegLayout& L, uint64_t* keys, uint32_t* vals,
