@@ -83,8 +83,11 @@ constexpr int kDiagFields = 10;      // doubles per diagnostics record
 // blocks of the next kernel resident beside the current one's made it take
 // over the predecessor's split of the SM between L1 and shared memory (N =
 // 1e7 step 5.35 -> 5.70 ms with an early release; 5.36 ms without).  What
-// is gained is the gap between launches, 0.6 us each: step 148 -> 139 us at
-// N = 1021, 245 -> 233 us at 1e5.
+// is gained is the gap between launches, 0.6 us each.
+// Such a kernel's life begins while its predecessor still writes, so none of its
+// loads may go by the non-coherent path, which is for memory that nothing writes
+// while the kernel lives: no __ldg, and no const __restrict__ parameters that the
+// compiler could turn into it.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -113,7 +116,7 @@ __device__ __forceinline__ int seg_find(const int64_t* a, int n, int64_t v) {
   int lo = 0, hi = n;  // invariant a[lo] <= v < a[hi]
   while (hi - lo > 1) {
     int mid = (lo + hi) >> 1;
-    if (__ldg(a + mid) <= v) lo = mid; else hi = mid;
+    if (a[mid] <= v) lo = mid; else hi = mid;
   }
   return lo;
 }
@@ -435,13 +438,13 @@ __device__ __forceinline__ Draws<kTaus> draws_of(const Seg& S, int c, uint32_t i
   d.seed = S.seed[c];
   d.id = id;
   d.step = step;
-  if (kTaus) d.z = S.taus[__ldg(S.taus_base + c) + id];
+  if (kTaus) d.z = S.taus[S.taus_base[c] + id];
   return d;
 }
 
 template <bool kTaus>
 __device__ __forceinline__ void draws_keep(const Seg& S, int c, const Draws<kTaus>& d) {
-  if (kTaus) S.taus[__ldg(S.taus_base + c) + d.id] = d.z;
+  if (kTaus) S.taus[S.taus_base[c] + d.id] = d.z;
 }
 
 // Non-inlined copies of div_rn and sqrt_rn for the relaxation kernel: its
@@ -598,17 +601,17 @@ __device__ __forceinline__ int64_t shell_of(const Table64& t, double q) {
   int64_t lo = -1, hi = t.nb;
   while (hi - lo > 1) {
     int64_t mid = lo + ((hi - lo) >> 1);
-    if (__ldg(rb + mid) <= qb) lo = mid; else hi = mid;
+    if (rb[mid] <= qb) lo = mid; else hi = mid;
   }
   return lo;
 }
 
 // Eq. 6 inside shell i (i = -1: central constant)
 __device__ __forceinline__ double phi_in_shell(const Table64& t, int64_t i, double q) {
-  if (i < 0) return __ldg(t.phi);
+  if (i < 0) return *t.phi;
   double x = div_rn(1.0, q);
-  double xj = __ldg(t.x + i), pj = __ldg(t.phi + i), xj1, pj1;
-  if (i + 1 < t.nb) { xj1 = __ldg(t.x + i + 1); pj1 = __ldg(t.phi + i + 1); }
+  double xj = t.x[i], pj = t.phi[i], xj1, pj1;
+  if (i + 1 < t.nb) { xj1 = t.x[i + 1]; pj1 = t.phi[i + 1]; }
   else { xj1 = 0.0; pj1 = 0.0; }
   double den = xj - xj1;
   if (!(den > 0.0)) return pj;

@@ -139,10 +139,9 @@ __host__ __device__ __forceinline__ BinShape bin_shape(int bs, bool by_pairs) {
 }
 
 template <bool kCentral, bool kPairs>
-__global__ void __launch_bounds__(kBinThreads) k_bins(Seg S, int bs, double pref, const double* r,
-                                                      const double* vr, const double* vt,
-                                                      const double* m, double* nbin,
-                                                      Central C) {
+__global__ void __launch_bounds__(kBinThreads, kCentral ? 5 : 6) k_bins(
+    Seg S, int bs, double pref, const double* r, const double* vr, const double* vt,
+    const double* m, double* nbin, Central C) {
   pdl_enter();
   int64_t blk = blockIdx.x;
   if (kCentral) {
@@ -484,7 +483,7 @@ __global__ void k_taus_init(int64_t slots, int n_seg, const int64_t* base, const
       const uint32_t* col = P + ((size_t)j * 32 + b) * 32;
       uint32_t r = 0u;
       for (int i = 0; i < 32; ++i)
-        if ((v[j] >> i) & 1u) r ^= __ldg(col + i);
+        if ((v[j] >> i) & 1u) r ^= col[i];
       v[j] = r;
     }
   table[e] = make_uint4(v[0], v[1], v[2], v[3]);

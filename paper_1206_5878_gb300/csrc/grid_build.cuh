@@ -58,13 +58,13 @@ __device__ __forceinline__ void grid_build(const Seg& S, const int64_t* esc, con
   float rel = 0.0f;
   if (g < pr.z) {
     if (fused && g == 0) {
-      gaux[c].x = (float)__ldg(phi + sb);
+      gaux[c].x = (float)phi[sb];
       gaux[c].y = (float)node[sb + nb - 1].w;
     }
     const double xg = (double)__uint_as_float((uint32_t)pr.x + ((uint32_t)g << pr.y));
     const double xn = (double)__uint_as_float((uint32_t)pr.x + ((uint32_t)(g + 1) << pr.y));
     const int64_t lo = gshell[p];
-    double ph = __ldg(phi + sb);
+    double ph = phi[sb];
     if (lo >= 0) {
       const double2 a = node_xp(node + sb + lo);
       ph = a.y + slope(lo) * (a.x - xg);

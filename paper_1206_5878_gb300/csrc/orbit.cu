@@ -38,17 +38,17 @@ __device__ __forceinline__ double Qv(const Star& s, double x, double p) {
 }
 
 __device__ __forceinline__ double Q_node64(const Table64& T, const Star& s, int64_t i) {
-  double L = s.J * __ldg(T.x + i);
-  return scale_up<1>(s.E - __ldg(T.phi + i)) - L * L;
+  double L = s.J * T.x[i];
+  return scale_up<1>(s.E - T.phi[i]) - L * L;
 }
 
 // root of Q inside shell j (nodes j, j+1; node nb is 1/r = 0, Phi = 0)
 __device__ __forceinline__ double shell_root64(const Table64& T, const Star& s, int64_t j,
                                                bool outer) {
-  const double rj = __ldg(T.r + j), xj = __ldg(T.x + j), pj = __ldg(T.phi + j);
+  const double rj = T.r[j], xj = T.x[j], pj = T.phi[j];
   double rj1, xj1, pj1;
   const bool has_next = j + 1 < T.nb;
-  if (has_next) { rj1 = __ldg(T.r + j + 1); xj1 = __ldg(T.x + j + 1); pj1 = __ldg(T.phi + j + 1); }
+  if (has_next) { rj1 = T.r[j + 1]; xj1 = T.x[j + 1]; pj1 = T.phi[j + 1]; }
   else { rj1 = __longlong_as_double(0x7FF0000000000000ll); xj1 = 0.0; pj1 = 0.0; }
   if (!(xj - xj1 > 0.0)) return rj;
   const double B = div_rn(pj1 - pj, xj - xj1);
@@ -124,7 +124,7 @@ __device__ __forceinline__ double rmin_core(const Star& s, bool central, double 
 // compares of the radii's bits) from a guess i by a bounded walk, then a
 // bisection, on the node records; a receives that shell's record (node 0's
 // for -1).  The records of the guess and its successor are loaded together.
-__device__ __forceinline__ int64_t fix_shell_nodes(const double4_32a* __restrict__ nd, int64_t nb,
+__device__ __forceinline__ int64_t fix_shell_nodes(const double4_32a* nd, int64_t nb,
                                                    int64_t i, double q, double4_32a& a) {
   if (!ge0(q)) {
     a = nd[0];
@@ -161,9 +161,9 @@ __device__ __forceinline__ int64_t fix_shell_nodes(const double4_32a* __restrict
 }
 
 __device__ __forceinline__ double central_root64(const Table64& T, const Star& s) {
-  double rmin = div_rn(s.J, sqrt_rn(scale_up<1>(s.E - __ldg(T.phi))));
+  double rmin = div_rn(s.J, sqrt_rn(scale_up<1>(s.E - *T.phi)));
   if (!(rmin >= 0.0)) rmin = 0.0;
-  const double r0 = __ldg(T.r);
+  const double r0 = *T.r;
   if (rmin > r0) rmin = r0;
   return rmin;
 }
@@ -237,7 +237,7 @@ struct Buckets {
 // (about 47 G/s).
 // K queries at once, so that their looks at the index overlap.
 template <int K>
-__device__ __forceinline__ void near_shells(const double4_32a* __restrict__ nd, int nb,
+__device__ __forceinline__ void near_shells(const double4_32a* nd, int nb,
                                             const Buckets& B, const float (&xq)[K],
                                             int (&out)[K]) {
   int s0[K], s1[K];
@@ -247,8 +247,8 @@ __device__ __forceinline__ void near_shells(const double4_32a* __restrict__ nd, 
     const long long b = d >> B.shift;
     s0[q] = s1[q] = -1;
     if (d >= 0 && b < B.nbk && CMC_IN(b + 1, B.nbk + 1)) {
-      s0[q] = __ldg(B.start + b);
-      s1[q] = __ldg(B.start + b + 1);
+      s0[q] = B.start[b];
+      s1[q] = B.start[b + 1];
     }
   }
 #pragma unroll
@@ -302,14 +302,14 @@ __device__ __forceinline__ Grid grid_of(const BucketArgs& B, int c) {
 __device__ __forceinline__ float grid_phi(const Grid& G, float xq) {
   const uint32_t key = __float_as_uint(xq);
   if (key >= G.kmax) return G.phi0;                               // inside the first star
-  if (key < G.key0) return __ldg(G.phi) + G.mb * (G.x0 - xq);     // beyond the last
+  if (key < G.key0) return *G.phi + G.mb * (G.x0 - xq);     // beyond the last
   const uint32_t d = key - G.key0;
   const int g = (int)(d >> G.sh);
   if (!CMC_IN(g + 1, G.cells)) return G.phi0;
   // f = (d mod 2^sh) 2^-sh, exact: 1 + f assembled from its bits, minus 1
   const float f =
       __uint_as_float(0x3F800000u | ((d & ((1u << G.sh) - 1u)) << (23 - G.sh))) - 1.0f;
-  const float a = __ldg(G.phi + g), b = __ldg(G.phi + g + 1);
+  const float a = G.phi[g], b = G.phi[g + 1];
   return a + f * (b - a);
 }
 
@@ -333,7 +333,7 @@ __device__ __forceinline__ float g32_grid(const Grid& G, float E, float J, float
 
 // about the shell of the point r(s) (bucket index), the start of the FP64
 // shell walk of an accepted or edge point
-__device__ __forceinline__ int shell32_of(const double4_32a* __restrict__ nd, int nb,
+__device__ __forceinline__ int shell32_of(const double4_32a* nd, int nb,
                                           const Buckets& B, float c0, float c1, float sv) {
   const float rs = c0 + c1 * (sv * (3.0f - sv * sv));
   float xq;
@@ -347,7 +347,7 @@ __device__ __forceinline__ int shell32_of(const double4_32a* __restrict__ nd, in
 // Mixed mode: the orbit point r(s) in FP64 from an FP32 shell index sh
 // (moved to the exact shell), Phi from the enclosed-mass slope of its
 // shell (Eq. 6: Phi = Phi_i + M_i (1/r_i - 1/r)), L = J / r and Q.
-__device__ __forceinline__ void point64(const double4_32a* __restrict__ nd, int64_t nb,
+__device__ __forceinline__ void point64(const double4_32a* nd, int64_t nb,
                                         const Star& st, double c0, double c1, double sv, int sh,
                                         double& rs, double& xs, double& ph, double& L,
                                         double& Q, int& i64) {
@@ -366,7 +366,7 @@ __device__ __forceinline__ void point64(const double4_32a* __restrict__ nd, int6
 // statement of the method, as phi_in_shell), L = J / r and Q.
 // sa = s (3 - s^2), the factor of c1 in r(s) (a table entry at the
 // envelope's samples)
-__device__ __forceinline__ void point64_div_sa(const double4_32a* __restrict__ nd, int64_t nb,
+__device__ __forceinline__ void point64_div_sa(const double4_32a* nd, int64_t nb,
                                                const Star& st, double c0, double c1, double sa,
                                                int sh, double& rs, double& ph, double& Q,
                                                double& L, double& xq, int& i) {
@@ -390,7 +390,7 @@ __device__ __forceinline__ void point64_div_sa(const double4_32a* __restrict__ n
   Q = scale_up<1>(st.E - ph) - L * L;
 }
 
-__device__ __forceinline__ void point64_div(const double4_32a* __restrict__ nd, int64_t nb,
+__device__ __forceinline__ void point64_div(const double4_32a* nd, int64_t nb,
                                             const Star& st, double c0, double c1, double sv,
                                             int sh, double& rs, double& ph, double& Q,
                                             double& L, double& xq, int& i) {
@@ -507,7 +507,7 @@ struct Bracket {
 };
 
 __device__ __forceinline__ bool walk_sign(const Star& s, const WalkStar& W,
-                                          const double4_32a* __restrict__ nd, int nb, int p,
+                                          const double4_32a* nd, int nb, int p,
                                           int lo, int hi, bool at_hi, double2 at, Bracket& B) {
   const unsigned long long xb = ubits(at.x), pb = ubits(at.y);
   const float ex = pow2_of(xb), ep = pow2_of(pb);
@@ -557,7 +557,7 @@ __device__ __forceinline__ bool walk_sign(const Star& s, const WalkStar& W,
 // Q in FP32 at grid point g (1/r from the grid key, Phi from the grid)
 __device__ __forceinline__ float grid_q(const Grid& G, float E, float J2, int g, float& xg) {
   xg = __uint_as_float(G.key0 + ((uint32_t)g << G.sh));
-  return __fmaf_rn(-J2 * xg, xg, 2.0f * (E - __ldg(G.phi + g)));
+  return __fmaf_rn(-J2 * xg, xg, 2.0f * (E - G.phi[g]));
 }
 
 // Node brackets of both turning points: r_max's node j with Q >= 0 (the star
@@ -576,7 +576,7 @@ __device__ __forceinline__ float grid_q(const Grid& G, float E, float J2, int g,
 // FP64 walks where uncertified 1.27 ms, 338 B.  Both walks in one loop (1.08),
 // four-way grid rounds (1.08), the grid's top levels in shared memory (1.01)
 // and 40 to 64 registers (0.98 to 1.01) gave nothing.
-__device__ __forceinline__ bool grid_brackets(const Grid& G, const double4_32a* __restrict__ nd,
+__device__ __forceinline__ bool grid_brackets(const Grid& G, const double4_32a* nd,
                                               const Buckets& BK, const Star& s, int nb, int k,
                                               float xk, float qk, Bracket& bmax,
                                               Bracket& bmin) {
@@ -643,7 +643,7 @@ __device__ __forceinline__ bool grid_brackets(const Grid& G, const double4_32a* 
 // grid and the nodes, or where a walk gives up by FP64 bisection, then the FP64
 // roots inside the bracketing shells (Eq. 12).
 __device__ __forceinline__ void turning_mixed(const Table64& T,
-                                              const double4_32a* __restrict__ nd, const Grid& G,
+                                              const double4_32a* nd, const Grid& G,
                                               const Buckets& BK, const Star& s, float xk,
                                               float qk, double& rmin, double& rmax) {
   const int nb = (int)T.nb, k = (int)s.k;
@@ -683,7 +683,7 @@ __global__ void __launch_bounds__(256, kMinB) k_turning_mixed(
   const double rk = r[p], vrk = vr[p], vtk = vt[p];
   Star s;
   s.k = k;
-  s.E = __ldg(T.phi + k) + scale_down<1>(vrk * vrk + vtk * vtk);
+  s.E = T.phi[k] + scale_down<1>(vrk * vrk + vtk * vtk);
   s.J = rk * vtk;
   // E < 0 on the bit pattern (negative, nonzero, not NaN); otherwise an
   // escaper, which the sampling kernel handles
@@ -848,7 +848,7 @@ __global__ void k_env_tables() {
 }
 
 // FP64 g at sample j of a star (one copy for the list and the spill loops)
-__device__ __noinline__ double g64_sample(const double4_32a* __restrict__ nd, int64_t nb,
+__device__ __noinline__ double g64_sample(const double4_32a* nd, int64_t nb,
                                           const Buckets& BK, double E, double J, double c0,
                                           double c1, int j) {
   Star s;
@@ -1101,7 +1101,7 @@ __global__ void __launch_bounds__(256, kMinB) k_sample32(Seg S, int max_trials,
       const Grid GD = grid_of(BA, c);
       bool degenerate;
       if (kExact) {
-        const double F64 = 1.2 * __ldg(Fx + p);
+        const double F64 = 1.2 * Fx[p];
         F32 = f32_rn(F64);
         degenerate = !gt_pos(c1, 0.0) || !(F64 > 0.0);
       } else {
@@ -1314,7 +1314,7 @@ __device__ __forceinline__ void pending_star(Seg S, int max_trials, const uint32
         const double c0 = o.z, c1 = o.w;
         const float c0f = f32_rn(c0), c1f = f32_rn(c1);
         const double F =
-            kExact ? 1.2 * __ldg(Fx + p) : (double)__uint_as_float((uint32_t)(res >> 32));
+            kExact ? 1.2 * Fx[p] : (double)__uint_as_float((uint32_t)(res >> 32));
         uint32_t st = kSmpCap;
         int t = (int)(res & 0x3FFFFFFFull);
         // stream mode: the blocks of trials 0 .. t-1 were the FP32 sampler's
@@ -1521,18 +1521,18 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
     c0o = o.z;
     c1o = o.w;
   } else {
-    s.E = __ldg(T.phi + k) + scale_down<1>(vrk * vrk + vtk * vtk);
+    s.E = T.phi[k] + scale_down<1>(vrk * vrk + vtk * vtk);
     s.J = rk * vtk;
   }
   Draws<kTaus> g = draws_of<kTaus>(S, c, idk, *step_p);
-  double ph_new = __ldg(T.phi + k);
+  double ph_new = T.phi[k];
 
   if (!lt0(s.E)) {
     escaped = true;
     code = 1;
     r_new = inf;
     // energy carried off: the star's energy in the field of the others
-    B.c = __ldg(T.phi + k) + div_rn(A.m, rk) + scale_down<1>(vrk * vrk + vtk * vtk);
+    B.c = T.phi[k] + div_rn(A.m, rk) + scale_down<1>(vrk * vrk + vtk * vtk);
   } else {
     int64_t jmax, jmin;
     Buckets BK;
@@ -1550,8 +1550,8 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
       jmin = bisect_rmin64(T, s);
     } else if (dbg.rmin) {
       // turning points from k_turning_mixed (for the stage outputs)
-      rmin = __ldg(tp_min + p);
-      rmax = __ldg(tp_max + p);
+      rmin = tp_min[p];
+      rmax = tp_max[p];
     }
     if (kPrec == 0) {
       rmax = shell_root64(T, s, jmax, true);
@@ -1603,7 +1603,7 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
           x_new = div_rn(1.0, rs_a);
           B.vr = (sg.x & 1u) ? -sq : sq;
           B.vt = div_rn(s.J, rs_a);
-          B.c = __ldg(T.phi + k) - ph_a;
+          B.c = T.phi[k] - ph_a;
           ph_new = ph_a;
         }
       }
@@ -1613,7 +1613,7 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
       const uint64_t res = keys[p];
       const uint32_t st = (uint32_t)(res >> 30) & 3u;
       int t = (int)(res & 0x3FFFFFFFull);
-      F = kPrec == 2 ? 1.2 * __ldg(Fx + p) : (double)__uint_as_float((uint32_t)(res >> 32));
+      F = kPrec == 2 ? 1.2 * Fx[p] : (double)__uint_as_float((uint32_t)(res >> 32));
       if (st == kSmpDegenerate) {
         code = 2;
       } else if (st == kSmpCap) {
@@ -1652,7 +1652,7 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
           r_new = rs;
           B.vr = (sg.x & 1u) ? -sq : sq;
           B.vt = vtn;
-          B.c = __ldg(T.phi + k) - ph;
+          B.c = T.phi[k] - ph;
           ph_new = ph;
         }
       }
@@ -1660,7 +1660,7 @@ __global__ void __launch_bounds__(256, kMinB) k_orbit(Seg S, int max_trials, con
   }
   // a star that stays in place has no point from the way: its shell by bisection
   if (!escaped && shell == -2) {
-    x_new = __ldg(T.x + k);
+    x_new = T.x[k];
     if (bo.bin) shell = (int)shell_of(T, rk);
   }
   A.r = r_new;
@@ -1740,10 +1740,10 @@ __global__ void k_grid_shells(Seg S, const int64_t* esc, bool sub, const double*
   const int64_t sb = S.off[c], k = p - sb;
   const int4 pr = B.gprm[c];
   const bool live = k < nb;
-  grid_shells_of(mask, live, (int)k, (int)nb, live ? grid_last_cell(__ldg(x + p), pr) : -1,
-                 live && k + 1 < nb ? grid_last_cell(__ldg(x + p + 1), pr) : -1, pr,
+  grid_shells_of(mask, live, (int)k, (int)nb, live ? grid_last_cell(x[p], pr) : -1,
+                 live && k + 1 < nb ? grid_last_cell(x[p + 1], pr) : -1, pr,
                  gshell + B.goff[c]);
-  if (live && k == 0) grid_close(grid_last_cell(__ldg(x + p), pr), pr, gshell + B.goff[c], 0, 1);
+  if (live && k == 0) grid_close(grid_last_cell(x[p], pr), pr, gshell + B.goff[c], 0, 1);
 }
 
 __global__ void k_grid_build(Seg S, const int64_t* esc, GridBuild G) {

@@ -65,10 +65,10 @@ __device__ __forceinline__ TileRange tile_range(const int64_t* off, const int64_
                                                 int n_seg, int64_t t, int tile) {
   TileRange R;
   R.seg = seg_find(tile_off, n_seg, t);
-  R.lt = t - __ldg(tile_off + R.seg);
-  R.seg_begin = __ldg(off + R.seg);
+  R.lt = t - tile_off[R.seg];
+  R.seg_begin = off[R.seg];
   R.begin = R.seg_begin + R.lt * tile;
-  int64_t se = __ldg(off + R.seg + 1);
+  int64_t se = off[R.seg + 1];
   R.end = R.begin + tile < se ? R.begin + tile : se;
   return R;
 }
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kThreads) k_upsweep(const int64_t* off, const 
   TileRange R = tile_range(off, tile_off, n_seg, blockIdx.x, kTile);
   uint32_t* hw = h + (size_t)warp * passes * kBins;
   for (int64_t p = R.begin + threadIdx.x; p < R.end; p += kThreads) {
-    const uint64_t k = __ldg(keys + p);
+    const uint64_t k = keys[p];
     for (int q = 0; q < passes; ++q)
       atomicAdd(&hw[q * kBins + (int)((k >> (8 * (first_pass + q))) & 0xFF)], 1u);
   }
@@ -177,8 +177,8 @@ constexpr int kRankBallot = 1;  // nine __ballot_sync
 template <bool kValIdentity, int IPT, int kRank>
 __global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 6 : 3))
     k_pass(const int64_t* off, const int64_t* tile_off, int n_seg, int64_t n_tiles,
-           const uint64_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
-           uint64_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out, int pass, int q,
+           const uint64_t* keys_in, const uint32_t* vals_in,
+           uint64_t* keys_out, uint32_t* vals_out, int pass, int q,
            int passes, const uint32_t* base, unsigned long long* desc, uint32_t* tickets,
            uint32_t* err) {
   pdl_enter();
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 6 : 3))
 
   // contiguous runs per digit go out coalesced; a destination outside the
   // segment (possible only after a timed-out look-back) is dropped
-  const int64_t seg_end = __ldg(off + R.seg + 1);
+  const int64_t seg_end = off[R.seg + 1];
   for (int lp = tid; lp < n_items; lp += kThreads) {
     uint64_t kk = S.key[lp];
     int dd = (int)((kk >> shift) & 0xFF);
@@ -328,7 +328,7 @@ __global__ void k_tiefix(const int64_t* off, int n_seg, int64_t n, uint64_t* key
     return;
   }
   int c = seg_find(off, n_seg, p);
-  int64_t sb = __ldg(off + c), se = __ldg(off + c + 1);
+  int64_t sb = off[c], se = off[c + 1];
   const uint64_t kp = keys[p], hp = kp >> shift;
   if (p + 1 >= se || (keys[p + 1] >> shift) != hp) return;
   if (p > sb && (keys[p - 1] >> shift) == hp) return;  // not the start of the run
