@@ -281,7 +281,8 @@ void record_step(cmc_ctx* c, cudaStream_t st, cudaEvent_t* ev = nullptr) {
   mark(4);
   uint32_t* ord = c->W.vals_alt;
   if (binned) {
-    launch_bin_sort(L, c->bins, c->vals, c->ra, ord, c->order, counted, c->err, st);
+    launch_bin_sort(L, c->bins, c->vals, c->ra, ord, c->order, c->keys, c->W.keys_alt, counted,
+                    c->err, st);
   } else {
     // radix passes over bits 24-63 of the radius keys; runs equal in those
     // bits (radii within 2^-28 of each other, escapers whose ids differ in

@@ -221,18 +221,31 @@ __device__ __forceinline__ void store_rec(RecB* p, const RecB& b) {
 // order inside a bin, which the gather settles by (r, id).  Bins of segment
 // c: cbase[c] + s + 1 for the stars in shell s = -1 .. nb - 1, then the
 // escapers by id >> esh[c].  Runs of more than kRunMax stars in one bin are
-// listed and sorted by one block each.
+// listed and sorted by a kernel of their own (k_long_runs).
 struct BinWork {
   int64_t* cbase = nullptr;             // n_seg + 1 first bins
   int* esh = nullptr;                   // per segment: ids per escaper bin (a shift)
   uint32_t* cnt = nullptr;              // counts, then positions; zero between steps
   unsigned long long* desc = nullptr;   // look-back words of the scan; zero between steps
-  uint32_t* ctl = nullptr;              // [0] scan tickets, [1] listed runs; zero between steps
-  uint2* runs = nullptr;                // listed runs: first position, length
+  uint32_t* ctl = nullptr;              // kCtl words; zero between steps
+  uint2* runs = nullptr;                // listed runs of up to kRunTile: first position, length
+  uint4* big = nullptr;                 // longer ones: first position, length, their tiles
   std::vector<int64_t> h_cbase;
   int64_t n_bins = 0, n_tiles = 0;      // bins padded to whole scan tiles
 };
 constexpr int kRunMax = 32;
+constexpr int kRunTile = 2048;          // stars of a long run per block
+enum : int {
+  kCtlScan,   // the scan's tickets
+  kCtlRuns,   // listed runs of up to kRunTile
+  kCtlBig,    // longer ones
+  kCtlTiles,  // their tiles
+  kCtlMost,   // tiles of the longest
+  kCtlNext,   // k_long_runs' tickets
+  kCtlDone,   // tiles it has done, over all passes
+  kCtlLeft,   // blocks that have left it
+  kCtlWords
+};
 constexpr int kBinTile = 4096;          // bins per block of the scan
 cudaError_t alloc_bins(BinWork& B, const SegLayout& L, cudaStream_t st);
 void free_bins(BinWork& B, cudaStream_t st);
@@ -242,10 +255,10 @@ cudaError_t set_bin_ids(BinWork& B, const SegLayout& L, const unsigned int* max_
 // order (n indices): the stars' indices in bin order, the order inside a bin
 // left to the gather except in the listed runs, which are in (r, id) order.
 // bin (n): each star's bin; counted: the orbit step has counted the bins.
-// scratch: n indices.
+// scratch: n indices; keys, keys_scratch: n keys each (long runs).
 void launch_bin_sort(const SegLayout& L, BinWork& B, const uint32_t* bin, const RecA* rec,
-                     uint32_t* order, uint32_t* scratch, bool counted, uint32_t* err,
-                     cudaStream_t st);
+                     uint32_t* order, uint32_t* scratch, uint64_t* keys, uint64_t* keys_scratch,
+                     bool counted, uint32_t* err, cudaStream_t st);
 
 // keys of the current state (radius_key of r, id)
 void launch_make_keys(const SegLayout& L, const double* r, const uint32_t* id, uint64_t* keys,

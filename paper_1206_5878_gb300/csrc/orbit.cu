@@ -1433,7 +1433,17 @@ __device__ __forceinline__ void put_star(const Seg& S, const BinOut& O, uint64_t
     if (s < 0) s = nc + 1 + (int64_t)(A.id >> O.esh[c]);
     A.bin = (uint32_t)(O.cbase[c] + s);
     O.bin[p] = A.bin;
-    if (O.cnt) atomicAdd(O.cnt + A.bin, 1u);
+    if (O.cnt) {
+      // (stars crowding into few bins: the lanes of a bin together, as k_bin_count)
+      const unsigned on = __activemask();
+      const uint32_t lane = threadIdx.x & 31u, next = __shfl_down_sync(on, A.bin, 1);
+      if (__any_sync(on, next == A.bin && lane < 31u)) {
+        const unsigned peers = __match_any_sync(on, A.bin);
+        if ((int)lane == __ffs(peers) - 1) atomicAdd(O.cnt + A.bin, (uint32_t)__popc(peers));
+      } else {
+        atomicAdd(O.cnt + A.bin, 1u);
+      }
+    }
   } else {
     keys[p] = radius_key(A.r, A.id);
   }

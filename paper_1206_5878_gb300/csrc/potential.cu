@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kGatThreads, kGatThreads == 512 ? 3 : kGatThre
           equal += eq;
         };
         for (int q = wp - 1; q >= 0 && left < kRunMax && bin_at(q) == b; --q, ++left) look(q);
-        for (int q = wp + 1; q < kGatWin && right < kRunMax && bin_at(q) == b; ++q, ++right)
+        for (int q = wp + 1; q < kGatWin && left + right < kRunMax && bin_at(q) == b; ++q, ++right)
           look(q);
         if (left + 1 + right <= kRunMax) f = wp - left + before;
         else equal = left > 0 && r_at(wp - 1) == r ? (left > 1 && r_at(wp - 2) == r ? 2 : 1) : 0;
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kGatThreads, kGatThreads == 512 ? 3 : kGatThre
     uint4* c4 = reinterpret_cast<uint4*>(cnt);
     for (int64_t i = g; i < n_bins / 4; i += step) c4[i] = make_uint4(0u, 0u, 0u, 0u);
     for (int64_t i = g; i < n_desc; i += step) desc[i] = 0ull;
-    if (g < 2) ctl[g] = 0u;
+    if (g < kCtlWords) ctl[g] = 0u;
   }
 }
 

@@ -371,12 +371,35 @@ __global__ void k_tiefix(const int64_t* off, int n_seg, int64_t n, uint64_t* key
 // by random atomics and 4-byte stores in the L2, against 0.54 ms for the five
 // 8-bit radix passes it replaced in the timestep (keys with the index packed
 // into their low bits, histograms, tie fix).
+// Stars crowding into few bins: a warp in which a thread finds all its four in one
+// adds to each bin with its lanes together (atomics on one address go at 2.4 a
+// nanosecond: 10^6 stars in two bins counted in 424 us, 28 so).  (Two neighbours in one bin are common
+// enough among few stars to make the sort of 1021 slower, 11.3 us against 10.0.)
+__device__ __forceinline__ bool crowded(const uint4& b) {
+  return __any_sync(__activemask(), b.x == b.y && b.y == b.z && b.z == b.w);
+}
+// this lane's place among the lanes that add to the same counter
+__device__ __forceinline__ uint32_t add_together(uint32_t* a, uint32_t bin) {
+  const unsigned peers = __match_any_sync(__activemask(), bin), lane = threadIdx.x & 31;
+  const int first = __ffs(peers) - 1;
+  uint32_t old = 0u;
+  if ((int)lane == first) old = atomicAdd(a + bin, (uint32_t)__popc(peers));
+  return __shfl_sync(peers, old, first) + __popc(peers & ((1u << lane) - 1u));
+}
+
 __global__ void __launch_bounds__(256) k_bin_count(int64_t n, const uint32_t* bin,
                                                    uint32_t* cnt) {
   pdl_enter();
   const int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (p0 + 4 <= n) {
     const uint4 b = *reinterpret_cast<const uint4*>(bin + p0);
+    if (crowded(b)) {
+      add_together(cnt, b.x);
+      add_together(cnt, b.y);
+      add_together(cnt, b.z);
+      add_together(cnt, b.w);
+      return;
+    }
     atomicAdd(cnt + b.x, 1u);
     atomicAdd(cnt + b.y, 1u);
     atomicAdd(cnt + b.z, 1u);
@@ -390,24 +413,25 @@ __global__ void __launch_bounds__(256) k_bin_count(int64_t n, const uint32_t* bi
 // ticket order, the sum of the tiles before by decoupled look-back, one warp
 // reading 32 tiles' words at a time.  Each wait is bounded (g_spin_cap polls
 // of a window that is not complete).  Bins with more than kRunMax stars are
-// listed.
+// listed, those with more than kRunTile with their share of the work's tiles.
 __global__ void __launch_bounds__(kThreads) k_bin_scan(uint32_t* cnt, unsigned long long* desc,
-                                                       uint32_t* ctl, uint2* runs,
+                                                       uint32_t* ctl, uint2* runs, uint4* big,
                                                        uint32_t* err) {
   pdl_enter();
   __shared__ uint32_t s_warp[kWarps];
   __shared__ uint32_t s_tile, s_excl;
   constexpr int kPer = kBinTile / kThreads;  // 16 consecutive bins per thread
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_tile = atomicAdd(ctl, 1u);
+  if (tid == 0) s_tile = atomicAdd(ctl + kCtlScan, 1u);
   __syncthreads();
   const int64_t t = s_tile;
   uint4* mine = reinterpret_cast<uint4*>(cnt + t * kBinTile + tid * kPer);
   uint4 c[kPer / 4];
-  uint32_t sum = 0;
+  uint32_t sum = 0, most = 0;
 #pragma unroll
   for (int i = 0; i < kPer / 4; ++i) {
     c[i] = mine[i];
+    most = max(max(max(c[i].x, c[i].y), max(c[i].z, c[i].w)), most);
     sum += c[i].x + c[i].y + c[i].z + c[i].w;
   }
   const uint32_t before = block_excl_scan_u32(sum, s_warp);
@@ -449,10 +473,24 @@ __global__ void __launch_bounds__(kThreads) k_bin_scan(uint32_t* cnt, unsigned l
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       o[k] = at;
-      if (v[k] > (uint32_t)kRunMax) runs[atomicAdd(ctl + 1, 1u)] = make_uint2(at, v[k]);
       at += v[k];
     }
     mine[i] = make_uint4(o[0], o[1], o[2], o[3]);
+  }
+  if (most <= (uint32_t)kRunMax) return;
+  const uint32_t* from = reinterpret_cast<const uint32_t*>(mine);
+#pragma unroll 1
+  for (int i = 0; i < kPer; ++i) {
+    const uint32_t p = from[i], len = (i + 1 < kPer ? from[i + 1] : at) - p;
+    if (len <= (uint32_t)kRunMax) continue;
+    const uint32_t nt = (len + kRunTile - 1) / kRunTile;
+    if (nt == 1u) {
+      runs[atomicAdd(ctl + kCtlRuns, 1u)] = make_uint2(p, len);
+    } else {
+      atomicMax(ctl + kCtlMost, nt);
+      const uint32_t b = atomicAdd(ctl + kCtlTiles, nt);
+      big[atomicAdd(ctl + kCtlBig, 1u)] = make_uint4(p, len, b, b + nt);
+    }
   }
 }
 
@@ -469,8 +507,14 @@ __global__ void __launch_bounds__(256) k_bin_scatter(int64_t n, const uint32_t* 
   };
   if (p0 + 4 <= n) {
     const uint4 b = *reinterpret_cast<const uint4*>(bin + p0);
-    const uint32_t a0 = atomicAdd(at + b.x, 1u), a1 = atomicAdd(at + b.y, 1u),
-                   a2 = atomicAdd(at + b.z, 1u), a3 = atomicAdd(at + b.w, 1u);
+    uint32_t a0, a1, a2, a3;
+    if (crowded(b)) {
+      a0 = add_together(at, b.x), a1 = add_together(at, b.y);
+      a2 = add_together(at, b.z), a3 = add_together(at, b.w);
+    } else {
+      a0 = atomicAdd(at + b.x, 1u), a1 = atomicAdd(at + b.y, 1u);
+      a2 = atomicAdd(at + b.z, 1u), a3 = atomicAdd(at + b.w, 1u);
+    }
     put(a0, p0);
     put(a1, p0 + 1);
     put(a2, p0 + 2);
@@ -482,118 +526,248 @@ __global__ void __launch_bounds__(256) k_bin_scatter(int64_t n, const uint32_t* 
 
 // The listed runs (more than kRunMax stars in one bin: new radii crowding
 // into one shell of the old table, as when a thin shell of stars spreads out)
-// in (r, id) order: one block per run, a stable radix sort of the run's
-// indices by id, then by the bits of r, over the digits that differ.  A step
-// without such runs finds the list empty.
-constexpr int kRunItems = 8;  // indices per thread and chunk
-__global__ void __launch_bounds__(kThreads) k_long_runs(int64_t n, const uint32_t* ctl,
-                                                        const uint2* runs, const RecA* rec,
-                                                        uint32_t* order, uint32_t* scratch,
-                                                        const uint32_t* err) {
-  pdl_enter();
-  if (*err & kErrTimeout) {
-    // After a timed-out look-back the order is not a permutation: the stars stay
-    // where they are, so that what follows up to the report reads stars only.
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * blockDim.x)
-      order[p] = (uint32_t)p;
-    return;
-  }
-  __shared__ uint32_t whist[kWarps][kBins];
-  __shared__ uint32_t base[kBins], s_warp[kWarps];
-  __shared__ unsigned long long s_dr;
-  __shared__ uint32_t s_di;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const unsigned lt_mask = lanemask_lt();
-  const uint32_t nr = ctl[1];
-  for (uint32_t l = blockIdx.x; l < nr; l += gridDim.x) {
-    const uint2 run = runs[l];
-    const uint32_t len = run.y;
-    if ((int64_t)run.x + len > n) continue;  // only after a timed-out look-back
-    uint32_t* in = order + run.x;
-    uint32_t* out = scratch + run.x;
-    // the bits in which the run's radii and ids differ
-    if (tid == 0) {
-      s_dr = 0ull;
-      s_di = 0u;
-    }
-    __syncthreads();
-    bool ok = true;
-    unsigned long long dr = 0ull;
-    uint32_t di = 0u;
-    const uint32_t first = in[0];
-    if ((int64_t)first < n) {
-      const unsigned long long r0 = ubits(rec[first].r);
-      const uint32_t i0 = rec[first].id;
-      for (uint32_t i = tid; i < len; i += kThreads) {
-        const uint32_t v = in[i];
-        if ((int64_t)v >= n) { ok = false; break; }
-        dr |= ubits(rec[v].r) ^ r0;
-        di |= rec[v].id ^ i0;
-      }
+// in (r, id) order.  A step without such runs finds the lists empty.
+//
+// A run of up to kRunTile stars is sorted by one block in shared memory.  A longer
+// one is a merge sort over all blocks: its tiles are sorted like that, then every
+// pass merges pairs of sorted stretches, one tile of the result per block, whose
+// part of the two stretches a search along the merge's diagonal finds.  (r, id) is
+// a strict order, so the result is the one order whatever the input's, which the
+// scatter's atomics decide.  Blocks take their work by ticket in the order tiles,
+// short runs, first pass, second pass ...; a tile of a pass waits until all of the
+// pass before it are done, which were all taken by blocks that run already.
+// Each wait is bounded (g_spin_cap polls).
+//
+// Nearly all stars in two runs, sort stage of 3 x 10^4, 2 x 10^5, 10^6, 10^7 stars: 0.10,
+// 0.16, 0.30, 2.3 ms (at 10^6 0.24 of it this kernel); by the radix passes 0.07, 0.08,
+// 0.13, 0.76; with one block to a run, as the first three were before, 0.76, 5.2, 27.
+constexpr int64_t kRunBlocks = 608;  // four to an SM (two: the million's 0.28 ms)
+struct RunSmem {
+  unsigned long long key[kRunTile];
+  uint32_t idx[kRunTile], id[kRunTile];
+  uint32_t item, cut[2];
+  uint4 run;
+  bool ok;
+};
+
+// order[0 .. len) -> out, by (r, id); keys (may be null): the bits of r
+__device__ __forceinline__ void sort_run_tile(RunSmem& S, const RecA* rec, const uint32_t* in,
+                                              uint32_t* out, unsigned long long* keys,
+                                              uint32_t len) {
+  const uint32_t tid = threadIdx.x;
+  uint32_t size = 64;
+  while (size < len) size <<= 1;
+  for (uint32_t i = tid; i < size; i += kThreads) {
+    const uint32_t v = i < len ? in[i] : 0u;
+    if (i < len) {
+      const RecA A = load_rec(rec + v);
+      S.key[i] = ubits(A.r);
+      S.id[i] = A.id;
     } else {
-      ok = false;
+      S.key[i] = ~0ull;  // (above every radius: stays at the end)
+      S.id[i] = ~0u;
     }
-    atomicOr(&s_dr, dr);
-    atomicOr(&s_di, di);
-    ok = __syncthreads_and(ok);
-    if (!ok) continue;  // only after a timed-out look-back
-    dr = s_dr;
-    di = s_di;
-    for (int q = 0; q < 12; ++q) {
-      const bool by_id = q < 4;
-      const int shift = 8 * (by_id ? q : q - 4);
-      if (!(by_id ? (di >> shift) & 255u : (uint32_t)(dr >> shift) & 255u)) continue;
-      auto digit = [&](uint32_t v) {
-        return (int)((by_id ? (unsigned long long)rec[v].id : ubits(rec[v].r)) >> shift) & 255;
-      };
-      base[tid] = 0u;
-      __syncthreads();
-      for (uint32_t i = tid; i < len; i += kThreads) atomicAdd(&base[digit(in[i])], 1u);
-      __syncthreads();
-      const uint32_t excl = block_excl_scan_u32(base[tid], s_warp);
-      __syncthreads();
-      base[tid] = excl;
-      for (uint32_t c0 = 0; c0 < len; c0 += kThreads * kRunItems) {
-        for (int i = tid; i < kWarps * kBins; i += kThreads) (&whist[0][0])[i] = 0u;
-        __syncthreads();
-        // warp w owns a contiguous stretch of the chunk (as k_pass)
-        uint32_t v[kRunItems], rank[kRunItems];
-        int dg[kRunItems];
-#pragma unroll
-        for (int i = 0; i < kRunItems; ++i) {
-          const uint32_t e = c0 + (uint32_t)(warp * (32 * kRunItems) + i * 32 + lane);
-          v[i] = e < len ? in[e] : 0u;
-          dg[i] = e < len ? digit(v[i]) : kBins;
-          const unsigned peers = __match_any_sync(0xffffffffu, dg[i]);
-          uint32_t old = 0u;
-          if (lane == __ffs(peers) - 1 && dg[i] < kBins)
-            old = atomicAdd(&whist[warp][dg[i]], (uint32_t)__popc(peers));
-          __syncwarp();
-          rank[i] = __shfl_sync(0xffffffffu, old, __ffs(peers) - 1) + __popc(peers & lt_mask);
-        }
-        __syncthreads();
-        uint32_t at = base[tid];
-        for (int w = 0; w < kWarps; ++w) {
-          const uint32_t k = whist[w][tid];
-          whist[w][tid] = at;
-          at += k;
-        }
-        base[tid] = at;
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < kRunItems; ++i)
-          if (dg[i] < kBins) out[whist[warp][dg[i]] + rank[i]] = v[i];
-        __syncthreads();
-      }
-      uint32_t* sw = in;
-      in = out;
-      out = sw;
-    }
-    if (in != order + run.x)
-      for (uint32_t i = tid; i < len; i += kThreads) out[i] = in[i];
-    __syncthreads();
+    S.idx[i] = v;
   }
+  __syncthreads();
+  // bitonic sort; a warp's 32 pairs lie in 64 neighbours while j <= 32
+  for (uint32_t k = 2; k <= size; k <<= 1)
+    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+      for (uint32_t t = tid; t < size / 2; t += kThreads) {
+        const uint32_t a = 2 * t - (t & (j - 1)), b = a + j;
+        const unsigned long long ka = S.key[a], kb = S.key[b];
+        const uint32_t ia = S.id[a], ib = S.id[b];
+        const bool a_first = ka < kb || (ka == kb && ia < ib);
+        if (a_first != ((a & k) == 0u)) {
+          S.key[a] = kb;
+          S.key[b] = ka;
+          S.id[a] = ib;
+          S.id[b] = ia;
+          const uint32_t v = S.idx[a];
+          S.idx[a] = S.idx[b];
+          S.idx[b] = v;
+        }
+      }
+      if (j > 32 || (j == 1 && k >= 64)) __syncthreads();
+      else __syncwarp();
+    }
+  for (uint32_t i = tid; i < len; i += kThreads) {
+    out[i] = S.idx[i];
+    if (keys) keys[i] = S.key[i];
+  }
+}
+
+struct RunBuf {
+  unsigned long long* key;
+  uint32_t* idx;
+};
+
+// Of the first d of the merge of stretches a (na) and b (nb), how many come from
+// a: by one warp, 32 probes a round.  (Written by other blocks of this kernel: read
+// past the L1.)
+__device__ __forceinline__ uint32_t merge_cut(const RunBuf& in, const RecA* rec, uint32_t a,
+                                              uint32_t na, uint32_t b, uint32_t nb, uint32_t d) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t lo = d > nb ? d - nb : 0u, hi = d < na ? d : na;
+  while (lo < hi) {
+    const unsigned long long span = hi - lo;
+    const uint32_t m = lo + (uint32_t)(span * lane / 32u);
+    const uint32_t pa = a + m, pb = b + (d - 1u - m);
+    const unsigned long long ka = __ldcg(in.key + pa), kb = __ldcg(in.key + pb);
+    const bool from_a =
+        ka < kb || (ka == kb && rec[__ldcg(in.idx + pa)].id < rec[__ldcg(in.idx + pb)].id);
+    const uint32_t k = (uint32_t)__popc(__ballot_sync(0xffffffffu, from_a));
+    // the first k probes come from a (probes rise with the lane)
+    if (k == 0) return lo;
+    hi = k == 32u ? hi : lo + (uint32_t)(span * k / 32u);
+    lo = lo + (uint32_t)(span * (k - 1u) / 32u) + 1u;
+  }
+  return lo;
+}
+
+// tile t of a run of len stars from first on: merged from the stretches of width w
+__device__ __forceinline__ void merge_run_tile(RunSmem& S, const RecA* rec, const RunBuf& in,
+                                               const RunBuf& out, uint32_t first, uint32_t len,
+                                               uint32_t t, uint32_t w) {
+  const uint32_t tid = threadIdx.x, o = t * kRunTile, pair = o / (2u * w) * (2u * w);
+  const uint32_t rest = len - pair;  // (w <= len: the last pass has 2 w >= len > w)
+  const uint32_t na = rest < w ? rest : w, nb = rest - na < w ? rest - na : w;
+  const uint32_t a = first + pair, b = a + na;
+  const uint32_t d0 = o - pair;
+  const uint32_t d1 = d0 + kRunTile < na + nb ? d0 + kRunTile : na + nb;
+  if (tid < 64) {
+    const uint32_t cut = merge_cut(in, rec, a, na, b, nb, tid < 32 ? d0 : d1);
+    if ((tid & 31u) == 0u) S.cut[tid >> 5] = cut;
+  }
+  __syncthreads();
+  const uint32_t c0 = S.cut[0], ta = S.cut[1] - c0, all = d1 - d0, tb = all - ta;
+  for (uint32_t i = tid; i < all; i += kThreads) {
+    const uint32_t p = i < ta ? a + c0 + i : b + (d0 - c0) + (i - ta);
+    S.key[i] = __ldcg(in.key + p);
+    S.idx[i] = __ldcg(in.idx + p);
+  }
+  __syncthreads();
+  auto from_a = [&](uint32_t x, uint32_t y) {
+    const unsigned long long ka = S.key[x], kb = S.key[y];
+    return ka < kb || (ka == kb && rec[S.idx[x]].id < rec[S.idx[y]].id);
+  };
+  constexpr uint32_t kPer = kRunTile / kThreads;
+  const uint32_t e = tid * kPer;
+  unsigned long long k[kPer];
+  uint32_t v[kPer];
+  if (e < all) {
+    uint32_t lo = e > tb ? e - tb : 0u, hi = e < ta ? e : ta;
+    while (lo < hi) {
+      const uint32_t m = (lo + hi) >> 1;
+      if (from_a(m, ta + (e - 1u - m))) lo = m + 1u; else hi = m;
+    }
+    uint32_t x = lo, y = ta + (e - lo);
+#pragma unroll
+    for (uint32_t i = 0; i < kPer; ++i) {
+      const bool left = x < ta && (y >= all || from_a(x, y));
+      const uint32_t q = left ? x++ : (y < all ? y++ : all - 1u);  // (past the end: not stored)
+      k[i] = S.key[q];
+      v[i] = S.idx[q];
+    }
+  }
+  __syncthreads();
+  if (e < all) {
+#pragma unroll
+    for (uint32_t i = 0; i < kPer; ++i) {
+      S.key[e + i] = k[i];
+      S.idx[e + i] = v[i];
+    }
+  }
+  __syncthreads();
+  for (uint32_t i = tid; i < all; i += kThreads) {
+    out.key[first + o + i] = S.key[i];
+    out.idx[first + o + i] = S.idx[i];
+  }
+}
+
+// the listed runs' work, by all blocks; false: a wait gave up
+__device__ __forceinline__ bool long_runs(RunSmem& S, uint32_t* ctl, const uint2* runs,
+                                          const uint4* big, const RecA* rec, const RunBuf& home,
+                                          const RunBuf& away, uint32_t nr, uint32_t nt,
+                                          uint32_t* err) {
+  const uint32_t passes = nt ? 32u - (uint32_t)__clz((int)(ctl[kCtlMost] - 1u)) : 0u;
+  const uint32_t total = nt + nr + passes * nt, nb = ctl[kCtlBig];
+  const int cap = g_spin_cap;
+  // the long run that tile i belongs to: first star, length, tile there
+  auto run_of = [&](uint32_t i) {
+    for (uint32_t l = threadIdx.x; l < nb; l += kThreads) {
+      const uint4 t = big[l];
+      if (t.z <= i && i < t.w) S.run = make_uint4(t.x, t.y, i - t.z, 0u);
+    }
+    __syncthreads();
+    return S.run;
+  };
+  for (;;) {
+    if (threadIdx.x == 0) S.item = atomicAdd(ctl + kCtlNext, 1u);
+    __syncthreads();
+    const uint32_t item = S.item;
+    if (item >= total) return true;
+    if (item >= nt && item < nt + nr) {
+      const uint2 run = runs[item - nt];
+      sort_run_tile(S, rec, home.idx + run.x, home.idx + run.x, nullptr, run.y);
+      __syncthreads();
+      continue;
+    }
+    if (item < nt) {
+      // the passes end at home
+      const RunBuf& out = passes & 1u ? away : home;
+      const uint4 t = run_of(item);
+      const uint32_t o = t.z * kRunTile, len = t.y - o < kRunTile ? t.y - o : kRunTile;
+      sort_run_tile(S, rec, home.idx + t.x + o, out.idx + t.x + o, out.key + t.x + o, len);
+    } else {
+      const uint32_t q = (item - nt - nr) / nt;
+      if (threadIdx.x == 0) {
+        int spins = 0;
+        S.ok = true;
+        while (*(volatile uint32_t*)(ctl + kCtlDone) < (q + 1u) * nt) {
+          if (++spins > cap || (*(volatile uint32_t*)err & kErrTimeout)) {
+            set_err(err, kErrTimeout);
+            S.ok = false;
+            break;
+          }
+          if (spins > 32) __nanosleep(64);
+        }
+        __threadfence();
+      }
+      __syncthreads();
+      if (!S.ok) return false;
+      const uint4 t = run_of((item - nt - nr) % nt);
+      const bool from_home = ((passes ^ q) & 1u) == 0u;
+      merge_run_tile(S, rec, from_home ? home : away, from_home ? away : home, t.x, t.y, t.z,
+                     (uint32_t)kRunTile << q);
+    }
+    __threadfence();  // this tile before its mark
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(ctl + kCtlDone, 1u);
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) k_long_runs(int64_t n, uint32_t* ctl,
+                                                        const uint2* runs, const uint4* big,
+                                                        const RecA* rec, RunBuf home, RunBuf away,
+                                                        uint32_t* err) {
+  pdl_enter();
+  const uint32_t nr = ctl[kCtlRuns], nt = ctl[kCtlTiles];
+  bool lost = *err & kErrTimeout;
+  if (nr + nt == 0u && !lost) return;
+  __shared__ RunSmem S;
+  if (!lost) long_runs(S, ctl, runs, big, rec, home, away, nr, nt, err);
+  // After a wait that gave up, here or in the scan, the order is not a permutation:
+  // the last block to leave puts the stars where they are, so that what follows up
+  // to the report reads stars only.
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    S.ok = atomicAdd(ctl + kCtlLeft, 1u) == gridDim.x - 1u && (*(volatile uint32_t*)err & kErrTimeout);
+  }
+  __syncthreads();
+  if (S.ok)
+    for (int64_t p = threadIdx.x; p < n; p += kThreads) home.idx[p] = (uint32_t)p;
 }
 
 __global__ void k_philox(int64_t n, const uint32_t* ctr, uint64_t seed, uint32_t* out) {
@@ -776,19 +950,21 @@ cudaError_t alloc_bins(BinWork& B, const SegLayout& L, cudaStream_t st) {
   if ((e = cudaMallocAsync((void**)&B.esh, sizeof(int) * L.n_seg, st))) return e;
   if ((e = cudaMallocAsync((void**)&B.cnt, sizeof(uint32_t) * B.n_bins, st))) return e;
   if ((e = cudaMallocAsync((void**)&B.desc, sizeof(unsigned long long) * B.n_tiles, st))) return e;
-  if ((e = cudaMallocAsync((void**)&B.ctl, sizeof(uint32_t) * 2, st))) return e;
+  if ((e = cudaMallocAsync((void**)&B.ctl, sizeof(uint32_t) * kCtlWords, st))) return e;
   if ((e = cudaMallocAsync((void**)&B.runs, sizeof(uint2) * (L.n / kRunMax + 1), st))) return e;
+  if ((e = cudaMallocAsync((void**)&B.big, sizeof(uint4) * (L.n / kRunTile + 1), st)))
+    return e;
   e = cudaMemcpyAsync(B.cbase, o.data(), sizeof(int64_t) * o.size(), cudaMemcpyHostToDevice, st);
   if (!e) e = cudaMemsetAsync(B.cnt, 0, sizeof(uint32_t) * B.n_bins, st);
   if (!e) e = cudaMemsetAsync(B.desc, 0, sizeof(unsigned long long) * B.n_tiles, st);
-  if (!e) e = cudaMemsetAsync(B.ctl, 0, sizeof(uint32_t) * 2, st);
+  if (!e) e = cudaMemsetAsync(B.ctl, 0, sizeof(uint32_t) * kCtlWords, st);
   if (e) return e;
   const std::vector<unsigned int> any((size_t)L.n_seg, 0xFFFFFFFFu);
   return set_bin_ids(B, L, any.data(), st);
 }
 
 void free_bins(BinWork& B, cudaStream_t st) {
-  void* ps[] = {B.cbase, B.esh, B.cnt, B.desc, B.ctl, B.runs};
+  void* ps[] = {B.cbase, B.esh, B.cnt, B.desc, B.ctl, B.runs, B.big};
   for (void* p : ps)
     if (p) cudaFreeAsync(p, st);
   B = BinWork();
@@ -808,16 +984,19 @@ cudaError_t set_bin_ids(BinWork& B, const SegLayout& L, const unsigned int* max_
 }
 
 void launch_bin_sort(const SegLayout& L, BinWork& B, const uint32_t* bin, const RecA* rec,
-                     uint32_t* order, uint32_t* scratch, bool counted, uint32_t* err,
-                     cudaStream_t st) {
+                     uint32_t* order, uint32_t* scratch, uint64_t* keys, uint64_t* keys_scratch,
+                     bool counted, uint32_t* err, cudaStream_t st) {
   if (L.n == 0) return;
   const unsigned grid = (unsigned)((L.n + 1023) / 1024);
   if (!counted) launch_k(k_bin_count, grid, 256, 0, st, L.n, bin, B.cnt);
-  launch_k(k_bin_scan, (unsigned)B.n_tiles, kThreads, 0, st, B.cnt, B.desc, B.ctl, B.runs, err);
+  launch_k(k_bin_scan, (unsigned)B.n_tiles, kThreads, 0, st, B.cnt, B.desc, B.ctl, B.runs, B.big,
+           err);
   launch_k(k_bin_scatter, grid, 256, 0, st, L.n, bin, B.cnt, order, err);
   const int64_t most = L.n / kRunMax + 1;  // listed runs at most
-  launch_k(k_long_runs, (unsigned)(most < 152 ? most : 152), kThreads, 0, st, L.n, B.ctl, B.runs,
-           rec, order, scratch, err);
+  const RunBuf home{reinterpret_cast<unsigned long long*>(keys), order};
+  const RunBuf away{reinterpret_cast<unsigned long long*>(keys_scratch), scratch};
+  launch_k(k_long_runs, (unsigned)(most < kRunBlocks ? most : kRunBlocks), kThreads, 0, st, L.n,
+           B.ctl, B.runs, B.big, rec, home, away, err);
 }
 
 void launch_philox(int64_t n, const uint32_t* ctr, uint64_t seed, uint32_t* out,

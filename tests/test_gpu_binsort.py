@@ -54,6 +54,64 @@ def test_runs_in_one_shell(g_stage, n, precision):
     assert np.all(np.diff(sa["r"][fin]) >= 0)
 
 
+@pytest.mark.parametrize("n", [300_000, 1_000_003])
+def test_runs_of_many_tiles(g_stage, n):
+    """The new radii of a thin shell: two runs of hundreds of tiles, merged in many
+    passes, the bins counted in the orbit step's kernels (300,000) or apart."""
+    _same(g_stage, _thin_shell(n, n, 1.2), [3], precision=1, steps=2)
+
+
+def test_very_many_runs_of_all_lengths(g_stage):
+    """Shells of 40 to 10,000 stars far apart, whose new radii lie just inside and just
+    outside of them: more listed runs than blocks, short ones and ones of several
+    tiles."""
+    g = np.random.default_rng(8)
+    lengths = np.concatenate([g.integers(40, 140, 900), [4000, 4096, 4200, 8000, 8192, 10_000]])
+    g.shuffle(lengths)
+    at = np.repeat(np.geomspace(1e-3, 1e3, len(lengths)), lengths)
+    n = len(at)
+    d = {"r": at * (1.0 + 1e-9 * g.random(n)), "m": np.full(n, 1.0 / n),
+         "id": g.permutation(n).astype(np.uint32)}
+    order = np.argsort(d["r"])
+    inside = np.empty(n)
+    inside[order] = (np.arange(n) + 1.0) / n
+    v = np.sqrt(inside / d["r"])
+    d["vr"], d["vt"] = 1e-3 * v * g.standard_normal(n), v * (1.0 + 1e-3 * g.standard_normal(n))
+    _same(g_stage, d, [3], precision=1)
+    _same(g_stage, d, [3], precision=0, max_trials=1)
+
+
+@pytest.mark.parametrize("length", [32, 33, 64, 65, 2047, 2048, 2049, 4096, 4097, 9000])
+def test_run_of_exactly(g_stage, length):
+    """One radius many times over, by id: escapers in one bin (one star's large id
+    makes the bins of ids that wide), as many as fill a list's entry, a tile, two."""
+    n = 20_000
+    d = ic.plummer(n, seed=5)
+    g = np.random.default_rng(length)
+    d["id"] = g.permutation(n).astype(np.uint32)
+    fast = g.choice(n, length + 1, replace=False)
+    d["id"][fast[0]] = 2**32 - 1
+    d["vr"][fast[1:]] *= 100.0
+    d["vt"][fast[1:]] *= 100.0
+    for precision in (0, 1):
+        sa = _same(g_stage, d, [5], precision=precision, steps=1, gamma=1e-9)  # no relaxation
+        out = ~np.isfinite(sa["r"])
+        assert out.sum() == length and np.all(np.diff(sa["id"][out].astype(np.int64)) > 0)
+
+
+def test_no_slow_case_where_radii_crowd(g_stage):
+    """The sort of a million stars in two bins within a small multiple of the radix
+    passes' time (twice measured; one block for each run took two hundred times)."""
+    d, t = _thin_shell(1_000_000, 2, 1.2), {}
+    for packed in (0, 1):
+        c = g_stage.Cluster(d, [3], precision=1, autotune=0, sort_packed=packed)
+        st, t[packed] = c.get_state(), np.inf
+        for _ in range(4):
+            c.set_state(st, 0)
+            t[packed] = min(t[packed], c.step_profiled(1)["sort"])
+    assert t[1] < 10.0 * t[0]
+
+
 def test_runs_across_tile_edges(g_stage):
     """Two thin shells inside a Plummer sphere: long runs beside runs of one
     or two stars, starting and ending anywhere in the tiles."""
