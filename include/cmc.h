@@ -109,13 +109,18 @@ typedef struct {
     int32_t max_trials;         /* rejection trials per star per step (1000) */
     int32_t energy_correction;  /* 1: apply the section 2.1 step 6 correction */
     int32_t orbit_block;        /* threads per block of the orbit kernel: 0 (auto) or a multiple of 32 up to 256 */
-    int32_t autotune;           /* 1: at cmc_init, time the sort shapes (and the
-                                   orbit block size when orbit_block is 0) on
-                                   the real state and keep the fastest; results
-                                   do not depend on the choice (default 1) */
+    int32_t autotune;           /* 1: at cmc_init, time on the real state, and keep
+                                   the fastest of, the orbit block sizes (when
+                                   orbit_block is 0), the orbit and relaxation
+                                   variants where they apply and, with
+                                   sort_packed = 0, the radix sort's shapes;
+                                   results do not depend on the choice
+                                   (default 1) */
     int32_t orbit_variant;      /* FP32 sampler kernel variant, precision 0 and 1 (listed at
                                    cmc_get_tuning): -1 = the autotuner's choice
-                                   (0 without autotune), or 0..6 (default -1) */
+                                   (0 without autotune), or 0..6 (default -1).
+                                   Only for more than 49,152 stars in all: with
+                                   fewer, lanes share a star, in one shape */
     int32_t rng;                /* 0: counter-based Philox4x32-10 draws keyed by
                                    (star id, step, purpose, trial) (default);
                                    1: the paper's combined Tausworthe generator
@@ -131,7 +136,10 @@ typedef struct {
                                    sampler runs one launch shape */
     int32_t relax_variant;      /* relaxation kernel variant (listed at
                                    cmc_get_tuning): -1 = the autotuner's choice
-                                   (0 without autotune), or 0..2 (default -1) */
+                                   (0 without autotune), or 0..2 (default -1).
+                                   Only for more than 16,384 pairs (or rng = 1):
+                                   with fewer, two lanes share a pair, in one
+                                   shape */
     int32_t collisions;         /* 1: stars carry radii (cmc_set_radii): the
                                    collision timestep of Eq. 8 joins Eq. 7's, and
                                    relaxation pairs may merge as sticky spheres
@@ -295,13 +303,15 @@ enum {
  * identical to cmc_step. */
 cmc_status cmc_step_profiled(cmc_ctx *ctx, int32_t n_steps, double *stage_ms);
 
-/* Kernel shapes in use (chosen by autotune or the configuration): out
- * (host, 5) = {orbit threads per block, sort keys per thread, sort
- * multisplit (0: match, 1: ballot), mixed-mode orbit variant (registers per
- * thread capped for 1 (no cap), 2, 3, 4, 5, 6 or 8 resident 256-thread
- * blocks per SM: variants 0..6), relaxation variant (registers per thread
- * capped for 1 (no cap), 6 or 8 resident 128-thread blocks per SM:
- * variants 0..2)}.  All shapes give bit-identical results. */
+/* Kernel shapes chosen by autotune or the configuration: out (host, 5) =
+ * {orbit threads per block, radix sort keys per thread, radix sort multisplit
+ * (0: match, 1: ballot), orbit variant (registers per thread of the FP32 sampler
+ * capped for 1 (no cap), 2, 3, 4, 5, 6 or 8 resident 256-thread blocks per SM:
+ * variants 0..6), relaxation variant (registers per thread capped for 1 (no
+ * cap), 6 or 8 resident 128-thread blocks per SM: variants 0..2)}.  The radix
+ * shapes are those of states set in no order, and of the timesteps only with
+ * sort_packed = 0; the variants run only where they apply (cmc_config), and
+ * autotune leaves them at 0 elsewhere.  All shapes give bit-identical results. */
 cmc_status cmc_get_tuning(const cmc_ctx *ctx, int32_t *out);
 
 /* Number of kernels one cmc_step timestep launches. */

@@ -603,14 +603,15 @@ cmc_status autotune(cmc_ctx* c) {
     }
     return best;
   };
-  // orbit block size and (sampled step) kernel variant
-  const int n_var = tab ? kOrbitVariants : 1;
+  // orbit block size and, where the sampler has them, kernel variant
+  const int n_var = tab && sampler_has_variants(L) ? kOrbitVariants : 1;
   int blk_best = c->cfg.orbit_block ? c->cfg.orbit_block : 64, var_best = c->orbit_variant;
   float tb = 3.4e38f;
-  for (int var = 0; var < n_var; ++var)
+  for (int v = 0; v < n_var; ++v)
     for (int blk : {64, 128, 256}) {
+      const int var = n_var > 1 ? v : c->orbit_variant;
       if (c->cfg.orbit_block && blk != c->cfg.orbit_block) continue;
-      if (tab && c->cfg.orbit_variant >= 0 && var != c->cfg.orbit_variant) continue;
+      if (n_var > 1 && c->cfg.orbit_variant >= 0 && var != c->cfg.orbit_variant) continue;
       const float ms = time_it([&] { run_orbit(blk, var); });
       if (ms < tb) { tb = ms; blk_best = blk; var_best = var; }
     }
@@ -619,7 +620,7 @@ cmc_status autotune(cmc_ctx* c) {
   // relaxation kernel variant: on copies of the velocities (r_old and cc
   // are free scratch here), after the bins of this state; the timestep the
   // bins leave is put back
-  if (c->cfg.relax_variant < 0 && L.n_pairs) {
+  if (c->cfg.relax_variant < 0 && L.n_pairs && !relax_two_lanes(L)) {
     uint64_t* dt_saved = reinterpret_cast<uint64_t*>(c->tile_c);
     cudaMemcpyAsync(dt_saved, L.dt_bits, sizeof(uint64_t) * L.n_seg, cudaMemcpyDeviceToDevice,
                     st);

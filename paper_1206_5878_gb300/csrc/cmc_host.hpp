@@ -442,6 +442,17 @@ void launch_potential_tables(const SegLayout& L, const double* r, const double* 
                              bool nb_sub, bool sums_ready, BucketWork& B, cudaStream_t st,
                              GridBuild* later = nullptr, double* recip = nullptr);
 
+// Lanes to a star in the kernels that share a star's samples and trials among
+// lanes while there are few stars (k_env_screen, k_sample32: times there).
+inline int star_lanes(const SegLayout& L) { return L.n <= 16384 ? 8 : L.n <= 49152 ? 4 : 1; }
+// ... in the sampler: one where draws come in sequence.  With more than one, and
+// in stream mode, it has one shape, whatever variant is asked for.
+inline int sampler_lanes(const SegLayout& L) { return L.taus ? 1 : star_lanes(L); }
+inline bool sampler_has_variants(const SegLayout& L) { return !L.taus && sampler_lanes(L) == 1; }
+// two lanes to a pair in the relaxation while there are few pairs (k_relax), in one
+// shape
+inline bool relax_two_lanes(const SegLayout& L) { return !L.taus && L.n_pairs <= 16384; }
+
 // launch_orbit writes the stars' records, and with bins their sort bins (count:
 // counted too) or else their sort keys.  precision 1 (mixed): it runs four kernels (turning points,
 // FP32 sampler, FP64 continuation of the pending stars, finishing) and

@@ -297,8 +297,7 @@ struct Collide {
 // angles, takes one of each two roots that do not depend on each other, and
 // finishes one of the stars: the stage of 10^3, 10^4, 3 x 10^4 stars 16.3, 17.4, 17.9 us
 // with a lane a pair, 14.5, 14.9, 16.9 with two; 22.4 and 28.9 at 10^5, where the
-// FP64 pipe has work enough.
-constexpr int64_t kTwoLanes = 16384;
+// FP64 pipe has work enough (the rule is relax_two_lanes).
 
 template <bool kTaus, int kMinB, bool kCol, bool kTwo>
 __global__ void __launch_bounds__(128, kMinB) k_relax(Seg S, int bs, double* vr, double* vt,
@@ -520,7 +519,7 @@ template <int kMinB>
 static void relax_shape(const SegLayout& L, double* vr, double* vt, double* m,
                         const uint32_t* id, const double* nbin, const uint32_t* step,
                         const Collide& col, cudaStream_t st) {
-  const bool two = !L.taus && L.n_pairs <= kTwoLanes;
+  const bool two = relax_two_lanes(L);
   const unsigned grid = (unsigned)((L.n_pairs * (two ? 2 : 1) + 127) / 128);
   // (the collision code only in the kernels that need it: it costs
   // registers)

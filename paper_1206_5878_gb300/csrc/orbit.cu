@@ -1065,7 +1065,7 @@ enum : uint32_t { kSmpAccepted = 0, kSmpPending = 1, kSmpDegenerate = 2, kSmpCap
 // take kG trials at a time, the first one that is accepted or undecided counts.
 // Orbit stage of 10^3, 10^4, 3 x 10^4, 6 x 10^4 stars 24.9, 29.1, 30.8, 32.9 us with a
 // lane, 22.4, 23.8, 26.7, 32.9 with four, 20.4, 22.8, 28.6, 36.3 with eight.
-constexpr int64_t kSample8 = 16384, kSample4 = 49152;
+// (The rule is sampler_lanes.)
 constexpr int kOwnTrials = 2;
 
 template <int kMinB, bool kTaus, bool kExact, int kG>
@@ -1996,7 +1996,7 @@ void launch_orbit(const SegLayout& L, int precision, int max_trials, const doubl
   do {                                                                                      \
     if (with_turning) CMC_TURN(B);                                                          \
     if (X) {                                                                                \
-      const int g = L.n <= kSample8 ? 8 : L.n <= kSample4 ? 4 : 1;                          \
+      const int g = star_lanes(L);                                                          \
       launch_k(g == 8   ? k_env_screen<8>                                                   \
                : g == 4 ? k_env_screen<4>                                                   \
                         : k_env_screen<1>,                                                  \
@@ -2004,7 +2004,7 @@ void launch_orbit(const SegLayout& L, int precision, int max_trials, const doubl
                L.dev(), ba, orb, W, L.n);                                                   \
       launch_k(k_env_eval, egrid, kEnvThreads, 0, st, L.dev(), ba, W);                             \
     }                                                                                       \
-    const int ahead = T ? 1 : L.n <= kSample8 ? 8 : L.n <= kSample4 ? 4 : 1;                 \
+    const int ahead = sampler_lanes(L);                                                     \
     launch_k(ahead == 8   ? k_sample32<4, false, X, 8>                                      \
              : ahead == 4 ? k_sample32<4, false, X, 4>                                      \
                           : k_sample32<B, T, X, 1>,                                         \

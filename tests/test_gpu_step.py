@@ -227,6 +227,20 @@ def test_autotuned_shapes_do_not_change_bits(g, precision):
     assert a.stats() == b.stats()
 
 
+@pytest.mark.parametrize("n,rng,orbit,relax", [(2000, 0, False, False), (32_769, 0, False, False),
+                                               (49_152, 0, False, True), (49_153, 0, True, True),
+                                               (2000, 1, False, True)])
+def test_variants_are_tuned_where_they_apply(g, n, rng, orbit, relax):
+    """The tuner leaves the variants of kernels that have one shape at 0 (of seven and
+    three, so three contexts would hardly all give 0 by timing); a forced one is kept."""
+    d = ic.plummer(n, seed=6)
+    got = [_cluster(g, d, 6, precision=1, rng=rng).tuning() for _ in range(3)]
+    assert orbit or [t["orbit_variant"] for t in got] == [0, 0, 0]
+    assert relax or [t["relax_variant"] for t in got] == [0, 0, 0]
+    t = _cluster(g, d, 6, precision=1, rng=rng, orbit_variant=3, relax_variant=1).tuning()
+    assert t["orbit_variant"] == 3 and t["relax_variant"] == 1
+
+
 def test_host_and_device_inputs_agree(g):
     import torch
     d = ic.plummer(5000, seed=8)
