@@ -44,7 +44,7 @@ struct cmc_ctx {
   std::vector<unsigned int> taus_max_id;  // per segment: the last id with a stream (rng 1)
   double *r_old = nullptr, *cc = nullptr, *nbin = nullptr;
   double *tile_a = nullptr, *tile_b = nullptr, *tile_c = nullptr,
-         *out3 = nullptr, *fr = nullptr, *lag = nullptr;
+         *out3 = nullptr;
   uint32_t* err = nullptr;
   uint32_t* step = nullptr;
   uint32_t* pcount = nullptr;  // pending stars of the sampled orbit step
@@ -352,8 +352,7 @@ void free_ctx(cmc_ctx* c) {
   for (cudaGraphExec_t e : c->exec)
     if (e) cudaGraphExecDestroy(e);
   double** ds[] = {&c->r_alt, &c->x_alt, &c->r, &c->x, &c->vr, &c->vt, &c->m, &c->phi, &c->r_old,
-                   &c->cc, &c->nbin, &c->tile_a, &c->tile_b, &c->tile_c, &c->out3,
-                   &c->fr, &c->lag};
+                   &c->cc, &c->nbin, &c->tile_a, &c->tile_b, &c->tile_c, &c->out3};
   for (double** p : ds) dfree(*p, st);
   dfree(c->id, st);
   dfree(c->R, st);

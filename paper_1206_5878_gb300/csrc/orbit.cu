@@ -30,13 +30,6 @@ struct Star {
   int64_t k;
 };
 
-
-// Q = 2 (E - Phi) - (J x)^2 from node values, as Q_node64 evaluates it
-__device__ __forceinline__ double Qv(const Star& s, double x, double p) {
-  const double L = s.J * x;
-  return 2.0 * (s.E - p) - L * L;
-}
-
 __device__ __forceinline__ double Q_node64(const Table64& T, const Star& s, int64_t i) {
   double L = s.J * T.x[i];
   return scale_up<1>(s.E - T.phi[i]) - L * L;
