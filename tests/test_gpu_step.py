@@ -188,9 +188,10 @@ def test_resume_is_bit_identical(g):
     np.testing.assert_array_equal(a.escaped(), c.escaped())
 
 
+@pytest.mark.parametrize("n", [20_000, 70_001])  # one shape of shared lanes; all variants
 @pytest.mark.parametrize("precision", [0, 1, 2])
-def test_launch_shape_does_not_change_bits(g, precision):
-    d = ic.plummer(20_000, seed=4)
+def test_launch_shape_does_not_change_bits(g, precision, n):
+    d = ic.plummer(n, seed=4)
     outs = []
     shapes = [(32, 0, 0), (128, 0, 1), (256, 0, 2)]
     if precision != 2:
@@ -207,9 +208,10 @@ def test_launch_shape_does_not_change_bits(g, precision):
         assert st == outs[0][1]
 
 
+@pytest.mark.parametrize("n", [30_001, 70_001])
 @pytest.mark.parametrize("precision", [0, 1, 2])
-def test_autotuned_shapes_do_not_change_bits(g, precision):
-    d = ic.plummer(30_001, seed=6, masses="salpeter")
+def test_autotuned_shapes_do_not_change_bits(g, precision, n):
+    d = ic.plummer(n, seed=6, masses="salpeter")
     a = _cluster(g, d, 6, autotune=0, precision=precision)
     b = _cluster(g, d, 6, autotune=1, precision=precision)
     ta, tb = a.tuning(), b.tuning()
@@ -217,7 +219,7 @@ def test_autotuned_shapes_do_not_change_bits(g, precision):
                   "orbit_variant": 0, "relax_variant": 0}
     assert tb["relax_variant"] in (0, 1, 2)
     assert tb["orbit_block"] in (64, 128, 256)
-    assert tb["sort_keys_per_thread"] in (8, 16, 24, 32)  # 24 and 32: packed keys only
+    assert tb["sort_keys_per_thread"] == 16 and tb["sort_multisplit"] == "match"  # not tuned
     assert b.stats()[0]["trials"] == 0  # the tuner's dry run left no trace
     a.step(3)
     b.step(3)
@@ -371,11 +373,11 @@ def test_fp64_paths_agree_over_steps(g, n, masses, rng):
 
 
 @pytest.mark.parametrize("precision", [0, 1])
-def test_packed_sort_keys_change_nothing(g_stage, precision):
-    """The timestep's sort on packed keys (each key's low 24 bits, which the
-    radix passes leave to the tie fix, carrying the star's index) against
-    the keys-and-values sort: the same states, bit for bit, after several
-    steps of one cluster and of a ragged ensemble (escapers included)."""
+def test_either_sort_gives_the_same_steps(g_stage, precision):
+    """The timestep's counting sort on the shells (sort_packed = 1) against its radix
+    sort of keys and values (0), as a user runs them: the same states and
+    statistics, bit for bit, after several steps of one cluster and of a ragged
+    ensemble (escapers included)."""
     g = g_stage
     sizes = [1, 3, 20, 4097, 9000, 2, 12_289]
     seeds = [500 + i for i in range(len(sizes))]
@@ -398,12 +400,11 @@ def test_packed_sort_keys_change_nothing(g_stage, precision):
 
 
 def test_unsorted_state_after_the_tuned_sort_shape(g):
-    """A new state in no particular order is ordered by the keys-and-values
-    sort, which takes tiles of 16 keys per thread whatever shape the tuner
-    chose for the timestep's packed keys (24 or 32 at large N), and puts the
-    tuned shape back: the same sorted state, bit for bit, and steps go on."""
+    """A new state in no particular order is ordered by the radix sort in whatever
+    shape the tuner chose for the timestep's: the same sorted state, bit for bit, and
+    steps go on."""
     d = ic.plummer(2_000_000, seed=12)
-    c = _cluster(g, d, 12)
+    c = _cluster(g, d, 12, sort_packed=0)
     tuned = c.tuning()
     c.step(1)
     st = c.get_state()

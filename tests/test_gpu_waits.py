@@ -1,11 +1,11 @@
 """The sort's bounded device waits run out, on purpose, without faulting or
-hanging anything: with a look-back limit of one poll, a timestep whose many
-escapers hand its sort to the radix passes gives up on earlier tiles,
-reports CMC_ETIMEOUT and poisons its context (later calls return
-CMC_EPOISONED), while another context on the device is unaffected; with a tie-fix limit of a few moves the stage sort of a run of
-equal radii falls back to sorting by id, then by radius, and still returns
-the (r, id) order.  Every wait bound is host-set (cmc_set_wait_limits) and
-restored to its default afterwards."""
+hanging anything: with a look-back limit of one poll a timestep's sort, by
+counting or by radix passes, gives up on earlier tiles, reports CMC_ETIMEOUT and
+poisons its context (later calls return CMC_EPOISONED), while another context on
+the device is unaffected; so does the merge of a long run on the pass before; with
+a tie-fix limit of a few moves the stage sort of a run of equal radii falls back to
+sorting by id, then by radius, and still returns the (r, id) order.  Every wait
+bound is host-set (cmc_set_wait_limits) and restored to its default afterwards."""
 import numpy as np
 import pytest
 
@@ -27,22 +27,13 @@ def _cluster(g, n, seed):
     return g.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, [seed], autotune=0)
 
 
-def _unbound(n, seed, n_fast):
-    """A Plummer sample with n_fast stars sent out at ten times their
-    speed (E > 0: they escape in the first step)."""
-    d = ic.plummer(n, seed=seed)
-    fast = np.random.default_rng(seed).choice(n, n_fast, replace=False)
-    d["vr"][fast] *= 10.0
-    d["vt"][fast] *= 10.0
-    return d
-
-
-def test_lookback_limit_times_out_and_poisons(g):
-    """More escapers in one step than the shell sort lists hand the step to
-    the radix sort, whose look-back then runs out."""
+@pytest.mark.parametrize("packed", [0, 1])
+def test_lookback_limit_times_out_and_poisons(g, packed):
+    """The counting sort's scan (550 tiles) and the radix passes (489)."""
     other = _cluster(g, 50_000, 2)  # built before the limit: unaffected later
-    d = _unbound(2_000_000, 1, 6000)  # 489 sort tiles, > 4096 escapers
-    c = g.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, [1], autotune=0)
+    d = ic.plummer(2_000_000, seed=1)
+    c = g.Cluster({k: d[k] for k in ("r", "vr", "vt", "m", "id")}, [1], autotune=0,
+                  sort_packed=packed)
     try:
         g.set_wait_limits(lookback_polls=1)
         with pytest.raises(g.CMCError) as ei:
@@ -85,6 +76,33 @@ def test_tie_move_limit_falls_back_and_keeps_the_order(g, orc):
     finally:
         g.set_wait_limits()
     np.testing.assert_array_equal(perm.astype(np.int64), orc.sort_perm(r, ids))
+
+
+def test_the_merge_of_a_long_run_gives_up(g):
+    """A thin shell that falls in: all stars in the innermost bin, two tiles to merge, and
+    few enough bins for one tile of the scan, which then has nothing to wait for.
+    The stars stay where they are, and a state set afterwards goes on as in a new
+    context."""
+    n = 3600
+    q = np.random.default_rng(1)
+    c = 2.0 * q.random(n) - 1.0
+    d = {"r": 1.0 + 1e-6 * q.random(n), "vr": 0.5 * c, "vt": 0.5 * np.sqrt(1.0 - c * c),
+         "m": np.full(n, 1.0 / n), "id": q.permutation(n).astype(np.uint32)}
+    a, b = (g.Cluster(d, [1], autotune=0, precision=1) for _ in range(2))
+    st = a.get_state()
+    try:
+        g.set_wait_limits(lookback_polls=1)
+        with pytest.raises(g.CMCError) as ei:
+            a.step(1)
+        assert ei.value.status == 5  # CMC_ETIMEOUT
+    finally:
+        g.set_wait_limits()
+    a.set_state(st, 0)
+    a.step(2)
+    b.step(2)
+    sa, sb = a.get_state(), b.get_state()
+    for k in ("r", "vr", "vt", "m", "id", "phi"):
+        np.testing.assert_array_equal(sa[k], sb[k], err_msg=k)
 
 
 def test_wait_limit_arguments(g):
