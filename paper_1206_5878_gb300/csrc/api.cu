@@ -1,6 +1,7 @@
 // C ABI (include/cmc.h): the context that advances clusters timestep by
 // timestep, and the stage functions that run one step of the hot path on
 // caller arrays.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -33,12 +34,16 @@ struct cmc_ctx {
   double *r_alt = nullptr, *x_alt = nullptr;
   int side = 0;
   uint32_t* id = nullptr;
-  // scratch
-  uint64_t* keys = nullptr;
+  // Scratch.  Arrays whose lives do not meet share memory: the orbit step's and the
+  // sorts' keys lie where the next 1/r goes (x_alt, which the gather writes after
+  // the last look at them), the radix sort's other keys and its look-back words in
+  // r_old and cc (written by the gather too), the stars' old indices at their new
+  // positions (order) over their pending list and their bins.
+  uint64_t* keys() const { return reinterpret_cast<uint64_t*>(x_alt); }
   uint32_t* vals = nullptr;
+  uint32_t* order() const { return vals; }
   RecA* ra = nullptr;
   RecB* rb = nullptr;
-  uint32_t* order = nullptr;   // the stars' old indices at their new positions
   BinWork bins;                // the timestep's counting sort (cfg.sort_packed)
   std::vector<unsigned int> max_id;  // per segment, as the bins have it
   std::vector<unsigned int> taus_max_id;  // per segment: the last id with a stream (rng 1)
@@ -189,8 +194,8 @@ bool order_in_place(cmc_ctx* c, const std::vector<unsigned long long>& bitoff,
     return false;
   }
   // the bitmap lives in the key scratch (64 bits per star)
-  cudaMemsetAsync(c->keys, 0, sizeof(uint64_t) * (size_t)L.n, st);
-  launch_place(L, c->r, c->id, dbo, reinterpret_cast<unsigned long long*>(c->keys), c->err, st);
+  cudaMemsetAsync(c->keys(), 0, sizeof(uint64_t) * (size_t)L.n, st);
+  launch_place(L, c->r, c->id, dbo, reinterpret_cast<unsigned long long*>(c->keys()), c->err, st);
   dfree(block, st);
   return true;
 }
@@ -200,7 +205,7 @@ bool order_in_place(cmc_ctx* c, const std::vector<unsigned long long>& bitoff,
 void finish_order(cmc_ctx* c, bool placed, cudaStream_t st) {
   const SegLayout& L = c->L;
   double* recip = placed ? c->x : nullptr;
-  if (!placed) launch_nb_from_keys(L, c->keys, st);
+  if (!placed) launch_nb_from_keys(L, c->keys(), st);
   cudaMemsetAsync(L.esc_step, 0, sizeof(int64_t) * L.n_seg, st);
   // the float tables, node records and indexes of the sampled orbit step
   // (precision 0 and 1)
@@ -224,11 +229,11 @@ void order_state(cmc_ctx* c, cudaStream_t st) {
   const bool placed =
       L.n > 0 && staged_in_order(c, bitoff, st, max_id) && order_in_place(c, bitoff, st);
   if (!placed) {
-    launch_id_keys(L, c->id, c->keys, st);
-    sort_segments(L, c->W, c->keys, c->vals, 0, 4, true, c->err, st);
-    launch_check_ids(L, c->keys, c->err, st);
-    launch_rekey_radius(L, c->vals, c->r, c->id, c->keys, st);
-    sort_segments(L, c->W, c->keys, c->vals, 0, 8, false, c->err, st);
+    launch_id_keys(L, c->id, c->keys(), st);
+    sort_segments(L, c->W, c->keys(), c->vals, 0, 4, true, c->err, st);
+    launch_check_ids(L, c->keys(), c->err, st);
+    launch_rekey_radius(L, c->vals, c->r, c->id, c->keys(), st);
+    sort_segments(L, c->W, c->keys(), c->vals, 0, 8, false, c->err, st);
     launch_make_records(L, c->r, c->vr, c->vt, c->m, c->id, c->ra, c->rb, st);
     launch_gather(L, c->vals, c->ra, c->rb, c->r, c->x, c->vr, c->vt, c->m, c->id, st);
   }
@@ -274,27 +279,27 @@ void record_step(cmc_ctx* c, cudaStream_t st, cudaEvent_t* ev = nullptr) {
   const bool binned = c->cfg.sort_packed != 0;
   const bool counted = L.n <= kCountInOrbit;
   launch_orbit(L, c->cfg.precision, c->cfg.max_trials, c->r, c->x, c->phi, c->vr, c->vt, c->m, c->id,
-               c->step, c->keys, c->ra, c->rb, nullptr, c->cfg.orbit_block, c->orbit_variant,
+               c->step, c->keys(), c->ra, c->rb, nullptr, c->cfg.orbit_block, c->orbit_variant,
                c->bk.args(), c->r_old, c->cc, c->vals, c->pcount, st, false, c->R, c->Rp,
                c->cfg.precision == 0 ? &c->env : nullptr, c->A, c->Ap, c->orb,
                binned ? &c->bins : nullptr, c->vals, counted);
   mark(4);
   uint32_t* ord = c->W.vals_alt;
   if (binned) {
-    launch_bin_sort(L, c->bins, c->vals, c->ra, ord, c->order, c->keys, c->W.keys_alt, counted,
+    launch_bin_sort(L, c->bins, c->vals, c->ra, ord, c->order(), c->keys(), c->W.keys_alt, counted,
                     c->err, st);
   } else {
     // radix passes over bits 24-63 of the radius keys; runs equal in those
     // bits (radii within 2^-28 of each other, escapers whose ids differ in
     // their low 4 bits) are put in (key, id) order after
     uint64_t* sk = nullptr;
-    sort_segments(L, c->W, c->keys, c->vals, 3, 5, true, c->err, st, &sk, &ord);
+    sort_segments(L, c->W, c->keys(), c->vals, 3, 5, true, c->err, st, &sk, &ord);
     launch_tiefix(L, sk, ord, &c->ra[0].id, (int)(sizeof(RecA) / sizeof(uint32_t)), c->err, st,
                   24);
   }
   mark(5);
   launch_gather_step(L, binned ? &c->bins : nullptr, ord, c->ra, c->rb, c->r, c->r_alt, c->x_alt,
-                     c->m, c->id, c->order, c->r_old, c->cc, c->tile_a, c->tile_b, c->Rp, c->R,
+                     c->m, c->id, c->order(), c->r_old, c->cc, c->tile_a, c->tile_b, c->Rp, c->R,
                      c->Ap, c->A, !binned, st);
   mark(6);
   const bool correct = c->cfg.energy_correction != 0;
@@ -314,7 +319,7 @@ void record_step(cmc_ctx* c, cudaStream_t st, cudaEvent_t* ev = nullptr) {
     launch_phi_old(L, c->r, c->x, c->r_alt, c->x_alt, c->phi, c->bk.node, c->rb, !mixed, st,
                    tab ? &grid : nullptr);
   // (and the end of the step: escapers' budgets, counters)
-  launch_velocities(L, c->order, c->rb, c->phi, c->m, c->vr, c->vt, correct, c->r_old, c->cc,
+  launch_velocities(L, c->order(), c->rb, c->phi, c->m, c->vr, c->vt, correct, c->r_old, c->cc,
                     c->step, st);
   mark(8);
   if (c->ring) {
@@ -359,11 +364,9 @@ void free_ctx(cmc_ctx* c) {
   dfree(c->Rp, st);
   dfree(c->A, st);
   dfree(c->Ap, st);
-  dfree(c->keys, st);
   dfree(c->vals, st);
   dfree(c->ra, st);
   dfree(c->rb, st);
-  dfree(c->order, st);
   free_bins(c->bins, st);
   dfree(c->err, st);
   dfree(c->step, st);
@@ -585,7 +588,7 @@ cmc_status autotune(cmc_ctx* c) {
   }
   auto run_orbit = [&](int blk, int var) {
     launch_orbit(L, c->cfg.precision, c->cfg.max_trials, c->r, c->x, c->phi, c->vr, c->vt, c->m,
-                 c->id, c->step, c->keys, c->ra, c->rb, nullptr, blk, var, c->bk.args(), c->r_old,
+                 c->id, c->step, c->keys(), c->ra, c->rb, nullptr, blk, var, c->bk.args(), c->r_old,
                  c->cc, c->vals, c->pcount, st, true, nullptr, nullptr,
                  c->cfg.precision == 0 ? &c->env : nullptr, nullptr, nullptr, c->orb);
   };
@@ -643,16 +646,16 @@ cmc_status autotune(cmc_ctx* c) {
   // keys the orbit step produced
   cudaError_t e = cudaSuccess;
   if (!c->cfg.sort_packed) {
-    uint64_t* saved = reinterpret_cast<uint64_t*>(c->cc);  // scratch of the same size
-    cudaMemcpyAsync(saved, c->keys, sizeof(uint64_t) * L.n, cudaMemcpyDeviceToDevice, st);
+    uint64_t* saved = reinterpret_cast<uint64_t*>(c->r_alt);  // scratch of the same size
+    cudaMemcpyAsync(saved, c->keys(), sizeof(uint64_t) * L.n, cudaMemcpyDeviceToDevice, st);
     int best_ipt = 16, best_rank = 0;
     float tbest = 3.4e38f;
     for (int ipt : {8, 16})
       for (int rank : {0, 1}) {
         if (sort_set_shape(L, c->W, ipt, rank, st)) continue;
         const float ms = time_it([&] {
-          cudaMemcpyAsync(c->keys, saved, sizeof(uint64_t) * L.n, cudaMemcpyDeviceToDevice, st);
-          sort_segments(L, c->W, c->keys, c->vals, 3, 5, true, c->err, st);
+          cudaMemcpyAsync(c->keys(), saved, sizeof(uint64_t) * L.n, cudaMemcpyDeviceToDevice, st);
+          sort_segments(L, c->W, c->keys(), c->vals, 3, 5, true, c->err, st);
         });
         if (ms < tbest) { tbest = ms; best_ipt = ipt; best_rank = rank; }
       }
@@ -819,15 +822,13 @@ cmc_status cmc_init(cmc_ctx** out, const cmc_config* cfg_in, int32_t n_clusters,
     if (!e) e = cudaMemsetAsync(c->ring, 0, sizeof(double) * (size_t)n_clusters *
                                                 cfg.diag_ring * kDiagFields, st);
   }
-  CMC_ALLOC(c->keys, n);
   CMC_ALLOC(c->vals, n);
   CMC_ALLOC(c->ra, n);
   CMC_ALLOC(c->rb, n);
-  CMC_ALLOC(c->order, n);
   CMC_ALLOC(c->r_alt, n);
   CMC_ALLOC(c->x_alt, n);
   CMC_ALLOC(c->r_old, n);
-  CMC_ALLOC(c->cc, n);
+  CMC_ALLOC(c->cc, std::max(n, (sort_zeroed_bytes(L, 8) + 7) / 8));
   CMC_ALLOC(c->nbin, (size_t)L.n_bins);
   CMC_ALLOC(c->tile_a, (size_t)L.n_tiles);
   CMC_ALLOC(c->tile_b, (size_t)L.n_tiles);
@@ -848,7 +849,7 @@ cmc_status cmc_init(cmc_ctx** out, const cmc_config* cfg_in, int32_t n_clusters,
     if (!e) e = cudaMemsetAsync(c->A, 0, sizeof(double) * n, st);
   }
 #undef CMC_ALLOC
-  if (!e) e = alloc_sort(c->W, L, 8, st);
+  if (!e) e = alloc_sort(c->W, L, 8, st, reinterpret_cast<uint64_t*>(c->r_old), c->cc);
   if (!e && cfg.sort_packed) e = alloc_bins(c->bins, L, st);
   if (!e && cfg.precision != 2) e = alloc_buckets(c->bk, L, st);
   if (e) { cmc_status s = cuda_fail(nullptr, e, "cmc_init: allocation"); free_ctx(c); return s; }

@@ -127,7 +127,6 @@ struct SortWork {
   uint32_t* hist = nullptr;             // [n_seg][passes][256]
   uint32_t* tickets = nullptr;          // [passes]
   uint32_t* done = nullptr;             // [n_seg] upsweep blocks finished
-  size_t zero_bytes = 0;                // hist + tickets + done, then desc
   size_t zero_head = 0;                 // bytes before desc (zeroed with it per sort)
   void* zero_base = nullptr;
   int max_passes = 0;
@@ -149,7 +148,11 @@ cudaError_t alloc_layout(SegLayout& L, const std::vector<int64_t>& sizes,
                          const std::vector<uint64_t>& seeds, const std::vector<double>& lnL,
                          int bin_size, cudaStream_t st);
 void free_layout(SegLayout& L, cudaStream_t st);
-cudaError_t alloc_sort(SortWork& W, const SegLayout& L, int max_passes, cudaStream_t st);
+// keys, zeroed: memory for its keys and counters (n keys and sort_zeroed_bytes;
+// the caller's), null: its own
+cudaError_t alloc_sort(SortWork& W, const SegLayout& L, int max_passes, cudaStream_t st,
+                       uint64_t* keys = nullptr, void* zeroed = nullptr);
+size_t sort_zeroed_bytes(const SegLayout& L, int max_passes);
 void free_sort(SortWork& W, cudaStream_t st);
 
 // ------------------------------------------------------------- launchers

@@ -844,37 +844,42 @@ cudaError_t sort_set_shape(const SegLayout& L, SortWork& W, int ipt, int rank,
   return cudaSuccess;
 }
 
-cudaError_t alloc_sort(SortWork& W, const SegLayout& L, int max_passes, cudaStream_t st) {
-  W.max_passes = max_passes;
-  size_t n = (size_t)L.n;
+// Histograms, tickets and done counters first, then the look-back words: a sort
+// zeroes the counters and the words of its own passes and tiles.
+static size_t sort_head_bytes(const SegLayout& L, int max_passes) {
+  const size_t hist = sizeof(uint32_t) * (size_t)L.n_seg * max_passes * kBins;
+  return (hist + sizeof(uint32_t) * (16 + (size_t)L.n_seg) + 255) / 256 * 256;
+}
+size_t sort_zeroed_bytes(const SegLayout& L, int max_passes) {
   // look-back words for the smallest tiles (the most tiles)
   const int64_t max_tiles = sort_tile_offsets(L, kThreads * 8)[L.n_seg];
-  size_t desc_b = sizeof(unsigned long long) * (size_t)max_passes * max_tiles * kBins;
-  size_t hist_b = sizeof(uint32_t) * (size_t)L.n_seg * max_passes * kBins;
-  size_t tick_b = sizeof(uint32_t) * 16;
-  size_t done_b = sizeof(uint32_t) * (size_t)L.n_seg;
-  // histograms, tickets and done counters first, then the look-back words:
-  // a sort zeroes the counters and the words of its own passes and tiles
-  const size_t head_b = (hist_b + tick_b + done_b + 255) / 256 * 256;
-  W.zero_bytes = head_b + desc_b;
-  W.zero_head = head_b;
+  return sort_head_bytes(L, max_passes) +
+         sizeof(unsigned long long) * (size_t)max_passes * max_tiles * kBins;
+}
+
+cudaError_t alloc_sort(SortWork& W, const SegLayout& L, int max_passes, cudaStream_t st,
+                       uint64_t* keys, void* zeroed) {
+  W.max_passes = max_passes;
+  W.zero_head = sort_head_bytes(L, max_passes);
   W.ipt = 16;
   W.rank = 0;
   const std::vector<int64_t> o = sort_tile_offsets(L, kThreads * W.ipt);
   W.n_stiles = o[L.n_seg];
-  unsigned char* zeroed = nullptr;
+  unsigned char* own = nullptr;
   Carve C;
   C.put(W.stile_off, o.data(), o.size());
-  C.add(W.keys_alt, n);
-  C.add(W.vals_alt, n);
-  C.add(zeroed, W.zero_bytes);
+  C.add(W.vals_alt, (size_t)L.n);
+  if (!keys) C.add(W.keys_alt, (size_t)L.n);
+  if (!zeroed) C.add(own, sort_zeroed_bytes(L, max_passes));
   const cudaError_t e = C.alloc(W.block, st);
   if (e) return e;
-  W.zero_base = zeroed;
-  W.hist = (uint32_t*)W.zero_base;
-  W.tickets = (uint32_t*)((char*)W.zero_base + hist_b);
-  W.done = (uint32_t*)((char*)W.zero_base + hist_b + tick_b);
-  W.desc = (unsigned long long*)((char*)W.zero_base + head_b);
+  if (keys) W.keys_alt = keys;
+  unsigned char* base = zeroed ? (unsigned char*)zeroed : own;
+  W.zero_base = base;
+  W.hist = (uint32_t*)base;
+  W.tickets = W.hist + (size_t)L.n_seg * max_passes * kBins;
+  W.done = W.tickets + 16;
+  W.desc = (unsigned long long*)(base + W.zero_head);
   return cudaSuccess;
 }
 

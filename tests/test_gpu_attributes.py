@@ -62,3 +62,25 @@ def test_a_failed_call_leaves_nothing_to_the_next(g_stage):
     c.set_radii(np.full(n, 1e-9))
     refused()
     c.step(1)
+
+
+@pytest.mark.parametrize("precision,most", [(0, 304), (1, 240), (2, 168)])
+def test_memory_per_star(g_stage, precision, most):
+    """A context's device memory, which bounds the largest cluster, of 2 x 10^7 stars:
+    the state (12 B and 5 doubles), the step's records and tables (241, 177 and 109 B),
+    a few per cent for the allocator's granularity."""
+    import gc
+
+    import torch
+    n = 20_000_000
+    q = np.random.default_rng(1)
+    d = {"r": q.random(n) + 0.5, "vr": np.zeros(n), "vt": q.random(n) * 0.1,
+         "m": np.full(n, 1.0 / n), "id": np.arange(n, dtype=np.uint32)}
+    gc.collect()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    c = g_stage.Cluster(d, [1], precision=precision, autotune=0)
+    torch.cuda.synchronize()
+    used = free - torch.cuda.mem_get_info()[0]
+    c.step(1)
+    assert 0 < used <= most * n, used / n
