@@ -147,7 +147,8 @@ typedef struct {
     int32_t diag_ring;          /* records per cluster of the per-step
                                    diagnostics ring (cmc_get_diagnostics), 0 =
                                    off (default); on, every step also computes
-                                   K and W (four more kernels per step) */
+                                   K and W (three or four more kernels per
+                                   step) */
     int32_t binaries;           /* 1: stars carry semi-major axes
                                    (cmc_set_binaries; 0 for a single star, a
                                    binary's mass its total): the binary-binary

@@ -345,7 +345,7 @@ int count_step_kernels(const cmc_ctx* c) {
   // evaluation], Phi_new(r_old) with the grid's values or those alone
   const int p = c->cfg.precision;
   const int sort = c->cfg.sort_packed ? (c->L.n <= kCountInOrbit ? 3 : 4) : 7;
-  return (c->L.n <= kEndWithVelocities ? 6 : 7) + sort + (c->ring ? 4 : 0) +
+  return (c->L.n <= kEndWithVelocities ? 6 : 7) + sort + (c->ring ? 1 + energy_kernels(c->L) : 0) +
          (p == 1 ? 3 : p == 0 ? 5 : 0) +
          (c->cfg.energy_correction || p != 2 ? 1 : 0);
 }

@@ -87,7 +87,7 @@ struct SegLayout {
   int64_t n_bins = 0;     // bin slots (ceil(n_c / bin_size) summed)
   int bin_size = 20;
   std::vector<int64_t> h_off, h_tile_off, h_pair_off, h_bin_off;
-  int64_t max_tiles_per_seg = 0;
+  int64_t max_seg = 0;    // stars of the largest segment
   // device arrays, all in one block
   void* block = nullptr;
   int64_t* off = nullptr;
@@ -518,6 +518,7 @@ constexpr int kRelaxVariants = 3;  // relaxation kernel register caps (launch_re
 void launch_energy(const SegLayout& L, const double* r, const double* vr, const double* vt,
                    const double* m, double* tile_m, double* tile_k, double* tile_w,
                    double* out3, cudaStream_t st);
+int energy_kernels(const SegLayout& L);  // that it launches
 // the mass up to and including every bound star
 void launch_masses(const SegLayout& L, const double* m, double* tile_m, double* Mout,
                    cudaStream_t st);

@@ -1250,6 +1250,95 @@ __global__ void __launch_bounds__(kDiagThreads, 3) k_core_tiles(Seg S, const dou
 }
 constexpr size_t kDiagSmem = sizeof(double) * 2 * (kPad16N + 8);
 
+// The same sums where every cluster has at most kDiagSmall stars: a warp per cluster,
+// a run of 16 stars to a lane (the runs, scans and trees above with nothing but
+// zeros beyond the warp's), no shared memory and no barriers.  20,000 clusters of
+// two stars: sums of the energy 2.3 ms by whole tiles' blocks, 0.07 so, of the core 1.5, 0.03.
+constexpr int64_t kDiagSmall = 32 * kPer;
+constexpr int kSmallWarps = 8;
+
+__device__ __forceinline__ double warp_tree(double v) {
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1) v = v + __shfl_down_sync(0xFFFFFFFFu, v, w);
+  return v;
+}
+
+template <bool kMass>
+__global__ void __launch_bounds__(32 * kSmallWarps) k_energy_small(
+    Seg S, int64_t n_tiles, const double* r, const double* vr, const double* vt, const double* m,
+    double* tile_k, double* tile_w, double* Mout) {
+  pdl_enter();
+  const int64_t tile = (int64_t)blockIdx.x * kSmallWarps + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (tile >= n_tiles) return;
+  const TR R = tile_of(S, nullptr, tile, false);
+  const int64_t p0 = R.begin + lane * kPer;
+  auto mass = [&](int64_t p) { return p < R.end && p < R.bound_end ? m[p] : 0.0; };
+  double am = 0.0;
+  for (int i = 0; i < kPer && p0 + i < R.end; ++i) am = am + mass(p0 + i);
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double a = __shfl_up_sync(0xFFFFFFFFu, am, o);
+    if (lane >= o) am = a + am;
+  }
+  const double below = __shfl_up_sync(0xFFFFFFFFu, am, 1), base = lane > 0 ? below : 0.0;
+  double run = 0.0, ak = 0.0, aw = 0.0;
+  for (int i = 0; i < kPer && p0 + i < R.end; ++i) {
+    const int64_t p = p0 + i;
+    const bool in = p < R.bound_end;
+    const double mi = in ? m[p] : 0.0, inside = base + run;
+    run = run + mi;
+    if (kMass) {
+      Mout[p] = in ? base + run : 0.0;
+    } else if (in) {
+      ak = ak + mul_rn(mi, mul_rn(vr[p], vr[p]) + mul_rn(vt[p], vt[p]));
+      aw = aw + div_rn(mul_rn(mi, inside), r[p]);
+    }
+  }
+  if (kMass) return;
+  const double tk = warp_tree(ak), tw = warp_tree(aw);
+  if (lane == 0) {
+    tile_k[tile] = tk;
+    tile_w[tile] = tw;
+  }
+}
+
+__global__ void __launch_bounds__(32 * kSmallWarps) k_core_small(Seg S, int64_t n_tiles,
+                                                                 const double* r, const double* m,
+                                                                 double* tile_s1, double* tile_s2,
+                                                                 double* tile_sr, double* tile_n) {
+  pdl_enter();
+  const int64_t tile = (int64_t)blockIdx.x * kSmallWarps + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (tile >= n_tiles) return;
+  const TR R = tile_of(S, nullptr, tile, false);
+  const double c43 = (4.0 * kPi) / 3.0;
+  double a1 = 0.0, a2 = 0.0, ar = 0.0;
+  int count = 0;
+  for (int i = 0; i < kPer; ++i) {
+    const int64_t p = R.begin + lane * kPer + i;
+    if (p + 3 >= R.bound_end) break;
+    if (p - R.seg_begin < 3) continue;
+    const double ro = r[p + 3], ri = r[p - 3];
+    const double vol = mul_rn(c43, mul_rn(ro * ro, ro) - mul_rn(ri * ri, ri));
+    if (!pos_num(vol)) continue;
+    const double q =
+        div_rn((((m[p - 2] + m[p - 1]) + m[p]) + m[p + 1]) + m[p + 2], vol);
+    a1 = a1 + q;
+    a2 = a2 + mul_rn(q, q);
+    ar = ar + mul_rn(q, r[p]);
+    ++count;
+  }
+  const double t1 = warp_tree(a1), t2 = warp_tree(a2), tr = warp_tree(ar);
+  count = __reduce_add_sync(0xFFFFFFFFu, count);
+  if (lane == 0) {
+    tile_s1[tile] = t1;
+    tile_s2[tile] = t2;
+    tile_sr[tile] = tr;
+    tile_n[tile] = (double)count;
+  }
+}
+
 // per cluster: rho_c = sum rho^2 / sum rho, r_c = sum rho r / sum rho and the
 // number of estimates (3 doubles per cluster)
 __global__ void __launch_bounds__(kThreads) k_core_final(Seg S, const double* tile_s1,
@@ -1569,7 +1658,7 @@ cudaError_t alloc_layout(SegLayout& L, const std::vector<int64_t>& sizes,
   L.h_tile_off.assign(L.n_seg + 1, 0);
   L.h_pair_off.assign(L.n_seg + 1, 0);
   L.h_bin_off.assign(L.n_seg + 1, 0);
-  L.max_tiles_per_seg = 0;
+  L.max_seg = 0;
   for (int c = 0; c < L.n_seg; ++c) {
     int64_t nc = sizes[c];
     int64_t nt = (nc + kTile - 1) / kTile;
@@ -1577,7 +1666,7 @@ cudaError_t alloc_layout(SegLayout& L, const std::vector<int64_t>& sizes,
     L.h_tile_off[c + 1] = L.h_tile_off[c] + nt;
     L.h_pair_off[c + 1] = L.h_pair_off[c] + nc / 2;
     L.h_bin_off[c + 1] = L.h_bin_off[c] + (nc + bin_size - 1) / bin_size;
-    if (nt > L.max_tiles_per_seg) L.max_tiles_per_seg = nt;
+    if (nc > L.max_seg) L.max_seg = nc;
   }
   L.n = L.h_off[L.n_seg];
   L.n_tiles = L.h_tile_off[L.n_seg];
@@ -1761,16 +1850,28 @@ void launch_energy(const SegLayout& L, const double* r, const double* vr, const 
                    double* out3, cudaStream_t st) {
   if (!L.n_tiles) return;
   Seg S = L.dev();
-  launch_tile_sums<kSumsMass>(L, false, nullptr, m, tile_m, nullptr, nullptr, st);
-  launch_k(k_energy_tiles<false>, (unsigned)L.n_tiles, kDiagThreads, kDiagSmem, st, S, r, vr, vt, m,
-           tile_m, tile_k, tile_w, nullptr);
+  if (L.max_seg <= kDiagSmall) {
+    launch_k(k_energy_small<false>, blocks_for(L.n_tiles, kSmallWarps), 32 * kSmallWarps, 0, st, S,
+             L.n_tiles, r, vr, vt, m, tile_k, tile_w, nullptr);
+  } else {
+    launch_tile_sums<kSumsMass>(L, false, nullptr, m, tile_m, nullptr, nullptr, st);
+    launch_k(k_energy_tiles<false>, (unsigned)L.n_tiles, kDiagThreads, kDiagSmem, st, S, r, vr, vt,
+             m, tile_m, tile_k, tile_w, nullptr);
+  }
   launch_k(k_energy_final, (unsigned)L.n_seg, kThreads, 0, st, S, tile_k, tile_w, out3);
 }
+
+int energy_kernels(const SegLayout& L) { return L.max_seg <= kDiagSmall ? 2 : 3; }
 
 void launch_masses(const SegLayout& L, const double* m, double* tile_m, double* Mout,
                    cudaStream_t st) {
   if (!L.n_tiles) return;
   Seg S = L.dev();
+  if (L.max_seg <= kDiagSmall) {
+    launch_k(k_energy_small<true>, blocks_for(L.n_tiles, kSmallWarps), 32 * kSmallWarps, 0, st, S,
+             L.n_tiles, nullptr, nullptr, nullptr, m, nullptr, nullptr, Mout);
+    return;
+  }
   launch_tile_sums<kSumsMass>(L, false, nullptr, m, tile_m, nullptr, nullptr, st);
   launch_k(k_energy_tiles<true>, (unsigned)L.n_tiles, kDiagThreads, kDiagSmem, st, S, nullptr,
            nullptr, nullptr, m, tile_m, nullptr, nullptr, Mout);
@@ -1788,8 +1889,12 @@ void launch_core(const SegLayout& L, const double* r, const double* m, double* t
   if (!L.n_tiles) return;
   Seg S = L.dev();
   const int64_t t = L.n_tiles;
-  launch_k(k_core_tiles, (unsigned)t, kDiagThreads, kDiagSmem, st, S, r, m, tiles4, tiles4 + t,
-           tiles4 + 2 * t, tiles4 + 3 * t);
+  if (L.max_seg <= kDiagSmall)
+    launch_k(k_core_small, blocks_for(t, kSmallWarps), 32 * kSmallWarps, 0, st, S, t, r, m, tiles4,
+             tiles4 + t, tiles4 + 2 * t, tiles4 + 3 * t);
+  else
+    launch_k(k_core_tiles, (unsigned)t, kDiagThreads, kDiagSmem, st, S, r, m, tiles4, tiles4 + t,
+             tiles4 + 2 * t, tiles4 + 3 * t);
   launch_k(k_core_final, (unsigned)L.n_seg, kThreads, 0, st, S, tiles4, tiles4 + t, tiles4 + 2 * t,
                                                        tiles4 + 3 * t, out3);
 }

@@ -103,13 +103,15 @@ def test_sums_in_order(g_stage, n, steps):
     _check(c, 0, *(st[k][b] for k in ("r", "vr", "vt", "m")))
 
 
-def test_ensemble(g_stage):
-    sizes = [9, 4097, 300, 20_000]
+@pytest.mark.parametrize("sizes", [[9, 4097, 300, 20_000],
+                                   [1, 2, 6, 7, 8, 15, 16, 17, 31, 33, 300, 511, 512, 5],  # a warp each
+                                   [1, 2, 6, 7, 8, 15, 16, 17, 31, 33, 300, 511, 513, 5]])
+def test_ensemble(g_stage, sizes):
     parts = [ic.plummer(n, seed=n, masses="salpeter") for n in sizes]
     cat = {k: np.concatenate([p[k] for p in parts]) for k in ("r", "vr", "vt", "m", "id")}
-    c = g_stage.Cluster(cat, [1, 2, 3, 4], sizes=sizes, precision=1)
+    c = g_stage.Cluster(cat, list(range(len(sizes))), sizes=sizes, precision=1)
     st, o = c.get_state(), np.concatenate([[0], np.cumsum(sizes)])
-    for i in range(4):
+    for i in range(len(sizes)):
         _check(c, i, *(st[k][o[i]:o[i + 1]] for k in ("r", "vr", "vt", "m")))
 
 
