@@ -286,15 +286,21 @@ int32_t cmc_is_debug_build(void);
 
 /* Stages of one timestep, as timed by cmc_step_profiled. */
 enum {
-    CMC_STAGE_TIMESTEP = 0,    /* Eq. 7 bins and the minimum over bins */
+    CMC_STAGE_TIMESTEP = 0,    /* Eq. 7 bins and the minimum over bins; Eqs. 8-10 */
     CMC_STAGE_RELAX = 1,       /* two-body relaxation of neighbour pairs */
-    CMC_STAGE_TURNING = 2,     /* turning points (mixed mode; FP64 mode: in ORBIT) */
-    CMC_STAGE_ORBIT = 3,       /* rejection sampling (FP64 mode: and turning points) */
-    CMC_STAGE_SORT = 4,        /* radix passes and the id order of ties */
-    CMC_STAGE_GATHER = 5,      /* payload into the sorted arrays */
-    CMC_STAGE_POTENTIAL = 6,   /* shell potential (Eqs. 1-5) and mixed-mode tables */
-    CMC_STAGE_CORRECTION = 7,  /* energy correction */
-    CMC_STAGE_END = 8,         /* bookkeeping of the step */
+    CMC_STAGE_TURNING = 2,     /* turning points (precision 2: in ORBIT) */
+    CMC_STAGE_ORBIT = 3,       /* rejection sampling, the stars' new shells and, up to
+                                  262,144 stars, their count (precision 2: and
+                                  turning points) */
+    CMC_STAGE_SORT = 4,        /* counting sort on the shells (sort_packed = 0: radix
+                                  passes and the order of keys equal in them) */
+    CMC_STAGE_GATHER = 5,      /* order inside a shell, stars into their new places */
+    CMC_STAGE_POTENTIAL = 6,   /* shell potential (Eqs. 1-5), orbit tables (the
+                                  potential grid's values are in CORRECTION when
+                                  that is on) */
+    CMC_STAGE_CORRECTION = 7,  /* energy correction, the velocities into their new
+                                  places, escapers' budget and the step's counters */
+    CMC_STAGE_END = 8,         /* the diagnostics ring's record, when it is on */
     CMC_NSTAGES = 9
 };
 
@@ -342,9 +348,10 @@ cmc_status cmc_rng_philox(int64_t n, const uint32_t *ctr, uint64_t seed, uint32_
                           void *stream);
 
 /* Sort by radius (section 2.1 step 6): perm[j] = input index of the star
- * that goes to slot j, order (r, id) with r = +inf last by id.  This is the
- * timestep's sort: a stable radix sort by r followed by ordering equal
- * radii by id. */
+ * that goes to slot j, order (r, id) with r = +inf last by id: a stable radix
+ * sort by r's upper 40 bits, then radii equal in those by (r, id).  (States set
+ * in no order and timesteps with sort_packed = 0 sort by radix too; other
+ * timesteps by counting, to the same order.) */
 cmc_status cmc_sort_radius(int64_t n, const double *r, const uint32_t *id, uint32_t *perm,
                            void *stream);
 
@@ -442,7 +449,8 @@ double cmc_tse(double M, double T_prev, double dm_se);
 /* Limits of the sort's bounded device waits on the current device, for all
  * contexts and stage calls there (read by the kernels at launch, so graphs
  * captured earlier follow them): lookback_polls = polls of an earlier
- * tile's look-back word before a tile gives up on it (the step then
+ * tile's look-back word, or of the count of tiles done in the merge of a long
+ * run of one shell, before a tile gives up on it (the step then
  * returns CMC_ETIMEOUT and the context is poisoned; cmc_sort_radius
  * returns CMC_ETIMEOUT); tie_moves = moves of the insertion sort that puts a
  * run of equal sort keys in id order before it gives up on the run (a step

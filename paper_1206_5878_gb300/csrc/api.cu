@@ -444,10 +444,6 @@ cmc_status load_state(cmc_ctx* c, const double* r, const double* vr, const doubl
   return CMC_OK;
 }
 
-// Time the shapes of the sort passes and of the orbit kernel on this state
-// and keep the fastest.  The orbit kernel runs once as a dry run (it writes
-// only keys and payload scratch) to give the sort realistic input; counters
-// it touched are reset.  Results never depend on the shapes.
 // ------------------------------------------------ Tausworthe streams (host)
 // Components (k, q, s) of the combined generator (section 3.6; L'Ecuyer
 // 1999) and one step of a component word; every step is linear over GF(2).
@@ -571,6 +567,10 @@ cmc_status check_stream_ids(cmc_ctx* c, const double* r, const uint32_t* id, int
   return CMC_OK;
 }
 
+// Time the shapes of the orbit and relaxation kernels, and of the radix passes
+// where the timestep uses them, on this state and keep the fastest.  The orbit
+// kernels run dry (they write only records, keys and scratch); the velocities are
+// copies; counters touched are reset.  Results never depend on the shapes.
 cmc_status autotune(cmc_ctx* c) {
   const SegLayout& L = c->L;
   cudaStream_t st = c->stream;
@@ -1304,8 +1304,8 @@ cmc_status cmc_sort_radius(int64_t n, const double* r, const uint32_t* id, uint3
   uint64_t* keys = nullptr;
   uint32_t* err = nullptr;
   cudaError_t e = alloc_sort(W, S.L, 8, st);
-  // ballots: 301 us a call against 310 with matches at 10^6 stars, 966 against 1014
-  // at 8 x 10^6 (8 keys a thread 330, 1032)
+  // (ballots, 16 keys a thread: calls one after the other on 10^6 and 8 x 10^6 stars in
+  // no order 204, 719 us; with matches 215, 782, with 8 keys 233, 964)
   W.rank = 1;
   uint32_t he = 0;
   void* block = nullptr;
@@ -1316,8 +1316,7 @@ cmc_status cmc_sort_radius(int64_t n, const double* r, const uint32_t* id, uint3
   if (!e) {
     sort_prepare();
     launch_make_keys(S.L, r, id, keys, st);
-    // as in the timestep: passes over bits 24-63, then runs equal in those
-    // bits in (r, id) order
+    // passes over bits 24-63, then runs equal in those bits in (r, id) order
     sort_segments(S.L, W, keys, perm, 3, 5, true, err, st);
     launch_tiefix(S.L, keys, perm, id, 1, err, st, 24);
     e = cudaMemcpyAsync(&he, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);

@@ -27,7 +27,7 @@ constexpr uint32_t kTagSgn = 3;      // orbit: sign of the new v_r
 constexpr uint32_t kTagCol = 4;      // relaxation pair: sticky-sphere collision draw
 
 // escaped stars sort after every finite radius, by id: key 0x7FF0...0 | id
-// << 20, above every finite radius (the timestep's sort orders by the top
+// << 20, above every finite radius (the radix sort orders by the top
 // 40 bits and puts runs equal in them -- escapers whose ids differ only in
 // their low 4 bits -- in (key, id) order, which for these keys is id order)
 constexpr uint64_t kEscKeyBase = 0x7FF0000000000000ull;

@@ -988,7 +988,7 @@ __global__ void __launch_bounds__(kPotThreads, 3) k_potential(
       // the slope of Eq. 6 in 1/r across shell k, (Phi_{k+1} - Phi_k) / (x_k -
       // x_{k+1}) with Phi = 0 at 1/r = 0 beyond the last bound star (the FP64
       // orbit step's shell parameter); a tile's last star, whose neighbour is
-      // in the next tile, gets its slope from k_grid_build
+      // in the next tile, gets its slope from grid_build
       double w = 0.0;
       if (bound && (p + 1 >= R.bound_end || e + 1 < kTile)) {
         const bool last = p + 1 >= R.bound_end;

@@ -27,6 +27,7 @@ def _same(g, d, seeds, sizes=None, steps=3, **cfg):
             np.testing.assert_array_equal(sa[k], sb[k], err_msg=k)
     np.testing.assert_array_equal(a.nbound(), b.nbound())
     np.testing.assert_array_equal(a.escaped(), b.escaped())
+    assert a.stats() == b.stats()
     return sa
 
 
