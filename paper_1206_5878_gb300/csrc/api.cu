@@ -551,16 +551,17 @@ cmc_status init_streams(cmc_ctx* c, const uint64_t* seeds) {
 // largest id at cmc_init): asked before anything of the state is replaced.
 cmc_status check_stream_ids(cmc_ctx* c, const double* r, const uint32_t* id, int32_t ptr_kind) {
   const SegLayout& L = c->L;
-  std::vector<unsigned int> max_id((size_t)L.n_seg, 0u);
-  if (ptr_kind == 0) {
-    for (int s = 0; s < L.n_seg; ++s)
-      for (int64_t p = L.h_off[s]; p < L.h_off[s + 1]; ++p)
-        if (id[p] > max_id[s]) max_id[s] = id[p];
-  } else {
-    bool ordered = false;
-    const cudaError_t e = check_order(L, r, id, c->stream, ordered, max_id);
-    if (e) return cuda_fail(c, e, "cmc_set_state: streams");
+  std::vector<unsigned int> max_id;
+  bool ordered = false;
+  cudaError_t e = cudaSuccess;
+  if (ptr_kind == 0) {  // (host ids by way of scratch; r only says whether they are in order)
+    e = cudaMemcpyAsync(c->vals, id, sizeof(uint32_t) * (size_t)L.n, cudaMemcpyHostToDevice,
+                        c->stream);
+    r = c->r;
+    id = c->vals;
   }
+  if (!e) e = check_order(L, r, id, c->stream, ordered, max_id);
+  if (e) return cuda_fail(c, e, "cmc_set_state: streams");
   for (int s = 0; s < L.n_seg; ++s)
     if (max_id[s] > c->taus_max_id[s])
       return fail(c, CMC_EINVAL, "cmc_set_state: an id above those that have a Tausworthe stream");

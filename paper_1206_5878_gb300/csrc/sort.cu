@@ -373,8 +373,9 @@ __global__ void k_tiefix(const int64_t* off, int n_seg, int64_t n, uint64_t* key
 // into their low bits, histograms, tie fix).
 // Stars crowding into few bins: a warp in which a thread finds all its four in one
 // adds to each bin with its lanes together (atomics on one address go at 2.4 a
-// nanosecond: 10^6 stars in two bins counted in 424 us, 28 so).  (Two neighbours in one bin are common
-// enough among few stars to make the sort of 1021 slower, 11.3 us against 10.0.)
+// nanosecond: 10^6 stars in two bins counted in 424 us, 28 so).  Two neighbours in
+// one bin are common enough among few stars that the sort of 1021 would take 11.3
+// us instead of 10.0.
 __device__ __forceinline__ bool crowded(const uint4& b) {
   return __any_sync(__activemask(), b.x == b.y && b.y == b.z && b.z == b.w);
 }
