@@ -764,7 +764,9 @@ __global__ void __launch_bounds__(kThreads) k_long_runs(int64_t n, uint32_t* ctl
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    S.ok = atomicAdd(ctl + kCtlLeft, 1u) == gridDim.x - 1u && (*(volatile uint32_t*)err & kErrTimeout);
+    S.ok = atomicAdd(ctl + kCtlLeft, 1u) == gridDim.x - 1u &&
+           (*(volatile uint32_t*)err & kErrTimeout);
+    __threadfence();
   }
   __syncthreads();
   if (S.ok)
